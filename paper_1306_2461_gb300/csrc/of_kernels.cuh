@@ -5,6 +5,7 @@
 #include <float.h>
 
 #include <climits>
+#include <type_traits>
 
 #include "async_copy.cuh"
 #include "of_internal.cuh"
@@ -366,18 +367,68 @@ __device__ __forceinline__ float bil_at(const T *I, int pitch, int H, int W, int
     return bil<NC>(I, pitch, H, W, pos_floor_clamped(x, fu), u - fu, pos_floor_clamped(y, fv), v - fv);
 }
 
-// sample_grad by five clamped bilinear samples. Where no sample is clamped these are the
-// interior branch's interpolations in the same order, so the two agree bit for bit.
+// sample_grad near the image border: each of the five bilinear samples at p, p +- (1, 0),
+// p +- (0, 1) is clamped to the image on its own. Together they read the 12 taps of the
+// interior form at clamped columns and rows, and a sample whose position leaves the image
+// takes fraction 0 along that axis (its clamped end pixel exactly): three fractions per
+// axis, one each for the samples at -1, 0 and +1. Where no sample is clamped the fractions
+// are equal and this is the interior form bit for bit. ld(col, row) reads one tap.
+// What bounds it is instructions: with 20 taps in 5 separate clamped samples per pixel a
+// 64 x 24 border tile took 16-23k cycles alone on an SM against 12.7k for an interior one,
+// which set the time of every launch of a few tiles (1024^2 pair 233 -> 200 us, 64 pairs
+// of 1024^2 6020 -> 5250 us with this form, the choice of form per warp and the region
+// check per tile, see stage1_pair).
+template <typename LD>
+__device__ __forceinline__ void sample_grad_taps(LD ld, int H, int W, int bx, int by, float ax, float ay, float &Iw,
+                                                 float &gx, float &gy)
+{
+    const float axm = (unsigned)(bx - 1) < (unsigned)(W - 1) ? ax : 0.0f;
+    const float axc = (unsigned)bx < (unsigned)(W - 1) ? ax : 0.0f;
+    const float axp = (unsigned)(bx + 1) < (unsigned)(W - 1) ? ax : 0.0f;
+    const float aym = (unsigned)(by - 1) < (unsigned)(H - 1) ? ay : 0.0f;
+    const float ayc = (unsigned)by < (unsigned)(H - 1) ? ay : 0.0f;
+    const float ayp = (unsigned)(by + 1) < (unsigned)(H - 1) ? ay : 0.0f;
+    const int cm = clampi(bx - 1, 0, W - 1), c0 = clampi(bx, 0, W - 1);
+    const int c1 = clampi(bx + 1, 0, W - 1), c2 = clampi(bx + 2, 0, W - 1);
+    const int rm = clampi(by - 1, 0, H - 1), r0 = clampi(by, 0, H - 1);
+    const int r1 = clampi(by + 1, 0, H - 1), r2 = clampi(by + 2, 0, H - 1);
+    const float a0 = ld(c0, rm), a1 = ld(c1, rm);
+    const float bm = ld(cm, r0), b0 = ld(c0, r0), b1 = ld(c1, r0), b2 = ld(c2, r0);
+    const float dm = ld(cm, r1), d0 = ld(c0, r1), d1 = ld(c1, r1), d2 = ld(c2, r1);
+    const float e0 = ld(c0, r2), e1 = ld(c1, r2);
+    const float top = lerpf(b0, b1, axc), bot = lerpf(d0, d1, axc);
+    Iw = lerpf(top, bot, ayc);
+    gx = __fmul_rn(__fsub_rn(lerpf(lerpf(b1, b2, axp), lerpf(d1, d2, axp), ayc),
+                             lerpf(lerpf(bm, b0, axm), lerpf(dm, d0, axm), ayc)), 0.5f);
+    gy = __fmul_rn(__fsub_rn(lerpf(bot, lerpf(e0, e1, axc), ayp), lerpf(lerpf(a0, a1, axc), top, aym)), 0.5f);
+}
+
+// The same from the image in global memory.
 template <bool NC, typename T>
 __device__ __forceinline__ void sample_grad_clamped(const T *I, int pitch, int H, int W, int x, int y, float u,
                                                     float v, float &Iw, float &gx, float &gy)
 {
     const float fu = floorf(u), fv = floorf(v);
-    const float ax = u - fu, ay = v - fv;
+    sample_grad_taps([=](int c, int r) { return ldf<NC>(I + (r * pitch + c)); }, H, W, pos_floor_clamped(x, fu),
+                     pos_floor_clamped(y, fv), u - fu, v - fv, Iw, gx, gy);
+}
+
+// The same from the staged window `win` (WW x WH elements, first at image (wx0, wy0)) when
+// all clamped taps lie in it, else from global memory.
+template <bool NC, int WW, int WH, typename T>
+__device__ __forceinline__ void sample_grad_clamped_win(const T *I, int pitch, int H, int W, const T *win, int wx0,
+                                                        int wy0, int x, int y, float u, float v, float &Iw,
+                                                        float &gx, float &gy)
+{
+    const float fu = floorf(u), fv = floorf(v);
     const int bx = pos_floor_clamped(x, fu), by = pos_floor_clamped(y, fv);
-    Iw = bil<NC>(I, pitch, H, W, bx, ax, by, ay);
-    gx = (bil<NC>(I, pitch, H, W, bx + 1, ax, by, ay) - bil<NC>(I, pitch, H, W, bx - 1, ax, by, ay)) * 0.5f;
-    gy = (bil<NC>(I, pitch, H, W, bx, ax, by + 1, ay) - bil<NC>(I, pitch, H, W, bx, ax, by - 1, ay)) * 0.5f;
+    if (win && clampi(bx - 1, 0, W - 1) >= wx0 && clampi(bx + 2, 0, W - 1) < wx0 + WW &&
+        clampi(by - 1, 0, H - 1) >= wy0 && clampi(by + 2, 0, H - 1) < wy0 + WH)
+        sample_grad_taps([=](int c, int r) { return ldf<false>(win + ((r - wy0) * WW + (c - wx0))); }, H, W, bx, by,
+                         u - fu, v - fv, Iw, gx, gy);
+    else
+        sample_grad_taps([=](int c, int r) { return ldf<NC>(I + (r * pitch + c)); }, H, W, bx, by, u - fu, v - fv, Iw,
+                         gx, gy);
 }
 
 // I2 at p = (x + u, y + v) and its gradient at p: central difference of the bilinear
@@ -1054,20 +1105,23 @@ __device__ __forceinline__ void box_v_planes(const float2 *P01, const float2 *P2
 // Stage 1 of the fixed-radius tile for the pixel pair (x, y), (x + 1, y): warp I2 by the
 // current estimate, its gradient there, e~ and the five products, on both pixels at
 // once when both sample the interior (taps from the staged window or global memory),
-// pixel by pixel near the border or at the image's last column. sflow: the pair's staged
-// estimates (NULL: read them from fin). Out-of-image pixels get zero products. Returns the
-// products in the planes' layout.
-template <typename T, bool NC, int MODE, int WW>
+// pixel by pixel near the border or at the image's last column. The form is chosen per
+// warp (all of its pairs take the border form if one has to: it gives the same bits, and
+// running both forms one after the other costs more). INNER: the tile's whole region and
+// its staged window lie inside the image, so that no pair needs a bounds check and a
+// footprint inside the window is inside the image. sflow: the pair's staged estimates
+// (NULL: read them from fin). Out-of-image pixels get zero products. Returns the products
+// in the planes' layout.
+template <typename T, bool NC, int MODE, int WW, int WH, bool INNER>
 __device__ __forceinline__ void stage1_pair(const IterArgs &a, int x, int y, float2 ref, const float4 *sflow,
-                                            const T *win, bool win_in_image, int wx0, int wy0, int WH, float4 &s01,
-                                            float4 &s23, float2 &s4)
+                                            const T *win, int wx0, int wy0, float4 &s01, float4 &s23, float2 &s4)
 {
     s01 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     s23 = s01;
     s4 = f2(0.0f, 0.0f);
-    const bool rowin = (unsigned)y < (unsigned)a.H;
-    const bool inp = rowin && (unsigned)x < (unsigned)a.W;
-    const bool inq = rowin && (unsigned)(x + 1) < (unsigned)a.W;   // implies inp (x even)
+    const bool rowin = INNER || (unsigned)y < (unsigned)a.H;
+    const bool inp = rowin && (INNER || (unsigned)x < (unsigned)a.W);
+    const bool inq = rowin && (INNER || (unsigned)(x + 1) < (unsigned)a.W);   // implies inp (x even)
     if (!inp) return;
     const T *I1 = static_cast<const T *>(a.I1);
     const T *I2 = static_cast<const T *>(a.I2);
@@ -1083,24 +1137,27 @@ __device__ __forceinline__ void stage1_pair(const IterArgs &a, int x, int y, flo
     float2 IW, GX, GY;
     // The positions' integer parts and fractions (exact; pos_floor). Both pixels sample
     // the interior (their 4x4 footprints inside the image) and, with a staged window, the
-    // footprints' corners (x0 - 1, y0 - 1) inside it. When the whole window lies inside
-    // the image, a footprint inside the window is inside the image, which is the interior
-    // condition, so only the window is tested.
+    // footprints' corners (x0 - 1, y0 - 1) inside it.
     const float2 FU = f2(floorf(fp.x), floorf(fq.x)), FV = f2(floorf(fp.y), floorf(fq.y));
     const float2 AX = sub2(f2(fp.x, fq.x), FU), AY = sub2(f2(fp.y, fq.y), FV);
     const int xp = pos_floor(x, FU.x), yp = pos_floor(y, FV.x);
     const int xq = pos_floor(x + 1, FU.y), yq = pos_floor(y, FV.y);
     const int cpx = (int)((unsigned)xp - 1u - (unsigned)wx0), cpy = (int)((unsigned)yp - 1u - (unsigned)wy0);
     const int cqx = (int)((unsigned)xq - 1u - (unsigned)wx0), cqy = (int)((unsigned)yq - 1u - (unsigned)wy0);
-    const bool inwin = win && (unsigned)cpx < (unsigned)(WW - 3) && (unsigned)cqx < (unsigned)(WW - 3) &&
+    const bool inwin = (INNER || win) && (unsigned)cpx < (unsigned)(WW - 3) && (unsigned)cqx < (unsigned)(WW - 3) &&
                        (unsigned)cpy < (unsigned)(WH - 3) && (unsigned)cqy < (unsigned)(WH - 3);
-    const unsigned ws = interior_span(a.W), hs = interior_span(a.H);
-    if (inq && (win_in_image ? inwin : (interior(xp, yp, ws, hs) && interior(xq, yq, ws, hs)))) {
-        sample_grad2<NC, WW>(I2, a.pitch, win, inwin, cpx, cpy, cqx, cqy, xp, yp, xq, yq, AX, AY, IW, GX, GY);
+    bool both = inwin;
+    if constexpr (!INNER) {
+        const unsigned ws = interior_span(a.W), hs = interior_span(a.H);
+        both = __all_sync(__activemask(), inq && interior(xp, yp, ws, hs) && interior(xq, yq, ws, hs));
+    }
+    if (both) {
+        sample_grad2<NC, WW>(I2, a.pitch, win, INNER || inwin, cpx, cpy, cqx, cqy, xp, yp, xq, yq, AX, AY, IW, GX, GY);
     } else {
         float iw0, gx0, gy0, iw1 = 0.0f, gx1 = 0.0f, gy1 = 0.0f;
-        sample_grad_clamped<NC>(I2, a.pitch, a.H, a.W, x, y, fp.x, fp.y, iw0, gx0, gy0);
-        if (inq) sample_grad_clamped<NC>(I2, a.pitch, a.H, a.W, x + 1, y, fq.x, fq.y, iw1, gx1, gy1);
+        const T *w = INNER ? nullptr : win;   // INNER comes here only with taps outside the window
+        sample_grad_clamped_win<NC, WW, WH>(I2, a.pitch, a.H, a.W, w, wx0, wy0, x, y, fp.x, fp.y, iw0, gx0, gy0);
+        if (inq) sample_grad_clamped_win<NC, WW, WH>(I2, a.pitch, a.H, a.W, w, wx0, wy0, x + 1, y, fq.x, fq.y, iw1, gx1, gy1);
         IW = f2(iw0, iw1);
         GX = f2(gx0, gx1);
         GY = f2(gy0, gy1);
@@ -1257,46 +1314,53 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
     // stage 1: products over region rows r0..RH-1 (the tile and its halo), by pixel pairs
     constexpr int NPR = F::RWE / 2;   // pairs per region row
     const T *wt = staged ? reinterpret_cast<const T *>(win) : nullptr;
-    const bool win_in_image = staged && wx0 >= 0 && wy0 >= 0 && wx0 + WW <= a.W && wy0 + F::WIN_H <= a.H;
-    auto pair = [&](int ry, int cx) {
+    auto pair = [&](auto inner, int ry, int cx) {
         const int k2 = ry * (F::RWP2 / 2) + cx;   // float4 slot of the pair in the pair planes
         float4 s01, s23;
         float2 s4;
-        stage1_pair<T, NC, MODE, WW>(a, tx0 - F::RE + 2 * cx, ty0 - R + ry, ref,
-                                     ry < brow_end ? reinterpret_cast<const float4 *>(P01) + k2 : nullptr, wt,
-                                     win_in_image, wx0, wy0, F::WIN_H, s01, s23, s4);
+        stage1_pair<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(
+            a, tx0 - F::RE + 2 * cx, ty0 - R + ry, ref,
+            ry < brow_end ? reinterpret_cast<const float4 *>(P01) + k2 : nullptr, wt, wx0, wy0, s01, s23, s4);
         reinterpret_cast<float4 *>(P01)[k2] = s01;
         reinterpret_cast<float4 *>(P23)[k2] = s23;
         reinterpret_cast<float2 *>(P4)[ry * (F::RWP1 / 2) + cx] = s4;
     };
-    if constexpr (CM == 2) {
-        // strips: thread t takes pixel pair cx = t mod NPR of rows r0 + t / NPR, then RPI
-        // rows further each round, so that what depends on the pair's column is the same on
-        // every row it takes (5% fewer instructions per pixel-iteration at r = 4)
-        constexpr int RPI = LK_THREADS / NPR;   // rows per round
-        const int cx = threadIdx.x % NPR, rs = threadIdx.x / NPR;
-        if (rs < RPI) {
+    auto rows = [&](auto inner) {
+        if constexpr (CM == 2) {
+            // strips: thread t takes pixel pair cx = t mod NPR of rows r0 + t / NPR, then RPI
+            // rows further each round, so that what depends on the pair's column is the same on
+            // every row it takes (5% fewer instructions per pixel-iteration at r = 4)
+            constexpr int RPI = LK_THREADS / NPR;   // rows per round
+            const int cx = threadIdx.x % NPR, rs = threadIdx.x / NPR;
+            if (rs < RPI) {
 #pragma unroll 1
-            for (int ry = r0 + rs; ry < F::RH; ry += RPI) pair(ry, cx);
-        }
-    } else {
-        // single tiles: pair j = threadIdx.x + k LK_THREADS is (row ry, pair cx) of the rows
-        // computed, stepped without a division (LK_THREADS = DY rows + DX pairs); it
-        // compiles without spills where the form above does not
-        constexpr int DY = LK_THREADS / NPR, DX = LK_THREADS % NPR;
-        const int npair = (F::RH - r0) * NPR;
-        int ry = r0 + threadIdx.x / NPR, cx = threadIdx.x % NPR;
+                for (int ry = r0 + rs; ry < F::RH; ry += RPI) pair(inner, ry, cx);
+            }
+        } else {
+            // single tiles: pair j = threadIdx.x + k LK_THREADS is (row ry, pair cx) of the rows
+            // computed, stepped without a division (LK_THREADS = DY rows + DX pairs); it
+            // compiles without spills where the form above does not
+            constexpr int DY = LK_THREADS / NPR, DX = LK_THREADS % NPR;
+            const int npair = (F::RH - r0) * NPR;
+            int ry = r0 + threadIdx.x / NPR, cx = threadIdx.x % NPR;
 #pragma unroll 1
-        for (int j = threadIdx.x; j < npair; j += LK_THREADS) {
-            pair(ry, cx);
-            ry += DY;
-            cx += DX;
-            if (cx >= NPR) {
-                cx -= NPR;
-                ++ry;
+            for (int j = threadIdx.x; j < npair; j += LK_THREADS) {
+                pair(inner, ry, cx);
+                ry += DY;
+                cx += DX;
+                if (cx >= NPR) {
+                    cx -= NPR;
+                    ++ry;
+                }
             }
         }
-    }
+    };
+    // the staged window and the region both inside the image: no pair needs a bounds check
+    if (staged && wx0 >= 0 && wy0 >= 0 && wx0 + WW <= a.W && wy0 + F::WIN_H <= a.H && tx0 >= F::RE && ty0 >= R &&
+        tx0 + LK_TW + F::RE <= a.W && ty0 + TH + R <= a.H)
+        rows(std::true_type());
+    else
+        rows(std::false_type());
     __syncthreads();
     if constexpr (CM == 2 && OF_EARLY_WINDOW) {
         // the window is free: request the next tile's, which lands while this tile
@@ -1433,8 +1497,8 @@ __device__ __forceinline__ void lk_tile_fused2(const IterArgs &a, int tile, floa
             const int k2 = ry * (A::RWP2 / 2) + cx;
             float4 s01, s23;
             float2 s4;
-            stage1_pair<T, NC, FLOW_SAME, 1>(a, ax0 - A::RE + 2 * cx, ay0 - R + ry, ref, nullptr, nullptr, false, 0,
-                                             0, 0, s01, s23, s4);
+            stage1_pair<T, NC, FLOW_SAME, 4, 4, false>(a, ax0 - A::RE + 2 * cx, ay0 - R + ry, ref, nullptr, nullptr, 0,
+                                                       0, s01, s23, s4);
             reinterpret_cast<float4 *>(Q01)[k2] = s01;
             reinterpret_cast<float4 *>(Q23)[k2] = s23;
             reinterpret_cast<float2 *>(Q4)[ry * (A::RWP1 / 2) + cx] = s4;
@@ -1488,9 +1552,9 @@ __device__ __forceinline__ void lk_tile_fused2(const IterArgs &a, int tile, floa
             const int k2 = ry * (B::RWP2 / 2) + cx;
             float4 s01, s23;
             float2 s4;
-            stage1_pair<T, NC, FLOW_SAME, 1>(a, tx0 - B::RE + 2 * cx, ty0 - R + ry, ref,
-                                             reinterpret_cast<const float4 *>(FB) + k2, nullptr, false, 0, 0, 0, s01,
-                                             s23, s4);
+            stage1_pair<T, NC, FLOW_SAME, 4, 4, false>(a, tx0 - B::RE + 2 * cx, ty0 - R + ry, ref,
+                                                       reinterpret_cast<const float4 *>(FB) + k2, nullptr, 0, 0, s01,
+                                                       s23, s4);
             reinterpret_cast<float4 *>(P01)[k2] = s01;
             reinterpret_cast<float4 *>(P23)[k2] = s23;
             reinterpret_cast<float2 *>(P4)[ry * (B::RWP1 / 2) + cx] = s4;

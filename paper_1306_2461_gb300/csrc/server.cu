@@ -84,6 +84,7 @@ struct of_server {
     std::condition_variable cv_work, cv_done;
     std::thread worker;
     bool stop = false;
+    bool forming = false;                          // the worker is queueing a tick (without the lock)
     int error = OF_OK;
     // statistics
     int64_t ticks = 0, pairs = 0;
@@ -124,20 +125,31 @@ void retire(of_server *s)
     }
 }
 
-// Take the next frame of every stream that has one into a new tick and launch it.
-int form_tick(of_server *s)
+// Take the next frame of every stream that has one into a new tick and launch it. The
+// frames are taken with the lock held; the copies and launches (a few microseconds each,
+// 17 launches per tick of the default method) are queued without it, so that frames
+// submitted meanwhile join the next tick instead of waiting for the lock. Only the worker
+// changes ticks, retires them and uses the handles; a stream with work in the tick being
+// formed is not closed (its last_tick is not retired).
+int form_tick(of_server *s, std::unique_lock<std::mutex> &lk)
 {
+    struct Copy {
+        void *dst;
+        const void *src;
+        size_t bytes;
+        cudaEvent_t after;   // the staging buffer's last reader, when still in flight
+    };
     const int slot = (int)(s->next_seq % s->cfg.max_inflight);
     Tick t;
     t.seq = s->next_seq;
     t.slot = slot;
     t.copied = s->ev_copied[slot];
     t.done = s->ev_done[slot];
+    std::vector<Copy> copies;
     std::vector<of_handle> hs;
     std::vector<const void *> I1s, I2s;
     std::vector<float *> us, vs;
     const size_t n = s->streams.size();
-    bool any = false;
     for (size_t k = 0; k < n && (int)hs.size() < s->cfg.max_batch; ++k) {
         Stream &st = s->streams[(s->rr + k) % n];
         if (!st.open || st.queue.empty()) continue;
@@ -146,12 +158,9 @@ int form_tick(of_server *s)
         --s->pending;
         const int b = (int)(st.frames % 2);
         // the staging buffer is free once the tick that last read it is done
-        if (st.last_reader[b] >= 0 && in_flight(s, st.last_reader[b])) {
-            cudaEvent_t e = done_event_of(s, st.last_reader[b]);
-            if (e && cudaStreamWaitEvent(s->copy, e, 0) != cudaSuccess) return OF_ECUDA;
-        }
-        if (cudaMemcpyAsync(st.raw[b], rq.frame, st.frame_bytes, cudaMemcpyHostToDevice, s->copy) != cudaSuccess)
-            return OF_ECUDA;
+        cudaEvent_t after = nullptr;
+        if (st.last_reader[b] >= 0 && in_flight(s, st.last_reader[b])) after = done_event_of(s, st.last_reader[b]);
+        copies.push_back(Copy{st.raw[b], rq.frame, st.frame_bytes, after});
         of_result r;
         memset(&r, 0, sizeof(r));
         r.stream = (int32_t)((s->rr + k) % n);
@@ -173,21 +182,31 @@ int form_tick(of_server *s)
         st.last_tick = t.seq;
         st.frames += 1;
         t.results.push_back(r);
-        any = true;
     }
-    if (!any) return OF_OK;
+    if (copies.empty()) return OF_OK;
     s->rr = (s->rr + 1) % (n ? n : 1);
-    if (cudaEventRecord(t.copied, s->copy) != cudaSuccess || cudaStreamWaitEvent(s->compute, t.copied, 0) != cudaSuccess)
-        return OF_ECUDA;
     for (auto &r : t.results) r.batch = (int32_t)hs.size();
-    if (!hs.empty()) {
-        const int rc = of::batch_run_slot(s->slots[slot], (int32_t)hs.size(), hs.data(), I1s.data(), I2s.data(),
-                                          us.data(), vs.data(), s->compute);
-        if (rc) return rc;
-        s->pairs += (int64_t)hs.size();
-    }
-    if (cudaEventRecord(t.done, s->compute) != cudaSuccess) return OF_ECUDA;
+    s->forming = true;
+    lk.unlock();
+    int rc = OF_OK;
+    for (const Copy &c : copies)
+        if ((c.after && cudaStreamWaitEvent(s->copy, c.after, 0) != cudaSuccess) ||
+            cudaMemcpyAsync(c.dst, c.src, c.bytes, cudaMemcpyHostToDevice, s->copy) != cudaSuccess) {
+            rc = OF_ECUDA;
+            break;
+        }
+    if (rc == OF_OK && (cudaEventRecord(t.copied, s->copy) != cudaSuccess ||
+                        cudaStreamWaitEvent(s->compute, t.copied, 0) != cudaSuccess))
+        rc = OF_ECUDA;
+    if (rc == OF_OK && !hs.empty())
+        rc = of::batch_run_slot(s->slots[slot], (int32_t)hs.size(), hs.data(), I1s.data(), I2s.data(), us.data(),
+                                vs.data(), s->compute);
+    if (rc == OF_OK && cudaEventRecord(t.done, s->compute) != cudaSuccess) rc = OF_ECUDA;
     t.launch_ns = now_ns();
+    lk.lock();
+    s->forming = false;
+    if (rc) return rc;
+    s->pairs += (int64_t)hs.size();
     s->inflight.push_back(std::move(t));
     ++s->next_seq;
     ++s->ticks;
@@ -201,8 +220,11 @@ void worker_main(of_server *s)
     while (!s->stop) {
         retire(s);
         if (s->pending > 0 && (int)s->inflight.size() < s->cfg.max_inflight && s->error == OF_OK) {
-            const int rc = form_tick(s);
-            if (rc) s->error = rc;
+            const int rc = form_tick(s, lk);
+            if (rc) {
+                s->error = rc;
+                s->cv_done.notify_all();
+            }
             continue;
         }
         if (!s->inflight.empty())
@@ -376,7 +398,7 @@ int of_server_drain(of_server_t s, int32_t timeout_ms)
     if (!s) return OF_EINVAL;
     std::unique_lock<std::mutex> lk(s->mu);
     const bool ok = s->cv_done.wait_for(lk, std::chrono::milliseconds(timeout_ms < 0 ? 0 : timeout_ms), [s] {
-        return (s->pending == 0 && s->inflight.empty()) || s->error;
+        return (s->pending == 0 && s->inflight.empty() && !s->forming) || s->error;
     });
     if (s->error) return s->error;
     return ok ? OF_OK : OF_ETIMEOUT;

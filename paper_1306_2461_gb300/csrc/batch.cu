@@ -349,14 +349,15 @@ static cudaError_t enqueue_chain(const BatchPair *pairs, int n, const of_plan &p
             I.npairs = m;
             I.ahead = prefetch_ahead;
             // strips as long as the tuning's while the launch keeps OF_STRIP_WAVES blocks per
-            // resident block slot (4 per SM) or more; the fields do not depend on the strip length
+            // resident block slot (4 per SM) or more; small tiles where there are few (of the
+            // default tile without a prefetch); the fields do not depend on either
             int kl = strip;
-            if (kl > 1) {
-                long tiles_l = 0;
-                for (int i = 0; i < m; ++i)
-                    tiles_l += strip_units(bp[i].H[l], bp[i].W[l], tile_h, 1);
-                while (kl > 1 && tiles_l < (long)kl * OF_STRIP_WAVES * 4 * sms) kl /= 2;
-            }
+            long tiles_l = 0;
+            for (int i = 0; i < m; ++i) tiles_l += strip_units(bp[i].H[l], bp[i].W[l], tile_h, 1);
+            while (kl > 1 && tiles_l < (long)kl * OF_STRIP_WAVES * 4 * sms) kl /= 2;
+            const bool small = !i1grad && !two && tile_h == LK_TH && !t.generic_sums && radius_specialised(p0.radius) &&
+                               prefetch_ahead == 0 && use_small_tiles(tiles_l, sms);
+            const int th_l = small ? SM_TH : tile_h;
             for (int i = 0; i < m; ++i) {
                 IterArgs &a = I.a[i];
                 a.I1 = bp[i].pyr[0] + bp[i].off[l];
@@ -390,14 +391,18 @@ static cudaError_t enqueue_chain(const BatchPair *pairs, int n, const of_plan &p
                 a.tiles = strip_units(a.H, a.W, th, a.strip);
                 a.status = bp[i].status;
                 a.stage_i2 = (i1grad || two) ? 0 : stage;   // the fused kernel gathers
-                if (a.stage_i2) fill_stage_maps(a, I.m[i], level_elem(p0, l), p0.radius, tile_h);   // else gathered
+                if (small) {
+                    a.tiles_x = small_tiles_x(a.W);
+                    a.tiles = small_units(a.H, a.W);
+                }
+                if (a.stage_i2) fill_stage_maps(a, I.m[i], level_elem(p0, l), p0.radius, th_l);   // else gathered
                 a.hess = bp[i].hess;
                 a.hess_pitch = bp[i].pitch[l];
                 I.prefix[i + 1] = I.prefix[i] + a.tiles;
             }
             e = i1grad ? launch_phase_i1_iter(I, level_elem(p0, l), p0.radius, t.generic_sums != 0, p0.fp64_cond, st)
                 : two  ? launch_phase_iter2(I, level_elem(p0, l), p0.radius, p0.fp64_cond, st)
-                       : launch_phase_iter(I, level_elem(p0, l), p0.radius, t.generic_sums != 0, p0.fp64_cond, tile_h,
+                       : launch_phase_iter(I, level_elem(p0, l), p0.radius, t.generic_sums != 0, p0.fp64_cond, th_l,
                                            st);
             if (e != cudaSuccess) return e;
             if (two) ++k;   // both iterations done

@@ -67,13 +67,13 @@ bool fill_stage_maps(IterArgs &a, StageMaps &m, int elem, int radius, int tile_h
 }
 
 #define OF_CASE_LK(R) \
-    case R: return lk_launch<R>(a, m, elem, radius, fp64_cond, s);
-cudaError_t launch_lk_iter(const IterArgs &a, const StageMaps &m, int elem, int radius, float fp64_cond,
+    case R: return lk_launch<R>(a, m, elem, radius, fp64_cond, small, s);
+cudaError_t launch_lk_iter(const IterArgs &a, const StageMaps &m, int elem, int radius, float fp64_cond, bool small,
                            cudaStream_t s)
 {
     switch (radius) {
         OF_RADII(OF_CASE_LK)
-    default: return lk_launch<0>(a, m, elem, radius, fp64_cond, s);
+    default: return lk_launch<0>(a, m, elem, radius, fp64_cond, false, s);
     }
 }
 

@@ -167,6 +167,8 @@ cudaError_t enqueue_pair(of_ctx *h, const void *I1, const void *I2, float *u, fl
     }
     // iterations
     const bool i1grad = (p.flags & OF_FLAG_I1GRAD) != 0;
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     int cur = 0;
     for (int l = p.levels - 1; l >= 0; --l) {
         if (i1grad) {
@@ -219,13 +221,19 @@ cudaError_t enqueue_pair(of_ctx *h, const void *I1, const void *I2, float *u, fl
             a.stage_i2 = !(p.flags & OF_FLAG_GATHER) && !i1grad ? 1 : 0;
             StageMaps maps;
             memset(&maps, 0, sizeof(maps));
-            if (a.stage_i2) fill_stage_maps(a, maps, level_elem(p, l), p.radius, LK_TH);   // else gathered
+            // few tiles: small ones, so that the launch is spread over the SMs
+            const bool small = !i1grad && radius_specialised(p.radius) && use_small_tiles(a.tiles, sms);
+            if (small) {
+                a.tiles_x = small_tiles_x(a.W);
+                a.tiles = small_units(a.H, a.W);
+            }
+            if (a.stage_i2) fill_stage_maps(a, maps, level_elem(p, l), p.radius, small ? SM_TH : LK_TH);   // else gathered
             if (i1grad) {
                 a.hess = h->hess;
                 a.hess_pitch = L.pitch[l];
                 e = launch_i1_iter(a, level_elem(p, l), p.radius, p.fp64_cond, st);
             } else {
-                e = launch_lk_iter(a, maps, level_elem(p, l), p.radius, p.fp64_cond, st);
+                e = launch_lk_iter(a, maps, level_elem(p, l), p.radius, p.fp64_cond, small, st);
             }
             if (e != cudaSuccess) return e;
             cur = 1 - cur;

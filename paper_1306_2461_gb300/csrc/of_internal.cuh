@@ -159,6 +159,18 @@ constexpr int LK_TW = 64;    // iteration output tile width
 #endif
 constexpr int LK_TH = OF_LK_TH;
 static_assert(LK_TH % 4 == 0, "the vertical box pass takes 4 rows at a time");
+// Small iteration tile, for launches whose 64 x LK_TH tiles are fewer than 4/3 of the SMs:
+// such a launch lasts as long as one tile alone on an SM, a serial chain of five rounds of
+// stage 1, two of the horizontal pass and six solves per thread, and leaves SMs idle. A
+// 32 x 12 tile has two rounds, one and two solves, and a quarter of the area. One same-level
+// iteration of one pair at r = 4 (us per launch in a graph, 64 x 24 -> 32 x 12 tiles): 128^2
+// 7.7 -> 4.5, 256^2 8.0 -> 5.0, 384^2 7.9 -> 6.0, 512^2 (176 tiles) 9.9 -> 8.7, 640^2 (270
+// tiles) 10.1 -> 11.1; four 256^2 pairs (176) 10.7 -> 9.3, two 512^2 (352) 13.3 -> 14.2: the
+// line lies between 176 and 270 tiles, beyond it the wider halo (400 pixel pairs computed for
+// 192 written) costs more than the shorter chain saves. Others measured: 64 x 12 5.8 at
+// 256^2, 32 x 6 5.3, 32 x 12 with 512 threads 4.6 (but 10.7 at 512^2).
+constexpr int SM_TW = 32, SM_TH = 12, SM_THREADS = 256, SM_MIN_BLOCKS = 4;
+inline bool use_small_tiles(long tiles, int sms) { return 3 * tiles < 4 * (long)sms; }
 // The other iteration tile height the tuning can choose for the phase launches (64 x ALT_TH).
 #ifndef OF_ALT_TH
 #define OF_ALT_TH 32
@@ -176,6 +188,10 @@ inline __host__ __device__ int strip_units(int H, int W, int tile_h, int strip)
     const int tx = (W + LK_TW - 1) / LK_TW, ty = (H + tile_h - 1) / tile_h, k = strip_len(strip);
     return tx * ((ty + k - 1) / k);
 }
+
+// Small tiles of one level.
+inline int small_tiles_x(int W) { return (W + SM_TW - 1) / SM_TW; }
+inline int small_units(int H, int W) { return small_tiles_x(W) * ((H + SM_TH - 1) / SM_TH); }
 
 // Output tile height of the first-image-gradient variant's kernels (two product planes,
 // so a taller tile still leaves room for many blocks per SM).
@@ -213,7 +229,7 @@ inline bool radius_specialised(int r)
 cudaError_t launch_pyr_first(const PyrArgs &a, int in_format, int storage, cudaStream_t s);
 cudaError_t launch_pyr_down(const PyrArgs &a, int storage, cudaStream_t s);
 cudaError_t launch_znssd(const ZnArgs &a, int in_format, int storage, cudaStream_t s);
-cudaError_t launch_lk_iter(const IterArgs &a, const StageMaps &m, int elem, int radius, float fp64_cond,
+cudaError_t launch_lk_iter(const IterArgs &a, const StageMaps &m, int elem, int radius, float fp64_cond, bool small,
                            cudaStream_t s);
 cudaError_t launch_window_sums(const float *ch, int H, int W, int r, float *out, cudaStream_t s);
 // The variant linearised with the first image's gradient: window matrix of one level,
@@ -223,6 +239,7 @@ cudaError_t launch_i1_iter(const IterArgs &a, int elem, int radius, float fp64_c
 // Phase launches of the batched method (grid = P.prefix[P.npairs] blocks).
 cudaError_t launch_phase_pyr(const PyrPhase &P, bool first, int in_format, int storage, cudaStream_t s);
 cudaError_t launch_phase_zn(const ZnPhase &P, int in_format, int storage, cudaStream_t s);
+// (tile_h SM_TH: small tiles)
 cudaError_t launch_phase_iter(const IterPhase &P, int elem, int radius, bool generic, float fp64_cond, int tile_h,
                               cudaStream_t s);
 // Two same-level FLOW_SAME iterations in one launch per tile (fixed radii, tile height
@@ -255,7 +272,8 @@ constexpr int ET_FLOW2 = 100;
 
 // Per-radius instantiations (radius_<R>.cu; R = 0 is the generic kernel).
 template <int R>
-cudaError_t lk_launch(const IterArgs &a, const StageMaps &m, int elem, int r, float fp64_cond, cudaStream_t s);
+cudaError_t lk_launch(const IterArgs &a, const StageMaps &m, int elem, int r, float fp64_cond, bool small,
+                      cudaStream_t s);
 template <int R> cudaError_t ws_launch(const float *ch, int H, int W, int r, float *out, cudaStream_t s);
 template <int R> cudaError_t i1h_launch(const HessArgs &a, int elem, int r, cudaStream_t s);
 template <int R> cudaError_t phase_launch(const IterPhase &P, int elem, int r, float fp64_cond, int tile_h, cudaStream_t s);

@@ -689,8 +689,9 @@ template <int R, int TH = LK_TH, int TW = LK_TW> struct FixedTile {
     // first tile, TH / 2R for the others), else one box of TH rows at row 2R; elsewhere one
     // box of TH rows at row 0 for a strip's first tile, the other rows' estimates read from
     // global memory.
+    // Tiles narrower than LK_TW are never part of a strip: one box of the whole region.
     static constexpr bool FLOW_BOX_BELOW = (2 * R * RWP2 * 8) % 128 == 0;
-    static constexpr int FLOW_BH = FLOW_BOX_BELOW && TH % (2 * R) == 0 ? 2 * R : TH;
+    static constexpr int FLOW_BH = TW < 64 ? RH : (FLOW_BOX_BELOW && TH % (2 * R) == 0 ? 2 * R : TH);
     static constexpr int FLOW_BOX_BYTES = RWP2 * FLOW_BH * 8;
 #ifndef OF_LK_MIN_BLOCKS
 #define OF_LK_MIN_BLOCKS 4   // resident blocks per SM the fixed-radius kernels are compiled for (R <= 6)
@@ -940,26 +941,28 @@ __device__ __forceinline__ void box4v(const V *v, V o[4])
 
 // Horizontal pass of one pair plane, in place, over rows r0..RH-1: row ry becomes, at
 // columns 0..TW-1, the window sums of its outputs (two channels per float2). Chunk c of
-// rows goes to warp (c + woff) mod WARPS. For 64-wide tiles a warp takes
-// two rows and a quarter warp 4 groups of 4 outputs of each (with rows RWP2 = 2 mod 4
+// rows goes to warp (c + woff) mod WARPS. For 64- and 32-wide tiles a warp takes two or
+// four rows and a quarter warp 4 groups of 4 outputs of two of them (with rows RWP2 = 2 mod 4
 // float2 long, its 16-byte reads hit distinct banks); other widths take one row per warp,
 // one group per lane. Each row is read and rewritten by one warp.
-template <int R, int TH, int TW = LK_TW>
+template <int R, int TH, int TW = LK_TW, int NT = LK_THREADS>
 __device__ __forceinline__ void box_h_pairs(float2 *P, int r0 = 0, int woff = 0)
 {
     using F = FixedTile<R, TH, TW>;
-    static_assert(LK_THREADS % 32 == 0, "whole warps");
-    constexpr int WARPS = LK_THREADS / 32;
+    static_assert(NT % 32 == 0, "whole warps");
+    constexpr int WARPS = NT / 32;
     constexpr int RW4 = F::RWP2 / 2;   // float4 per row
     const int lane = threadIdx.x & 31;
-    constexpr bool TWO = TW == 64;
     constexpr int NG = TW / 4;
-    const int rsub = TWO ? (lane >> 2) & 1 : 0, g = TWO ? (((lane >> 3) << 2) | (lane & 3)) : lane;
-    const int rows = TWO ? (F::RH - r0) / 2 : F::RH - r0;   // warp-sized chunks (r0, RH - r0 even)
+    constexpr int RPC = TW == 64 ? 2 : (TW == 32 ? 4 : 1);   // rows per warp-sized chunk (r0, RH - r0 even)
+    const int rsub = RPC == 1 ? 0 : ((lane >> 2) & 1) | (RPC == 4 ? (lane >> 4) << 1 : 0);
+    const int g = RPC == 1 ? lane : (lane & 3) | ((lane >> 3) << 2 & (NG - 1));
+    const int chunks = (F::RH - r0 + RPC - 1) / RPC;
 #pragma unroll 1
-    for (int chunk = ((threadIdx.x >> 5) + WARPS - woff) % WARPS; chunk < rows; chunk += WARPS) {
-        const bool act = TWO || g < NG;
-        float4 *row = reinterpret_cast<float4 *>(P) + ((r0 + (TWO ? 2 * chunk + rsub : chunk)) * RW4 + 2 * g);
+    for (int chunk = ((threadIdx.x >> 5) + WARPS - woff) % WARPS; chunk < chunks; chunk += WARPS) {
+        const int ry = r0 + RPC * chunk + rsub;
+        const bool act = (RPC != 1 || g < NG) && (RPC != 4 || ry < F::RH);
+        float4 *row = reinterpret_cast<float4 *>(P) + (ry * RW4 + 2 * g);
         float2 o[4];
         if (act) {
             float2 v[4 * F::NVE];
@@ -979,20 +982,20 @@ __device__ __forceinline__ void box_h_pairs(float2 *P, int r0 = 0, int woff = 0)
     }
 }
 
-// Horizontal pass of the float plane P4, in place, over rows r0..RH-1: for 64-wide tiles
-// the 16 items of a row in 16 lanes, else one row per warp.
-template <int R, int TH, int TW = LK_TW>
+// Horizontal pass of the float plane P4, in place, over rows r0..RH-1: for 64- and 32-wide
+// tiles the items of a row lie in one warp, else one row per warp.
+template <int R, int TH, int TW = LK_TW, int NT = LK_THREADS>
 __device__ __forceinline__ void box_h_single(float *P, int r0 = 0)
 {
     using F = FixedTile<R, TH, TW>;
     constexpr int NG = TW / 4;
-    if constexpr (TW == LK_TW && NG == 16) {
-        constexpr int IT = (F::RH * NG + LK_THREADS - 1) / LK_THREADS;
+    if constexpr (TW == 64 || TW == 32) {
+        constexpr int IT = (F::RH * NG + NT - 1) / NT;
         const int nitems = (F::RH - r0) * NG;
         float4 res[IT];
 #pragma unroll
         for (int k = 0; k < IT; ++k) {
-            const int i = threadIdx.x + k * LK_THREADS;
+            const int i = threadIdx.x + k * NT;
             if (i < nitems) {
                 const int ry = r0 + i / NG, g = i % NG;
                 const float4 *src = reinterpret_cast<const float4 *>(P + ry * F::RWP1 + 4 * g);
@@ -1013,14 +1016,14 @@ __device__ __forceinline__ void box_h_single(float *P, int r0 = 0)
         __syncwarp();
 #pragma unroll
         for (int k = 0; k < IT; ++k) {
-            const int i = threadIdx.x + k * LK_THREADS;
+            const int i = threadIdx.x + k * NT;
             if (i < nitems) {
                 const int ry = r0 + i / NG, g = i % NG;
                 *reinterpret_cast<float4 *>(P + ry * F::RWP1 + 4 * g) = res[k];
             }
         }
     } else {
-        constexpr int WARPS = LK_THREADS / 32;
+        constexpr int WARPS = NT / 32;
         const int g = threadIdx.x & 31;
 #pragma unroll 1
         for (int ry = r0 + (threadIdx.x >> 5); ry < F::RH; ry += WARPS) {
@@ -1102,6 +1105,69 @@ __device__ __forceinline__ void box_v_planes(const float2 *P01, const float2 *P2
     }
 }
 
+// Outputs J and J + 1 of a group of v_rows output rows alone (the items of a small tile, which
+// has fewer groups than threads), each the additions of box6v or box4v in their order: v[0 ..
+// 2R+1] are the group's rows J .. J + 2R + 1.
+template <int R, int VR, int J, typename V> __device__ __forceinline__ void box2v(const V *v, V o[2])
+{
+    if constexpr (VR == 6) {
+        V m = v[5 - J];
+#pragma unroll
+        for (int k = 6; k <= 2 * R; ++k) m = vadd(m, v[k - J]);
+#pragma unroll
+        for (int j = J; j < J + 2; ++j) {
+            V t = m;   // lf[j] + m, then + rt[j]
+            if (j < 5) {
+                V lf = v[4 - J];
+#pragma unroll
+                for (int k = 3; k >= j; --k) lf = vadd(v[k - J], lf);
+                t = vadd(lf, m);
+            }
+            if (j >= 1) {
+                V rt = v[2 * R + 1 - J];
+#pragma unroll
+                for (int k = 2; k <= j; ++k) rt = vadd(rt, v[2 * R + k - J]);
+                t = vadd(t, rt);
+            }
+            o[j - J] = t;
+        }
+    } else {
+        V m = v[3 - J];
+#pragma unroll
+        for (int k = 4; k <= 2 * R; ++k) m = vadd(m, v[k - J]);
+        if constexpr (J == 0) {
+            o[0] = vadd(vadd(vadd(v[0], v[1]), v[2]), m);
+            o[1] = vadd(vadd(vadd(v[1], v[2]), m), v[2 * R + 1]);
+        } else {
+            o[0] = vadd(vadd(vadd(v[2 - J], m), v[2 * R + 1 - J]), v[2 * R + 2 - J]);
+            o[1] = vadd(vadd(vadd(m, v[2 * R + 1 - J]), v[2 * R + 2 - J]), v[2 * R + 3 - J]);
+        }
+    }
+}
+
+template <int R, int TH, int TW, int J>
+__device__ __forceinline__ void box_v_two(const float2 *P01, const float2 *P23, const float *P4, int g, int tx,
+                                          float2 s01[2], float2 s23[2], float s4[2])
+{
+    using F = FixedTile<R, TH, TW>;
+    constexpr int VR = v_rows<R, TH>(), NV = 2 * R + 2;
+    const int row = VR * g + J;
+    {
+        float2 v[NV], w[NV];
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+            v[q] = P01[(row + q) * F::RWP2 + tx];
+            w[q] = P23[(row + q) * F::RWP2 + tx];
+        }
+        box2v<R, VR, J>(v, s01);
+        box2v<R, VR, J>(w, s23);
+    }
+    float v[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v[q] = P4[(row + q) * F::RWP1 + tx];
+    box2v<R, VR, J>(v, s4);
+}
+
 // Stage 1 of the fixed-radius tile for the pixel pair (x, y), (x + 1, y): warp I2 by the
 // current estimate, its gradient there, e~ and the five products, on both pixels at
 // once when both sample the interior (taps from the staged window or global memory),
@@ -1176,21 +1242,21 @@ __device__ __forceinline__ void stage1_pair(const IterArgs &a, int x, int y, flo
     }
 }
 
-// The estimate that places the staged window of the 64 x TH tile at (tx0, ty0): the one at
+// The estimate that places the staged window of the TW x TH tile at (tx0, ty0): the one at
 // the tile's centre.
-template <bool NC, int MODE, int TH>
+template <bool NC, int MODE, int TH, int TW = LK_TW>
 __device__ __forceinline__ float2 win_ref(const IterArgs &a, int tx0, int ty0)
 {
-    return flow_mode<NC, MODE>(a, min(tx0 + LK_TW / 2, a.W - 1), min(ty0 + TH / 2, a.H - 1));
+    return flow_mode<NC, MODE>(a, min(tx0 + TW / 2, a.W - 1), min(ty0 + TH / 2, a.H - 1));
 }
 
 // First element (wx0, wy0) of the staged window of the tile at (tx0, ty0) for the estimate
 // w at its centre: the tile's region displaced by w rounded, widened by the margin and the
 // tap footprint, wx0 rounded down to a multiple of 16 bytes.
-template <int R, int TH, int S>
+template <int R, int TH, int S, int TW = LK_TW>
 __device__ __forceinline__ void win_origin(const IterArgs &a, int tx0, int ty0, float2 w, int &wx0, int &wy0)
 {
-    using F = FixedTile<R, TH>;
+    using F = FixedTile<R, TH, TW>;
     constexpr int E = 16 / S;
     const int ox = __float2int_rn(fminf(fmaxf(w.x, -(float)a.W), (float)a.W));
     const int oy = __float2int_rn(fminf(fmaxf(w.y, -(float)a.H), (float)a.H));
@@ -1200,10 +1266,10 @@ __device__ __forceinline__ void win_origin(const IterArgs &a, int tx0, int ty0, 
 }
 
 // The tile's mbarrier: initialised once per block, before the first tile.
-template <int R, int TH = LK_TH> __device__ __forceinline__ void lk_tile_init(float *smem)
+template <int R, int TH = LK_TH, int TW = LK_TW> __device__ __forceinline__ void lk_tile_init(float *smem)
 {
     if (threadIdx.x == 0) {
-        mbar_init(reinterpret_cast<uint64_t *>(smem + FixedTile<R, TH>::OFF_BAR), 1);
+        mbar_init(reinterpret_cast<uint64_t *>(smem + FixedTile<R, TH, TW>::OFF_BAR), 1);
         fence_proxy_async_smem();
     }
     __syncthreads();
@@ -1216,13 +1282,13 @@ template <int R, int TH = LK_TH> __device__ __forceinline__ void lk_tile_init(fl
 // when `next` (a tile of the same strip follows): that tile's window is then requested as
 // soon as this tile's stage 1 is done, and a later tile of a strip requests only its flow
 // boxes. Returns false if a staging copy did not complete in time.
-template <typename T, bool NC, int R, int MODE, int TH, int CM>
+template <typename T, bool NC, int R, int MODE, int TH, int CM, int TW = LK_TW, int NT = LK_THREADS>
 __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps *maps, int tx0, int ty0, float2 ref,
                                              float fp64_cond, float *smem, uint32_t &phase, bool carry_rt,
                                              const float2 *wrefs = nullptr, bool next = false)
 {
     const bool CARRY = CM == 2 ? carry_rt : CM == 1;
-    using F = FixedTile<R, TH>;
+    using F = FixedTile<R, TH, TW>;
     unsigned char *win = reinterpret_cast<unsigned char *>(smem + F::OFF_WIN);
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + F::OFF_BAR);
     constexpr int S = (int)sizeof(T);
@@ -1237,9 +1303,9 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
     if (CARRY) {
         // region rows TH .. TH+2R-1 of the tile above are rows 0 .. 2R-1 of this one:
         // their window sums along x (columns 0..TW-1 of each plane) move up
-        constexpr int Q2 = LK_TW / 2, Q1 = LK_TW / 4;   // float4 per row: pair planes, P4
+        constexpr int Q2 = TW / 2, Q1 = TW / 4;   // float4 per row: pair planes, P4
         constexpr int N = 2 * R * (2 * Q2 + Q1);
-        for (int i = threadIdx.x; i < N; i += LK_THREADS) {
+        for (int i = threadIdx.x; i < N; i += NT) {
             const int row = i / (2 * Q2 + Q1), c = i - row * (2 * Q2 + Q1);
             float4 *dst, *src;
             if (c < 2 * Q2) {
@@ -1261,7 +1327,7 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
     // P01: stage 1 reads each pair's estimate there before storing the pair's products
     // in the same place (the estimates of rows no box covers are read from global memory).
     const bool box = SAME && staged && (!CARRY || F::FLOW_BOX_BELOW);
-    constexpr bool ALL = F::FLOW_BH == 2 * R;   // boxes cover a first tile's whole region
+    constexpr bool ALL = F::FLOW_BH == 2 * R || F::FLOW_BH == F::RH;   // boxes cover a first tile's whole region
     const int bx0 = CARRY ? 2 * R : 0;          // first row of the boxes; rows below brow_end read them
     const int nbox = !box ? 0 : (CARRY ? TH / F::FLOW_BH : (ALL ? F::RH / F::FLOW_BH : 1));
     const int brow_end = box ? ((CARRY || ALL) ? F::RH : TH) : 0;
@@ -1269,7 +1335,7 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
     if (staged) {
         // a later tile of a strip: its window was requested by the tile above
         const bool early = OF_EARLY_WINDOW && CM == 2 && CARRY;
-        win_origin<R, TH, S>(a, tx0, ty0, CM == 2 ? wrefs[0] : win_ref<NC, MODE, TH>(a, tx0, ty0), wx0, wy0);
+        win_origin<R, TH, S, TW>(a, tx0, ty0, CM == 2 ? wrefs[0] : win_ref<NC, MODE, TH, TW>(a, tx0, ty0), wx0, wy0);
         if (threadIdx.x == 0) {
             fence_proxy_async_smem();
             mbar_arrive_expect_tx(bar, (uint32_t)((early ? 0 : F::win_bytes(S)) + nbox * F::FLOW_BOX_BYTES));
@@ -1291,7 +1357,7 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
             constexpr int CRH = F::RH / 2 + 2, CLPR = ((F::RWE / 2 + 2) * 8 + 127) / 128 + 1;
             const int n1 = (F::RH - r0) * LPR;
             const int n = n1 + (MODE == FLOW_UPSAMPLE ? CRH * CLPR : 0);
-            for (int i = threadIdx.x; i < n; i += LK_THREADS) {
+            for (int i = threadIdx.x; i < n; i += NT) {
                 if (i < n1)
                     prefetch_lines_l1(a.I1, a.pitch, S, a.H, a.W, ty0 - R + r0, ty0 - R + F::RH, tx0 - F::RE,
                                       tx0 - F::RE + F::RWE, LPR, i);
@@ -1330,21 +1396,21 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
             // strips: thread t takes pixel pair cx = t mod NPR of rows r0 + t / NPR, then RPI
             // rows further each round, so that what depends on the pair's column is the same on
             // every row it takes (5% fewer instructions per pixel-iteration at r = 4)
-            constexpr int RPI = LK_THREADS / NPR;   // rows per round
+            constexpr int RPI = NT / NPR;   // rows per round
             const int cx = threadIdx.x % NPR, rs = threadIdx.x / NPR;
             if (rs < RPI) {
 #pragma unroll 1
                 for (int ry = r0 + rs; ry < F::RH; ry += RPI) pair(inner, ry, cx);
             }
         } else {
-            // single tiles: pair j = threadIdx.x + k LK_THREADS is (row ry, pair cx) of the rows
-            // computed, stepped without a division (LK_THREADS = DY rows + DX pairs); it
+            // single tiles: pair j = threadIdx.x + k NT is (row ry, pair cx) of the rows
+            // computed, stepped without a division (NT = DY rows + DX pairs); it
             // compiles without spills where the form above does not
-            constexpr int DY = LK_THREADS / NPR, DX = LK_THREADS % NPR;
+            constexpr int DY = NT / NPR, DX = NT % NPR;
             const int npair = (F::RH - r0) * NPR;
             int ry = r0 + threadIdx.x / NPR, cx = threadIdx.x % NPR;
 #pragma unroll 1
-            for (int j = threadIdx.x; j < npair; j += LK_THREADS) {
+            for (int j = threadIdx.x; j < npair; j += NT) {
                 pair(inner, ry, cx);
                 ry += DY;
                 cx += DX;
@@ -1357,7 +1423,7 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
     };
     // the staged window and the region both inside the image: no pair needs a bounds check
     if (staged && wx0 >= 0 && wy0 >= 0 && wx0 + WW <= a.W && wy0 + F::WIN_H <= a.H && tx0 >= F::RE && ty0 >= R &&
-        tx0 + LK_TW + F::RE <= a.W && ty0 + TH + R <= a.H)
+        tx0 + TW + F::RE <= a.W && ty0 + TH + R <= a.H)
         rows(std::true_type());
     else
         rows(std::false_type());
@@ -1367,7 +1433,7 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
         // finishes (the barrier's next phase completes only on that tile's arrival)
         if (staged && next && threadIdx.x == 0) {
             int nx0, ny0;
-            win_origin<R, TH, S>(a, tx0, ty0 + TH, wrefs[1], nx0, ny0);
+            win_origin<R, TH, S, TW>(a, tx0, ty0 + TH, wrefs[1], nx0, ny0);
             fence_proxy_async_smem();
             mbar_expect_tx(bar, (uint32_t)F::win_bytes(S));
             tma_load_2d(win, &maps->i2, nx0, ny0, bar);
@@ -1375,24 +1441,34 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
     }
     // P23's chunks start at warp 4, so that when the rows leave some warps an extra chunk
     // of P01 and of P4 (24 rows: 12 chunks and 384 items) the other warps take P23's
-    box_h_pairs<R, TH>(P01, r0);
-    box_h_pairs<R, TH>(P23, r0, LK_THREADS / 64);
-    box_h_single<R, TH>(P4, r0);
+    box_h_pairs<R, TH, TW, NT>(P01, r0);
+    box_h_pairs<R, TH, TW, NT>(P23, r0, NT / 64);
+    box_h_single<R, TH, TW, NT>(P4, r0);
     __syncthreads();
-    // vertical sums, solve and write, VR rows of one column per item
+    // vertical sums, solve and write: VO rows of one column per item (all VR rows of a group, or
+    // two of them where the tile has fewer groups than threads)
     constexpr int VR = v_rows<R, TH>();
-    constexpr int VITEMS = LK_TW * (TH / VR);
+    constexpr int NGRP = TW * (TH / VR);
+    constexpr int VO = NGRP < NT ? 2 : VR;
 #pragma unroll 1
-    for (int i = threadIdx.x; i < VITEMS; i += LK_THREADS) {
-        const int tx = i % LK_TW, g = i / LK_TW;
-        const int x = tx0 + tx;
-        if (x >= a.W || ty0 + VR * g >= a.H) continue;
-        float2 s01[VR], s23[VR];
-        float s4[VR];
-        box_v_planes<R, TH>(P01, P23, P4, g, tx, s01, s23, s4);
+    for (int i = threadIdx.x; i < NGRP * (VR / VO); i += NT) {
+        const int part = VO == VR ? 0 : i / NGRP;   // the same for a whole warp
+        const int k = i - part * NGRP;
+        const int tx = k % TW, g = k / TW;
+        const int x = tx0 + tx, yb = ty0 + VR * g + VO * part;
+        if (x >= a.W || yb >= a.H) continue;
+        float2 s01[VO], s23[VO];
+        float s4[VO];
+        if constexpr (VO == VR) {
+            box_v_planes<R, TH, TW>(P01, P23, P4, g, tx, s01, s23, s4);
+        } else {
+            if (part == 0) box_v_two<R, TH, TW, 0>(P01, P23, P4, g, tx, s01, s23, s4);
+            else if (VR == 4 || part == 1) box_v_two<R, TH, TW, 2>(P01, P23, P4, g, tx, s01, s23, s4);
+            else box_v_two<R, TH, TW, VR == 6 ? 4 : 2>(P01, P23, P4, g, tx, s01, s23, s4);
+        }
 #pragma unroll
-        for (int j = 0; j < VR; ++j) {
-            const int y = ty0 + VR * g + j;
+        for (int j = 0; j < VO; ++j) {
+            const int y = yb + j;
             if (y >= a.H) break;
             const float sj[5] = {s01[j].x, s01[j].y, s23[j].x, s23[j].y, s4[j]};
             float xu, xv;
@@ -1447,6 +1523,24 @@ __device__ __forceinline__ bool lk_tile_fixed(const IterArgs &a, const StageMaps
                 return false;
         return true;
     }
+}
+
+// One small tile of the fixed-radius iteration (SM_TW x SM_TH outputs, SM_THREADS threads),
+// for launches with too few 64 x LK_TH tiles to fill the GPU: same reference flows (the
+// groups of the 64 x LK_TH tiles) and the same groups of window sums, so the same bits.
+static_assert(LK_TW % SM_TW == 0 && LK_TH % SM_TH == 0, "small tiles inside the default tiles, group-aligned");
+template <typename T, bool NC, int R, int MODE>
+__device__ __forceinline__ bool lk_tile_small(const IterArgs &a, const StageMaps *maps, int unit, float fp64_cond,
+                                              float *smem)
+{
+    static_assert(v_rows<R, SM_TH>() == v_rows<R, LK_TH>(), "the same groups of window sums");
+    uint32_t phase = 0;
+    const int uy = unit / a.tiles_x;
+    const int tx0 = (unit - uy * a.tiles_x) * SM_TW, ty0 = uy * SM_TH;
+    const int gx0 = tx0 / LK_TW * LK_TW, gy0 = ty0 / (REF_GROUP * LK_TH) * (REF_GROUP * LK_TH);
+    const float2 ref = flow_mode<NC, MODE>(a, min(gx0 + LK_TW / 2, a.W - 1), min(gy0 + REF_GROUP * LK_TH / 2, a.H - 1));
+    return lk_tile_step<T, NC, R, MODE, SM_TH, 0, SM_TW, SM_THREADS>(a, maps, tx0, ty0, ref, fp64_cond, smem, phase,
+                                                                     false);
 }
 
 // ------------------------------------------------ two iterations fused in one tile

@@ -24,6 +24,40 @@ lk_iter_kernel(const __grid_constant__ IterArgs a, const __grid_constant__ Stage
     lk_tile<T, true, R, -1, LK_TH, false>(a, &m, blockIdx.x, r, fp64_cond, smem, phase);   // a.strip is 1
 }
 
+// The same on small tiles.
+template <typename T, int R>
+__global__ void __launch_bounds__(SM_THREADS, SM_MIN_BLOCKS)
+lk_small_kernel(const __grid_constant__ IterArgs a, const __grid_constant__ StageMaps m, float fp64_cond)
+{
+    extern __shared__ __align__(128) float4 smem4[];
+    float *smem = reinterpret_cast<float *>(smem4);
+    if constexpr (R != 0) {
+        lk_tile_init<R, SM_TH, SM_TW>(smem);
+        if (a.mode == FLOW_SAME) lk_tile_small<T, true, R, FLOW_SAME>(a, &m, blockIdx.x, fp64_cond, smem);
+        else lk_tile_small<T, true, R, -1>(a, &m, blockIdx.x, fp64_cond, smem);
+    }
+}
+
+template <typename T, int R, int MODE>
+__global__ void __launch_bounds__(SM_THREADS, SM_MIN_BLOCKS)
+phase_small_kernel(const __grid_constant__ IterPhase P, float fp64_cond)
+{
+    extern __shared__ __align__(128) float4 smem4[];
+    float *smem = reinterpret_cast<float *>(smem4);
+    if constexpr (R != 0) {
+        const int p = phase_pair(P.prefix, P.npairs, blockIdx.x);
+        lk_tile_init<R, SM_TH, SM_TW>(smem);
+        lk_tile_small<T, true, R, MODE>(P.a[p], &P.m[p], blockIdx.x - P.prefix[p], fp64_cond, smem);
+    }
+}
+
+template <int R> int small_smem_floats(bool stage_i2, int elem_bytes)
+{
+    if constexpr (R == 0) return 0;
+    else if (stage_i2) return FixedTile<R, SM_TH, SM_TW>::smem_staged(elem_bytes);
+    else return FixedTile<R, SM_TH, SM_TW>::SMEM_NOSTAGE;
+}
+
 // One iteration of up to PHASE_PAIRS pairs on one level: block b runs tile
 // b - prefix[p] of pair p. The same tile code as lk_iter_kernel, so the same results.
 template <typename T, int R, int MODE, int TH>
@@ -148,8 +182,16 @@ template <int R> size_t radius_smem_bytes(int r, bool stage_i2)
 }
 
 template <typename T, int R>
-static cudaError_t lk_for(const IterArgs &a, const StageMaps &m, int r, float fp64_cond, cudaStream_t s)
+static cudaError_t lk_for(const IterArgs &a, const StageMaps &m, int r, float fp64_cond, bool small, cudaStream_t s)
 {
+    if constexpr (R != 0) {
+        if (small) {
+            lk_small_kernel<T, R><<<a.tiles, SM_THREADS,
+                                    sizeof(float) * small_smem_floats<R>(a.stage_i2 != 0, (int)sizeof(T)), s>>>(
+                a, m, fp64_cond);
+            return cudaGetLastError();
+        }
+    }
     lk_iter_kernel<T, R><<<a.tiles, LK_THREADS,
                            sizeof(float) * lk_tile_smem_floats<R>(r, a.stage_i2 != 0, (int)sizeof(T)), s>>>(
         a, m, r, fp64_cond);
@@ -157,14 +199,15 @@ static cudaError_t lk_for(const IterArgs &a, const StageMaps &m, int r, float fp
 }
 
 template <int R>
-cudaError_t lk_launch(const IterArgs &a, const StageMaps &m, int elem, int r, float fp64_cond, cudaStream_t s)
+cudaError_t lk_launch(const IterArgs &a, const StageMaps &m, int elem, int r, float fp64_cond, bool small,
+                      cudaStream_t s)
 {
     switch (elem) {
-    case ET_U8: return lk_for<uint8_t, R>(a, m, r, fp64_cond, s);
-    case ET_U16: return lk_for<uint16_t, R>(a, m, r, fp64_cond, s);
-    case ET_F32: return lk_for<float, R>(a, m, r, fp64_cond, s);
-    case ET_F16: return lk_for<__half, R>(a, m, r, fp64_cond, s);
-    default: return lk_for<__nv_bfloat16, R>(a, m, r, fp64_cond, s);
+    case ET_U8: return lk_for<uint8_t, R>(a, m, r, fp64_cond, small, s);
+    case ET_U16: return lk_for<uint16_t, R>(a, m, r, fp64_cond, small, s);
+    case ET_F32: return lk_for<float, R>(a, m, r, fp64_cond, small, s);
+    case ET_F16: return lk_for<__half, R>(a, m, r, fp64_cond, small, s);
+    default: return lk_for<__nv_bfloat16, R>(a, m, r, fp64_cond, small, s);
     }
 }
 
@@ -197,6 +240,18 @@ template <typename T, int R>
 static cudaError_t phase_for(const IterPhase &P, int r, float fp64_cond, int tile_h, cudaStream_t s)
 {
     if constexpr (R != 0) {
+        if (tile_h == SM_TH) {
+            bool stage = false;
+            for (int i = 0; i < P.npairs; ++i) stage = stage || P.a[i].stage_i2 != 0;
+            const size_t smem = sizeof(float) * small_smem_floats<R>(stage, (int)sizeof(T));
+            const int blocks = P.prefix[P.npairs];
+            switch (P.a[0].mode) {
+            case FLOW_ZERO: phase_small_kernel<T, R, FLOW_ZERO><<<blocks, SM_THREADS, smem, s>>>(P, fp64_cond); break;
+            case FLOW_SAME: phase_small_kernel<T, R, FLOW_SAME><<<blocks, SM_THREADS, smem, s>>>(P, fp64_cond); break;
+            default: phase_small_kernel<T, R, FLOW_UPSAMPLE><<<blocks, SM_THREADS, smem, s>>>(P, fp64_cond); break;
+            }
+            return cudaGetLastError();
+        }
         if (tile_h == ALT_TH) return phase_for_th<T, R, ALT_TH>(P, r, fp64_cond, s);
     }
     return phase_for_th<T, R, LK_TH>(P, r, fp64_cond, s);
@@ -317,9 +372,9 @@ template <int R> cudaError_t phase_i1_launch(const IterPhase &P, int elem, int r
 
 // The tensor maps of the staged fixed-radius tile of height TH: the estimate in boxes
 // of the tile's region (RWP2 x RH elements of 8 bytes) and I2 in boxes of the window.
-template <int R, int TH> static bool stage_maps_th(const IterArgs &a, StageMaps &m, int elem)
+template <int R, int TH, int TW = LK_TW> static bool stage_maps_th(const IterArgs &a, StageMaps &m, int elem)
 {
-    using F = FixedTile<R, TH>;
+    using F = FixedTile<R, TH, TW>;
     const int S = elem_bytes(elem);
     if (a.mode == FLOW_SAME &&
         !encode_tile_map(&m.flow, ET_FLOW2, a.fin, a.W, a.H, (size_t)a.fin_pitch * 8, F::RWP2, F::FLOW_BH))
@@ -332,6 +387,7 @@ template <int R> bool radius_stage_maps(const IterArgs &a, StageMaps &m, int ele
     if constexpr (R == 0) {
         return false;
     } else {
+        if (tile_h == SM_TH) return stage_maps_th<R, SM_TH, SM_TW>(a, m, elem);
         return tile_h == ALT_TH ? stage_maps_th<R, ALT_TH>(a, m, elem) : stage_maps_th<R, LK_TH>(a, m, elem);
     }
 }
@@ -383,6 +439,21 @@ template <int R> cudaError_t radius_configure()
 #undef OF_SET_ALT
     }
     OF_SET((window_sums_kernel<R>));
+    if constexpr (R != 0) {   // small tiles
+        const int sb = (int)sizeof(float) * small_smem_floats<R>(true, 4);
+#define OF_SET_SM(T)                                                                                        \
+    for (const void *fn : {(const void *)lk_small_kernel<T, R>, (const void *)phase_small_kernel<T, R, FLOW_ZERO>, \
+                           (const void *)phase_small_kernel<T, R, FLOW_SAME>,                               \
+                           (const void *)phase_small_kernel<T, R, FLOW_UPSAMPLE>})                          \
+        if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sb)) != cudaSuccess) \
+            return e;
+        OF_SET_SM(uint8_t)
+        OF_SET_SM(uint16_t)
+        OF_SET_SM(float)
+        OF_SET_SM(__half)
+        OF_SET_SM(__nv_bfloat16)
+#undef OF_SET_SM
+    }
     if constexpr (R != 0) {   // the fused two-iteration kernels
         const int fb = (int)fused2_smem_bytes<R>();
         for (const void *fn : {(const void *)phase_iter2_kernel<uint8_t, R>, (const void *)phase_iter2_kernel<uint16_t, R>,
@@ -416,7 +487,7 @@ template <int R> cudaError_t radius_configure()
     return cudaSuccess;
 }
 
-template cudaError_t lk_launch<OF_RADIUS>(const IterArgs &, const StageMaps &, int, int, float, cudaStream_t);
+template cudaError_t lk_launch<OF_RADIUS>(const IterArgs &, const StageMaps &, int, int, float, bool, cudaStream_t);
 template cudaError_t ws_launch<OF_RADIUS>(const float *, int, int, int, float *, cudaStream_t);
 template cudaError_t i1h_launch<OF_RADIUS>(const HessArgs &, int, int, cudaStream_t);
 template cudaError_t phase_launch<OF_RADIUS>(const IterPhase &, int, int, float, int, cudaStream_t);

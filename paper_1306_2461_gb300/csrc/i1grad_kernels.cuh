@@ -64,7 +64,7 @@ __device__ __forceinline__ void i1_hess_tile(const HessArgs &a, int tile, int r,
         float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f;
         if ((unsigned)y < (unsigned)a.H && (unsigned)x < (unsigned)a.W) {
             float c, gx, gy;
-            i1_grad<true>(I1, a.pitch, a.H, a.W, x, y, c, gx, gy);
+            i1_grad<false>(I1, a.pitch, a.H, a.W, x, y, c, gx, gy);
             p0 = gx * gx;
             p1 = gx * gy;
             p2 = gy * gy;
@@ -113,7 +113,7 @@ __device__ __forceinline__ void i1_iter_tile(const IterArgs &a, int tile, int r,
     const int ty0 = tyi * I1_TH, tx0 = (tile - tyi * a.tiles_x) * LK_TW;
     const T *I1 = static_cast<const T *>(a.I1);
     const T *I2 = static_cast<const T *>(a.I2);
-    const float2 ref = flow_at<true>(a, min(tx0 + LK_TW / 2, a.W - 1), min(ty0 + I1_TH / 2, a.H - 1));
+    const float2 ref = flow_at<false>(a, min(tx0 + LK_TW / 2, a.W - 1), min(ty0 + I1_TH / 2, a.H - 1));
     const int rr = R == 0 ? r : R;
     const int RH = I1_TH + 2 * rr, RW = LK_TW + 2 * rr;
     const int plane = i1_plane<R>(RH, RW);
@@ -131,7 +131,7 @@ __device__ __forceinline__ void i1_iter_tile(const IterArgs &a, int tile, int r,
             const int ry = i / RW, rx = i - ry * RW;
             const int y = ty0 - rr + ry, x = tx0 - rr + rx;
             in[k] = i < nreg && (unsigned)y < (unsigned)a.H && (unsigned)x < (unsigned)a.W;
-            f[k] = in[k] ? flow_at<true>(a, x, y) : make_float2(0.0f, 0.0f);
+            f[k] = in[k] ? flow_at<false>(a, x, y) : make_float2(0.0f, 0.0f);
         }
 #pragma unroll
         for (int k = 0; k < S1; ++k) {
@@ -142,8 +142,8 @@ __device__ __forceinline__ void i1_iter_tile(const IterArgs &a, int tile, int r,
             float p0 = 0.0f, p1 = 0.0f;
             if (in[k]) {
                 float c, gx, gy;
-                i1_grad<true>(I1, a.pitch, a.H, a.W, x, y, c, gx, gy);
-                const float Iw = bil_at<true>(I2, a.pitch, a.H, a.W, x, y, f[k].x, f[k].y);
+                i1_grad<false>(I1, a.pitch, a.H, a.W, x, y, c, gx, gy);
+                const float Iw = bil_at<false>(I2, a.pitch, a.H, a.W, x, y, f[k].x, f[k].y);
                 const float e = resid(c, Iw, gx, gy, f[k].x - ref.x, f[k].y - ref.y);
                 p0 = gx * e;
                 p1 = gy * e;
@@ -154,11 +154,11 @@ __device__ __forceinline__ void i1_iter_tile(const IterArgs &a, int tile, int r,
         }
     }
     __syncthreads();
-    auto finish = [&](int x, int y, float d, float e) {
-        const float4 h = __ldg(a.hess + (size_t)y * a.hess_pitch + x);
+    auto matrix = [&](int x, int y) { return a.hess[(size_t)y * a.hess_pitch + x]; };
+    auto finish = [&](int x, int y, float4 h, float d, float e) {
         const float s[5] = {h.x, h.y, h.z, d, e};
         float xu, xv;
-        const float2 f = solve2(s, fp64_cond, xu, xv) ? make_float2(ref.x + xu, ref.y + xv) : flow_at<true>(a, x, y);
+        const float2 f = solve2(s, fp64_cond, xu, xv) ? make_float2(ref.x + xu, ref.y + xv) : flow_at<false>(a, x, y);
         if (a.fout) {
             a.fout[(size_t)y * a.fout_pitch + x] = f;
         } else {
@@ -176,7 +176,7 @@ __device__ __forceinline__ void i1_iter_tile(const IterArgs &a, int tile, int r,
             if (y >= a.H || x >= a.W) continue;
             float s[2];
             box_vsum<2>(S, RH, r, ty, tx, s);
-            finish(x, y, s[0], s[1]);
+            finish(x, y, matrix(x, y), s[0], s[1]);
         }
     } else {
         box_h_inplace<R, 2, I1_TH>(smem);
@@ -185,13 +185,16 @@ __device__ __forceinline__ void i1_iter_tile(const IterArgs &a, int tile, int r,
             const int tx = i % LK_TW, g = i / LK_TW;
             const int x = tx0 + tx;
             if (x >= a.W || ty0 + 4 * g >= a.H) continue;
+            float4 h[4];   // loaded together, before the first row is written
+#pragma unroll
+            for (int j = 0; j < 4; ++j) h[j] = matrix(x, min(ty0 + 4 * g + j, a.H - 1));
             float s[2][4];
             box_v4<R, 2, I1_TH>(smem, g, tx, s);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int y = ty0 + 4 * g + j;
                 if (y >= a.H) break;
-                finish(x, y, s[0][j], s[1][j]);
+                finish(x, y, h[j], s[0][j], s[1][j]);
             }
         }
     }
@@ -201,6 +204,7 @@ template <typename T, int R>
 __global__ void __launch_bounds__(LK_THREADS) i1_hess_kernel(HessArgs a, int r)
 {
     extern __shared__ float4 smem4[];
+    chain_begin();
     i1_hess_tile<T, R>(a, blockIdx.x, r, reinterpret_cast<float *>(smem4));
 }
 
@@ -211,6 +215,7 @@ template <typename T, int R>
 __global__ void __launch_bounds__(LK_THREADS, OF_I1_MIN_BLOCKS) i1_iter_kernel(IterArgs a, int r, float fp64_cond)
 {
     extern __shared__ float4 smem4[];
+    chain_begin();
     i1_iter_tile<T, R>(a, blockIdx.x, r, fp64_cond, reinterpret_cast<float *>(smem4));
 }
 
@@ -219,6 +224,7 @@ template <typename T, int R>
 __global__ void __launch_bounds__(LK_THREADS) phase_hess_kernel(const __grid_constant__ HessPhase P, int r)
 {
     extern __shared__ float4 smem4[];
+    chain_begin();
     const int p = phase_pair(P.prefix, P.npairs, blockIdx.x);
     i1_hess_tile<T, R>(P.a[p], blockIdx.x - P.prefix[p], r, reinterpret_cast<float *>(smem4));
 }
@@ -228,6 +234,7 @@ __global__ void __launch_bounds__(LK_THREADS, OF_I1_MIN_BLOCKS)
 phase_i1_iter_kernel(const __grid_constant__ IterPhase P, int r, float fp64_cond)
 {
     extern __shared__ float4 smem4[];
+    chain_begin();
     if constexpr (R != 0) {
         const int t2 = blockIdx.x + P.ahead;
         if (P.ahead > 0 && t2 < P.prefix[P.npairs]) {

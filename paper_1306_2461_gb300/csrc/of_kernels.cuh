@@ -236,7 +236,7 @@ template <typename Tin, typename Tout, bool FIRST>
 __device__ __forceinline__ void pyr_tile(const PyrArgs &a, int tile, int img)
 {
     __shared__ float smem[PYR_SMEM_FLOATS];
-    pyr_tile_smem<Tin, Tout, FIRST, true>(a, tile, img, smem);
+    pyr_tile_smem<Tin, Tout, FIRST, FIRST>(a, tile, img, smem);   // later passes read what the launch before wrote
 }
 
 // ---------------------------------------------------------- normalisation tile

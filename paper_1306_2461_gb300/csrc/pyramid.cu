@@ -16,6 +16,8 @@ namespace of {
 template <typename Tin, typename Tout, bool FIRST>
 __global__ void __launch_bounds__(PYR_THREADS) pyr_kernel(PyrArgs a)
 {
+    if constexpr (FIRST) chain_next();   // the sequence's first launch
+    else chain_begin();
     pyr_tile<Tin, Tout, FIRST>(a, blockIdx.x, blockIdx.y + a.first_image);
 }
 
@@ -43,17 +45,17 @@ cudaError_t launch_pyr_down(const PyrArgs &a, int storage, cudaStream_t s)
 {
     dim3 grid(a.tiles, 2 - a.first_image);
     switch (storage) {
-    case OF_F32: pyr_kernel<float, float, false><<<grid, PYR_THREADS, 0, s>>>(a); break;
-    case OF_F16: pyr_kernel<__half, __half, false><<<grid, PYR_THREADS, 0, s>>>(a); break;
-    default: pyr_kernel<__nv_bfloat16, __nv_bfloat16, false><<<grid, PYR_THREADS, 0, s>>>(a); break;
+    case OF_F32: return launch_chained(pyr_kernel<float, float, false>, grid, PYR_THREADS, 0, s, a);
+    case OF_F16: return launch_chained(pyr_kernel<__half, __half, false>, grid, PYR_THREADS, 0, s, a);
+    default: return launch_chained(pyr_kernel<__nv_bfloat16, __nv_bfloat16, false>, grid, PYR_THREADS, 0, s, a);
     }
-    return cudaGetLastError();
 }
 
 template <typename Tin, typename Tout>
 __global__ void __launch_bounds__(256) znssd_kernel(ZnArgs a)
 {
     __shared__ float smem[ZN_SMEM_FLOATS];
+    chain_next();   // the sequence's first launch
     znssd_tile<Tin, Tout, true>(a, blockIdx.x, blockIdx.y + a.first_image, smem);
 }
 
@@ -80,6 +82,8 @@ cudaError_t launch_znssd(const ZnArgs &a, int in_format, int storage, cudaStream
 template <typename Tin, typename Tout, bool FIRST>
 __global__ void __launch_bounds__(PYR_THREADS) phase_pyr_kernel(const __grid_constant__ PyrPhase P)
 {
+    if constexpr (FIRST) chain_next();   // the sequence's first launch
+    else chain_begin();
     const int p = phase_pair(P.prefix, P.npairs, blockIdx.x);
     const PyrArgs &a = P.a[p];
     const int j = blockIdx.x - P.prefix[p];
@@ -109,17 +113,17 @@ cudaError_t launch_phase_pyr(const PyrPhase &P, bool first, int in_format, int s
         }
     }
     switch (storage) {
-    case OF_F32: phase_pyr_kernel<float, float, false><<<blocks, PYR_THREADS, 0, s>>>(P); break;
-    case OF_F16: phase_pyr_kernel<__half, __half, false><<<blocks, PYR_THREADS, 0, s>>>(P); break;
-    default: phase_pyr_kernel<__nv_bfloat16, __nv_bfloat16, false><<<blocks, PYR_THREADS, 0, s>>>(P); break;
+    case OF_F32: return launch_chained(phase_pyr_kernel<float, float, false>, blocks, PYR_THREADS, 0, s, P);
+    case OF_F16: return launch_chained(phase_pyr_kernel<__half, __half, false>, blocks, PYR_THREADS, 0, s, P);
+    default: return launch_chained(phase_pyr_kernel<__nv_bfloat16, __nv_bfloat16, false>, blocks, PYR_THREADS, 0, s, P);
     }
-    return cudaGetLastError();
 }
 
 template <typename Tin, typename Tout>
 __global__ void __launch_bounds__(256) phase_zn_kernel(const __grid_constant__ ZnPhase P)
 {
     __shared__ float smem[ZN_SMEM_FLOATS];
+    chain_next();   // the sequence's first launch
     const int p = phase_pair(P.prefix, P.npairs, blockIdx.x);
     const ZnArgs &a = P.a[p];
     const int j = blockIdx.x - P.prefix[p];

@@ -21,7 +21,8 @@ lk_iter_kernel(const __grid_constant__ IterArgs a, const __grid_constant__ Stage
     float *smem = reinterpret_cast<float *>(smem4);
     uint32_t phase = 0;
     lk_tile_prepare<R>(smem);
-    lk_tile<T, true, R, -1, LK_TH, false>(a, &m, blockIdx.x, r, fp64_cond, smem, phase);   // a.strip is 1
+    chain_begin();
+    lk_tile<T, false, R, -1, LK_TH, false>(a, &m, blockIdx.x, r, fp64_cond, smem, phase);   // a.strip is 1
 }
 
 // The same on small tiles.
@@ -33,8 +34,9 @@ lk_small_kernel(const __grid_constant__ IterArgs a, const __grid_constant__ Stag
     float *smem = reinterpret_cast<float *>(smem4);
     if constexpr (R != 0) {
         lk_tile_init<R, SM_TH, SM_TW>(smem);
-        if (a.mode == FLOW_SAME) lk_tile_small<T, true, R, FLOW_SAME>(a, &m, blockIdx.x, fp64_cond, smem);
-        else lk_tile_small<T, true, R, -1>(a, &m, blockIdx.x, fp64_cond, smem);
+        chain_begin();
+        if (a.mode == FLOW_SAME) lk_tile_small<T, false, R, FLOW_SAME>(a, &m, blockIdx.x, fp64_cond, smem);
+        else lk_tile_small<T, false, R, -1>(a, &m, blockIdx.x, fp64_cond, smem);
     }
 }
 
@@ -47,7 +49,8 @@ phase_small_kernel(const __grid_constant__ IterPhase P, float fp64_cond)
     if constexpr (R != 0) {
         const int p = phase_pair(P.prefix, P.npairs, blockIdx.x);
         lk_tile_init<R, SM_TH, SM_TW>(smem);
-        lk_tile_small<T, true, R, MODE>(P.a[p], &P.m[p], blockIdx.x - P.prefix[p], fp64_cond, smem);
+        chain_begin();
+        lk_tile_small<T, false, R, MODE>(P.a[p], &P.m[p], blockIdx.x - P.prefix[p], fp64_cond, smem);
     }
 }
 
@@ -66,6 +69,10 @@ phase_iter_kernel(const __grid_constant__ IterPhase P, int r, float fp64_cond)
 {
     extern __shared__ __align__(128) float4 smem4[];
     float *smem = reinterpret_cast<float *>(smem4);
+    const int p = phase_pair(P.prefix, P.npairs, blockIdx.x);
+    uint32_t phase = 0;
+    lk_tile_prepare<R, TH>(smem);
+    chain_begin();
     if constexpr (R != 0) {
         const int t2 = blockIdx.x + P.ahead;
         if (P.ahead > 0 && t2 < P.prefix[P.npairs]) {
@@ -73,10 +80,7 @@ phase_iter_kernel(const __grid_constant__ IterPhase P, int r, float fp64_cond)
             prefetch_tile<T, MODE, TH>(P.a[q], t2 - P.prefix[q], R);
         }
     }
-    const int p = phase_pair(P.prefix, P.npairs, blockIdx.x);
-    uint32_t phase = 0;
-    lk_tile_prepare<R, TH>(smem);
-    lk_tile<T, true, R, MODE, TH>(P.a[p], &P.m[p], blockIdx.x - P.prefix[p], r, fp64_cond, smem, phase);
+    lk_tile<T, false, R, MODE, TH>(P.a[p], &P.m[p], blockIdx.x - P.prefix[p], r, fp64_cond, smem, phase);
 }
 
 // Two same-level iterations of up to PHASE_PAIRS pairs in one launch (iteration fusion
@@ -97,7 +101,8 @@ phase_iter2_kernel(const __grid_constant__ IterPhase P, float fp64_cond)
     extern __shared__ __align__(128) float4 smem4[];
     if constexpr (R != 0) {
         const int p = phase_pair(P.prefix, P.npairs, blockIdx.x);
-        lk_tile_fused2<T, true, R, LK_TH>(P.a[p], blockIdx.x - P.prefix[p], fp64_cond,
+        chain_begin();
+        lk_tile_fused2<T, false, R, LK_TH>(P.a[p], blockIdx.x - P.prefix[p], fp64_cond,
                                           reinterpret_cast<float *>(smem4));
     }
 }
@@ -186,16 +191,10 @@ static cudaError_t lk_for(const IterArgs &a, const StageMaps &m, int r, float fp
 {
     if constexpr (R != 0) {
         if (small) {
-            lk_small_kernel<T, R><<<a.tiles, SM_THREADS,
-                                    sizeof(float) * small_smem_floats<R>(a.stage_i2 != 0, (int)sizeof(T)), s>>>(
-                a, m, fp64_cond);
-            return cudaGetLastError();
+            return launch_chained(lk_small_kernel<T, R>, a.tiles, SM_THREADS, sizeof(float) * small_smem_floats<R>(a.stage_i2 != 0, (int)sizeof(T)), s, a, m, fp64_cond);
         }
     }
-    lk_iter_kernel<T, R><<<a.tiles, LK_THREADS,
-                           sizeof(float) * lk_tile_smem_floats<R>(r, a.stage_i2 != 0, (int)sizeof(T)), s>>>(
-        a, m, r, fp64_cond);
-    return cudaGetLastError();
+    return launch_chained(lk_iter_kernel<T, R>, a.tiles, LK_THREADS, sizeof(float) * lk_tile_smem_floats<R>(r, a.stage_i2 != 0, (int)sizeof(T)), s, a, m, r, fp64_cond);
 }
 
 template <int R>
@@ -229,11 +228,10 @@ static cudaError_t phase_for_th(const IterPhase &P, int r, float fp64_cond, cuda
     const size_t smem = sizeof(float) * lk_tile_smem_floats<R, TH>(r, stage, (int)sizeof(T));
     const int blocks = P.prefix[P.npairs];
     switch (P.a[0].mode) {
-    case FLOW_ZERO: phase_iter_kernel<T, R, FLOW_ZERO, TH><<<blocks, LK_THREADS, smem, s>>>(P, r, fp64_cond); break;
-    case FLOW_SAME: phase_iter_kernel<T, R, FLOW_SAME, TH><<<blocks, LK_THREADS, smem, s>>>(P, r, fp64_cond); break;
-    default: phase_iter_kernel<T, R, FLOW_UPSAMPLE, TH><<<blocks, LK_THREADS, smem, s>>>(P, r, fp64_cond); break;
+    case FLOW_ZERO: return launch_chained(phase_iter_kernel<T, R, FLOW_ZERO, TH>, blocks, LK_THREADS, smem, s, P, r, fp64_cond);
+    case FLOW_SAME: return launch_chained(phase_iter_kernel<T, R, FLOW_SAME, TH>, blocks, LK_THREADS, smem, s, P, r, fp64_cond);
+    default: return launch_chained(phase_iter_kernel<T, R, FLOW_UPSAMPLE, TH>, blocks, LK_THREADS, smem, s, P, r, fp64_cond);
     }
-    return cudaGetLastError();
 }
 
 template <typename T, int R>
@@ -246,11 +244,10 @@ static cudaError_t phase_for(const IterPhase &P, int r, float fp64_cond, int til
             const size_t smem = sizeof(float) * small_smem_floats<R>(stage, (int)sizeof(T));
             const int blocks = P.prefix[P.npairs];
             switch (P.a[0].mode) {
-            case FLOW_ZERO: phase_small_kernel<T, R, FLOW_ZERO><<<blocks, SM_THREADS, smem, s>>>(P, fp64_cond); break;
-            case FLOW_SAME: phase_small_kernel<T, R, FLOW_SAME><<<blocks, SM_THREADS, smem, s>>>(P, fp64_cond); break;
-            default: phase_small_kernel<T, R, FLOW_UPSAMPLE><<<blocks, SM_THREADS, smem, s>>>(P, fp64_cond); break;
+            case FLOW_ZERO: return launch_chained(phase_small_kernel<T, R, FLOW_ZERO>, blocks, SM_THREADS, smem, s, P, fp64_cond);
+            case FLOW_SAME: return launch_chained(phase_small_kernel<T, R, FLOW_SAME>, blocks, SM_THREADS, smem, s, P, fp64_cond);
+            default: return launch_chained(phase_small_kernel<T, R, FLOW_UPSAMPLE>, blocks, SM_THREADS, smem, s, P, fp64_cond);
             }
-            return cudaGetLastError();
         }
         if (tile_h == ALT_TH) return phase_for_th<T, R, ALT_TH>(P, r, fp64_cond, s);
     }
@@ -278,8 +275,7 @@ template <int R> size_t fused2_smem_bytes()
 
 template <typename T, int R> static cudaError_t phase2_for(const IterPhase &P, float fp64_cond, cudaStream_t s)
 {
-    phase_iter2_kernel<T, R><<<P.prefix[P.npairs], LK_THREADS, fused2_smem_bytes<R>(), s>>>(P, fp64_cond);
-    return cudaGetLastError();
+    return launch_chained(phase_iter2_kernel<T, R>, P.prefix[P.npairs], LK_THREADS, fused2_smem_bytes<R>(), s, P, fp64_cond);
 }
 
 template <int R> cudaError_t phase2_launch(const IterPhase &P, int elem, float fp64_cond, cudaStream_t s)
@@ -300,8 +296,7 @@ template <int R> cudaError_t phase2_launch(const IterPhase &P, int elem, float f
 
 template <typename T, int R> static cudaError_t i1h_for(const HessArgs &a, int r, cudaStream_t s)
 {
-    i1_hess_kernel<T, R><<<a.tiles, LK_THREADS, sizeof(float) * i1_smem_floats<R>(r, 3), s>>>(a, r);
-    return cudaGetLastError();
+    return launch_chained(i1_hess_kernel<T, R>, a.tiles, LK_THREADS, sizeof(float) * i1_smem_floats<R>(r, 3), s, a, r);
 }
 
 template <int R> cudaError_t i1h_launch(const HessArgs &a, int elem, int r, cudaStream_t s)
@@ -317,8 +312,7 @@ template <int R> cudaError_t i1h_launch(const HessArgs &a, int elem, int r, cuda
 
 template <typename T, int R> static cudaError_t i1_for(const IterArgs &a, int r, float fp64_cond, cudaStream_t s)
 {
-    i1_iter_kernel<T, R><<<a.tiles, LK_THREADS, sizeof(float) * i1_smem_floats<R>(r, 2), s>>>(a, r, fp64_cond);
-    return cudaGetLastError();
+    return launch_chained(i1_iter_kernel<T, R>, a.tiles, LK_THREADS, sizeof(float) * i1_smem_floats<R>(r, 2), s, a, r, fp64_cond);
 }
 
 template <int R> cudaError_t i1_launch(const IterArgs &a, int elem, int r, float fp64_cond, cudaStream_t s)
@@ -334,8 +328,7 @@ template <int R> cudaError_t i1_launch(const IterArgs &a, int elem, int r, float
 
 template <typename T, int R> static cudaError_t phase_hess_for(const HessPhase &P, int r, cudaStream_t s)
 {
-    phase_hess_kernel<T, R><<<P.prefix[P.npairs], LK_THREADS, sizeof(float) * i1_smem_floats<R>(r, 3), s>>>(P, r);
-    return cudaGetLastError();
+    return launch_chained(phase_hess_kernel<T, R>, P.prefix[P.npairs], LK_THREADS, sizeof(float) * i1_smem_floats<R>(r, 3), s, P, r);
 }
 
 template <int R> cudaError_t phase_hess_launch(const HessPhase &P, int elem, int r, cudaStream_t s)
@@ -353,9 +346,7 @@ template <int R> cudaError_t phase_hess_launch(const HessPhase &P, int elem, int
 template <typename T, int R>
 static cudaError_t phase_i1_for(const IterPhase &P, int r, float fp64_cond, cudaStream_t s)
 {
-    phase_i1_iter_kernel<T, R><<<P.prefix[P.npairs], LK_THREADS, sizeof(float) * i1_smem_floats<R>(r, 2), s>>>(
-        P, r, fp64_cond);
-    return cudaGetLastError();
+    return launch_chained(phase_i1_iter_kernel<T, R>, P.prefix[P.npairs], LK_THREADS, sizeof(float) * i1_smem_floats<R>(r, 2), s, P, r, fp64_cond);
 }
 
 template <int R> cudaError_t phase_i1_launch(const IterPhase &P, int elem, int r, float fp64_cond, cudaStream_t s)

@@ -193,7 +193,9 @@ int of_compute_batch_host(int32_t n, const of_handle *hs, const void *const *hI1
  *   phased         1: one ordinary launch per phase (pyramid pass, iteration) over all
  *                  pairs' tiles, the pairs' arguments passed as kernel parameters, in
  *                  place of the one persistent launch with grid barriers (then
- *                  blocks_per_sm must be 0)
+ *                  blocks_per_sm must be 0). The persistent launch with grouped sums exists
+ *                  for radii 2-6, 8 and 10 (as do tile_h 32 and fusion 2); other radii from 7
+ *                  to 16 run as phase launches instead
  *   prefetch       phase launches: each iteration block warms L2 with the rows the block
  *                  prefetch x (number of SMs) tiles later will read first (0: off, <= 16)
  *   tile_h         phase launches with grouped sums: height of the 64-wide iteration tile,

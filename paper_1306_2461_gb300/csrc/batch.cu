@@ -260,7 +260,7 @@ static cudaError_t enqueue_chain(const BatchPair *pairs, int n, const of_plan &p
     // iteration tile height: the tuned one for the grouped sums of a specialised radius
     const int tile_h = (t.tile_h == ALT_TH && !t.generic_sums && radius_specialised(p0.radius)) ? ALT_TH : LK_TH;
     // tiles per block of the fixed-radius kernels (the run-time-radius kernel takes one)
-    const int strip = (!t.generic_sums && radius_specialised(p0.radius)) ? strip_len(tuning_strip(t)) : 1;
+    const int strip = (!t.generic_sums && radius_strips(p0.radius, tile_h)) ? strip_len(tuning_strip(t)) : 1;
     cudaError_t e;
     for (int g0 = 0; g0 < n; g0 += PHASE_PAIRS) {
         const int m = n - g0 < PHASE_PAIRS ? n - g0 : PHASE_PAIRS;
@@ -355,7 +355,7 @@ static cudaError_t enqueue_chain(const BatchPair *pairs, int n, const of_plan &p
             long tiles_l = 0;
             for (int i = 0; i < m; ++i) tiles_l += strip_units(bp[i].H[l], bp[i].W[l], tile_h, 1);
             while (kl > 1 && tiles_l < (long)kl * OF_STRIP_WAVES * 4 * sms) kl /= 2;
-            const bool small = !i1grad && !two && tile_h == LK_TH && !t.generic_sums && radius_specialised(p0.radius) &&
+            const bool small = !i1grad && !two && tile_h == LK_TH && !t.generic_sums && radius_grouped(p0.radius) &&
                                prefetch_ahead == 0 && use_small_tiles(tiles_l, sms);
             const int th_l = small ? SM_TH : tile_h;
             for (int i = 0; i < m; ++i) {
@@ -510,6 +510,10 @@ static Tuning effective(const of_plan &p0, Tuning t)
         t.stage_i2 = 0;
         t.tile_h = 0;
         t.fusion = 0;
+    }
+    if (!t.generic_sums && radius_grouped(p0.radius) && !radius_specialised(p0.radius)) {
+        t.phased = 1;   // no persistent kernel with grouped sums for these radii
+        t.blocks_per_sm = 0;
     }
     if (!t.phased || t.generic_sums || !radius_specialised(p0.radius) || (t.tile_h != 0 && t.tile_h != LK_TH))
         t.fusion = 0;

@@ -1,6 +1,7 @@
 // Dispatch of the iteration, window-sum and batch kernels to their per-radius
 // instantiations (radius_<R>.cu): a specialised kernel for the radii listed in
-// OF_RADII, the generic one (radius at run time) for any other.
+// OF_RADII (and, but for the persistent and the fused form, OF_RADII_MORE), the generic one
+// (radius at run time) for any other.
 #include <cudaTypedefs.h>
 
 #include <mutex>
@@ -58,7 +59,7 @@ bool fill_stage_maps(IterArgs &a, StageMaps &m, int elem, int radius, int tile_h
     bool ok = false;
     if (a.stage_i2) {
         switch (radius) {
-            OF_RADII(OF_CASE_SMAP)
+            OF_RADII(OF_CASE_SMAP) OF_RADII_MORE(OF_CASE_SMAP)
         default: ok = false;
         }
     }
@@ -72,7 +73,7 @@ cudaError_t launch_lk_iter(const IterArgs &a, const StageMaps &m, int elem, int 
                            cudaStream_t s)
 {
     switch (radius) {
-        OF_RADII(OF_CASE_LK)
+        OF_RADII(OF_CASE_LK) OF_RADII_MORE(OF_CASE_LK)
     default: return lk_launch<0>(a, m, elem, radius, fp64_cond, false, s);
     }
 }
@@ -82,7 +83,7 @@ cudaError_t launch_lk_iter(const IterArgs &a, const StageMaps &m, int elem, int 
 cudaError_t launch_window_sums(const float *ch, int H, int W, int r, float *out, cudaStream_t s)
 {
     switch (r) {
-        OF_RADII(OF_CASE_WS)
+        OF_RADII(OF_CASE_WS) OF_RADII_MORE(OF_CASE_WS)
     default: return ws_launch<0>(ch, H, W, r, out, s);
     }
 }
@@ -92,7 +93,7 @@ cudaError_t launch_window_sums(const float *ch, int H, int W, int r, float *out,
 cudaError_t launch_i1_hess(const HessArgs &a, int elem, int radius, cudaStream_t s)
 {
     switch (radius) {
-        OF_RADII(OF_CASE_I1H)
+        OF_RADII(OF_CASE_I1H) OF_RADII_MORE(OF_CASE_I1H)
     default: return i1h_launch<0>(a, elem, radius, s);
     }
 }
@@ -102,7 +103,7 @@ cudaError_t launch_i1_hess(const HessArgs &a, int elem, int radius, cudaStream_t
 cudaError_t launch_i1_iter(const IterArgs &a, int elem, int radius, float fp64_cond, cudaStream_t s)
 {
     switch (radius) {
-        OF_RADII(OF_CASE_I1)
+        OF_RADII(OF_CASE_I1) OF_RADII_MORE(OF_CASE_I1)
     default: return i1_launch<0>(a, elem, radius, fp64_cond, s);
     }
 }
@@ -114,7 +115,7 @@ cudaError_t launch_phase_iter(const IterPhase &P, int elem, int radius, bool gen
 {
     if (generic) return phase_launch<0>(P, elem, radius, fp64_cond, LK_TH, s);
     switch (radius) {
-        OF_RADII(OF_CASE_PH)
+        OF_RADII(OF_CASE_PH) OF_RADII_MORE(OF_CASE_PH)
     default: return phase_launch<0>(P, elem, radius, fp64_cond, LK_TH, s);
     }
 }
@@ -135,7 +136,7 @@ cudaError_t launch_phase_hess(const HessPhase &P, int elem, int radius, bool gen
 {
     if (generic) return phase_hess_launch<0>(P, elem, radius, s);
     switch (radius) {
-        OF_RADII(OF_CASE_PHH)
+        OF_RADII(OF_CASE_PHH) OF_RADII_MORE(OF_CASE_PHH)
     default: return phase_hess_launch<0>(P, elem, radius, s);
     }
 }
@@ -147,7 +148,7 @@ cudaError_t launch_phase_i1_iter(const IterPhase &P, int elem, int radius, bool 
 {
     if (generic) return phase_i1_launch<0>(P, elem, radius, fp64_cond, s);
     switch (radius) {
-        OF_RADII(OF_CASE_PHI)
+        OF_RADII(OF_CASE_PHI) OF_RADII_MORE(OF_CASE_PHI)
     default: return phase_i1_launch<0>(P, elem, radius, fp64_cond, s);
     }
 }
@@ -181,6 +182,7 @@ cudaError_t configure_lk_kernels()
 {
     cudaError_t e;
     OF_RADII(OF_CFG)
+    OF_RADII_MORE(OF_CFG)
     OF_CFG(0)
     return cudaSuccess;
 }

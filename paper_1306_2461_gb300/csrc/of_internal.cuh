@@ -212,17 +212,30 @@ constexpr int PYR_THREADS = 256;
 #endif
 constexpr int MAX_RADIUS = OF_MAX_RADIUS;
 
-// Window radii with a kernel specialised at compile time (the workloads' and the
-// paper's radii); any other radius runs the generic kernel.
+// Window radii with kernels specialised at compile time (grouped window sums, staging, strips
+// and small tiles). OF_RADII (the workloads' and the paper's radii) have every form of the
+// batched launch; OF_RADII_MORE the per-pair and phase launches at the default tile height,
+// which keeps the build short. Radius 1 runs the run-time-radius kernel, whose 3-term sums
+// leave nothing to share. Four 499 x 701 pairs at r = 7: 704 us with the run-time-radius
+// kernel (per-output sums, gathered taps), 318 us specialised.
 #define OF_RADII(X) X(2) X(3) X(4) X(5) X(6) X(8) X(10)
+#define OF_RADII_MORE(X) X(7) X(9) X(11) X(12) X(13) X(14) X(15) X(16)
 
-inline bool radius_specialised(int r)
+constexpr bool radius_specialised(int r)   // all forms
 {
 #define OF_IS_RADIUS(R) if (r == R) return true;
     OF_RADII(OF_IS_RADIUS)
-#undef OF_IS_RADIUS
     return false;
 }
+constexpr bool radius_grouped(int r)   // the per-pair and phase launches at least
+{
+    OF_RADII_MORE(OF_IS_RADIUS)
+#undef OF_IS_RADIUS
+    return radius_specialised(r);
+}
+// Strips take over 2r rows of sums from the tile above, which must lie below that tile's own
+// 2r first rows.
+constexpr bool radius_strips(int r, int tile_h) { return radius_grouped(r) && tile_h >= 2 * r; }
 
 // ------------------------------------------------------------- chained launches
 // The launches of a method's sequence after its first, when they go to a stream directly (no

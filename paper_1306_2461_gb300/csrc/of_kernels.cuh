@@ -1501,7 +1501,7 @@ __device__ __forceinline__ bool lk_tile_fixed(const IterArgs &a, const StageMaps
 {
     using F = FixedTile<R, TH>;
     static_assert(REF_GROUP % 4 == 0, "strips of 1, 2 or 4 tiles inside a group");
-    static_assert(TH >= 2 * R && TH % 2 == 0, "the rows taken over lie below the tile above's own 2R first rows");
+    static_assert(!MULTI || (TH >= 2 * R && TH % 2 == 0), "the rows taken over lie below the tile above's own 2R first rows");
     const int K = strip_len(a.strip);
     const int uy = unit / a.tiles_x;
     const int tx0 = (unit - uy * a.tiles_x) * LK_TW;

@@ -13,6 +13,10 @@
 
 namespace of {
 
+// Radii with every form of the batched launch (0: the run-time-radius kernel); the others
+// have the per-pair and phase launches at the default tile height.
+template <int R> constexpr bool all_forms() { return R == 0 || radius_specialised(R); }
+
 template <typename T, int R>
 __global__ void __launch_bounds__(LK_THREADS, lk_min_blocks<R>())
 lk_iter_kernel(const __grid_constant__ IterArgs a, const __grid_constant__ StageMaps m, int r, float fp64_cond)
@@ -80,7 +84,7 @@ phase_iter_kernel(const __grid_constant__ IterPhase P, int r, float fp64_cond)
             prefetch_tile<T, MODE, TH>(P.a[q], t2 - P.prefix[q], R);
         }
     }
-    lk_tile<T, false, R, MODE, TH>(P.a[p], &P.m[p], blockIdx.x - P.prefix[p], r, fp64_cond, smem, phase);
+    lk_tile<T, false, R, MODE, TH, (TH >= 2 * R)>(P.a[p], &P.m[p], blockIdx.x - P.prefix[p], r, fp64_cond, smem, phase);
 }
 
 // Two same-level iterations of up to PHASE_PAIRS pairs in one launch (iteration fusion
@@ -249,7 +253,8 @@ static cudaError_t phase_for(const IterPhase &P, int r, float fp64_cond, int til
             default: return launch_chained(phase_small_kernel<T, R, FLOW_UPSAMPLE>, blocks, SM_THREADS, smem, s, P, fp64_cond);
             }
         }
-        if (tile_h == ALT_TH) return phase_for_th<T, R, ALT_TH>(P, r, fp64_cond, s);
+        if constexpr (all_forms<R>())
+            if (tile_h == ALT_TH) return phase_for_th<T, R, ALT_TH>(P, r, fp64_cond, s);
     }
     return phase_for_th<T, R, LK_TH>(P, r, fp64_cond, s);
 }
@@ -280,7 +285,7 @@ template <typename T, int R> static cudaError_t phase2_for(const IterPhase &P, f
 
 template <int R> cudaError_t phase2_launch(const IterPhase &P, int elem, float fp64_cond, cudaStream_t s)
 {
-    if constexpr (R == 0) {
+    if constexpr (R == 0 || !all_forms<R>()) {
         return cudaErrorInvalidValue;   // fusion needs a fixed-radius kernel
     } else {
         if (P.prefix[P.npairs] == 0) return cudaSuccess;
@@ -367,6 +372,12 @@ template <int R, int TH, int TW = LK_TW> static bool stage_maps_th(const IterArg
 {
     using F = FixedTile<R, TH, TW>;
     const int S = elem_bytes(elem);
+    // a window that leaves one block per SM where two would fit gathered (r = 16, and r = 13
+    // on with 4-byte levels) costs more than it saves: eight 1024^2 pairs at r = 16 3147 us
+    // staged, 2574 gathered
+    constexpr int SM_BYTES = 228 * 1024, BLOCK_BYTES = 1024;   // shared memory per SM, and reserved per block
+    if (2 * (4 * F::smem_staged(S) + BLOCK_BYTES) > SM_BYTES && 2 * (4 * F::SMEM_NOSTAGE + BLOCK_BYTES) <= SM_BYTES)
+        return false;
     if (a.mode == FLOW_SAME &&
         !encode_tile_map(&m.flow, ET_FLOW2, a.fin, a.W, a.H, (size_t)a.fin_pitch * 8, F::RWP2, F::FLOW_BH))
         return false;
@@ -379,7 +390,7 @@ template <int R> bool radius_stage_maps(const IterArgs &a, StageMaps &m, int ele
         return false;
     } else {
         if (tile_h == SM_TH) return stage_maps_th<R, SM_TH, SM_TW>(a, m, elem);
-        return tile_h == ALT_TH ? stage_maps_th<R, ALT_TH>(a, m, elem) : stage_maps_th<R, LK_TH>(a, m, elem);
+        return tile_h == ALT_TH && all_forms<R>() ? stage_maps_th<R, ALT_TH>(a, m, elem) : stage_maps_th<R, LK_TH>(a, m, elem);
     }
 }
 
@@ -414,7 +425,7 @@ template <int R> cudaError_t radius_configure()
     OF_SET_PH(__half);
     OF_SET_PH(__nv_bfloat16);
 #undef OF_SET_PH
-    if constexpr (R != 0) {   // the other tile height of the phase kernels
+    if constexpr (R != 0 && all_forms<R>()) {   // the other tile height of the phase kernels
         const int alt = (int)sizeof(float) * lk_tile_smem_floats<R, ALT_TH>(R, true);
 #define OF_SET_ALT(T)                                                                                       \
     for (const void *fn : {(const void *)phase_iter_kernel<T, R, FLOW_ZERO, ALT_TH>,                        \
@@ -445,7 +456,7 @@ template <int R> cudaError_t radius_configure()
         OF_SET_SM(__nv_bfloat16)
 #undef OF_SET_SM
     }
-    if constexpr (R != 0) {   // the fused two-iteration kernels
+    if constexpr (R != 0 && all_forms<R>()) {   // the fused two-iteration kernels
         const int fb = (int)fused2_smem_bytes<R>();
         for (const void *fn : {(const void *)phase_iter2_kernel<uint8_t, R>, (const void *)phase_iter2_kernel<uint16_t, R>,
                                (const void *)phase_iter2_kernel<float, R>, (const void *)phase_iter2_kernel<__half, R>,
@@ -472,8 +483,9 @@ template <int R> cudaError_t radius_configure()
         OF_SET_I1(__nv_bfloat16)
 #undef OF_SET_I1
     }
-    for (int f = 0; f < 2; ++f)
-        for (int st = 0; st < 3; ++st) OF_SET(batch_kernel_ptr<R>(f, st));
+    if constexpr (all_forms<R>())
+        for (int f = 0; f < 2; ++f)
+            for (int st = 0; st < 3; ++st) OF_SET(batch_kernel_ptr<R>(f, st));
 #undef OF_SET
     return cudaSuccess;
 }
@@ -485,7 +497,9 @@ template cudaError_t phase_launch<OF_RADIUS>(const IterPhase &, int, int, float,
 template cudaError_t phase_hess_launch<OF_RADIUS>(const HessPhase &, int, int, cudaStream_t);
 template cudaError_t phase_i1_launch<OF_RADIUS>(const IterPhase &, int, int, float, cudaStream_t);
 template cudaError_t i1_launch<OF_RADIUS>(const IterArgs &, int, int, float, cudaStream_t);
+#ifndef OF_RADIUS_MORE   // one of OF_RADII_MORE
 template void *batch_kernel_ptr<OF_RADIUS>(int, int);
+#endif
 template bool radius_stage_maps<OF_RADIUS>(const IterArgs &, StageMaps &, int, int);
 template cudaError_t phase2_launch<OF_RADIUS>(const IterPhase &, int, float, cudaStream_t);
 template cudaError_t radius_configure<OF_RADIUS>();

@@ -156,11 +156,13 @@ int of_autotune_batch(int32_t n, const of_handle *hs, const void *const *I1s, co
     const int occ[6] = {-1, -2, -3, 0, 2, 1};   // < 0: phase launches with prefetch pf_of[-1 - b]
     const int pf_of[3] = {0, 1, 3};
     const bool variant = (p0.flags & OF_FLAG_I1GRAD) != 0;
-    for (int gs = radius_specialised(p0.radius) ? 0 : 1; gs <= 1; ++gs)
+    const bool more = radius_grouped(p0.radius) && !radius_specialised(p0.radius);   // phase launches, one tile height
+    for (int gs = radius_grouped(p0.radius) ? 0 : 1; gs <= 1; ++gs)
         for (int sg = 0; sg <= (gs ? 0 : 1); ++sg)
-            for (int th = 0; th <= ((gs || variant) ? 0 : 1); ++th)
+            for (int th = 0; th <= ((gs || variant || more) ? 0 : 1); ++th)
                 for (int b : occ) {
                     if (variant && (b >= 0 || sg)) continue;   // phase launches, gathered taps only
+                    if (more && !gs && b >= 0) continue;       // no persistent form
                     if (th && b >= 0) continue;                // the persistent launch has one tile height
                     if (sg && b >= 0) continue;                // and gathers its taps
                     Tuning t;
@@ -170,13 +172,13 @@ int of_autotune_batch(int32_t n, const of_handle *hs, const void *const *I1s, co
                     t.blocks_per_sm = b < 0 ? 0 : b;
                     t.prefetch = b < 0 ? pf_of[-1 - b] : 0;
                     t.tile_h = th ? ALT_TH : 0;
-                    t.strip = (t.phased && !gs) ? 0 : 1;
+                    t.strip = (t.phased && !gs && radius_strips(p0.radius, LK_TH)) ? 0 : 1;
                     cand.push_back(t);
                     if (t.phased && t.prefetch == 0 && n > 1) {
                         t.branches = 2;
                         cand.push_back(t);
                     }
-                    if (t.phased && !gs && sg && !th && t.prefetch == 0) {
+                    if (t.phased && !gs && sg && !th && t.prefetch == 0 && t.strip != 1) {
                         // one tile per block (every tile its own stage 1 and horizontal pass)
                         t.strip = 1;
                         t.branches = 0;

@@ -395,7 +395,7 @@ static cudaError_t enqueue_chain(const BatchPair *pairs, int n, const of_plan &p
                     a.tiles_x = small_tiles_x(a.W);
                     a.tiles = small_units(a.H, a.W);
                 }
-                if (a.stage_i2) fill_stage_maps(a, I.m[i], level_elem(p0, l), p0.radius, th_l);   // else gathered
+                if (a.stage_i2) fill_stage_maps(a, I.m[i], level_elem(p0, l), p0.radius, th_l, true);   // else gathered
                 a.hess = bp[i].hess;
                 a.hess_pitch = bp[i].pitch[l];
                 I.prefix[i + 1] = I.prefix[i] + a.tiles;

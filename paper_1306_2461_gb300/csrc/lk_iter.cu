@@ -53,8 +53,8 @@ bool encode_tile_map(CUtensorMap *m, int elem, const void *base, int W, int H, s
 }
 
 #define OF_CASE_SMAP(R) \
-    case R: ok = radius_stage_maps<R>(a, m, elem, tile_h); break;
-bool fill_stage_maps(IterArgs &a, StageMaps &m, int elem, int radius, int tile_h)
+    case R: ok = radius_stage_maps<R>(a, m, elem, tile_h, strips); break;
+bool fill_stage_maps(IterArgs &a, StageMaps &m, int elem, int radius, int tile_h, bool strips)
 {
     bool ok = false;
     if (a.stage_i2) {

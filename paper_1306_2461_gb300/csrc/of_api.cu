@@ -227,7 +227,7 @@ cudaError_t enqueue_pair(of_ctx *h, const void *I1, const void *I2, float *u, fl
                 a.tiles_x = small_tiles_x(a.W);
                 a.tiles = small_units(a.H, a.W);
             }
-            if (a.stage_i2) fill_stage_maps(a, maps, level_elem(p, l), p.radius, small ? SM_TH : LK_TH);   // else gathered
+            if (a.stage_i2) fill_stage_maps(a, maps, level_elem(p, l), p.radius, small ? SM_TH : LK_TH, false);   // else gathered
             if (i1grad) {
                 a.hess = h->hess;
                 a.hess_pitch = L.pitch[l];

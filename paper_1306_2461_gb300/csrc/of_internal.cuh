@@ -312,7 +312,8 @@ cudaError_t configure_lk_kernels();   // all kernels with dynamic shared memory,
 // height (level image type elem). Returns false (and clears a.stage_i2) when the radius
 // has no fixed-radius kernel or the tensor maps cannot be encoded; the tile then
 // gathers from global memory.
-bool fill_stage_maps(IterArgs &a, StageMaps &m, int elem, int radius, int tile_h);
+// strips: for the phase launches, whose 64-wide tiles come in strips.
+bool fill_stage_maps(IterArgs &a, StageMaps &m, int elem, int radius, int tile_h, bool strips);
 // Encode a 2-D tiled tensor map: W x H elements of elem_bytes with rows pitch_bytes apart,
 // boxes of box_w x box_h, zero fill outside. False if the driver entry point is missing or
 // the encoding fails.
@@ -334,7 +335,7 @@ template <int R> cudaError_t i1_launch(const IterArgs &a, int elem, int r, float
 template <int R> void *batch_kernel_ptr(int in_format, int storage);
 template <int R> cudaError_t radius_configure();
 template <int R> size_t radius_smem_bytes(int r, bool stage_i2);
-template <int R> bool radius_stage_maps(const IterArgs &a, StageMaps &m, int elem, int tile_h);
+template <int R> bool radius_stage_maps(const IterArgs &a, StageMaps &m, int elem, int tile_h, bool strips);
 template <int R> cudaError_t phase2_launch(const IterPhase &P, int elem, float fp64_cond, cudaStream_t s);
 
 }  // namespace of

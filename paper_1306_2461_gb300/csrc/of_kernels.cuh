@@ -531,30 +531,36 @@ __device__ __forceinline__ void box_vsum(const float *S, int RH, int r, int ty, 
 // det <= 1e-6 tr^2. Pixels with tr^2/det above fp64_cond (or det <= 0) form the
 // determinant and the numerators in FP64 from the FP32 sums; fp64_cond == 0 keeps
 // everything in FP32.
+// The well-conditioned pixels take one branch; the others decide in solve2_other.
+__device__ __forceinline__ bool solve2_other(float a, float b, float c, float d, float e, float fp64_cond, float tr,
+                                             float det, float &xu, float &xv)
+{
+    if (!(tr > 0.0f) || !(fp64_cond > 0.0f && !(det * fp64_cond > tr * tr))) return false;
+    // ill-conditioned: the determinant and the numerators, where the cancellation
+    // is, in FP64 from the FP32 sums (the products are exact, one rounding each);
+    // the final divisions in FP32
+    const double A = a, B = b, C = c, D = d, E = e;
+    const double T = A + C, dt = fma(A, C, -__dmul_rn(B, B));
+    if (!(dt > 1e-6 * T * T)) return false;
+    const float fdt = (float)dt;
+    if (!(fdt >= FLT_MIN)) return false;
+    xu = __fdiv_rn((float)fma(C, D, -__dmul_rn(B, E)), fdt);
+    xv = __fdiv_rn((float)fma(A, E, -__dmul_rn(B, D)), fdt);
+    return true;
+}
 __device__ __forceinline__ bool solve2(const float s[5], float fp64_cond, float &xu, float &xv)
 {
     const float a = s[0], b = s[1], c = s[2], d = s[3], e = s[4];
     const float tr = a + c;
-    if (!(tr > 0.0f)) return false;
     const float det = fmaf(a, c, -__fmul_rn(b, b));
-    if (fp64_cond > 0.0f && !(det * fp64_cond > tr * tr)) {
-        // ill-conditioned: the determinant and the numerators, where the cancellation
-        // is, in FP64 from the FP32 sums (the products are exact, one rounding each);
-        // the final divisions in FP32
-        const double A = a, B = b, C = c, D = d, E = e;
-        const double T = A + C, dt = fma(A, C, -__dmul_rn(B, B));
-        if (!(dt > 1e-6 * T * T)) return false;
-        const float fdt = (float)dt;
-        if (!(fdt >= FLT_MIN)) return false;
-        xu = __fdiv_rn((float)fma(C, D, -__dmul_rn(B, E)), fdt);
-        xv = __fdiv_rn((float)fma(A, E, -__dmul_rn(B, D)), fdt);
+    const bool well = !(fp64_cond > 0.0f) || det * fp64_cond > tr * tr;
+    if (tr > 0.0f & well & det > 1e-6f * tr * tr) {
+        const float inv = __fdividef(1.0f, det);   // det < 2^126 for any sums of 16-bit data
+        xu = fmaf(c, d, -__fmul_rn(b, e)) * inv;
+        xv = fmaf(a, e, -__fmul_rn(b, d)) * inv;
         return true;
     }
-    if (!(det > 1e-6f * tr * tr)) return false;
-    const float inv = __fdividef(1.0f, det);   // det < 2^126 for any sums of 16-bit data
-    xu = fmaf(c, d, -__fmul_rn(b, e)) * inv;
-    xv = fmaf(a, e, -__fmul_rn(b, d)) * inv;
-    return true;
+    return solve2_other(a, b, c, d, e, fp64_cond, tr, det, xu, xv);
 }
 
 inline __host__ __device__ int lk_smem_floats(int r)   // generic tile
@@ -677,21 +683,13 @@ template <int R, int TH = LK_TH, int TW = LK_TW> struct FixedTile {
     static constexpr int PLANES = 4 * PAIR_PLANE + RH * RWP1;  // floats of the three planes
     static_assert(PLANES % 4 == 0, "the barrier after the planes must be 8-byte aligned");
     static constexpr int OFF_BAR = PLANES;                    // 8-byte mbarrier
-    static constexpr int OFF_WREF = OFF_BAR + 2;              // a strip's tile-centre estimates (4 float2)
-    static constexpr int OFF_WIN = (OFF_WREF + 8 + 31) / 32 * 32;   // 128-byte aligned staging window
+    static constexpr int OFF_WIN = (OFF_BAR + 2 + 31) / 32 * 32;   // 128-byte aligned staging window
     static constexpr int SMEM_NOSTAGE = OFF_WIN;              // launches without staging
     static constexpr int smem_staged(int S) { return OFF_WIN + (win_bytes(S) + 15) / 16 * 4; }
     static constexpr int SMEM_FLOATS = smem_staged(4);        // the largest (FP32 storage)
-    // The staged flow estimate: TMA boxes of RWP2 x FLOW_BH 8-byte elements written over
-    // P01. Where row 2R (the first below the 2R rows a tile of a strip takes over from the
-    // tile above) starts on a 128-byte boundary (R a multiple of 4), boxes of 2R rows when
-    // they tile TH, so that every row of a region is staged (RH / 2R boxes for a strip's
-    // first tile, TH / 2R for the others), else one box of TH rows at row 2R; elsewhere one
-    // box of TH rows at row 0 for a strip's first tile, the other rows' estimates read from
-    // global memory.
-    // Tiles narrower than LK_TW are never part of a strip: one box of the whole region.
-    static constexpr bool FLOW_BOX_BELOW = (2 * R * RWP2 * 8) % 128 == 0;
-    static constexpr int FLOW_BH = TW < 64 ? RH : (FLOW_BOX_BELOW && TH % (2 * R) == 0 ? 2 * R : TH);
+    // The staged flow estimate: one TMA box of the region's RH rows of RWP2 8-byte elements,
+    // written over P01 (strips: see StripTile).
+    static constexpr int FLOW_BH = RH;
     static constexpr int FLOW_BOX_BYTES = RWP2 * FLOW_BH * 8;
 #ifndef OF_LK_MIN_BLOCKS
 #define OF_LK_MIN_BLOCKS 4   // resident blocks per SM the fixed-radius kernels are compiled for (R <= 6)
@@ -703,17 +701,33 @@ template <int R, int TH = LK_TH, int TW = LK_TW> struct FixedTile {
         TH == LK_TH ? (R <= 6 ? OF_LK_MIN_BLOCKS : 2) : (SMEM_FIT < 1 ? 1 : (SMEM_FIT > 5 ? 5 : SMEM_FIT));
 };
 
+// Shared memory of a strip's tiles: the planes are rings of RING rows. Region row ry of a tile
+// is in slot (ring + RPAD + ry) mod RING, ring a multiple of 8 that moves on by TH from tile to
+// tile; RPAD puts the first row after the 2R carried ones in a slot that is a multiple of 8
+// (a 128-byte boundary), so that the estimate of the rows a tile computes comes in TMA boxes
+// of 8 rows.
+template <int R, int TH> struct StripTile {
+    using F = FixedTile<R, TH>;
+    static_assert(TH % 8 == 0, "boxes of 8 rows");
+    static constexpr int RPAD = (8 - 2 * R % 8) % 8;
+    static constexpr int RING = RPAD + F::RH;
+    static constexpr int BOX = 8;
+    static constexpr int BOX_BYTES = F::RWP2 * BOX * 8;
+    static constexpr int PAIR_PLANE = RING * F::RWP2;
+    static constexpr int PLANES = 4 * PAIR_PLANE + RING * F::RWP1;
+    static constexpr int OFF_BAR = PLANES;
+    static constexpr int OFF_WREF = OFF_BAR + 2;              // the tile-centre estimates (4 float2)
+    static constexpr int OFF_WIN = (OFF_WREF + 8 + 31) / 32 * 32;
+    static constexpr int SMEM_NOSTAGE = OFF_WIN;
+    static constexpr int smem_staged(int S) { return OFF_WIN + (F::win_bytes(S) + 15) / 16 * 4; }
+};
+
 // Staged tile, while its boxes land: 0 no prefetch, 1 warm L2 with the region's I1 rows,
 // 2 bring the region's I1 lines (and, upsampling, the coarser estimate's) into L1. With 4
 // resident blocks per SM their lines (4.6 KB per 64 x 24 tile of 16-bit data) fit in what
 // the shared-memory carve-out leaves of L1; 2 measured 1.9% faster per batch step than 0.
 #ifndef OF_PREFETCH_I1
 #define OF_PREFETCH_I1 2
-#endif
-// Strips: request a later tile's window of I2 while the tile above finishes (1), or at
-// the tile's own staging (0).
-#ifndef OF_EARLY_WINDOW
-#define OF_EARLY_WINDOW 1
 #endif
 constexpr long long STAGE_TIMEOUT_NS = 200000000LL;   // 0.2 s for one tile's staging copies
 
@@ -939,14 +953,23 @@ __device__ __forceinline__ void box4v(const V *v, V o[4])
     o[3] = vadd(vadd(vadd(m, v[OFF + 2 * R + 1]), v[OFF + 2 * R + 2]), v[OFF + 2 * R + 3]);
 }
 
+// Slot of region row ry in a ring of RN rows whose row 0 is in slot `base` (0 .. RN-1); single
+// tiles (RN = 0) keep their rows in order.
+template <int RN> __device__ __forceinline__ int ring_slot(int ry, int base)
+{
+    if constexpr (RN == 0) return ry;
+    const int s = ry + base;
+    return s >= RN ? s - RN : s;
+}
+
 // Horizontal pass of one pair plane, in place, over rows r0..RH-1: row ry becomes, at
 // columns 0..TW-1, the window sums of its outputs (two channels per float2). Chunk c of
 // rows goes to warp (c + woff) mod WARPS. For 64- and 32-wide tiles a warp takes two or
 // four rows and a quarter warp 4 groups of 4 outputs of two of them (with rows RWP2 = 2 mod 4
 // float2 long, its 16-byte reads hit distinct banks); other widths take one row per warp,
 // one group per lane. Each row is read and rewritten by one warp.
-template <int R, int TH, int TW = LK_TW, int NT = LK_THREADS>
-__device__ __forceinline__ void box_h_pairs(float2 *P, int r0 = 0, int woff = 0)
+template <int R, int TH, int TW = LK_TW, int NT = LK_THREADS, int RN = 0>
+__device__ __forceinline__ void box_h_pairs(float2 *P, int r0 = 0, int woff = 0, int base = 0)
 {
     using F = FixedTile<R, TH, TW>;
     static_assert(NT % 32 == 0, "whole warps");
@@ -962,7 +985,7 @@ __device__ __forceinline__ void box_h_pairs(float2 *P, int r0 = 0, int woff = 0)
     for (int chunk = ((threadIdx.x >> 5) + WARPS - woff) % WARPS; chunk < chunks; chunk += WARPS) {
         const int ry = r0 + RPC * chunk + rsub;
         const bool act = (RPC != 1 || g < NG) && (RPC != 4 || ry < F::RH);
-        float4 *row = reinterpret_cast<float4 *>(P) + (ry * RW4 + 2 * g);
+        float4 *row = reinterpret_cast<float4 *>(P) + (ring_slot<RN>(ry, base) * RW4 + 2 * g);
         float2 o[4];
         if (act) {
             float2 v[4 * F::NVE];
@@ -984,8 +1007,8 @@ __device__ __forceinline__ void box_h_pairs(float2 *P, int r0 = 0, int woff = 0)
 
 // Horizontal pass of the float plane P4, in place, over rows r0..RH-1: for 64- and 32-wide
 // tiles the items of a row lie in one warp, else one row per warp.
-template <int R, int TH, int TW = LK_TW, int NT = LK_THREADS>
-__device__ __forceinline__ void box_h_single(float *P, int r0 = 0)
+template <int R, int TH, int TW = LK_TW, int NT = LK_THREADS, int RN = 0>
+__device__ __forceinline__ void box_h_single(float *P, int r0 = 0, int base = 0)
 {
     using F = FixedTile<R, TH, TW>;
     constexpr int NG = TW / 4;
@@ -998,7 +1021,7 @@ __device__ __forceinline__ void box_h_single(float *P, int r0 = 0)
             const int i = threadIdx.x + k * NT;
             if (i < nitems) {
                 const int ry = r0 + i / NG, g = i % NG;
-                const float4 *src = reinterpret_cast<const float4 *>(P + ry * F::RWP1 + 4 * g);
+                const float4 *src = reinterpret_cast<const float4 *>(P + ring_slot<RN>(ry, base) * F::RWP1 + 4 * g);
                 float v[4 * F::NVE];
 #pragma unroll
                 for (int q = 0; q < F::NVE; ++q) {
@@ -1019,7 +1042,7 @@ __device__ __forceinline__ void box_h_single(float *P, int r0 = 0)
             const int i = threadIdx.x + k * NT;
             if (i < nitems) {
                 const int ry = r0 + i / NG, g = i % NG;
-                *reinterpret_cast<float4 *>(P + ry * F::RWP1 + 4 * g) = res[k];
+                *reinterpret_cast<float4 *>(P + ring_slot<RN>(ry, base) * F::RWP1 + 4 * g) = res[k];
             }
         }
     } else {
@@ -1074,32 +1097,35 @@ __device__ __forceinline__ void box6v(const V *v, V o[6])
 template <int R, int TH> constexpr int v_rows() { return (TH % 6 == 0 && R >= 3) ? 6 : 4; }
 
 // Vertical pass for the VR = v_rows outputs of item g (rows VR g .. VR g + VR - 1, column
-// tx): sums of the three planes.
-template <int R, int TH, int TW = LK_TW>
+// tx): sums of the three planes. The rows read wrap around once at most in a ring.
+template <int R, int TH, int TW = LK_TW, int RN = 0>
 __device__ __forceinline__ void box_v_planes(const float2 *P01, const float2 *P23, const float *P4, int g, int tx,
                                              float2 s01[v_rows<R, TH>()], float2 s23[v_rows<R, TH>()],
-                                             float s4[v_rows<R, TH>()])
+                                             float s4[v_rows<R, TH>()], int base = 0)
 {
     using F = FixedTile<R, TH, TW>;
     constexpr int VR = v_rows<R, TH>(), NV = 2 * R + VR;
+    const int s0 = ring_slot<RN>(VR * g, base), nq = RN ? RN - s0 : NV;   // rows nq.. are in slots 0..
+    const int o2 = s0 * F::RWP2 + tx, w2 = o2 - RN * F::RWP2;
+    const int o1 = s0 * F::RWP1 + tx, w1 = o1 - RN * F::RWP1;
     {
         float2 v[NV];
 #pragma unroll
-        for (int q = 0; q < NV; ++q) v[q] = P01[(VR * g + q) * F::RWP2 + tx];
+        for (int q = 0; q < NV; ++q) v[q] = P01[(RN == 0 || q < nq ? o2 : w2) + q * F::RWP2];
         if constexpr (VR == 6) box6v<R>(v, s01);
         else box4v<R, 0>(v, s01);
     }
     {
         float2 v[NV];
 #pragma unroll
-        for (int q = 0; q < NV; ++q) v[q] = P23[(VR * g + q) * F::RWP2 + tx];
+        for (int q = 0; q < NV; ++q) v[q] = P23[(RN == 0 || q < nq ? o2 : w2) + q * F::RWP2];
         if constexpr (VR == 6) box6v<R>(v, s23);
         else box4v<R, 0>(v, s23);
     }
     {
         float v[NV];
 #pragma unroll
-        for (int q = 0; q < NV; ++q) v[q] = P4[(VR * g + q) * F::RWP1 + tx];
+        for (int q = 0; q < NV; ++q) v[q] = P4[(RN == 0 || q < nq ? o1 : w1) + q * F::RWP1];
         if constexpr (VR == 6) box6v<R>(v, s4);
         else box4v<R, 0>(v, s4);
     }
@@ -1266,184 +1292,158 @@ __device__ __forceinline__ void win_origin(const IterArgs &a, int tx0, int ty0, 
 }
 
 // The tile's mbarrier: initialised once per block, before the first tile.
-template <int R, int TH = LK_TH, int TW = LK_TW> __device__ __forceinline__ void lk_tile_init(float *smem)
+template <int R, int TH = LK_TH, int TW = LK_TW, bool MULTI = false> __device__ __forceinline__ void lk_tile_init(float *smem)
 {
     if (threadIdx.x == 0) {
-        mbar_init(reinterpret_cast<uint64_t *>(smem + FixedTile<R, TH, TW>::OFF_BAR), 1);
+        constexpr int off = [] {
+            if constexpr (MULTI) return StripTile<R, TH>::OFF_BAR;
+            else return FixedTile<R, TH, TW>::OFF_BAR;
+        }();
+        mbar_init(reinterpret_cast<uint64_t *>(smem + off), 1);
         fence_proxy_async_smem();
     }
     __syncthreads();
 }
 
-// One tile of a work unit (lk_tile_fixed). A tile after the first of its strip takes over
-// region rows 0..2R-1 from the tile above; CM = 0: a first tile, 1: a later one, 2: as
-// `carry_rt` says at run time (one body for both, the loop of a strip). At CM 2 with
-// staging, wrefs[0] is this tile's window estimate (win_ref) and wrefs[1] the next one's
-// when `next` (a tile of the same strip follows): that tile's window is then requested as
-// soon as this tile's stage 1 is done, and a later tile of a strip requests only its flow
-// boxes. Returns false if a staging copy did not complete in time.
-template <typename T, bool NC, int R, int MODE, int TH, int CM, int TW = LK_TW, int NT = LK_THREADS>
-__device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps *maps, int tx0, int ty0, float2 ref,
-                                             float fp64_cond, float *smem, uint32_t &phase, bool carry_rt,
-                                             const float2 *wrefs = nullptr, bool next = false)
+// The solve of one output pixel from its window sums, and the store of its new estimate
+// (pixels below the image, in: false, are computed and dropped).
+template <bool NC, int MODE>
+__device__ __forceinline__ void solve_store(const IterArgs &a, int x, int y, float2 ref, float fp64_cond, float2 s01,
+                                            float2 s23, float s4)
 {
-    const bool CARRY = CM == 2 ? carry_rt : CM == 1;
+    const float sj[5] = {s01.x, s01.y, s23.x, s23.y, s4};
+    float xu, xv;
+    const float2 f = solve2(sj, fp64_cond, xu, xv) ? make_float2(ref.x + xu, ref.y + xv) : flow_mode<NC, MODE>(a, x, y);
+    if (a.fout) {
+        a.fout[(size_t)y * a.fout_pitch + x] = f;
+    } else {
+        a.u_out[(size_t)y * a.W + x] = f.x;
+        a.v_out[(size_t)y * a.W + x] = f.y;
+    }
+}
+
+// While a tile's copies land: bring the lines of I1 that its stage 1 reads (region rows r0..)
+// into L1 (OF_PREFETCH_I1 2; 1: into L2), and at the first iteration of a level those of the
+// coarser estimate it upsamples. Threads [t0, NT) take part.
+template <int R, int MODE, int TH, int TW, int NT, int S>
+__device__ __forceinline__ void prefetch_region(const IterArgs &a, int tx0, int ty0, int r0, int t0)
+{
+    using F = FixedTile<R, TH, TW>;
+    const int t = (int)threadIdx.x - t0;
+    if (t < 0) return;
+#if OF_PREFETCH_I1 == 1
+    if (t < F::RH - r0)
+        prefetch_row(a.I1, a.pitch, S, a.H, a.W, ty0 - R + r0, ty0 - R + F::RH, tx0 - F::RE, tx0 - F::RE + F::RWE, t);
+#elif OF_PREFETCH_I1 == 2
+    constexpr int LPR = (F::RWE * S + 127) / 128 + 1;
+    constexpr int CRH = F::RH / 2 + 2, CLPR = ((F::RWE / 2 + 2) * 8 + 127) / 128 + 1;
+    const int n1 = (F::RH - r0) * LPR;
+    const int n = n1 + (MODE == FLOW_UPSAMPLE ? CRH * CLPR : 0);
+    for (int i = t; i < n; i += NT - t0) {
+        if (i < n1)
+            prefetch_lines_l1(a.I1, a.pitch, S, a.H, a.W, ty0 - R + r0, ty0 - R + F::RH, tx0 - F::RE,
+                              tx0 - F::RE + F::RWE, LPR, i);
+        else
+            prefetch_lines_l1(a.fin, a.fin_pitch, 8, a.Hc, a.Wc, (ty0 - R) >> 1, ((ty0 - R) >> 1) + CRH,
+                              (tx0 - F::RE) >> 1, ((tx0 - F::RE) >> 1) + F::RWE / 2 + 2, CLPR, i - n1);
+    }
+#endif
+}
+
+// Whether the tile's region and its staged window both lie inside the image: no pixel pair of
+// its stage 1 then needs a bounds check.
+template <int R, int TH, int TW, int S>
+__device__ __forceinline__ bool tile_inner(const IterArgs &a, int tx0, int ty0, int wx0, int wy0)
+{
+    using F = FixedTile<R, TH, TW>;
+    return wx0 >= 0 && wy0 >= 0 && wx0 + F::win_w(S) <= a.W && wy0 + F::WIN_H <= a.H && tx0 >= F::RE && ty0 >= R &&
+           tx0 + TW + F::RE <= a.W && ty0 + TH + R <= a.H;
+}
+
+// Wait for the copies of the barrier's current phase. False (for the whole block) if they did
+// not complete in time: recorded in the status word, and the block must stop.
+__device__ __forceinline__ bool stage_wait(const IterArgs &a, uint64_t *bar, uint32_t &phase)
+{
+    const bool done = mbar_wait_bounded(bar, phase, STAGE_TIMEOUT_NS);
+    if (__syncthreads_or(!done)) {
+        // give the copies in flight a further bounded wait before the block leaves
+        if (!done) mbar_wait_bounded(bar, phase, STAGE_TIMEOUT_NS);
+        if (threadIdx.x == 0 && a.status) atomicExch(a.status, DEV_TIMEOUT);
+        return false;
+    }
+    phase ^= 1u;
+    return true;
+}
+
+// A single tile (TW x TH outputs at (tx0, ty0), NT threads). Returns false if a staging copy
+// did not complete in time.
+template <typename T, bool NC, int R, int MODE, int TH, int TW = LK_TW, int NT = LK_THREADS>
+__device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps *maps, int tx0, int ty0, float2 ref,
+                                             float fp64_cond, float *smem, uint32_t &phase)
+{
     using F = FixedTile<R, TH, TW>;
     unsigned char *win = reinterpret_cast<unsigned char *>(smem + F::OFF_WIN);
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + F::OFF_BAR);
     constexpr int S = (int)sizeof(T);
     constexpr int WW = F::win_w(S);
-    constexpr bool SAME = MODE == FLOW_SAME;
     float2 *P01 = reinterpret_cast<float2 *>(smem);
     float2 *P23 = P01 + F::PAIR_PLANE;
     float *P4 = reinterpret_cast<float *>(P23 + F::PAIR_PLANE);
     const bool staged = maps && a.stage_i2 != 0;
-    const int r0 = CARRY ? 2 * R : 0;   // the first region row this tile computes
     __syncthreads();   // the previous tile's readers of smem are done
-    if (CARRY) {
-        // region rows TH .. TH+2R-1 of the tile above are rows 0 .. 2R-1 of this one:
-        // their window sums along x (columns 0..TW-1 of each plane) move up
-        constexpr int Q2 = TW / 2, Q1 = TW / 4;   // float4 per row: pair planes, P4
-        constexpr int N = 2 * R * (2 * Q2 + Q1);
-        for (int i = threadIdx.x; i < N; i += NT) {
-            const int row = i / (2 * Q2 + Q1), c = i - row * (2 * Q2 + Q1);
-            float4 *dst, *src;
-            if (c < 2 * Q2) {
-                float2 *P = c < Q2 ? P01 : P23;
-                const int q = c < Q2 ? c : c - Q2;
-                dst = reinterpret_cast<float4 *>(P + row * F::RWP2) + q;
-                src = reinterpret_cast<float4 *>(P + (row + TH) * F::RWP2) + q;
-            } else {
-                dst = reinterpret_cast<float4 *>(P4 + row * F::RWP1) + (c - 2 * Q2);
-                src = reinterpret_cast<float4 *>(P4 + (row + TH) * F::RWP1) + (c - 2 * Q2);
-            }
-            *dst = *src;
-        }
-        __syncthreads();
-    }
-    // Staging (a.stage_i2): one TMA box of I2, the tile's window displaced by the
-    // rounded estimate at the tile's centre, and at FLOW_SAME the boxes of the current
-    // estimate over the rows this tile computes (FixedTile::FLOW_BH), written over plane
-    // P01: stage 1 reads each pair's estimate there before storing the pair's products
-    // in the same place (the estimates of rows no box covers are read from global memory).
-    const bool box = SAME && staged && (!CARRY || F::FLOW_BOX_BELOW);
-    constexpr bool ALL = F::FLOW_BH == 2 * R || F::FLOW_BH == F::RH;   // boxes cover a first tile's whole region
-    const int bx0 = CARRY ? 2 * R : 0;          // first row of the boxes; rows below brow_end read them
-    const int nbox = !box ? 0 : (CARRY ? TH / F::FLOW_BH : (ALL ? F::RH / F::FLOW_BH : 1));
-    const int brow_end = box ? ((CARRY || ALL) ? F::RH : TH) : 0;
+    // Staging (a.stage_i2): one TMA box of I2, the tile's window displaced by the rounded
+    // estimate at the tile's centre, and at FLOW_SAME one of the current estimate over the
+    // region, written over plane P01: stage 1 reads each pair's estimate there before storing
+    // the pair's products in the same place.
+    const bool box = MODE == FLOW_SAME && staged;
     int wx0 = 0, wy0 = 0;
     if (staged) {
-        // a later tile of a strip: its window was requested by the tile above
-        const bool early = OF_EARLY_WINDOW && CM == 2 && CARRY;
-        win_origin<R, TH, S, TW>(a, tx0, ty0, CM == 2 ? wrefs[0] : win_ref<NC, MODE, TH, TW>(a, tx0, ty0), wx0, wy0);
+        win_origin<R, TH, S, TW>(a, tx0, ty0, win_ref<NC, MODE, TH, TW>(a, tx0, ty0), wx0, wy0);
         if (threadIdx.x == 0) {
             fence_proxy_async_smem();
-            mbar_arrive_expect_tx(bar, (uint32_t)((early ? 0 : F::win_bytes(S)) + nbox * F::FLOW_BOX_BYTES));
-            for (int b = 0; b < nbox; ++b)
-                tma_load_2d(P01 + (bx0 + b * F::FLOW_BH) * F::RWP2, &maps->flow, tx0 - F::RE,
-                            ty0 - R + bx0 + b * F::FLOW_BH, bar);
-            if (!early) tma_load_2d(win, &maps->i2, wx0, wy0, bar);
+            mbar_arrive_expect_tx(bar, (uint32_t)(F::win_bytes(S) + (box ? F::FLOW_BOX_BYTES : 0)));
+            if (box) tma_load_2d(P01, &maps->flow, tx0 - F::RE, ty0 - R, bar);
+            tma_load_2d(win, &maps->i2, wx0, wy0, bar);
         }
-#if OF_PREFETCH_I1 == 1
-        // while the boxes land: warm L2 with the region's rows of I1 (read by stage 1)
-        if (threadIdx.x >= 32 && threadIdx.x < 32 + F::RH - r0)
-            prefetch_row(a.I1, a.pitch, S, a.H, a.W, ty0 - R + r0, ty0 - R + F::RH, tx0 - F::RE,
-                         tx0 - F::RE + F::RWE, threadIdx.x - 32);
-#elif OF_PREFETCH_I1 == 2
-        // while the boxes land: bring the lines of I1 that stage 1 reads into L1, and at
-        // the first iteration of a level those of the coarser estimate it upsamples
-        {
-            constexpr int LPR = (F::RWE * S + 127) / 128 + 1;
-            constexpr int CRH = F::RH / 2 + 2, CLPR = ((F::RWE / 2 + 2) * 8 + 127) / 128 + 1;
-            const int n1 = (F::RH - r0) * LPR;
-            const int n = n1 + (MODE == FLOW_UPSAMPLE ? CRH * CLPR : 0);
-            for (int i = threadIdx.x; i < n; i += NT) {
-                if (i < n1)
-                    prefetch_lines_l1(a.I1, a.pitch, S, a.H, a.W, ty0 - R + r0, ty0 - R + F::RH, tx0 - F::RE,
-                                      tx0 - F::RE + F::RWE, LPR, i);
-                else
-                    prefetch_lines_l1(a.fin, a.fin_pitch, 8, a.Hc, a.Wc, (ty0 - R) >> 1,
-                                      ((ty0 - R) >> 1) + CRH, (tx0 - F::RE) >> 1,
-                                      ((tx0 - F::RE) >> 1) + F::RWE / 2 + 2, CLPR, i - n1);
-            }
-        }
-#endif
-        bool done = mbar_wait_bounded(bar, phase, STAGE_TIMEOUT_NS);
-        if (__syncthreads_or(!done)) {
-            // give the copies in flight a further bounded wait before the block leaves
-            if (!done) mbar_wait_bounded(bar, phase, STAGE_TIMEOUT_NS);
-            if (threadIdx.x == 0 && a.status) atomicExch(a.status, DEV_TIMEOUT);
-            return false;
-        }
-        phase ^= 1u;
+        prefetch_region<R, MODE, TH, TW, NT, S>(a, tx0, ty0, 0, 0);
+        if (!stage_wait(a, bar, phase)) return false;
     }
-    // stage 1: products over region rows r0..RH-1 (the tile and its halo), by pixel pairs
+    // stage 1: products over the region (the tile and its halo), by pixel pairs
     constexpr int NPR = F::RWE / 2;   // pairs per region row
     const T *wt = staged ? reinterpret_cast<const T *>(win) : nullptr;
-    auto pair = [&](auto inner, int ry, int cx) {
-        const int k2 = ry * (F::RWP2 / 2) + cx;   // float4 slot of the pair in the pair planes
-        float4 s01, s23;
-        float2 s4;
-        stage1_pair<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(
-            a, tx0 - F::RE + 2 * cx, ty0 - R + ry, ref,
-            ry < brow_end ? reinterpret_cast<const float4 *>(P01) + k2 : nullptr, wt, wx0, wy0, s01, s23, s4);
-        reinterpret_cast<float4 *>(P01)[k2] = s01;
-        reinterpret_cast<float4 *>(P23)[k2] = s23;
-        reinterpret_cast<float2 *>(P4)[ry * (F::RWP1 / 2) + cx] = s4;
-    };
     auto rows = [&](auto inner) {
-        if constexpr (CM == 2) {
-            // strips: thread t takes pixel pair cx = t mod NPR of rows r0 + t / NPR, then RPI
-            // rows further each round, so that what depends on the pair's column is the same on
-            // every row it takes (5% fewer instructions per pixel-iteration at r = 4)
-            constexpr int RPI = NT / NPR;   // rows per round
-            const int cx = threadIdx.x % NPR, rs = threadIdx.x / NPR;
-            if (rs < RPI) {
+        // pair j = threadIdx.x + k NT is (row ry, pair cx), stepped without a division (NT = DY
+        // rows + DX pairs)
+        constexpr int DY = NT / NPR, DX = NT % NPR;
+        constexpr int npair = F::RH * NPR;
+        int ry = threadIdx.x / NPR, cx = threadIdx.x % NPR;
 #pragma unroll 1
-                for (int ry = r0 + rs; ry < F::RH; ry += RPI) pair(inner, ry, cx);
-            }
-        } else {
-            // single tiles: pair j = threadIdx.x + k NT is (row ry, pair cx) of the rows
-            // computed, stepped without a division (NT = DY rows + DX pairs); it
-            // compiles without spills where the form above does not
-            constexpr int DY = NT / NPR, DX = NT % NPR;
-            const int npair = (F::RH - r0) * NPR;
-            int ry = r0 + threadIdx.x / NPR, cx = threadIdx.x % NPR;
-#pragma unroll 1
-            for (int j = threadIdx.x; j < npair; j += NT) {
-                pair(inner, ry, cx);
-                ry += DY;
-                cx += DX;
-                if (cx >= NPR) {
-                    cx -= NPR;
-                    ++ry;
-                }
+        for (int j = threadIdx.x; j < npair; j += NT) {
+            const int k2 = ry * (F::RWP2 / 2) + cx;   // float4 slot of the pair in the pair planes
+            float4 s01, s23;
+            float2 s4;
+            stage1_pair<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(
+                a, tx0 - F::RE + 2 * cx, ty0 - R + ry, ref, box ? reinterpret_cast<const float4 *>(P01) + k2 : nullptr,
+                wt, wx0, wy0, s01, s23, s4);
+            reinterpret_cast<float4 *>(P01)[k2] = s01;
+            reinterpret_cast<float4 *>(P23)[k2] = s23;
+            reinterpret_cast<float2 *>(P4)[ry * (F::RWP1 / 2) + cx] = s4;
+            ry += DY;
+            cx += DX;
+            if (cx >= NPR) {
+                cx -= NPR;
+                ++ry;
             }
         }
     };
-    // the staged window and the region both inside the image: no pair needs a bounds check
-    if (staged && wx0 >= 0 && wy0 >= 0 && wx0 + WW <= a.W && wy0 + F::WIN_H <= a.H && tx0 >= F::RE && ty0 >= R &&
-        tx0 + TW + F::RE <= a.W && ty0 + TH + R <= a.H)
-        rows(std::true_type());
-    else
-        rows(std::false_type());
+    if (staged && tile_inner<R, TH, TW, S>(a, tx0, ty0, wx0, wy0)) rows(std::true_type());
+    else rows(std::false_type());
     __syncthreads();
-    if constexpr (CM == 2 && OF_EARLY_WINDOW) {
-        // the window is free: request the next tile's, which lands while this tile
-        // finishes (the barrier's next phase completes only on that tile's arrival)
-        if (staged && next && threadIdx.x == 0) {
-            int nx0, ny0;
-            win_origin<R, TH, S, TW>(a, tx0, ty0 + TH, wrefs[1], nx0, ny0);
-            fence_proxy_async_smem();
-            mbar_expect_tx(bar, (uint32_t)F::win_bytes(S));
-            tma_load_2d(win, &maps->i2, nx0, ny0, bar);
-        }
-    }
-    // P23's chunks start at warp 4, so that when the rows leave some warps an extra chunk
-    // of P01 and of P4 (24 rows: 12 chunks and 384 items) the other warps take P23's
-    box_h_pairs<R, TH, TW, NT>(P01, r0);
-    box_h_pairs<R, TH, TW, NT>(P23, r0, NT / 64);
-    box_h_single<R, TH, TW, NT>(P4, r0);
+    // P23's chunks start at the middle warp, so that when the rows leave some warps an extra
+    // chunk of P01 and of P4 the other warps take P23's
+    box_h_pairs<R, TH, TW, NT>(P01);
+    box_h_pairs<R, TH, TW, NT>(P23, 0, NT / 64);
+    box_h_single<R, TH, TW, NT>(P4);
     __syncthreads();
     // vertical sums, solve and write: VO rows of one column per item (all VR rows of a group, or
     // two of them where the tile has fewer groups than threads)
@@ -1468,19 +1468,151 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
         }
 #pragma unroll
         for (int j = 0; j < VO; ++j) {
-            const int y = yb + j;
-            if (y >= a.H) break;
-            const float sj[5] = {s01[j].x, s01[j].y, s23[j].x, s23[j].y, s4[j]};
-            float xu, xv;
-            const float2 f = solve2(sj, fp64_cond, xu, xv) ? make_float2(ref.x + xu, ref.y + xv)
-                                                           : flow_mode<NC, MODE>(a, x, y);
-            if (a.fout) {
-                a.fout[(size_t)y * a.fout_pitch + x] = f;
-            } else {
-                a.u_out[(size_t)y * a.W + x] = f.x;
-                a.v_out[(size_t)y * a.W + x] = f.y;
-            }
+            if (yb + j >= a.H) break;
+            solve_store<NC, MODE>(a, x, yb + j, ref, fp64_cond, s01[j], s23[j], s4[j]);
         }
+    }
+    return true;
+}
+
+// Tiles t_first .. t_end-1 (64 x TH each) of one column of tiles at tx0, top to bottom. The
+// planes are rings (StripTile): a tile after the first finds the window sums along x of its
+// first 2R rows where the tile above left them and computes the TH rows below them. A tile's
+// I2 window is requested when the tile above has done stage 1 (the window buffer is free
+// then) and its estimate rows, written over P01's slots of the rows that leave, when the tile
+// above has read its vertical sums, so that both are in flight during the horizontal pass
+// and the solves. Before the rings (carried rows copied up, the estimate requested at the
+// tile's own start, or read pair by pair where 2R rows were no whole number of boxes) a later
+// tile of 32 pairs of 1024^2 at r = 4 took 15.8k cycles with 4 blocks on the SM, of which the
+// copy 1.1k and request and wait 2.4k; now 13.4k, request and wait 1.1k. Level-0 launch: r = 4
+// 358 -> 348 us, r = 5 462 -> 417, r = 10 680 -> 589. One bulk copy per row instead of the boxes
+// holds the issuing warp for 2k cycles per tile (410 us at r = 4).
+template <typename T, bool NC, int R, int MODE, int TH>
+__device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *maps, int tx0, int t_first, int t_end,
+                                         float2 ref, float fp64_cond, float *smem, uint32_t &phase)
+{
+    using F = FixedTile<R, TH>;
+    using X = StripTile<R, TH>;
+    constexpr int NT = LK_THREADS, TW = LK_TW, S = (int)sizeof(T), WW = F::win_w(S), RH = F::RH, RN = X::RING;
+    unsigned char *win = reinterpret_cast<unsigned char *>(smem + X::OFF_WIN);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + X::OFF_BAR);
+    float2 *wrefs = reinterpret_cast<float2 *>(smem + X::OFF_WREF);
+    float2 *P01 = reinterpret_cast<float2 *>(smem);
+    float2 *P23 = P01 + X::PAIR_PLANE;
+    float *P4 = reinterpret_cast<float *>(P23 + X::PAIR_PLANE);
+    const bool staged = maps && a.stage_i2 != 0;
+    const bool flows = MODE == FLOW_SAME && staged;   // the estimate is staged as well
+    // the window estimates of the strip's tiles (at most the 4 slots at OFF_WREF), loaded together
+    if (staged && (int)threadIdx.x < t_end - t_first)
+        wrefs[threadIdx.x] = win_ref<NC, MODE, TH>(a, tx0, (t_first + (int)threadIdx.x) * TH);
+    // Close the tile's phase of the barrier and request the estimate (one thread) in n boxes of
+    // 8 rows, the first at image row y in slot sl. extra: bytes requested besides.
+    auto request_rows = [&](int y, int sl, int n, uint32_t extra) {
+        fence_proxy_async_smem();
+        mbar_arrive_expect_tx(bar, extra + (flows ? (uint32_t)(n * X::BOX_BYTES) : 0u));
+        if (flows)
+            for (int k = 0; k < n; ++k, sl = sl + X::BOX < RN ? sl + X::BOX : 0)
+                tma_load_2d(P01 + sl * F::RWP2, &maps->flow, tx0 - F::RE, y + k * X::BOX, bar);
+    };
+    int base = X::RPAD;   // slot of the tile's region row 0
+    __syncthreads();   // wrefs
+#pragma unroll 1
+    for (int t = t_first; t < t_end; ++t) {
+        const int ty0 = t * TH;
+        const bool next = t + 1 < t_end;
+        const int r0 = t > t_first ? 2 * R : 0;   // the first region row this tile computes
+        int wx0 = 0, wy0 = 0;
+        if (staged) {
+            win_origin<R, TH, S>(a, tx0, ty0, wrefs[t - t_first], wx0, wy0);
+            if (t == t_first) {
+                if (threadIdx.x == 0) {
+                    request_rows(ty0 - R - X::RPAD, 0, RN / X::BOX, (uint32_t)F::win_bytes(S));
+                    tma_load_2d(win, &maps->i2, wx0, wy0, bar);
+                }
+                prefetch_region<R, MODE, TH, TW, NT, S>(a, tx0, ty0, 0, 32);
+            }
+            if (!stage_wait(a, bar, phase)) return false;
+        }
+        // stage 1 over region rows r0..RH-1, by pixel pairs
+        constexpr int NPR = F::RWE / 2;   // pairs per region row
+        const T *wt = staged ? reinterpret_cast<const T *>(win) : nullptr;
+        auto pair = [&](auto inner, int ry, int cx) {
+            const int sl = ring_slot<RN>(ry, base);
+            const int k2 = sl * (F::RWP2 / 2) + cx;   // float4 slot of the pair in the pair planes
+            float4 s01, s23;
+            float2 s4;
+            stage1_pair<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(
+                a, tx0 - F::RE + 2 * cx, ty0 - R + ry, ref, flows ? reinterpret_cast<const float4 *>(P01) + k2 : nullptr,
+                wt, wx0, wy0, s01, s23, s4);
+            reinterpret_cast<float4 *>(P01)[k2] = s01;
+            reinterpret_cast<float4 *>(P23)[k2] = s23;
+            reinterpret_cast<float2 *>(P4)[sl * (F::RWP1 / 2) + cx] = s4;
+        };
+        auto rows = [&](auto inner) {
+            // thread t takes pair cx = t mod NPR of rows r0 + t / NPR, then RPI rows further each
+            // round, so that what depends on the pair's column is the same on every row it takes
+            constexpr int RPI = NT / NPR;   // rows per round
+            const int cx = threadIdx.x % NPR, rs = threadIdx.x / NPR;
+            if (rs < RPI) {
+#pragma unroll 1
+                for (int ry = r0 + rs; ry < RH; ry += RPI) pair(inner, ry, cx);
+            }
+        };
+        if (staged && tile_inner<R, TH, TW, S>(a, tx0, ty0, wx0, wy0)) rows(std::true_type());
+        else rows(std::false_type());
+        __syncthreads();
+        if (staged && next) {
+            if (threadIdx.x == 0) {   // on the barrier's next phase, which request_rows closes
+                int nx0, ny0;
+                win_origin<R, TH, S>(a, tx0, ty0 + TH, wrefs[t - t_first + 1], nx0, ny0);
+                fence_proxy_async_smem();
+                mbar_expect_tx(bar, (uint32_t)F::win_bytes(S));
+                tma_load_2d(win, &maps->i2, nx0, ny0, bar);
+            }
+            prefetch_region<R, MODE, TH, TW, NT, S>(a, tx0, ty0 + TH, 2 * R, 32);
+        }
+        box_h_pairs<R, TH, TW, NT, RN>(P01, r0, 0, base);
+        box_h_pairs<R, TH, TW, NT, RN>(P23, r0, NT / 64, base);   // from the middle warp: the extra chunks fall on different warps
+        box_h_single<R, TH, TW, NT, RN>(P4, r0, base);
+        __syncthreads();
+        // vertical sums, solve and write, VR rows of one column per item
+        constexpr int VR = v_rows<R, TH>();
+        constexpr int NITEM = TW * (TH / VR);
+        const int base_next = ring_slot<RN>(TH, base);
+        if constexpr (NITEM == NT) {   // one item per thread: the planes are free before the solves
+            const int tx = threadIdx.x % TW, g = threadIdx.x / TW;
+            const int x = tx0 + tx, yb = ty0 + VR * g;
+            float2 s01[VR], s23[VR];
+            float s4[VR];
+            box_v_planes<R, TH, TW, RN>(P01, P23, P4, g, tx, s01, s23, s4, base);
+            __syncthreads();
+            if (staged && next && threadIdx.x == 0) request_rows(ty0 + TH + R, ring_slot<RN>(2 * R, base_next), TH / X::BOX, 0u);
+            if (x < a.W) {
+#pragma unroll
+                for (int j = 0; j < VR; ++j) {
+                    if (yb + j >= a.H) break;
+                    solve_store<NC, MODE>(a, x, yb + j, ref, fp64_cond, s01[j], s23[j], s4[j]);
+                }
+            }
+        } else {
+#pragma unroll 1
+            for (int i = threadIdx.x; i < NITEM; i += NT) {
+                const int tx = i % TW, g = i / TW;
+                const int x = tx0 + tx, yb = ty0 + VR * g;
+                if (x >= a.W || yb >= a.H) continue;
+                float2 s01[VR], s23[VR];
+                float s4[VR];
+                box_v_planes<R, TH, TW, RN>(P01, P23, P4, g, tx, s01, s23, s4, base);
+#pragma unroll
+                for (int j = 0; j < VR; ++j) {
+                    if (yb + j >= a.H) break;
+                    solve_store<NC, MODE>(a, x, yb + j, ref, fp64_cond, s01[j], s23[j], s4[j]);
+                }
+            }
+            __syncthreads();
+            if (staged && next && threadIdx.x == 0) request_rows(ty0 + TH + R, ring_slot<RN>(2 * R, base_next), TH / X::BOX, 0u);
+        }
+        base = base_next;
     }
     return true;
 }
@@ -1509,19 +1641,9 @@ __device__ __forceinline__ bool lk_tile_fixed(const IterArgs &a, const StageMaps
     const int gy0 = t_first / REF_GROUP * REF_GROUP * TH;
     const float2 ref = flow_mode<NC, MODE>(a, min(tx0 + LK_TW / 2, a.W - 1), min(gy0 + REF_GROUP * TH / 2, a.H - 1));
     if constexpr (!MULTI) {   // one tile per unit (a.strip 1)
-        return lk_tile_step<T, NC, R, MODE, TH, 0>(a, maps, tx0, t_first * TH, ref, fp64_cond, smem, phase, false);
+        return lk_tile_step<T, NC, R, MODE, TH>(a, maps, tx0, t_first * TH, ref, fp64_cond, smem, phase);
     } else {
-        // the window estimates of the strip's tiles (strip_len: at most the 4 slots at
-        // OFF_WREF), loaded together before the first tile's staging
-        float2 *wrefs = reinterpret_cast<float2 *>(smem + F::OFF_WREF);
-        if (maps && a.stage_i2 && (int)threadIdx.x < t_end - t_first)
-            wrefs[threadIdx.x] = win_ref<NC, MODE, TH>(a, tx0, (t_first + (int)threadIdx.x) * TH);
-#pragma unroll 1
-        for (int t = t_first; t < t_end; ++t)
-            if (!lk_tile_step<T, NC, R, MODE, TH, 2>(a, maps, tx0, t * TH, ref, fp64_cond, smem, phase, t > t_first,
-                                                     wrefs + (t - t_first), t + 1 < t_end))
-                return false;
-        return true;
+        return lk_strip<T, NC, R, MODE, TH>(a, maps, tx0, t_first, t_end, ref, fp64_cond, smem, phase);
     }
 }
 
@@ -1539,8 +1661,7 @@ __device__ __forceinline__ bool lk_tile_small(const IterArgs &a, const StageMaps
     const int tx0 = (unit - uy * a.tiles_x) * SM_TW, ty0 = uy * SM_TH;
     const int gx0 = tx0 / LK_TW * LK_TW, gy0 = ty0 / (REF_GROUP * LK_TH) * (REF_GROUP * LK_TH);
     const float2 ref = flow_mode<NC, MODE>(a, min(gx0 + LK_TW / 2, a.W - 1), min(gy0 + REF_GROUP * LK_TH / 2, a.H - 1));
-    return lk_tile_step<T, NC, R, MODE, SM_TH, 0, SM_TW, SM_THREADS>(a, maps, tx0, ty0, ref, fp64_cond, smem, phase,
-                                                                     false);
+    return lk_tile_step<T, NC, R, MODE, SM_TH, SM_TW, SM_THREADS>(a, maps, tx0, ty0, ref, fp64_cond, smem, phase);
 }
 
 // ------------------------------------------------ two iterations fused in one tile
@@ -1709,9 +1830,9 @@ __device__ __forceinline__ bool lk_tile(const IterArgs &a, const StageMaps *maps
     }
 }
 
-template <int R, int TH = LK_TH> __device__ __forceinline__ void lk_tile_prepare(float *smem)
+template <int R, int TH = LK_TH, bool MULTI = false> __device__ __forceinline__ void lk_tile_prepare(float *smem)
 {
-    if constexpr (R != 0) lk_tile_init<R, TH>(smem);
+    if constexpr (R != 0) lk_tile_init<R, TH, LK_TW, MULTI>(smem);
 }
 
 template <int R, int TH = LK_TH> constexpr int lk_min_blocks()
@@ -1732,10 +1853,11 @@ template <int R> constexpr int batch_min_blocks()
 
 // Dynamic shared memory of the iteration tile (floats); elem_bytes: the level image's
 // element size (the staged window's).
-template <int R, int TH = LK_TH>
+template <int R, int TH = LK_TH, bool MULTI = false>
 inline __host__ __device__ int lk_tile_smem_floats(int r, bool stage_i2, int elem_bytes = 4)
 {
     if constexpr (R == 0) return lk_smem_floats(r);
+    else if constexpr (MULTI) return stage_i2 ? StripTile<R, TH>::smem_staged(elem_bytes) : StripTile<R, TH>::SMEM_NOSTAGE;
     else return stage_i2 ? FixedTile<R, TH>::smem_staged(elem_bytes) : FixedTile<R, TH>::SMEM_NOSTAGE;
 }
 

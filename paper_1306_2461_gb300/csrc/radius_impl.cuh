@@ -15,6 +15,8 @@ namespace of {
 
 // Radii with every form of the batched launch (0: the run-time-radius kernel); the others
 // have the per-pair and phase launches at the default tile height.
+// Strips: the phase kernels whose tile height holds the rows carried from tile to tile.
+template <int R, int TH> constexpr bool strip_kernel() { return R != 0 && TH >= 2 * R; }
 template <int R> constexpr bool all_forms() { return R == 0 || radius_specialised(R); }
 
 template <typename T, int R>
@@ -75,7 +77,7 @@ phase_iter_kernel(const __grid_constant__ IterPhase P, int r, float fp64_cond)
     float *smem = reinterpret_cast<float *>(smem4);
     const int p = phase_pair(P.prefix, P.npairs, blockIdx.x);
     uint32_t phase = 0;
-    lk_tile_prepare<R, TH>(smem);
+    lk_tile_prepare<R, TH, strip_kernel<R, TH>()>(smem);
     chain_begin();
     if constexpr (R != 0) {
         const int t2 = blockIdx.x + P.ahead;
@@ -84,7 +86,7 @@ phase_iter_kernel(const __grid_constant__ IterPhase P, int r, float fp64_cond)
             prefetch_tile<T, MODE, TH>(P.a[q], t2 - P.prefix[q], R);
         }
     }
-    lk_tile<T, false, R, MODE, TH, (TH >= 2 * R)>(P.a[p], &P.m[p], blockIdx.x - P.prefix[p], r, fp64_cond, smem, phase);
+    lk_tile<T, false, R, MODE, TH, strip_kernel<R, TH>()>(P.a[p], &P.m[p], blockIdx.x - P.prefix[p], r, fp64_cond, smem, phase);
 }
 
 // Two same-level iterations of up to PHASE_PAIRS pairs in one launch (iteration fusion
@@ -183,7 +185,9 @@ window_sums_kernel(const float *ch, int H, int W, int r, int tiles_x, float *out
 
 template <int R> size_t radius_smem_bytes(int r, bool stage_i2)
 {
-    const size_t lk = sizeof(float) * (size_t)lk_tile_smem_floats<R>(r, stage_i2);
+    size_t lk = sizeof(float) * (size_t)lk_tile_smem_floats<R>(r, stage_i2);
+    const size_t st = sizeof(float) * (size_t)lk_tile_smem_floats<R, LK_TH, strip_kernel<R, LK_TH>()>(r, stage_i2);
+    if (st > lk) lk = st;
     size_t pyr = sizeof(float) * (size_t)PYR_SMEM_FLOATS;
     const size_t zn = sizeof(float) * (size_t)ZN_SMEM_FLOATS;
     if (zn > pyr) pyr = zn;
@@ -229,7 +233,7 @@ static cudaError_t phase_for_th(const IterPhase &P, int r, float fp64_cond, cuda
 {
     bool stage = false;   // shared memory for the staged window if any pair stages
     for (int i = 0; i < P.npairs; ++i) stage = stage || P.a[i].stage_i2 != 0;
-    const size_t smem = sizeof(float) * lk_tile_smem_floats<R, TH>(r, stage, (int)sizeof(T));
+    const size_t smem = sizeof(float) * lk_tile_smem_floats<R, TH, strip_kernel<R, TH>()>(r, stage, (int)sizeof(T));
     const int blocks = P.prefix[P.npairs];
     switch (P.a[0].mode) {
     case FLOW_ZERO: return launch_chained(phase_iter_kernel<T, R, FLOW_ZERO, TH>, blocks, LK_THREADS, smem, s, P, r, fp64_cond);
@@ -368,7 +372,7 @@ template <int R> cudaError_t phase_i1_launch(const IterPhase &P, int elem, int r
 
 // The tensor maps of the staged fixed-radius tile of height TH: the estimate in boxes
 // of the tile's region (RWP2 x RH elements of 8 bytes) and I2 in boxes of the window.
-template <int R, int TH, int TW = LK_TW> static bool stage_maps_th(const IterArgs &a, StageMaps &m, int elem)
+template <int R, int TH, int TW = LK_TW> static bool stage_maps_th(const IterArgs &a, StageMaps &m, int elem, bool strips)
 {
     using F = FixedTile<R, TH, TW>;
     const int S = elem_bytes(elem);
@@ -378,19 +382,22 @@ template <int R, int TH, int TW = LK_TW> static bool stage_maps_th(const IterArg
     constexpr int SM_BYTES = 228 * 1024, BLOCK_BYTES = 1024;   // shared memory per SM, and reserved per block
     if (2 * (4 * F::smem_staged(S) + BLOCK_BYTES) > SM_BYTES && 2 * (4 * F::SMEM_NOSTAGE + BLOCK_BYTES) <= SM_BYTES)
         return false;
+    int flow_rows = F::FLOW_BH;
+    if constexpr (TW == LK_TW && strip_kernel<R, TH>())
+        if (strips) flow_rows = StripTile<R, TH>::BOX;
     if (a.mode == FLOW_SAME &&
-        !encode_tile_map(&m.flow, ET_FLOW2, a.fin, a.W, a.H, (size_t)a.fin_pitch * 8, F::RWP2, F::FLOW_BH))
+        !encode_tile_map(&m.flow, ET_FLOW2, a.fin, a.W, a.H, (size_t)a.fin_pitch * 8, F::RWP2, flow_rows))
         return false;
     return encode_tile_map(&m.i2, elem, a.I2, a.W, a.H, (size_t)a.pitch * S, F::win_w(S), F::WIN_H);
 }
 
-template <int R> bool radius_stage_maps(const IterArgs &a, StageMaps &m, int elem, int tile_h)
+template <int R> bool radius_stage_maps(const IterArgs &a, StageMaps &m, int elem, int tile_h, bool strips)
 {
     if constexpr (R == 0) {
         return false;
     } else {
-        if (tile_h == SM_TH) return stage_maps_th<R, SM_TH, SM_TW>(a, m, elem);
-        return tile_h == ALT_TH && all_forms<R>() ? stage_maps_th<R, ALT_TH>(a, m, elem) : stage_maps_th<R, LK_TH>(a, m, elem);
+        if (tile_h == SM_TH) return stage_maps_th<R, SM_TH, SM_TW>(a, m, elem, strips);
+        return tile_h == ALT_TH && all_forms<R>() ? stage_maps_th<R, ALT_TH>(a, m, elem, strips) : stage_maps_th<R, LK_TH>(a, m, elem, strips);
     }
 }
 
@@ -426,7 +433,7 @@ template <int R> cudaError_t radius_configure()
     OF_SET_PH(__nv_bfloat16);
 #undef OF_SET_PH
     if constexpr (R != 0 && all_forms<R>()) {   // the other tile height of the phase kernels
-        const int alt = (int)sizeof(float) * lk_tile_smem_floats<R, ALT_TH>(R, true);
+        const int alt = (int)sizeof(float) * lk_tile_smem_floats<R, ALT_TH, strip_kernel<R, ALT_TH>()>(R, true);
 #define OF_SET_ALT(T)                                                                                       \
     for (const void *fn : {(const void *)phase_iter_kernel<T, R, FLOW_ZERO, ALT_TH>,                        \
                            (const void *)phase_iter_kernel<T, R, FLOW_SAME, ALT_TH>,                        \
@@ -500,7 +507,7 @@ template cudaError_t i1_launch<OF_RADIUS>(const IterArgs &, int, int, float, cud
 #ifndef OF_RADIUS_MORE   // one of OF_RADII_MORE
 template void *batch_kernel_ptr<OF_RADIUS>(int, int);
 #endif
-template bool radius_stage_maps<OF_RADIUS>(const IterArgs &, StageMaps &, int, int);
+template bool radius_stage_maps<OF_RADIUS>(const IterArgs &, StageMaps &, int, int, bool);
 template cudaError_t phase2_launch<OF_RADIUS>(const IterPhase &, int, float, cudaStream_t);
 template cudaError_t radius_configure<OF_RADIUS>();
 template size_t radius_smem_bytes<OF_RADIUS>(int, bool);

@@ -692,13 +692,15 @@ template <int R, int TH = LK_TH, int TW = LK_TW> struct FixedTile {
     static constexpr int FLOW_BH = RH;
     static constexpr int FLOW_BOX_BYTES = RWP2 * FLOW_BH * 8;
 #ifndef OF_LK_MIN_BLOCKS
-#define OF_LK_MIN_BLOCKS 4   // resident blocks per SM the fixed-radius kernels are compiled for (R <= 6)
+#define OF_LK_MIN_BLOCKS 4   // resident blocks per SM the fixed-radius kernels are compiled for (R <= 4)
 #endif
     // resident blocks per SM the kernels are compiled for: the measured choice for the
-    // default tile height, else as many as the shared memory holds (at most 5)
+    // default tile height, else as many as the shared memory holds (at most 5). At r = 5 and 6
+    // shared memory holds 3 blocks, which leaves 80 registers instead of 64: level-0 launch of 32
+    // pairs of 1024^2 at r = 5 416 -> 405 us, a pair 195 -> 193 us
     static constexpr int SMEM_FIT = 233472 / (4 * (PLANES + 4) + 1024);
     static constexpr int MIN_BLOCKS =
-        TH == LK_TH ? (R <= 6 ? OF_LK_MIN_BLOCKS : 2) : (SMEM_FIT < 1 ? 1 : (SMEM_FIT > 5 ? 5 : SMEM_FIT));
+        TH == LK_TH ? (R <= 4 ? OF_LK_MIN_BLOCKS : (R <= 6 ? 3 : 2)) : (SMEM_FIT < 1 ? 1 : (SMEM_FIT > 5 ? 5 : SMEM_FIT));
 };
 
 // Shared memory of a strip's tiles: the planes are rings of RING rows. Region row ry of a tile
@@ -1449,7 +1451,7 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
     // two of them where the tile has fewer groups than threads)
     constexpr int VR = v_rows<R, TH>();
     constexpr int NGRP = TW * (TH / VR);
-    constexpr int VO = NGRP < NT ? 2 : VR;
+    constexpr int VO = TW < LK_TW && NGRP < NT ? 2 : VR;
 #pragma unroll 1
     for (int i = threadIdx.x; i < NGRP * (VR / VO); i += NT) {
         const int part = VO == VR ? 0 : i / NGRP;   // the same for a whole warp
@@ -1487,13 +1489,13 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
 // copy 1.1k and request and wait 2.4k; now 13.4k, request and wait 1.1k. Level-0 launch: r = 4
 // 358 -> 348 us, r = 5 462 -> 417, r = 10 680 -> 589. One bulk copy per row instead of the boxes
 // holds the issuing warp for 2k cycles per tile (410 us at r = 4).
-template <typename T, bool NC, int R, int MODE, int TH>
+template <typename T, bool NC, int R, int MODE, int TH, int NT>
 __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *maps, int tx0, int t_first, int t_end,
                                          float2 ref, float fp64_cond, float *smem, uint32_t &phase)
 {
     using F = FixedTile<R, TH>;
     using X = StripTile<R, TH>;
-    constexpr int NT = LK_THREADS, TW = LK_TW, S = (int)sizeof(T), WW = F::win_w(S), RH = F::RH, RN = X::RING;
+    constexpr int TW = LK_TW, S = (int)sizeof(T), WW = F::win_w(S), RH = F::RH, RN = X::RING;
     unsigned char *win = reinterpret_cast<unsigned char *>(smem + X::OFF_WIN);
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + X::OFF_BAR);
     float2 *wrefs = reinterpret_cast<float2 *>(smem + X::OFF_WREF);
@@ -1579,15 +1581,16 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
         constexpr int VR = v_rows<R, TH>();
         constexpr int NITEM = TW * (TH / VR);
         const int base_next = ring_slot<RN>(TH, base);
-        if constexpr (NITEM == NT) {   // one item per thread: the planes are free before the solves
-            const int tx = threadIdx.x % TW, g = threadIdx.x / TW;
+        if constexpr (NITEM <= NT) {   // one item per thread: the planes are free before the solves
+            const bool has = NITEM == NT || threadIdx.x < NITEM;
+            const int tx = threadIdx.x % TW, g = has ? threadIdx.x / TW : 0;
             const int x = tx0 + tx, yb = ty0 + VR * g;
             float2 s01[VR], s23[VR];
             float s4[VR];
-            box_v_planes<R, TH, TW, RN>(P01, P23, P4, g, tx, s01, s23, s4, base);
+            if (has) box_v_planes<R, TH, TW, RN>(P01, P23, P4, g, tx, s01, s23, s4, base);
             __syncthreads();
             if (staged && next && threadIdx.x == 0) request_rows(ty0 + TH + R, ring_slot<RN>(2 * R, base_next), TH / X::BOX, 0u);
-            if (x < a.W) {
+            if (has && x < a.W) {
 #pragma unroll
                 for (int j = 0; j < VR; ++j) {
                     if (yb + j >= a.H) break;
@@ -1627,7 +1630,7 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
 // every a.strip. MULTI = false: a kernel whose units are single tiles (a.strip 1). Returns
 // false if a staging copy did not complete in time (then OF_ETIMEOUT is in *a.status,
 // nothing more of the unit was written, and the block must stop).
-template <typename T, bool NC, int R, int MODE, int TH = LK_TH, bool MULTI = true>
+template <typename T, bool NC, int R, int MODE, int TH = LK_TH, bool MULTI = true, int NT = LK_THREADS>
 __device__ __forceinline__ bool lk_tile_fixed(const IterArgs &a, const StageMaps *maps, int unit, float fp64_cond,
                                               float *smem, uint32_t &phase)
 {
@@ -1641,9 +1644,9 @@ __device__ __forceinline__ bool lk_tile_fixed(const IterArgs &a, const StageMaps
     const int gy0 = t_first / REF_GROUP * REF_GROUP * TH;
     const float2 ref = flow_mode<NC, MODE>(a, min(tx0 + LK_TW / 2, a.W - 1), min(gy0 + REF_GROUP * TH / 2, a.H - 1));
     if constexpr (!MULTI) {   // one tile per unit (a.strip 1)
-        return lk_tile_step<T, NC, R, MODE, TH>(a, maps, tx0, t_first * TH, ref, fp64_cond, smem, phase);
+        return lk_tile_step<T, NC, R, MODE, TH, LK_TW, NT>(a, maps, tx0, t_first * TH, ref, fp64_cond, smem, phase);
     } else {
-        return lk_strip<T, NC, R, MODE, TH>(a, maps, tx0, t_first, t_end, ref, fp64_cond, smem, phase);
+        return lk_strip<T, NC, R, MODE, TH, NT>(a, maps, tx0, t_first, t_end, ref, fp64_cond, smem, phase);
     }
 }
 
@@ -1818,7 +1821,7 @@ __device__ __forceinline__ void lk_tile_fused2(const IterArgs &a, int tile, floa
 // mode when it is known at compile time (-1: read a.mode at run time). maps: the staging
 // tensor maps in parameter space (NULL: gather from global memory). Returns false when
 // the block must stop (a staging copy timed out; recorded in *a.status).
-template <typename T, bool NC, int R, int MODE = -1, int TH = LK_TH, bool MULTI = true>
+template <typename T, bool NC, int R, int MODE = -1, int TH = LK_TH, bool MULTI = true, int NT = LK_THREADS>
 __device__ __forceinline__ bool lk_tile(const IterArgs &a, const StageMaps *maps, int tile, int r, float fp64_cond,
                                         float *smem, uint32_t &phase)
 {
@@ -1826,7 +1829,7 @@ __device__ __forceinline__ bool lk_tile(const IterArgs &a, const StageMaps *maps
         lk_tile_generic<T, NC>(a, tile, r, fp64_cond, smem);
         return true;
     } else {
-        return lk_tile_fixed<T, NC, R, MODE, TH, MULTI>(a, maps, tile, fp64_cond, smem, phase);
+        return lk_tile_fixed<T, NC, R, MODE, TH, MULTI, NT>(a, maps, tile, fp64_cond, smem, phase);
     }
 }
 
@@ -1840,6 +1843,12 @@ template <int R, int TH = LK_TH> constexpr int lk_min_blocks()
     if constexpr (R == 0) return 2;
     else return FixedTile<R, TH>::MIN_BLOCKS;
 }
+// Threads per block of the per-pair kernel: at r > 6 shared memory holds two blocks per SM, and
+// 384 threads each (12 warps instead of 8; 80 registers) shorten a tile: 1024^2 pair at r = 8
+// 257 -> 247 us, r = 10 291 -> 276 (512 threads: 245, 276). The strips of the phase kernels stay at
+// 256, where half the warps would have no output group: 384 threads 589 -> 597 us, 512 (64
+// registers, spills) 652 us per level-0 launch of 32 pairs at r = 10.
+template <int R> constexpr int pair_threads() { return R > 6 ? 384 : LK_THREADS; }
 
 #ifndef OF_BATCH_MIN_BLOCKS
 #define OF_BATCH_MIN_BLOCKS 3

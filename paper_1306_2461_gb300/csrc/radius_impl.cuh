@@ -20,7 +20,7 @@ template <int R, int TH> constexpr bool strip_kernel() { return R != 0 && TH >= 
 template <int R> constexpr bool all_forms() { return R == 0 || radius_specialised(R); }
 
 template <typename T, int R>
-__global__ void __launch_bounds__(LK_THREADS, lk_min_blocks<R>())
+__global__ void __launch_bounds__(pair_threads<R>(), lk_min_blocks<R>())
 lk_iter_kernel(const __grid_constant__ IterArgs a, const __grid_constant__ StageMaps m, int r, float fp64_cond)
 {
     extern __shared__ __align__(128) float4 smem4[];
@@ -28,7 +28,7 @@ lk_iter_kernel(const __grid_constant__ IterArgs a, const __grid_constant__ Stage
     uint32_t phase = 0;
     lk_tile_prepare<R>(smem);
     chain_begin();
-    lk_tile<T, false, R, -1, LK_TH, false>(a, &m, blockIdx.x, r, fp64_cond, smem, phase);   // a.strip is 1
+    lk_tile<T, false, R, -1, LK_TH, false, pair_threads<R>()>(a, &m, blockIdx.x, r, fp64_cond, smem, phase);   // a.strip is 1
 }
 
 // The same on small tiles.
@@ -86,7 +86,7 @@ phase_iter_kernel(const __grid_constant__ IterPhase P, int r, float fp64_cond)
             prefetch_tile<T, MODE, TH>(P.a[q], t2 - P.prefix[q], R);
         }
     }
-    lk_tile<T, false, R, MODE, TH, strip_kernel<R, TH>()>(P.a[p], &P.m[p], blockIdx.x - P.prefix[p], r, fp64_cond, smem, phase);
+    lk_tile<T, false, R, MODE, TH, strip_kernel<R, TH>(), LK_THREADS>(P.a[p], &P.m[p], blockIdx.x - P.prefix[p], r, fp64_cond, smem, phase);
 }
 
 // Two same-level iterations of up to PHASE_PAIRS pairs in one launch (iteration fusion
@@ -202,7 +202,7 @@ static cudaError_t lk_for(const IterArgs &a, const StageMaps &m, int r, float fp
             return launch_chained(lk_small_kernel<T, R>, a.tiles, SM_THREADS, sizeof(float) * small_smem_floats<R>(a.stage_i2 != 0, (int)sizeof(T)), s, a, m, fp64_cond);
         }
     }
-    return launch_chained(lk_iter_kernel<T, R>, a.tiles, LK_THREADS, sizeof(float) * lk_tile_smem_floats<R>(r, a.stage_i2 != 0, (int)sizeof(T)), s, a, m, r, fp64_cond);
+    return launch_chained(lk_iter_kernel<T, R>, a.tiles, pair_threads<R>(), sizeof(float) * lk_tile_smem_floats<R>(r, a.stage_i2 != 0, (int)sizeof(T)), s, a, m, r, fp64_cond);
 }
 
 template <int R>
@@ -236,9 +236,9 @@ static cudaError_t phase_for_th(const IterPhase &P, int r, float fp64_cond, cuda
     const size_t smem = sizeof(float) * lk_tile_smem_floats<R, TH, strip_kernel<R, TH>()>(r, stage, (int)sizeof(T));
     const int blocks = P.prefix[P.npairs];
     switch (P.a[0].mode) {
-    case FLOW_ZERO: return launch_chained(phase_iter_kernel<T, R, FLOW_ZERO, TH>, blocks, LK_THREADS, smem, s, P, r, fp64_cond);
-    case FLOW_SAME: return launch_chained(phase_iter_kernel<T, R, FLOW_SAME, TH>, blocks, LK_THREADS, smem, s, P, r, fp64_cond);
-    default: return launch_chained(phase_iter_kernel<T, R, FLOW_UPSAMPLE, TH>, blocks, LK_THREADS, smem, s, P, r, fp64_cond);
+    case FLOW_ZERO: return launch_chained((phase_iter_kernel<T, R, FLOW_ZERO, TH>), blocks, LK_THREADS, smem, s, P, r, fp64_cond);
+    case FLOW_SAME: return launch_chained((phase_iter_kernel<T, R, FLOW_SAME, TH>), blocks, LK_THREADS, smem, s, P, r, fp64_cond);
+    default: return launch_chained((phase_iter_kernel<T, R, FLOW_UPSAMPLE, TH>), blocks, LK_THREADS, smem, s, P, r, fp64_cond);
     }
 }
 

@@ -622,11 +622,21 @@ int run_batch(int32_t n, const of_handle *hs, const void *const *I1s, const void
 {
     if (n == 0) return OF_OK;
     if (!hs || !hs[0]) return OF_EINVAL;
-    const Tuning t = effective(hs[0]->plan, t_in);
+    Tuning t = effective(hs[0]->plan, t_in);
     BatchBuild b;
     int rc = build_batch(n, hs, I1s, I2s, us, vs, b);
     if (rc) return rc;
     const of_plan &p0 = hs[0]->plan;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const bool graphs = st != nullptr && !(p0.flags & OF_FLAG_NO_GRAPH) && cudaStreamIsCapturing(st, &cs) == cudaSuccess &&
+                        cs == cudaStreamCaptureStatusNone;
+    // Without a table entry: two concurrent sequences over halves of the batch where they are
+    // branches of a graph, so that each fills the last waves and the gaps between launches of
+    // the other (us, one and two sequences: 2 x 1024^2 280, 237; 8 x 512^2 296, 255; 16 x 256^2
+    // 239, 195; 64 x 1024^2 5070, 4840; three and four are no better). One where the launches
+    // are queued one by one, which twice as many would take longer, and for the variant,
+    // whose launches are nearer to the memory's rate (16 x 1024^2 1536, 1563).
+    if (t.branches == BRANCHES_AUTO) t.branches = graphs && n > 1 && !(p0.flags & OF_FLAG_I1GRAD) ? 2 : 0;
     const size_t pairs_bytes = sizeof(BatchPair) * n, prefix_bytes = sizeof(int32_t) * b.prefix.size();
     std::vector<char> key(pairs_bytes + prefix_bytes + sizeof(st) + 7 * sizeof(int));
     {
@@ -684,9 +694,6 @@ int run_batch(int32_t n, const of_handle *hs, const void *const *I1s, const void
         }
         // capture [reset barrier, persistent kernel] or the phase launches as a graph when
         // the stream allows it
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        const bool graphs = st != nullptr && !(p0.flags & OF_FLAG_NO_GRAPH) &&
-                            cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
         if (graphs) {
             cudaGraph_t g = nullptr;
             if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {

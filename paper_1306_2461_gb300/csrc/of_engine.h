@@ -70,6 +70,7 @@ void drop_graphs(of_ctx *h);
 // cudaMalloc that honours of_debug_fail_allocs (injected out-of-memory failures).
 cudaError_t dev_malloc(void **p, size_t bytes);
 
+constexpr int BRANCHES_AUTO = -1;
 // How one persistent batched launch is run (the autotuner's choice; see tune.cu).
 struct Tuning {
     int generic_sums = 0;    // 1: the run-time-radius kernel (per-output sums); 0: grouped fixed-radius sums
@@ -78,7 +79,8 @@ struct Tuning {
     int phased = 1;          // 1: one ordinary launch per phase; 0: the persistent launch with grid barriers
     int prefetch = 0;        // phase launches: warm L2 for the tile this many blocks per SM ahead (0: off)
     int tile_h = 0;          // phase launches with grouped sums: iteration tile height (0: the default)
-    int branches = 0;        // phase launches: concurrent launch sequences over parts of the batch (0: one)
+    int branches = 0;        // phase launches: concurrent launch sequences over parts of the batch (0: one;
+                             // BRANCHES_AUTO, without a table entry: run_batch chooses)
     int fusion = 0;          // phase launches: 2 fuses pairs of same-level iterations in one launch per tile
                              // (fixed radii, default tile height); 0 or 1: one iteration per launch
     int strip = 0;           // phase launches with grouped sums: tiles per block along y (1, 2, 4; 0: 4)

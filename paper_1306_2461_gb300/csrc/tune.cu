@@ -68,7 +68,10 @@ Tuning tuning_for(const of_plan &method, int size_class)
 {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_table.find(key_of(method, size_class));
-    return it == g_table.end() ? Tuning() : it->second;
+    if (it != g_table.end()) return it->second;
+    Tuning t;
+    t.branches = BRANCHES_AUTO;
+    return t;
 }
 
 int batch_size_class(int32_t n, const of_handle *hs)

@@ -321,7 +321,7 @@ def tuning_get(method: Plan, size_class: int) -> dict | None:
 
 def tuning_set(method: Plan, size_class: int, generic_sums=0, stage_i2=1, blocks_per_sm=0, phased=1, prefetch=0,
                tile_h=0, branches=0, fusion=1, strip=4):
-    """of_tuning_set; the defaults are the library's tuning without a table entry."""
+    """of_tuning_set; the defaults are the library's tuning without a table entry, in one sequence."""
     t = Tuning(int(generic_sums), int(stage_i2), int(blocks_per_sm), int(phased), int(prefetch), int(tile_h),
                int(branches), int(fusion), int(strip), 0.0)
     _check(_lib.of_tuning_set(ctypes.byref(method), int(size_class), ctypes.byref(t)), "of_tuning_set")

@@ -355,7 +355,7 @@ static cudaError_t enqueue_chain(const BatchPair *pairs, int n, const of_plan &p
             long tiles_l = 0;
             for (int i = 0; i < m; ++i) tiles_l += strip_units(bp[i].H[l], bp[i].W[l], tile_h, 1);
             while (kl > 1 && tiles_l < (long)kl * OF_STRIP_WAVES * 4 * sms) kl /= 2;
-            const bool small = !i1grad && !two && tile_h == LK_TH && !t.generic_sums && radius_grouped(p0.radius) &&
+            const bool small = !two && tile_h == LK_TH && !t.generic_sums && radius_grouped(p0.radius) &&
                                prefetch_ahead == 0 && use_small_tiles(tiles_l, sms);
             const int th_l = small ? SM_TH : tile_h;
             for (int i = 0; i < m; ++i) {
@@ -385,22 +385,22 @@ static cudaError_t enqueue_chain(const BatchPair *pairs, int n, const of_plan &p
                     a.fout_pitch = bp[i].pitch[l];
                 }
                 a.tiles_x = (a.W + LK_TW - 1) / LK_TW;
-                // the variant's kernels and the fused kernel have their own tile height
-                const int th = i1grad ? I1_TH : (two ? LK_TH : tile_h);
-                a.strip = (i1grad || two) ? 1 : kl;
+                // the variant's run-time-radius kernel and the fused kernel have their own tile height
+                const int th = i1grad && (t.generic_sums || !radius_grouped(p0.radius)) ? I1_TH : (two ? LK_TH : tile_h);
+                a.strip = two ? 1 : kl;
                 a.tiles = strip_units(a.H, a.W, th, a.strip);
                 a.status = bp[i].status;
-                a.stage_i2 = (i1grad || two) ? 0 : stage;   // the fused kernel gathers
+                a.hess = bp[i].hess;
+                a.hess_pitch = bp[i].pitch[l];
+                a.stage_i2 = two ? 0 : stage;   // the fused kernel gathers
                 if (small) {
                     a.tiles_x = small_tiles_x(a.W);
                     a.tiles = small_units(a.H, a.W);
                 }
                 if (a.stage_i2) fill_stage_maps(a, I.m[i], level_elem(p0, l), p0.radius, th_l, true);   // else gathered
-                a.hess = bp[i].hess;
-                a.hess_pitch = bp[i].pitch[l];
                 I.prefix[i + 1] = I.prefix[i] + a.tiles;
             }
-            e = i1grad ? launch_phase_i1_iter(I, level_elem(p0, l), p0.radius, t.generic_sums != 0, p0.fp64_cond, st)
+            e = i1grad ? launch_phase_i1_iter(I, level_elem(p0, l), p0.radius, t.generic_sums != 0, p0.fp64_cond, th_l, st)
                 : two  ? launch_phase_iter2(I, level_elem(p0, l), p0.radius, p0.fp64_cond, st)
                        : launch_phase_iter(I, level_elem(p0, l), p0.radius, t.generic_sums != 0, p0.fp64_cond, th_l,
                                            st);
@@ -501,13 +501,13 @@ static cudaError_t enqueue_phased(const std::vector<BatchPair> &pairs, const of_
 }
 
 // The variant with the first image's gradient runs as phase launches only (it has no
-// persistent form) and gathers its 4 taps (no staging).
+// persistent form).
 static Tuning effective(const of_plan &p0, Tuning t)
 {
     if (p0.flags & OF_FLAG_I1GRAD) {
         t.phased = 1;
         t.blocks_per_sm = 0;
-        t.stage_i2 = 0;
+        t.stage_i2 = t.generic_sums ? 0 : 1;
         t.tile_h = 0;
         t.fusion = 0;
     }

@@ -105,8 +105,9 @@ __device__ __forceinline__ void i1_hess_tile(const HessArgs &a, int tile, int r,
     }
 }
 
-// One iteration of the variant on one output tile.
-template <typename T, int R>
+// One iteration of the variant on one output tile, for any window radius r given at run time
+// (the fixed radii run the tiles of the main method with the variant's stage 1 and solve).
+template <typename T>
 __device__ __forceinline__ void i1_iter_tile(const IterArgs &a, int tile, int r, float fp64_cond, float *smem)
 {
     const int tyi = tile / a.tiles_x;
@@ -114,89 +115,37 @@ __device__ __forceinline__ void i1_iter_tile(const IterArgs &a, int tile, int r,
     const T *I1 = static_cast<const T *>(a.I1);
     const T *I2 = static_cast<const T *>(a.I2);
     const float2 ref = flow_at<false>(a, min(tx0 + LK_TW / 2, a.W - 1), min(ty0 + I1_TH / 2, a.H - 1));
-    const int rr = R == 0 ? r : R;
-    const int RH = I1_TH + 2 * rr, RW = LK_TW + 2 * rr;
-    const int plane = i1_plane<R>(RH, RW);
-    const int rowlen = i1_rowlen<R>(RW);
-    const int nreg = RH * RW;
-    // the current estimates of S1 region pixels are loaded before any is used
-    constexpr int S1 = 4;
-#pragma unroll 1
-    for (int i0 = threadIdx.x; i0 < nreg; i0 += S1 * LK_THREADS) {
-        float2 f[S1];
-        bool in[S1];
-#pragma unroll
-        for (int k = 0; k < S1; ++k) {
-            const int i = i0 + k * LK_THREADS;
-            const int ry = i / RW, rx = i - ry * RW;
-            const int y = ty0 - rr + ry, x = tx0 - rr + rx;
-            in[k] = i < nreg && (unsigned)y < (unsigned)a.H && (unsigned)x < (unsigned)a.W;
-            f[k] = in[k] ? flow_at<false>(a, x, y) : make_float2(0.0f, 0.0f);
+    const int RH = I1_TH + 2 * r, RW = LK_TW + 2 * r;
+    const int plane = RH * RW;
+    for (int i = threadIdx.x; i < plane; i += LK_THREADS) {
+        const int ry = i / RW, rx = i - ry * RW;
+        const int y = ty0 - r + ry, x = tx0 - r + rx;
+        float p0 = 0.0f, p1 = 0.0f;
+        if ((unsigned)y < (unsigned)a.H && (unsigned)x < (unsigned)a.W) {
+            const float2 f = flow_at<false>(a, x, y);
+            float c, gx, gy;
+            i1_grad<false>(I1, a.pitch, a.H, a.W, x, y, c, gx, gy);
+            const float Iw = bil_at<false>(I2, a.pitch, a.H, a.W, x, y, f.x, f.y);
+            const float e = resid(c, Iw, gx, gy, f.x - ref.x, f.y - ref.y);
+            p0 = gx * e;
+            p1 = gy * e;
         }
-#pragma unroll
-        for (int k = 0; k < S1; ++k) {
-            const int i = i0 + k * LK_THREADS;
-            if (i >= nreg) break;
-            const int ry = i / RW, rx = i - ry * RW;
-            const int y = ty0 - rr + ry, x = tx0 - rr + rx;
-            float p0 = 0.0f, p1 = 0.0f;
-            if (in[k]) {
-                float c, gx, gy;
-                i1_grad<false>(I1, a.pitch, a.H, a.W, x, y, c, gx, gy);
-                const float Iw = bil_at<false>(I2, a.pitch, a.H, a.W, x, y, f[k].x, f[k].y);
-                const float e = resid(c, Iw, gx, gy, f[k].x - ref.x, f[k].y - ref.y);
-                p0 = gx * e;
-                p1 = gy * e;
-            }
-            float *q = smem + ry * rowlen + rx;
-            q[0] = p0;
-            q[plane] = p1;
-        }
+        smem[i] = p0;
+        smem[plane + i] = p1;
     }
     __syncthreads();
-    auto matrix = [&](int x, int y) { return a.hess[(size_t)y * a.hess_pitch + x]; };
-    auto finish = [&](int x, int y, float4 h, float d, float e) {
-        const float s[5] = {h.x, h.y, h.z, d, e};
-        float xu, xv;
-        const float2 f = solve2(s, fp64_cond, xu, xv) ? make_float2(ref.x + xu, ref.y + xv) : flow_at<false>(a, x, y);
-        if (a.fout) {
-            a.fout[(size_t)y * a.fout_pitch + x] = f;
-        } else {
-            a.u_out[(size_t)y * a.W + x] = f.x;
-            a.v_out[(size_t)y * a.W + x] = f.y;
-        }
-    };
-    if constexpr (R == 0) {
-        float *S = smem + 2 * plane;
-        box_hsum<2>(smem, S, RH, RW, r);
-        __syncthreads();
-        for (int i = threadIdx.x; i < I1_TH * LK_TW; i += LK_THREADS) {
-            const int ty = i / LK_TW, tx = i - ty * LK_TW;
-            const int y = ty0 + ty, x = tx0 + tx;
-            if (y >= a.H || x >= a.W) continue;
-            float s[2];
-            box_vsum<2>(S, RH, r, ty, tx, s);
-            finish(x, y, matrix(x, y), s[0], s[1]);
-        }
-    } else {
-        box_h_inplace<R, 2, I1_TH>(smem);
-#pragma unroll 1
-        for (int i = threadIdx.x; i < LK_TW * (I1_TH / 4); i += LK_THREADS) {
-            const int tx = i % LK_TW, g = i / LK_TW;
-            const int x = tx0 + tx;
-            if (x >= a.W || ty0 + 4 * g >= a.H) continue;
-            float4 h[4];   // loaded together, before the first row is written
-#pragma unroll
-            for (int j = 0; j < 4; ++j) h[j] = matrix(x, min(ty0 + 4 * g + j, a.H - 1));
-            float s[2][4];
-            box_v4<R, 2, I1_TH>(smem, g, tx, s);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int y = ty0 + 4 * g + j;
-                if (y >= a.H) break;
-                finish(x, y, h[j], s[0][j], s[1][j]);
-            }
-        }
+    float *S = smem + 2 * plane;
+    box_hsum<2>(smem, S, RH, RW, r);
+    __syncthreads();
+    for (int i = threadIdx.x; i < I1_TH * LK_TW; i += LK_THREADS) {
+        const int ty = i / LK_TW, tx = i - ty * LK_TW;
+        const int y = ty0 + ty, x = tx0 + tx;
+        if (y >= a.H || x >= a.W) continue;
+        float s[2];
+        box_vsum<2>(S, RH, r, ty, tx, s);
+        const float4 h = a.hess[(size_t)y * a.hess_pitch + x];
+        const float sj[5] = {h.x, h.y, h.z, s[0], s[1]};
+        solve_store<false, -1>(a, x, y, ref, fp64_cond, sj);
     }
 }
 
@@ -208,15 +157,45 @@ __global__ void __launch_bounds__(LK_THREADS) i1_hess_kernel(HessArgs a, int r)
     i1_hess_tile<T, R>(a, blockIdx.x, r, reinterpret_cast<float *>(smem4));
 }
 
+// Resident blocks per SM. The iteration is bound by latency and then by memory (36 bytes per
+// pixel): as the main method's tiles, with one product plane, a level-0 launch of 16 pairs of
+// 1024^2 at r = 4 takes 153 us (157 with 4 blocks per SM, 160 with 6 at 40 registers; its bytes 89 us),
+// with tiles of their own that gathered every tap and estimate one pixel at a time 188; r = 10
+// 177 instead of 295. A 1024^2 pair 203 -> 158 us.
 #ifndef OF_I1_MIN_BLOCKS
-#define OF_I1_MIN_BLOCKS 6
+#define OF_I1_MIN_BLOCKS 5
 #endif
+template <int R> constexpr int i1_min_blocks() { return R == 0 ? 4 : (R <= 6 ? OF_I1_MIN_BLOCKS : (R <= 12 ? 4 : 3)); }
+
 template <typename T, int R>
-__global__ void __launch_bounds__(LK_THREADS, OF_I1_MIN_BLOCKS) i1_iter_kernel(IterArgs a, int r, float fp64_cond)
+__global__ void __launch_bounds__(LK_THREADS, i1_min_blocks<R>())
+i1_iter_kernel(const __grid_constant__ IterArgs a, const __grid_constant__ StageMaps m, int r, float fp64_cond)
 {
-    extern __shared__ float4 smem4[];
-    chain_begin();
-    i1_iter_tile<T, R>(a, blockIdx.x, r, fp64_cond, reinterpret_cast<float *>(smem4));
+    extern __shared__ __align__(128) float4 smem4[];
+    float *smem = reinterpret_cast<float *>(smem4);
+    if constexpr (R == 0) {
+        chain_begin();
+        i1_iter_tile<T>(a, blockIdx.x, r, fp64_cond, smem);
+    } else {
+        uint32_t phase = 0;
+        lk_tile_init<R, LK_TH, LK_TW, false, true>(smem);
+        chain_begin();
+        lk_tile_fixed<T, false, R, -1, LK_TH, false, LK_THREADS, true>(a, &m, blockIdx.x, fp64_cond, smem, phase);
+    }
+}
+
+// Small tiles of one pair.
+template <typename T, int R>
+__global__ void __launch_bounds__(SM_THREADS, i1_min_blocks<R>())
+i1_small_kernel(const __grid_constant__ IterArgs a, const __grid_constant__ StageMaps m, float fp64_cond)
+{
+    extern __shared__ __align__(128) float4 smem4[];
+    float *smem = reinterpret_cast<float *>(smem4);
+    if constexpr (R != 0) {
+        lk_tile_init<R, SM_TH, SM_TW, false, true>(smem);
+        chain_begin();
+        lk_tile_small<T, false, R, -1, true>(a, &m, blockIdx.x, fp64_cond, smem);
+    }
 }
 
 // The same over the tiles of up to PHASE_PAIRS pairs (batched form).
@@ -230,20 +209,61 @@ __global__ void __launch_bounds__(LK_THREADS) phase_hess_kernel(const __grid_con
 }
 
 template <typename T, int R>
-__global__ void __launch_bounds__(LK_THREADS, OF_I1_MIN_BLOCKS)
+__global__ void __launch_bounds__(LK_THREADS, i1_min_blocks<R>())
 phase_i1_iter_kernel(const __grid_constant__ IterPhase P, int r, float fp64_cond)
 {
-    extern __shared__ float4 smem4[];
-    chain_begin();
-    if constexpr (R != 0) {
+    extern __shared__ __align__(128) float4 smem4[];
+    float *smem = reinterpret_cast<float *>(smem4);
+    const int p = phase_pair(P.prefix, P.npairs, blockIdx.x);
+    const int unit = blockIdx.x - P.prefix[p];
+    if constexpr (R == 0) {
+        chain_begin();
+        i1_iter_tile<T>(P.a[p], unit, r, fp64_cond, smem);
+    } else {
+        constexpr bool MULTI = LK_TH >= 2 * R;
+        uint32_t phase = 0;
+        lk_tile_init<R, LK_TH, LK_TW, MULTI, true>(smem);
+        chain_begin();
         const int t2 = blockIdx.x + P.ahead;
         if (P.ahead > 0 && t2 < P.prefix[P.npairs]) {
             const int q = phase_pair(P.prefix, P.npairs, t2);
-            prefetch_tile<T, -1, I1_TH>(P.a[q], t2 - P.prefix[q], R);
+            prefetch_tile<T, -1, LK_TH>(P.a[q], t2 - P.prefix[q], R);
         }
+        lk_tile_fixed<T, false, R, -1, LK_TH, MULTI, LK_THREADS, true>(P.a[p], &P.m[p], unit, fp64_cond, smem, phase);
     }
-    const int p = phase_pair(P.prefix, P.npairs, blockIdx.x);
-    i1_iter_tile<T, R>(P.a[p], blockIdx.x - P.prefix[p], r, fp64_cond, reinterpret_cast<float *>(smem4));
+}
+
+template <typename T, int R>
+__global__ void __launch_bounds__(SM_THREADS, i1_min_blocks<R>())
+phase_i1_small_kernel(const __grid_constant__ IterPhase P, float fp64_cond)
+{
+    extern __shared__ __align__(128) float4 smem4[];
+    float *smem = reinterpret_cast<float *>(smem4);
+    if constexpr (R != 0) {
+        const int p = phase_pair(P.prefix, P.npairs, blockIdx.x);
+        lk_tile_init<R, SM_TH, SM_TW, false, true>(smem);
+        chain_begin();
+        lk_tile_small<T, false, R, -1, true>(P.a[p], &P.m[p], blockIdx.x - P.prefix[p], fp64_cond, smem);
+    }
+}
+
+// Dynamic shared memory of the variant's iteration kernels (bytes).
+template <int R> inline size_t i1_iter_smem(int r, bool strips, bool small, bool stage, int elem_bytes)
+{
+    if constexpr (R == 0) {
+        return sizeof(float) * (size_t)i1_smem_floats<0>(r, 2);
+    } else {
+        using S = FixedTile<R, SM_TH, SM_TW, true>;
+        using F = FixedTile<R, LK_TH, LK_TW, true>;
+        int f;
+        if (small) f = stage ? S::smem_staged(elem_bytes) : S::SMEM_NOSTAGE;
+        else f = stage ? F::smem_staged(elem_bytes) : F::SMEM_NOSTAGE;
+        if constexpr (LK_TH >= 2 * R) {
+            using X = StripTile<R, LK_TH, true>;
+            if (strips && !small) f = stage ? X::smem_staged(elem_bytes) : X::SMEM_NOSTAGE;
+        }
+        return sizeof(float) * (size_t)f;
+    }
 }
 
 }  // namespace of

@@ -99,12 +99,13 @@ cudaError_t launch_i1_hess(const HessArgs &a, int elem, int radius, cudaStream_t
 }
 
 #define OF_CASE_I1(R) \
-    case R: return i1_launch<R>(a, elem, radius, fp64_cond, s);
-cudaError_t launch_i1_iter(const IterArgs &a, int elem, int radius, float fp64_cond, cudaStream_t s)
+    case R: return i1_launch<R>(a, m, elem, radius, fp64_cond, small, s);
+cudaError_t launch_i1_iter(const IterArgs &a, const StageMaps &m, int elem, int radius, float fp64_cond, bool small,
+                           cudaStream_t s)
 {
     switch (radius) {
         OF_RADII(OF_CASE_I1) OF_RADII_MORE(OF_CASE_I1)
-    default: return i1_launch<0>(a, elem, radius, fp64_cond, s);
+    default: return i1_launch<0>(a, m, elem, radius, fp64_cond, false, s);
     }
 }
 
@@ -142,14 +143,14 @@ cudaError_t launch_phase_hess(const HessPhase &P, int elem, int radius, bool gen
 }
 
 #define OF_CASE_PHI(R) \
-    case R: return phase_i1_launch<R>(P, elem, radius, fp64_cond, s);
-cudaError_t launch_phase_i1_iter(const IterPhase &P, int elem, int radius, bool generic, float fp64_cond,
+    case R: return phase_i1_launch<R>(P, elem, radius, fp64_cond, tile_h, s);
+cudaError_t launch_phase_i1_iter(const IterPhase &P, int elem, int radius, bool generic, float fp64_cond, int tile_h,
                                  cudaStream_t s)
 {
-    if (generic) return phase_i1_launch<0>(P, elem, radius, fp64_cond, s);
+    if (generic) return phase_i1_launch<0>(P, elem, radius, fp64_cond, 0, s);
     switch (radius) {
         OF_RADII(OF_CASE_PHI) OF_RADII_MORE(OF_CASE_PHI)
-    default: return phase_i1_launch<0>(P, elem, radius, fp64_cond, s);
+    default: return phase_i1_launch<0>(P, elem, radius, fp64_cond, 0, s);
     }
 }
 

@@ -214,27 +214,26 @@ cudaError_t enqueue_pair(of_ctx *h, const void *I1, const void *I2, float *u, fl
                 a.fout_pitch = L.pitch[l];
             }
             a.tiles_x = (a.W + LK_TW - 1) / LK_TW;
-            const int th = i1grad ? I1_TH : LK_TH;   // the variant's kernels have their own tile height
+            const bool fixed = radius_grouped(p.radius);
             a.strip = 1;   // one tile per block: the most blocks for one pair
-            a.tiles = strip_units(a.H, a.W, th, a.strip);
+            a.tiles = strip_units(a.H, a.W, i1grad && !fixed ? I1_TH : LK_TH, a.strip);
             a.status = h->status;
-            a.stage_i2 = !(p.flags & OF_FLAG_GATHER) && !i1grad ? 1 : 0;
+            a.stage_i2 = p.flags & OF_FLAG_GATHER ? 0 : 1;
+            if (i1grad) {
+                a.hess = h->hess;
+                a.hess_pitch = L.pitch[l];
+            }
             StageMaps maps;
             memset(&maps, 0, sizeof(maps));
             // few tiles: small ones, so that the launch is spread over the SMs
-            const bool small = !i1grad && radius_grouped(p.radius) && use_small_tiles(a.tiles, sms);
+            const bool small = fixed && use_small_tiles(a.tiles, sms);
             if (small) {
                 a.tiles_x = small_tiles_x(a.W);
                 a.tiles = small_units(a.H, a.W);
             }
             if (a.stage_i2) fill_stage_maps(a, maps, level_elem(p, l), p.radius, small ? SM_TH : LK_TH, false);   // else gathered
-            if (i1grad) {
-                a.hess = h->hess;
-                a.hess_pitch = L.pitch[l];
-                e = launch_i1_iter(a, level_elem(p, l), p.radius, p.fp64_cond, st);
-            } else {
-                e = launch_lk_iter(a, maps, level_elem(p, l), p.radius, p.fp64_cond, small, st);
-            }
+            e = i1grad ? launch_i1_iter(a, maps, level_elem(p, l), p.radius, p.fp64_cond, small, st)
+                       : launch_lk_iter(a, maps, level_elem(p, l), p.radius, p.fp64_cond, small, st);
             if (e != cudaSuccess) return e;
             cur = 1 - cur;
         }

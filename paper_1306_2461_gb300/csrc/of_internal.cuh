@@ -193,8 +193,8 @@ inline __host__ __device__ int strip_units(int H, int W, int tile_h, int strip)
 inline int small_tiles_x(int W) { return (W + SM_TW - 1) / SM_TW; }
 inline int small_units(int H, int W) { return small_tiles_x(W) * ((H + SM_TH - 1) / SM_TH); }
 
-// Output tile height of the first-image-gradient variant's kernels (two product planes,
-// so a taller tile still leaves room for many blocks per SM).
+// Output tile height of the first-image-gradient variant's window-matrix kernel and of its
+// run-time-radius iteration.
 #ifndef OF_I1_TH
 #define OF_I1_TH 32
 #endif
@@ -286,7 +286,8 @@ cudaError_t launch_window_sums(const float *ch, int H, int W, int r, float *out,
 // The variant linearised with the first image's gradient: window matrix of one level,
 // then iterations that read it from a.hess.
 cudaError_t launch_i1_hess(const HessArgs &a, int elem, int radius, cudaStream_t s);
-cudaError_t launch_i1_iter(const IterArgs &a, int elem, int radius, float fp64_cond, cudaStream_t s);
+cudaError_t launch_i1_iter(const IterArgs &a, const StageMaps &m, int elem, int radius, float fp64_cond, bool small,
+                           cudaStream_t s);
 // Phase launches of the batched method (grid = P.prefix[P.npairs] blocks).
 cudaError_t launch_phase_pyr(const PyrPhase &P, bool first, int in_format, int storage, cudaStream_t s);
 cudaError_t launch_phase_zn(const ZnPhase &P, int in_format, int storage, cudaStream_t s);
@@ -299,7 +300,7 @@ cudaError_t launch_phase_iter(const IterPhase &P, int elem, int radius, bool gen
 cudaError_t launch_phase_iter2(const IterPhase &P, int elem, int radius, float fp64_cond, cudaStream_t s);
 // The first-image-gradient variant: window matrices of one level, then its iterations.
 cudaError_t launch_phase_hess(const HessPhase &P, int elem, int radius, bool generic, cudaStream_t s);
-cudaError_t launch_phase_i1_iter(const IterPhase &P, int elem, int radius, bool generic, float fp64_cond,
+cudaError_t launch_phase_i1_iter(const IterPhase &P, int elem, int radius, bool generic, float fp64_cond, int tile_h,
                                  cudaStream_t s);
 void *batch_kernel_for(int in_format, int storage, int radius);
 size_t batch_smem_bytes(int radius, bool stage_i2);
@@ -330,8 +331,11 @@ template <int R> cudaError_t ws_launch(const float *ch, int H, int W, int r, flo
 template <int R> cudaError_t i1h_launch(const HessArgs &a, int elem, int r, cudaStream_t s);
 template <int R> cudaError_t phase_launch(const IterPhase &P, int elem, int r, float fp64_cond, int tile_h, cudaStream_t s);
 template <int R> cudaError_t phase_hess_launch(const HessPhase &P, int elem, int r, cudaStream_t s);
-template <int R> cudaError_t phase_i1_launch(const IterPhase &P, int elem, int r, float fp64_cond, cudaStream_t s);
-template <int R> cudaError_t i1_launch(const IterArgs &a, int elem, int r, float fp64_cond, cudaStream_t s);
+template <int R>
+cudaError_t phase_i1_launch(const IterPhase &P, int elem, int r, float fp64_cond, int tile_h, cudaStream_t s);
+template <int R>
+cudaError_t i1_launch(const IterArgs &a, const StageMaps &m, int elem, int r, float fp64_cond, bool small,
+                      cudaStream_t s);
 template <int R> void *batch_kernel_ptr(int in_format, int storage);
 template <int R> cudaError_t radius_configure();
 template <int R> size_t radius_smem_bytes(int r, bool stage_i2);

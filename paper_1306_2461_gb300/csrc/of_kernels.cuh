@@ -640,7 +640,7 @@ __device__ __forceinline__ void lk_tile_generic(const IterArgs &a, int tile, int
 // at multiples of 4 in image coordinates (tiles are multiples of 4 wide and high), so
 // the order of the additions depends only on the pixel's position, not on the tiling:
 // the batched and the per-pair launches give the same bits.
-template <int R, int TH = LK_TH, int TW = LK_TW> struct FixedTile {
+template <int R, int TH = LK_TH, int TW = LK_TW, bool V = false> struct FixedTile {
     static_assert(R >= 2, "the grouped box sums need 2R >= 4");
     static constexpr int W = 2 * R + 1;                // window width
     static constexpr int NV4 = (2 * R + 4 + 3) / 4;    // float4 loads for 4 outputs' windows
@@ -680,7 +680,8 @@ template <int R, int TH = LK_TH, int TW = LK_TW> struct FixedTile {
     static constexpr int RWP2 = RWE + 2;
     static_assert(RWP1 % 4 == 0 && RWP2 % 4 == 2, "row lengths");
     static constexpr int PAIR_PLANE = RH * RWP2;             // float2 per pair plane
-    static constexpr int PLANES = 4 * PAIR_PLANE + RH * RWP1;  // floats of the three planes
+    // floats of the three planes (V: the variant with the first image's gradient, P01 alone)
+    static constexpr int PLANES = 2 * PAIR_PLANE + (V ? 0 : 2 * PAIR_PLANE + RH * RWP1);
     static_assert(PLANES % 4 == 0, "the barrier after the planes must be 8-byte aligned");
     static constexpr int OFF_BAR = PLANES;                    // 8-byte mbarrier
     static constexpr int OFF_WIN = (OFF_BAR + 2 + 31) / 32 * 32;   // 128-byte aligned staging window
@@ -708,15 +709,15 @@ template <int R, int TH = LK_TH, int TW = LK_TW> struct FixedTile {
 // tile; RPAD puts the first row after the 2R carried ones in a slot that is a multiple of 8
 // (a 128-byte boundary), so that the estimate of the rows a tile computes comes in TMA boxes
 // of 8 rows.
-template <int R, int TH> struct StripTile {
-    using F = FixedTile<R, TH>;
+template <int R, int TH, bool V = false> struct StripTile {
+    using F = FixedTile<R, TH, LK_TW, V>;
     static_assert(TH % 8 == 0, "boxes of 8 rows");
     static constexpr int RPAD = (8 - 2 * R % 8) % 8;
     static constexpr int RING = RPAD + F::RH;
     static constexpr int BOX = 8;
     static constexpr int BOX_BYTES = F::RWP2 * BOX * 8;
     static constexpr int PAIR_PLANE = RING * F::RWP2;
-    static constexpr int PLANES = 4 * PAIR_PLANE + RING * F::RWP1;
+    static constexpr int PLANES = 2 * PAIR_PLANE + (V ? 0 : 2 * PAIR_PLANE + RING * F::RWP1);
     static constexpr int OFF_BAR = PLANES;
     static constexpr int OFF_WREF = OFF_BAR + 2;              // the tile-centre estimates (4 float2)
     static constexpr int OFF_WIN = (OFF_WREF + 8 + 31) / 32 * 32;
@@ -1100,7 +1101,7 @@ template <int R, int TH> constexpr int v_rows() { return (TH % 6 == 0 && R >= 3)
 
 // Vertical pass for the VR = v_rows outputs of item g (rows VR g .. VR g + VR - 1, column
 // tx): sums of the three planes. The rows read wrap around once at most in a ring.
-template <int R, int TH, int TW = LK_TW, int RN = 0>
+template <int R, int TH, int TW = LK_TW, int RN = 0, bool V = false>
 __device__ __forceinline__ void box_v_planes(const float2 *P01, const float2 *P23, const float *P4, int g, int tx,
                                              float2 s01[v_rows<R, TH>()], float2 s23[v_rows<R, TH>()],
                                              float s4[v_rows<R, TH>()], int base = 0)
@@ -1117,6 +1118,7 @@ __device__ __forceinline__ void box_v_planes(const float2 *P01, const float2 *P2
         if constexpr (VR == 6) box6v<R>(v, s01);
         else box4v<R, 0>(v, s01);
     }
+    if constexpr (V) return;   // the variant's two channels
     {
         float2 v[NV];
 #pragma unroll
@@ -1173,7 +1175,7 @@ template <int R, int VR, int J, typename V> __device__ __forceinline__ void box2
     }
 }
 
-template <int R, int TH, int TW, int J>
+template <int R, int TH, int TW, int J, bool V>
 __device__ __forceinline__ void box_v_two(const float2 *P01, const float2 *P23, const float *P4, int g, int tx,
                                           float2 s01[2], float2 s23[2], float s4[2])
 {
@@ -1181,14 +1183,17 @@ __device__ __forceinline__ void box_v_two(const float2 *P01, const float2 *P23, 
     constexpr int VR = v_rows<R, TH>(), NV = 2 * R + 2;
     const int row = VR * g + J;
     {
-        float2 v[NV], w[NV];
+        float2 v[NV];
 #pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            v[q] = P01[(row + q) * F::RWP2 + tx];
-            w[q] = P23[(row + q) * F::RWP2 + tx];
-        }
+        for (int q = 0; q < NV; ++q) v[q] = P01[(row + q) * F::RWP2 + tx];
         box2v<R, VR, J>(v, s01);
-        box2v<R, VR, J>(w, s23);
+    }
+    if constexpr (V) return;
+    {
+        float2 v[NV];
+#pragma unroll
+        for (int q = 0; q < NV; ++q) v[q] = P23[(row + q) * F::RWP2 + tx];
+        box2v<R, VR, J>(v, s23);
     }
     float v[NV];
 #pragma unroll
@@ -1270,6 +1275,80 @@ __device__ __forceinline__ void stage1_pair(const IterArgs &a, int x, int y, flo
     }
 }
 
+// Stage 1 of the variant linearised with the first image's gradient, for the pixel pair: g1 is
+// the central difference of I1 at the pixels (neighbour indices clamped, halved), e~ = I1 -
+// I2(x + u) + g1 . (u - ref), and the products are the two right-hand-side channels g1 e~.
+template <typename T, bool NC, int MODE, int WW, int WH, bool INNER>
+__device__ __forceinline__ void stage1_pair_i1(const IterArgs &a, int x, int y, float2 ref, const float4 *sflow,
+                                               const T *win, int wx0, int wy0, float4 &s01)
+{
+    s01 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    const bool rowin = INNER || (unsigned)y < (unsigned)a.H;
+    const bool inp = rowin && (INNER || (unsigned)x < (unsigned)a.W);
+    const bool inq = rowin && (INNER || (unsigned)(x + 1) < (unsigned)a.W);   // implies inp (x even)
+    if (!inp) return;
+    const T *I1 = static_cast<const T *>(a.I1);
+    const T *I2 = static_cast<const T *>(a.I2);
+    float2 fp, fq;
+    if (sflow) {
+        const float4 w = *sflow;
+        fp = f2(w.x, w.y);
+        fq = f2(w.z, w.w);
+    } else {
+        flow_pair<NC, MODE>(a, x, y, inq, fp, fq);
+    }
+    const T *row = I1 + (y * a.pitch + x);
+    const float2 c = ld_pair<NC>(row, inq);
+    const float2 up = ld_pair<NC>(INNER || y > 0 ? row - a.pitch : row, inq);
+    const float2 dn = ld_pair<NC>(INNER || y + 1 < a.H ? row + a.pitch : row, inq);
+    const float lf = ldf<NC>(INNER || x > 0 ? row - 1 : row);
+    const float rt = INNER || x + 2 < a.W ? ldf<NC>(row + 2) : c.y;   // right of q (q is the last: itself)
+    const float2 half = f2(0.5f, 0.5f);
+    // p's right neighbour is q, or p itself at the last column
+    const float2 GX = mul2(sub2(f2(inq ? c.y : c.x, rt), f2(lf, c.x)), half);
+    const float2 GY = mul2(sub2(dn, up), half);
+    const float2 FU = f2(floorf(fp.x), floorf(fq.x)), FV = f2(floorf(fp.y), floorf(fq.y));
+    const float2 AX = sub2(f2(fp.x, fq.x), FU), AY = sub2(f2(fp.y, fq.y), FV);
+    const int xp = pos_floor(x, FU.x), yp = pos_floor(y, FV.x);
+    const int xq = pos_floor(x + 1, FU.y), yq = pos_floor(y, FV.y);
+    const int cpx = (int)((unsigned)xp - 1u - (unsigned)wx0), cpy = (int)((unsigned)yp - 1u - (unsigned)wy0);
+    const int cqx = (int)((unsigned)xq - 1u - (unsigned)wx0), cqy = (int)((unsigned)yq - 1u - (unsigned)wy0);
+    const bool inwin = (INNER || win) && (unsigned)cpx < (unsigned)(WW - 3) && (unsigned)cqx < (unsigned)(WW - 3) &&
+                       (unsigned)cpy < (unsigned)(WH - 3) && (unsigned)cqy < (unsigned)(WH - 3);
+    bool both = inwin;
+    if constexpr (!INNER) {
+        const unsigned ws = interior_span(a.W), hs = interior_span(a.H);
+        both = inq && interior(xp, yp, ws, hs) && interior(xq, yq, ws, hs);
+    }
+    float2 IW;
+    if (both) {
+        float2 B0, B1, C0, C1;
+        if (INNER || inwin) {
+            const T *p = win + ((cpy + 1) * WW + cpx + 1), *q = win + ((cqy + 1) * WW + cqx + 1);
+            B0 = f2(ldf<false>(p), ldf<false>(q));
+            B1 = f2(ldf<false>(p + 1), ldf<false>(q + 1));
+            C0 = f2(ldf<false>(p + WW), ldf<false>(q + WW));
+            C1 = f2(ldf<false>(p + WW + 1), ldf<false>(q + WW + 1));
+        } else {
+            const T *p = I2 + (yp * a.pitch + xp), *q = I2 + (yq * a.pitch + xq);
+            B0 = f2(ldf<NC>(p), ldf<NC>(q));
+            B1 = f2(ldf<NC>(p + 1), ldf<NC>(q + 1));
+            C0 = f2(ldf<NC>(p + a.pitch), ldf<NC>(q + a.pitch));
+            C1 = f2(ldf<NC>(p + a.pitch + 1), ldf<NC>(q + a.pitch + 1));
+        }
+        const float2 one = f2(1.0f, 1.0f);
+        const float2 OX = sub2(one, AX), OY = sub2(one, AY);
+        IW = lerp2(lerp2(B0, B1, AX, OX), lerp2(C0, C1, AX, OX), AY, OY);
+    } else {
+        IW.x = bil_at<NC>(I2, a.pitch, a.H, a.W, x, y, fp.x, fp.y);
+        IW.y = inq ? bil_at<NC>(I2, a.pitch, a.H, a.W, x + 1, y, fq.x, fq.y) : 0.0f;
+    }
+    const float2 DX = sub2(f2(fp.x, fq.x), f2(ref.x, ref.x)), DY = sub2(f2(fp.y, fq.y), f2(ref.y, ref.y));
+    const float2 E = fma2(GY, DY, fma2(GX, DX, sub2(c, IW)));
+    const float2 q0 = mul2(GX, E), q1 = mul2(GY, E);
+    s01 = inq ? make_float4(q0.x, q1.x, q0.y, q1.y) : make_float4(q0.x, q1.x, 0.0f, 0.0f);
+}
+
 // The estimate that places the staged window of the TW x TH tile at (tx0, ty0): the one at
 // the tile's centre.
 template <bool NC, int MODE, int TH, int TW = LK_TW>
@@ -1294,12 +1373,13 @@ __device__ __forceinline__ void win_origin(const IterArgs &a, int tx0, int ty0, 
 }
 
 // The tile's mbarrier: initialised once per block, before the first tile.
-template <int R, int TH = LK_TH, int TW = LK_TW, bool MULTI = false> __device__ __forceinline__ void lk_tile_init(float *smem)
+template <int R, int TH = LK_TH, int TW = LK_TW, bool MULTI = false, bool V = false>
+__device__ __forceinline__ void lk_tile_init(float *smem)
 {
     if (threadIdx.x == 0) {
         constexpr int off = [] {
-            if constexpr (MULTI) return StripTile<R, TH>::OFF_BAR;
-            else return FixedTile<R, TH, TW>::OFF_BAR;
+            if constexpr (MULTI) return StripTile<R, TH, V>::OFF_BAR;
+            else return FixedTile<R, TH, TW, V>::OFF_BAR;
         }();
         mbar_init(reinterpret_cast<uint64_t *>(smem + off), 1);
         fence_proxy_async_smem();
@@ -1307,13 +1387,11 @@ template <int R, int TH = LK_TH, int TW = LK_TW, bool MULTI = false> __device__ 
     __syncthreads();
 }
 
-// The solve of one output pixel from its window sums, and the store of its new estimate
-// (pixels below the image, in: false, are computed and dropped).
+// The solve of one output pixel from its window sums, and the store of its new estimate.
 template <bool NC, int MODE>
-__device__ __forceinline__ void solve_store(const IterArgs &a, int x, int y, float2 ref, float fp64_cond, float2 s01,
-                                            float2 s23, float s4)
+__device__ __forceinline__ void solve_store(const IterArgs &a, int x, int y, float2 ref, float fp64_cond,
+                                            const float (&sj)[5])
 {
-    const float sj[5] = {s01.x, s01.y, s23.x, s23.y, s4};
     float xu, xv;
     const float2 f = solve2(sj, fp64_cond, xu, xv) ? make_float2(ref.x + xu, ref.y + xv) : flow_mode<NC, MODE>(a, x, y);
     if (a.fout) {
@@ -1324,10 +1402,47 @@ __device__ __forceinline__ void solve_store(const IterArgs &a, int x, int y, flo
     }
 }
 
+// The N output rows from yb of column x. V: the window matrices come from a.hess, three rows'
+// loaded together before the first of them is written.
+template <bool NC, int MODE, bool V, int N>
+__device__ __forceinline__ void solve_rows(const IterArgs &a, int x, int yb, float2 ref, float fp64_cond,
+                                           const float2 *s01, const float2 *s23, const float *s4)
+{
+    if constexpr (V) {
+        constexpr int B = N % 3 == 0 ? 3 : 2;
+#pragma unroll
+        for (int j0 = 0; j0 < N; j0 += B) {
+            float4 h[B];
+#pragma unroll
+            for (int j = 0; j < B; ++j) h[j] = a.hess[(size_t)min(yb + j0 + j, a.H - 1) * a.hess_pitch + x];
+#pragma unroll
+            for (int j = 0; j < B; ++j)
+                if (yb + j0 + j < a.H) {
+                    const float sj[5] = {h[j].x, h[j].y, h[j].z, s01[j0 + j].x, s01[j0 + j].y};
+                    solve_store<NC, MODE>(a, x, yb + j0 + j, ref, fp64_cond, sj);
+                }
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            if (yb + j >= a.H) break;
+            const float sj[5] = {s01[j].x, s01[j].y, s23[j].x, s23[j].y, s4[j]};
+            solve_store<NC, MODE>(a, x, yb + j, ref, fp64_cond, sj);
+        }
+    }
+}
+
+// The flow mode is `m`, known at compile time (MODE) or at run time (MODE < 0).
+template <int MODE> __device__ __forceinline__ bool mode_is(const IterArgs &a, int m)
+{
+    return MODE >= 0 ? MODE == m : a.mode == m;
+}
+
 // While a tile's copies land: bring the lines of I1 that its stage 1 reads (region rows r0..)
 // into L1 (OF_PREFETCH_I1 2; 1: into L2), and at the first iteration of a level those of the
 // coarser estimate it upsamples. Threads [t0, NT) take part.
-template <int R, int MODE, int TH, int TW, int NT, int S>
+// V: also I1's rows and columns next to the region, and the tile's window matrices into L2.
+template <int R, int MODE, int TH, int TW, int NT, int S, bool V>
 __device__ __forceinline__ void prefetch_region(const IterArgs &a, int tx0, int ty0, int r0, int t0)
 {
     using F = FixedTile<R, TH, TW>;
@@ -1337,29 +1452,40 @@ __device__ __forceinline__ void prefetch_region(const IterArgs &a, int tx0, int 
     if (t < F::RH - r0)
         prefetch_row(a.I1, a.pitch, S, a.H, a.W, ty0 - R + r0, ty0 - R + F::RH, tx0 - F::RE, tx0 - F::RE + F::RWE, t);
 #elif OF_PREFETCH_I1 == 2
-    constexpr int LPR = (F::RWE * S + 127) / 128 + 1;
+    constexpr int B = V ? 1 : 0;
+    constexpr int LPR = ((F::RWE + 2 * B) * S + 127) / 128 + 1;
     constexpr int CRH = F::RH / 2 + 2, CLPR = ((F::RWE / 2 + 2) * 8 + 127) / 128 + 1;
-    const int n1 = (F::RH - r0) * LPR;
-    const int n = n1 + (MODE == FLOW_UPSAMPLE ? CRH * CLPR : 0);
+    const int n1 = (F::RH - r0 + 2 * B) * LPR;
+    const int n = n1 + (mode_is<MODE>(a, FLOW_UPSAMPLE) ? CRH * CLPR : 0);
     for (int i = t; i < n; i += NT - t0) {
         if (i < n1)
-            prefetch_lines_l1(a.I1, a.pitch, S, a.H, a.W, ty0 - R + r0, ty0 - R + F::RH, tx0 - F::RE,
-                              tx0 - F::RE + F::RWE, LPR, i);
+            prefetch_lines_l1(a.I1, a.pitch, S, a.H, a.W, ty0 - R + r0 - B, ty0 - R + F::RH + B, tx0 - F::RE - B,
+                              tx0 - F::RE + F::RWE + B, LPR, i);
         else
             prefetch_lines_l1(a.fin, a.fin_pitch, 8, a.Hc, a.Wc, (ty0 - R) >> 1, ((ty0 - R) >> 1) + CRH,
                               (tx0 - F::RE) >> 1, ((tx0 - F::RE) >> 1) + F::RWE / 2 + 2, CLPR, i - n1);
+    }
+    if constexpr (V) {
+        constexpr int HL = TW * 16 / 128;   // lines per row of the tile's matrices
+        for (int i = t; i < TH * HL; i += NT - t0) {
+            const int y = ty0 + i / HL, x = tx0 + (i % HL) * 8;
+            if (y < a.H && x < a.W)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(a.hess + ((size_t)y * a.hess_pitch + x)));
+        }
     }
 #endif
 }
 
 // Whether the tile's region and its staged window both lie inside the image: no pixel pair of
 // its stage 1 then needs a bounds check.
-template <int R, int TH, int TW, int S>
+// V: the region with a border of one pixel, for I1's gradient.
+template <int R, int TH, int TW, int S, bool V>
 __device__ __forceinline__ bool tile_inner(const IterArgs &a, int tx0, int ty0, int wx0, int wy0)
 {
     using F = FixedTile<R, TH, TW>;
-    return wx0 >= 0 && wy0 >= 0 && wx0 + F::win_w(S) <= a.W && wy0 + F::WIN_H <= a.H && tx0 >= F::RE && ty0 >= R &&
-           tx0 + TW + F::RE <= a.W && ty0 + TH + R <= a.H;
+    constexpr int B = V ? 1 : 0;
+    return wx0 >= 0 && wy0 >= 0 && wx0 + F::win_w(S) <= a.W && wy0 + F::WIN_H <= a.H && tx0 >= F::RE + B &&
+           ty0 >= R + B && tx0 + TW + F::RE + B <= a.W && ty0 + TH + R + B <= a.H;
 }
 
 // Wait for the copies of the barrier's current phase. False (for the whole block) if they did
@@ -1379,11 +1505,11 @@ __device__ __forceinline__ bool stage_wait(const IterArgs &a, uint64_t *bar, uin
 
 // A single tile (TW x TH outputs at (tx0, ty0), NT threads). Returns false if a staging copy
 // did not complete in time.
-template <typename T, bool NC, int R, int MODE, int TH, int TW = LK_TW, int NT = LK_THREADS>
+template <typename T, bool NC, int R, int MODE, int TH, int TW = LK_TW, int NT = LK_THREADS, bool V = false>
 __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps *maps, int tx0, int ty0, float2 ref,
                                              float fp64_cond, float *smem, uint32_t &phase)
 {
-    using F = FixedTile<R, TH, TW>;
+    using F = FixedTile<R, TH, TW, V>;
     unsigned char *win = reinterpret_cast<unsigned char *>(smem + F::OFF_WIN);
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + F::OFF_BAR);
     constexpr int S = (int)sizeof(T);
@@ -1397,7 +1523,7 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
     // estimate at the tile's centre, and at FLOW_SAME one of the current estimate over the
     // region, written over plane P01: stage 1 reads each pair's estimate there before storing
     // the pair's products in the same place.
-    const bool box = MODE == FLOW_SAME && staged;
+    const bool box = staged && mode_is<MODE>(a, FLOW_SAME);
     int wx0 = 0, wy0 = 0;
     if (staged) {
         win_origin<R, TH, S, TW>(a, tx0, ty0, win_ref<NC, MODE, TH, TW>(a, tx0, ty0), wx0, wy0);
@@ -1407,7 +1533,7 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
             if (box) tma_load_2d(P01, &maps->flow, tx0 - F::RE, ty0 - R, bar);
             tma_load_2d(win, &maps->i2, wx0, wy0, bar);
         }
-        prefetch_region<R, MODE, TH, TW, NT, S>(a, tx0, ty0, 0, 0);
+        prefetch_region<R, MODE, TH, TW, NT, S, V>(a, tx0, ty0, 0, 0);
         if (!stage_wait(a, bar, phase)) return false;
     }
     // stage 1: products over the region (the tile and its halo), by pixel pairs
@@ -1422,14 +1548,20 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
 #pragma unroll 1
         for (int j = threadIdx.x; j < npair; j += NT) {
             const int k2 = ry * (F::RWP2 / 2) + cx;   // float4 slot of the pair in the pair planes
-            float4 s01, s23;
-            float2 s4;
-            stage1_pair<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(
-                a, tx0 - F::RE + 2 * cx, ty0 - R + ry, ref, box ? reinterpret_cast<const float4 *>(P01) + k2 : nullptr,
-                wt, wx0, wy0, s01, s23, s4);
+            const float4 *sf = box ? reinterpret_cast<const float4 *>(P01) + k2 : nullptr;
+            const int x = tx0 - F::RE + 2 * cx, y = ty0 - R + ry;
+            float4 s01;
+            if constexpr (V) {
+                stage1_pair_i1<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(a, x, y, ref, sf, wt, wx0, wy0, s01);
+            } else {
+                float4 s23;
+                float2 s4;
+                stage1_pair<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(a, x, y, ref, sf, wt, wx0, wy0, s01, s23,
+                                                                               s4);
+                reinterpret_cast<float4 *>(P23)[k2] = s23;
+                reinterpret_cast<float2 *>(P4)[ry * (F::RWP1 / 2) + cx] = s4;
+            }
             reinterpret_cast<float4 *>(P01)[k2] = s01;
-            reinterpret_cast<float4 *>(P23)[k2] = s23;
-            reinterpret_cast<float2 *>(P4)[ry * (F::RWP1 / 2) + cx] = s4;
             ry += DY;
             cx += DX;
             if (cx >= NPR) {
@@ -1438,14 +1570,16 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
             }
         }
     };
-    if (staged && tile_inner<R, TH, TW, S>(a, tx0, ty0, wx0, wy0)) rows(std::true_type());
+    if (staged && tile_inner<R, TH, TW, S, V>(a, tx0, ty0, wx0, wy0)) rows(std::true_type());
     else rows(std::false_type());
     __syncthreads();
     // P23's chunks start at the middle warp, so that when the rows leave some warps an extra
     // chunk of P01 and of P4 the other warps take P23's
     box_h_pairs<R, TH, TW, NT>(P01);
-    box_h_pairs<R, TH, TW, NT>(P23, 0, NT / 64);
-    box_h_single<R, TH, TW, NT>(P4);
+    if constexpr (!V) {
+        box_h_pairs<R, TH, TW, NT>(P23, 0, NT / 64);
+        box_h_single<R, TH, TW, NT>(P4);
+    }
     __syncthreads();
     // vertical sums, solve and write: VO rows of one column per item (all VR rows of a group, or
     // two of them where the tile has fewer groups than threads)
@@ -1462,17 +1596,13 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
         float2 s01[VO], s23[VO];
         float s4[VO];
         if constexpr (VO == VR) {
-            box_v_planes<R, TH, TW>(P01, P23, P4, g, tx, s01, s23, s4);
+            box_v_planes<R, TH, TW, 0, V>(P01, P23, P4, g, tx, s01, s23, s4);
         } else {
-            if (part == 0) box_v_two<R, TH, TW, 0>(P01, P23, P4, g, tx, s01, s23, s4);
-            else if (VR == 4 || part == 1) box_v_two<R, TH, TW, 2>(P01, P23, P4, g, tx, s01, s23, s4);
-            else box_v_two<R, TH, TW, VR == 6 ? 4 : 2>(P01, P23, P4, g, tx, s01, s23, s4);
+            if (part == 0) box_v_two<R, TH, TW, 0, V>(P01, P23, P4, g, tx, s01, s23, s4);
+            else if (VR == 4 || part == 1) box_v_two<R, TH, TW, 2, V>(P01, P23, P4, g, tx, s01, s23, s4);
+            else box_v_two<R, TH, TW, VR == 6 ? 4 : 2, V>(P01, P23, P4, g, tx, s01, s23, s4);
         }
-#pragma unroll
-        for (int j = 0; j < VO; ++j) {
-            if (yb + j >= a.H) break;
-            solve_store<NC, MODE>(a, x, yb + j, ref, fp64_cond, s01[j], s23[j], s4[j]);
-        }
+        solve_rows<NC, MODE, V, VO>(a, x, yb, ref, fp64_cond, s01, s23, s4);
     }
     return true;
 }
@@ -1489,12 +1619,12 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
 // copy 1.1k and request and wait 2.4k; now 13.4k, request and wait 1.1k. Level-0 launch: r = 4
 // 358 -> 348 us, r = 5 462 -> 417, r = 10 680 -> 589. One bulk copy per row instead of the boxes
 // holds the issuing warp for 2k cycles per tile (410 us at r = 4).
-template <typename T, bool NC, int R, int MODE, int TH, int NT>
+template <typename T, bool NC, int R, int MODE, int TH, int NT, bool V = false>
 __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *maps, int tx0, int t_first, int t_end,
                                          float2 ref, float fp64_cond, float *smem, uint32_t &phase)
 {
-    using F = FixedTile<R, TH>;
-    using X = StripTile<R, TH>;
+    using F = FixedTile<R, TH, LK_TW, V>;
+    using X = StripTile<R, TH, V>;
     constexpr int TW = LK_TW, S = (int)sizeof(T), WW = F::win_w(S), RH = F::RH, RN = X::RING;
     unsigned char *win = reinterpret_cast<unsigned char *>(smem + X::OFF_WIN);
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + X::OFF_BAR);
@@ -1503,7 +1633,7 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
     float2 *P23 = P01 + X::PAIR_PLANE;
     float *P4 = reinterpret_cast<float *>(P23 + X::PAIR_PLANE);
     const bool staged = maps && a.stage_i2 != 0;
-    const bool flows = MODE == FLOW_SAME && staged;   // the estimate is staged as well
+    const bool flows = staged && mode_is<MODE>(a, FLOW_SAME);   // the estimate is staged as well
     // the window estimates of the strip's tiles (at most the 4 slots at OFF_WREF), loaded together
     if (staged && (int)threadIdx.x < t_end - t_first)
         wrefs[threadIdx.x] = win_ref<NC, MODE, TH>(a, tx0, (t_first + (int)threadIdx.x) * TH);
@@ -1531,7 +1661,7 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
                     request_rows(ty0 - R - X::RPAD, 0, RN / X::BOX, (uint32_t)F::win_bytes(S));
                     tma_load_2d(win, &maps->i2, wx0, wy0, bar);
                 }
-                prefetch_region<R, MODE, TH, TW, NT, S>(a, tx0, ty0, 0, 32);
+                prefetch_region<R, MODE, TH, TW, NT, S, V>(a, tx0, ty0, 0, 32);
             }
             if (!stage_wait(a, bar, phase)) return false;
         }
@@ -1541,14 +1671,20 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
         auto pair = [&](auto inner, int ry, int cx) {
             const int sl = ring_slot<RN>(ry, base);
             const int k2 = sl * (F::RWP2 / 2) + cx;   // float4 slot of the pair in the pair planes
-            float4 s01, s23;
-            float2 s4;
-            stage1_pair<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(
-                a, tx0 - F::RE + 2 * cx, ty0 - R + ry, ref, flows ? reinterpret_cast<const float4 *>(P01) + k2 : nullptr,
-                wt, wx0, wy0, s01, s23, s4);
+            const float4 *sf = flows ? reinterpret_cast<const float4 *>(P01) + k2 : nullptr;
+            const int x = tx0 - F::RE + 2 * cx, y = ty0 - R + ry;
+            float4 s01;
+            if constexpr (V) {
+                stage1_pair_i1<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(a, x, y, ref, sf, wt, wx0, wy0, s01);
+            } else {
+                float4 s23;
+                float2 s4;
+                stage1_pair<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(a, x, y, ref, sf, wt, wx0, wy0, s01, s23,
+                                                                               s4);
+                reinterpret_cast<float4 *>(P23)[k2] = s23;
+                reinterpret_cast<float2 *>(P4)[sl * (F::RWP1 / 2) + cx] = s4;
+            }
             reinterpret_cast<float4 *>(P01)[k2] = s01;
-            reinterpret_cast<float4 *>(P23)[k2] = s23;
-            reinterpret_cast<float2 *>(P4)[sl * (F::RWP1 / 2) + cx] = s4;
         };
         auto rows = [&](auto inner) {
             // thread t takes pair cx = t mod NPR of rows r0 + t / NPR, then RPI rows further each
@@ -1560,7 +1696,7 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
                 for (int ry = r0 + rs; ry < RH; ry += RPI) pair(inner, ry, cx);
             }
         };
-        if (staged && tile_inner<R, TH, TW, S>(a, tx0, ty0, wx0, wy0)) rows(std::true_type());
+        if (staged && tile_inner<R, TH, TW, S, V>(a, tx0, ty0, wx0, wy0)) rows(std::true_type());
         else rows(std::false_type());
         __syncthreads();
         if (staged && next) {
@@ -1571,11 +1707,13 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
                 mbar_expect_tx(bar, (uint32_t)F::win_bytes(S));
                 tma_load_2d(win, &maps->i2, nx0, ny0, bar);
             }
-            prefetch_region<R, MODE, TH, TW, NT, S>(a, tx0, ty0 + TH, 2 * R, 32);
+            prefetch_region<R, MODE, TH, TW, NT, S, V>(a, tx0, ty0 + TH, 2 * R, 32);
         }
         box_h_pairs<R, TH, TW, NT, RN>(P01, r0, 0, base);
-        box_h_pairs<R, TH, TW, NT, RN>(P23, r0, NT / 64, base);   // from the middle warp: the extra chunks fall on different warps
-        box_h_single<R, TH, TW, NT, RN>(P4, r0, base);
+        if constexpr (!V) {
+            box_h_pairs<R, TH, TW, NT, RN>(P23, r0, NT / 64, base);   // from the middle warp: the extra chunks fall on different warps
+            box_h_single<R, TH, TW, NT, RN>(P4, r0, base);
+        }
         __syncthreads();
         // vertical sums, solve and write, VR rows of one column per item
         constexpr int VR = v_rows<R, TH>();
@@ -1587,16 +1725,10 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
             const int x = tx0 + tx, yb = ty0 + VR * g;
             float2 s01[VR], s23[VR];
             float s4[VR];
-            if (has) box_v_planes<R, TH, TW, RN>(P01, P23, P4, g, tx, s01, s23, s4, base);
+            if (has) box_v_planes<R, TH, TW, RN, V>(P01, P23, P4, g, tx, s01, s23, s4, base);
             __syncthreads();
             if (staged && next && threadIdx.x == 0) request_rows(ty0 + TH + R, ring_slot<RN>(2 * R, base_next), TH / X::BOX, 0u);
-            if (has && x < a.W) {
-#pragma unroll
-                for (int j = 0; j < VR; ++j) {
-                    if (yb + j >= a.H) break;
-                    solve_store<NC, MODE>(a, x, yb + j, ref, fp64_cond, s01[j], s23[j], s4[j]);
-                }
-            }
+            if (has && x < a.W && yb < a.H) solve_rows<NC, MODE, V, VR>(a, x, yb, ref, fp64_cond, s01, s23, s4);
         } else {
 #pragma unroll 1
             for (int i = threadIdx.x; i < NITEM; i += NT) {
@@ -1605,12 +1737,8 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
                 if (x >= a.W || yb >= a.H) continue;
                 float2 s01[VR], s23[VR];
                 float s4[VR];
-                box_v_planes<R, TH, TW, RN>(P01, P23, P4, g, tx, s01, s23, s4, base);
-#pragma unroll
-                for (int j = 0; j < VR; ++j) {
-                    if (yb + j >= a.H) break;
-                    solve_store<NC, MODE>(a, x, yb + j, ref, fp64_cond, s01[j], s23[j], s4[j]);
-                }
+                box_v_planes<R, TH, TW, RN, V>(P01, P23, P4, g, tx, s01, s23, s4, base);
+                solve_rows<NC, MODE, V, VR>(a, x, yb, ref, fp64_cond, s01, s23, s4);
             }
             __syncthreads();
             if (staged && next && threadIdx.x == 0) request_rows(ty0 + TH + R, ring_slot<RN>(2 * R, base_next), TH / X::BOX, 0u);
@@ -1630,7 +1758,7 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
 // every a.strip. MULTI = false: a kernel whose units are single tiles (a.strip 1). Returns
 // false if a staging copy did not complete in time (then OF_ETIMEOUT is in *a.status,
 // nothing more of the unit was written, and the block must stop).
-template <typename T, bool NC, int R, int MODE, int TH = LK_TH, bool MULTI = true, int NT = LK_THREADS>
+template <typename T, bool NC, int R, int MODE, int TH = LK_TH, bool MULTI = true, int NT = LK_THREADS, bool V = false>
 __device__ __forceinline__ bool lk_tile_fixed(const IterArgs &a, const StageMaps *maps, int unit, float fp64_cond,
                                               float *smem, uint32_t &phase)
 {
@@ -1644,9 +1772,9 @@ __device__ __forceinline__ bool lk_tile_fixed(const IterArgs &a, const StageMaps
     const int gy0 = t_first / REF_GROUP * REF_GROUP * TH;
     const float2 ref = flow_mode<NC, MODE>(a, min(tx0 + LK_TW / 2, a.W - 1), min(gy0 + REF_GROUP * TH / 2, a.H - 1));
     if constexpr (!MULTI) {   // one tile per unit (a.strip 1)
-        return lk_tile_step<T, NC, R, MODE, TH, LK_TW, NT>(a, maps, tx0, t_first * TH, ref, fp64_cond, smem, phase);
+        return lk_tile_step<T, NC, R, MODE, TH, LK_TW, NT, V>(a, maps, tx0, t_first * TH, ref, fp64_cond, smem, phase);
     } else {
-        return lk_strip<T, NC, R, MODE, TH, NT>(a, maps, tx0, t_first, t_end, ref, fp64_cond, smem, phase);
+        return lk_strip<T, NC, R, MODE, TH, NT, V>(a, maps, tx0, t_first, t_end, ref, fp64_cond, smem, phase);
     }
 }
 
@@ -1654,7 +1782,7 @@ __device__ __forceinline__ bool lk_tile_fixed(const IterArgs &a, const StageMaps
 // for launches with too few 64 x LK_TH tiles to fill the GPU: same reference flows (the
 // groups of the 64 x LK_TH tiles) and the same groups of window sums, so the same bits.
 static_assert(LK_TW % SM_TW == 0 && LK_TH % SM_TH == 0, "small tiles inside the default tiles, group-aligned");
-template <typename T, bool NC, int R, int MODE>
+template <typename T, bool NC, int R, int MODE, bool V = false>
 __device__ __forceinline__ bool lk_tile_small(const IterArgs &a, const StageMaps *maps, int unit, float fp64_cond,
                                               float *smem)
 {
@@ -1664,7 +1792,7 @@ __device__ __forceinline__ bool lk_tile_small(const IterArgs &a, const StageMaps
     const int tx0 = (unit - uy * a.tiles_x) * SM_TW, ty0 = uy * SM_TH;
     const int gx0 = tx0 / LK_TW * LK_TW, gy0 = ty0 / (REF_GROUP * LK_TH) * (REF_GROUP * LK_TH);
     const float2 ref = flow_mode<NC, MODE>(a, min(gx0 + LK_TW / 2, a.W - 1), min(gy0 + REF_GROUP * LK_TH / 2, a.H - 1));
-    return lk_tile_step<T, NC, R, MODE, SM_TH, SM_TW, SM_THREADS>(a, maps, tx0, ty0, ref, fp64_cond, smem, phase);
+    return lk_tile_step<T, NC, R, MODE, SM_TH, SM_TW, SM_THREADS, V>(a, maps, tx0, ty0, ref, fp64_cond, smem, phase);
 }
 
 // ------------------------------------------------ two iterations fused in one tile

@@ -319,19 +319,23 @@ template <int R> cudaError_t i1h_launch(const HessArgs &a, int elem, int r, cuda
     }
 }
 
-template <typename T, int R> static cudaError_t i1_for(const IterArgs &a, int r, float fp64_cond, cudaStream_t s)
+template <typename T, int R>
+static cudaError_t i1_for(const IterArgs &a, const StageMaps &m, int r, float fp64_cond, bool small, cudaStream_t s)
 {
-    return launch_chained(i1_iter_kernel<T, R>, a.tiles, LK_THREADS, sizeof(float) * i1_smem_floats<R>(r, 2), s, a, r, fp64_cond);
+    const size_t smem = i1_iter_smem<R>(r, false, small, a.stage_i2 != 0, (int)sizeof(T));
+    if constexpr (R != 0)
+        if (small) return launch_chained(i1_small_kernel<T, R>, a.tiles, SM_THREADS, smem, s, a, m, fp64_cond);
+    return launch_chained(i1_iter_kernel<T, R>, a.tiles, LK_THREADS, smem, s, a, m, r, fp64_cond);
 }
 
-template <int R> cudaError_t i1_launch(const IterArgs &a, int elem, int r, float fp64_cond, cudaStream_t s)
+template <int R> cudaError_t i1_launch(const IterArgs &a, const StageMaps &m, int elem, int r, float fp64_cond, bool small, cudaStream_t s)
 {
     switch (elem) {
-    case ET_U8: return i1_for<uint8_t, R>(a, r, fp64_cond, s);
-    case ET_U16: return i1_for<uint16_t, R>(a, r, fp64_cond, s);
-    case ET_F32: return i1_for<float, R>(a, r, fp64_cond, s);
-    case ET_F16: return i1_for<__half, R>(a, r, fp64_cond, s);
-    default: return i1_for<__nv_bfloat16, R>(a, r, fp64_cond, s);
+    case ET_U8: return i1_for<uint8_t, R>(a, m, r, fp64_cond, small, s);
+    case ET_U16: return i1_for<uint16_t, R>(a, m, r, fp64_cond, small, s);
+    case ET_F32: return i1_for<float, R>(a, m, r, fp64_cond, small, s);
+    case ET_F16: return i1_for<__half, R>(a, m, r, fp64_cond, small, s);
+    default: return i1_for<__nv_bfloat16, R>(a, m, r, fp64_cond, small, s);
     }
 }
 
@@ -353,20 +357,27 @@ template <int R> cudaError_t phase_hess_launch(const HessPhase &P, int elem, int
 }
 
 template <typename T, int R>
-static cudaError_t phase_i1_for(const IterPhase &P, int r, float fp64_cond, cudaStream_t s)
+static cudaError_t phase_i1_for(const IterPhase &P, int r, float fp64_cond, int tile_h, cudaStream_t s)
 {
-    return launch_chained(phase_i1_iter_kernel<T, R>, P.prefix[P.npairs], LK_THREADS, sizeof(float) * i1_smem_floats<R>(r, 2), s, P, r, fp64_cond);
+    bool stage = false;
+    for (int i = 0; i < P.npairs; ++i) stage = stage || P.a[i].stage_i2 != 0;
+    const bool small = R != 0 && tile_h == SM_TH;
+    const size_t smem = i1_iter_smem<R>(r, true, small, stage, (int)sizeof(T));
+    const int blocks = P.prefix[P.npairs];
+    if constexpr (R != 0)
+        if (small) return launch_chained(phase_i1_small_kernel<T, R>, blocks, SM_THREADS, smem, s, P, fp64_cond);
+    return launch_chained(phase_i1_iter_kernel<T, R>, blocks, LK_THREADS, smem, s, P, r, fp64_cond);
 }
 
-template <int R> cudaError_t phase_i1_launch(const IterPhase &P, int elem, int r, float fp64_cond, cudaStream_t s)
+template <int R> cudaError_t phase_i1_launch(const IterPhase &P, int elem, int r, float fp64_cond, int tile_h, cudaStream_t s)
 {
     if (P.prefix[P.npairs] == 0) return cudaSuccess;
     switch (elem) {
-    case ET_U8: return phase_i1_for<uint8_t, R>(P, r, fp64_cond, s);
-    case ET_U16: return phase_i1_for<uint16_t, R>(P, r, fp64_cond, s);
-    case ET_F32: return phase_i1_for<float, R>(P, r, fp64_cond, s);
-    case ET_F16: return phase_i1_for<__half, R>(P, r, fp64_cond, s);
-    default: return phase_i1_for<__nv_bfloat16, R>(P, r, fp64_cond, s);
+    case ET_U8: return phase_i1_for<uint8_t, R>(P, r, fp64_cond, tile_h, s);
+    case ET_U16: return phase_i1_for<uint16_t, R>(P, r, fp64_cond, tile_h, s);
+    case ET_F32: return phase_i1_for<float, R>(P, r, fp64_cond, tile_h, s);
+    case ET_F16: return phase_i1_for<__half, R>(P, r, fp64_cond, tile_h, s);
+    default: return phase_i1_for<__nv_bfloat16, R>(P, r, fp64_cond, tile_h, s);
     }
 }
 
@@ -380,7 +391,7 @@ template <int R, int TH, int TW = LK_TW> static bool stage_maps_th(const IterArg
     // on with 4-byte levels) costs more than it saves: eight 1024^2 pairs at r = 16 3147 us
     // staged, 2574 gathered
     constexpr int SM_BYTES = 228 * 1024, BLOCK_BYTES = 1024;   // shared memory per SM, and reserved per block
-    if (2 * (4 * F::smem_staged(S) + BLOCK_BYTES) > SM_BYTES && 2 * (4 * F::SMEM_NOSTAGE + BLOCK_BYTES) <= SM_BYTES)
+    if (!a.hess && 2 * (4 * F::smem_staged(S) + BLOCK_BYTES) > SM_BYTES && 2 * (4 * F::SMEM_NOSTAGE + BLOCK_BYTES) <= SM_BYTES)
         return false;
     int flow_rows = F::FLOW_BH;
     if constexpr (TW == LK_TW && strip_kernel<R, TH>())
@@ -472,23 +483,25 @@ template <int R> cudaError_t radius_configure()
     }
     {
         const int r = R == 0 ? MAX_RADIUS : R;
-        const int hb = (int)sizeof(float) * i1_smem_floats<R>(r, 3), ib = (int)sizeof(float) * i1_smem_floats<R>(r, 2);
-#define OF_SET_I1(T)                                                                                       \
-    if ((e = cudaFuncSetAttribute((const void *)i1_hess_kernel<T, R>,                                     \
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, hb)) != cudaSuccess ||     \
-        (e = cudaFuncSetAttribute((const void *)i1_iter_kernel<T, R>,                                     \
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, ib)) != cudaSuccess ||     \
-        (e = cudaFuncSetAttribute((const void *)phase_hess_kernel<T, R>,                                  \
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, hb)) != cudaSuccess ||     \
-        (e = cudaFuncSetAttribute((const void *)phase_i1_iter_kernel<T, R>,                               \
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, ib)) != cudaSuccess)       \
+        const int hb = (int)sizeof(float) * i1_smem_floats<R>(r, 3);
+        const int ib = (int)i1_iter_smem<R>(r, false, false, true, 4), jb = (int)i1_iter_smem<R>(r, true, false, true, 4);
+#define OF_SET_TO(fn, bytes)                                                                                   \
+    if ((e = cudaFuncSetAttribute((const void *)(fn), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess) \
         return e;
+#define OF_SET_I1(T)                             \
+    OF_SET_TO((i1_hess_kernel<T, R>), hb)        \
+    OF_SET_TO((phase_hess_kernel<T, R>), hb)     \
+    OF_SET_TO((i1_iter_kernel<T, R>), ib)        \
+    OF_SET_TO((phase_i1_iter_kernel<T, R>), jb)  \
+    OF_SET_TO((i1_small_kernel<T, R>), ib)       \
+    OF_SET_TO((phase_i1_small_kernel<T, R>), jb)
         OF_SET_I1(uint8_t)
         OF_SET_I1(uint16_t)
         OF_SET_I1(float)
         OF_SET_I1(__half)
         OF_SET_I1(__nv_bfloat16)
 #undef OF_SET_I1
+#undef OF_SET_TO
     }
     if constexpr (all_forms<R>())
         for (int f = 0; f < 2; ++f)
@@ -502,8 +515,8 @@ template cudaError_t ws_launch<OF_RADIUS>(const float *, int, int, int, float *,
 template cudaError_t i1h_launch<OF_RADIUS>(const HessArgs &, int, int, cudaStream_t);
 template cudaError_t phase_launch<OF_RADIUS>(const IterPhase &, int, int, float, int, cudaStream_t);
 template cudaError_t phase_hess_launch<OF_RADIUS>(const HessPhase &, int, int, cudaStream_t);
-template cudaError_t phase_i1_launch<OF_RADIUS>(const IterPhase &, int, int, float, cudaStream_t);
-template cudaError_t i1_launch<OF_RADIUS>(const IterArgs &, int, int, float, cudaStream_t);
+template cudaError_t phase_i1_launch<OF_RADIUS>(const IterPhase &, int, int, float, int, cudaStream_t);
+template cudaError_t i1_launch<OF_RADIUS>(const IterArgs &, const StageMaps &, int, int, float, bool, cudaStream_t);
 #ifndef OF_RADIUS_MORE   // one of OF_RADII_MORE
 template void *batch_kernel_ptr<OF_RADIUS>(int, int);
 #endif

@@ -10,13 +10,13 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("storage,H,W", [("f16", 150, 200), ("f32", 97, 129), ("bf16", 121, 321)])
-@pytest.mark.parametrize("r", [2, 3, 4, 5, 6, 8, 10])
-def test_small_tiles_equal_wide_tiles(storage, H, W, r):
+@pytest.mark.parametrize("r,variant", [(r, False) for r in (2, 3, 4, 5, 6, 8, 10)] + [(r, True) for r in (2, 5, 10, 16)])
+def test_small_tiles_equal_wide_tiles(storage, H, W, r, variant):
     import torch
     from paper_1306_2461_gb300 import of
     p = synth.make_c1(H, W, seed=H + r)
     I1, I2 = to_dev(p.I1), to_dev(p.I2)
-    plan = of.Plan.make(H, W, 2, r, 3, bits=8, storage=storage)
+    plan = of.Plan.make(H, W, 2, r, 3, bits=8, storage=storage, flags=of.OF_FLAG_I1GRAD if variant else 0)
     tiles = -(-W // 64) * -(-H // 24)
     n = 4 * torch.cuda.get_device_properties(0).multi_processor_count // (3 * tiles) + 2
     with of.Flow(plan) as f:

@@ -183,7 +183,7 @@ int of_compute_batch_host(int32_t n, const of_handle *hs, const void *const *hI1
  * for bit (with the default tile height and fusion 1, whatever the strip). Without a table
  * entry a batch runs {generic_sums 0, stage_i2 1, blocks_per_sm 0, phased 1, prefetch 0,
  * tile_h 24, branches 2, fusion 1, strip 4} (branches 1 where the launches are not replayed from
- * a graph, and with OF_FLAG_I1GRAD).
+ * a graph).
  * A tuning:
  *   generic_sums   1: per-output window sums of the run-time-radius kernel;
  *                  0: grouped sums of the kernel specialised for the radius

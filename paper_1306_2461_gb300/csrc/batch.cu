@@ -633,10 +633,10 @@ int run_batch(int32_t n, const of_handle *hs, const void *const *I1s, const void
     // Without a table entry: two concurrent sequences over halves of the batch where they are
     // branches of a graph, so that each fills the last waves and the gaps between launches of
     // the other (us, one and two sequences: 2 x 1024^2 280, 237; 8 x 512^2 296, 255; 16 x 256^2
-    // 239, 195; 64 x 1024^2 5070, 4840; three and four are no better). One where the launches
-    // are queued one by one, which twice as many would take longer, and for the variant,
-    // whose launches are nearer to the memory's rate (16 x 1024^2 1536, 1563).
-    if (t.branches == BRANCHES_AUTO) t.branches = graphs && n > 1 && !(p0.flags & OF_FLAG_I1GRAD) ? 2 : 0;
+    // 239, 195; 64 x 1024^2 5070, 4840; the variant's 16 x 1024^2 1348, 1197; three and four are
+    // no better). One where the launches are queued one by one, which twice as many would take
+    // longer.
+    if (t.branches == BRANCHES_AUTO) t.branches = graphs && n > 1 ? 2 : 0;
     const size_t pairs_bytes = sizeof(BatchPair) * n, prefix_bytes = sizeof(int32_t) * b.prefix.size();
     std::vector<char> key(pairs_bytes + prefix_bytes + sizeof(st) + 7 * sizeof(int));
     {

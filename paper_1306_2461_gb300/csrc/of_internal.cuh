@@ -62,7 +62,8 @@ struct Level {
 enum FlowMode : int {
     FLOW_ZERO = 0,     // coarsest level, first iteration: u = v = 0
     FLOW_SAME = 1,     // previous iterate on this level
-    FLOW_UPSAMPLE = 2  // first iteration of a finer level: 2 * bilinear(coarse, x/2, y/2)
+    FLOW_UPSAMPLE = 2, // first iteration of a finer level: 2 * bilinear(coarse, x/2, y/2)
+    FLOW_FIRST = 3     // kernels only: a level's first iteration, zero or upsampled at run time
 };
 
 // Arguments of one Gauss-Newton iteration on one level of one pair.

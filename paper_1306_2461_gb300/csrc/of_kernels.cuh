@@ -493,6 +493,8 @@ template <bool NC, int MODE>
 __device__ __forceinline__ float2 flow_mode(const IterArgs &a, int x, int y)
 {
     if constexpr (MODE < 0) return flow_at<NC>(a, x, y);
+    else if constexpr (MODE == FLOW_FIRST)
+        return a.mode == FLOW_ZERO ? make_float2(0.0f, 0.0f) : flow_at_m<NC, FLOW_UPSAMPLE>(a, x, y);
     else return flow_at_m<NC, MODE>(a, x, y);
 }
 
@@ -844,6 +846,14 @@ template <bool NC> __device__ __forceinline__ float2 ld_pair(const __nv_bfloat16
     return __bfloat1622float2(w);
 }
 
+// The flow mode is `m`: known at compile time (MODE), at run time (MODE < 0), or one of a
+// level's first iteration (FLOW_FIRST).
+template <int MODE> __device__ __forceinline__ bool mode_is(const IterArgs &a, int m)
+{
+    if (MODE == FLOW_FIRST) return m != FLOW_SAME && a.mode == m;
+    return MODE >= 0 ? MODE == m : a.mode == m;
+}
+
 // The current estimates of the pixel pair (x, y), (x + 1, y) (x even; the second only
 // when q): one 16-byte load of the same-level flow, else pixel by pixel.
 template <bool NC, int MODE>
@@ -857,7 +867,7 @@ __device__ __forceinline__ void flow_pair(const IterArgs &a, int x, int y, bool 
             return;
         }
     }
-    if (MODE == FLOW_UPSAMPLE || (MODE < 0 && a.mode == FLOW_UPSAMPLE)) {
+    if (mode_is<MODE>(a, FLOW_UPSAMPLE)) {
         // flow_at_m's upsampling for x (weight 0) and x + 1 (weight 1/2), which share
         // their four coarse samples (x even), computed on both at once
         const int x0 = x >> 1, y0 = y >> 1;
@@ -1430,12 +1440,6 @@ __device__ __forceinline__ void solve_rows(const IterArgs &a, int x, int yb, flo
             solve_store<NC, MODE>(a, x, yb + j, ref, fp64_cond, sj);
         }
     }
-}
-
-// The flow mode is `m`, known at compile time (MODE) or at run time (MODE < 0).
-template <int MODE> __device__ __forceinline__ bool mode_is(const IterArgs &a, int m)
-{
-    return MODE >= 0 ? MODE == m : a.mode == m;
 }
 
 // While a tile's copies land: bring the lines of I1 that its stage 1 reads (region rows r0..)

@@ -41,12 +41,11 @@ lk_small_kernel(const __grid_constant__ IterArgs a, const __grid_constant__ Stag
     if constexpr (R != 0) {
         lk_tile_init<R, SM_TH, SM_TW>(smem);
         chain_begin();
-        if (a.mode == FLOW_SAME) lk_tile_small<T, false, R, FLOW_SAME>(a, &m, blockIdx.x, fp64_cond, smem);
-        else lk_tile_small<T, false, R, -1>(a, &m, blockIdx.x, fp64_cond, smem);
+        lk_tile_small<T, false, R, -1>(a, &m, blockIdx.x, fp64_cond, smem);
     }
 }
 
-template <typename T, int R, int MODE>
+template <typename T, int R>
 __global__ void __launch_bounds__(SM_THREADS, SM_MIN_BLOCKS)
 phase_small_kernel(const __grid_constant__ IterPhase P, float fp64_cond)
 {
@@ -56,7 +55,7 @@ phase_small_kernel(const __grid_constant__ IterPhase P, float fp64_cond)
         const int p = phase_pair(P.prefix, P.npairs, blockIdx.x);
         lk_tile_init<R, SM_TH, SM_TW>(smem);
         chain_begin();
-        lk_tile_small<T, false, R, MODE>(P.a[p], &P.m[p], blockIdx.x - P.prefix[p], fp64_cond, smem);
+        lk_tile_small<T, false, R, -1>(P.a[p], &P.m[p], blockIdx.x - P.prefix[p], fp64_cond, smem);
     }
 }
 
@@ -226,8 +225,14 @@ template <int R> cudaError_t ws_launch(const float *ch, int H, int W, int r, flo
     return cudaGetLastError();
 }
 
-// The flow mode is the same for every pair of a phase: one kernel per mode (and per
-// tile height; the run-time-radius kernel has only the default height).
+// The flow mode is the same for every pair of a phase: at the default tile height one kernel per
+// mode (for the radii with fewer forms one for both modes of a level's first iteration; with
+// that 64 pairs of 1024^2 at r = 4 take 4883 instead of 4840 us). The other tile height and the
+// small tiles read the mode at run time. Fewer kernels keep the build short.
+template <int R, int TH> constexpr int phase_mode(int mode)
+{
+    return TH != LK_TH ? -1 : (mode == FLOW_SAME || all_forms<R>() ? mode : (int)FLOW_FIRST);
+}
 template <typename T, int R, int TH>
 static cudaError_t phase_for_th(const IterPhase &P, int r, float fp64_cond, cudaStream_t s)
 {
@@ -236,9 +241,15 @@ static cudaError_t phase_for_th(const IterPhase &P, int r, float fp64_cond, cuda
     const size_t smem = sizeof(float) * lk_tile_smem_floats<R, TH, strip_kernel<R, TH>()>(r, stage, (int)sizeof(T));
     const int blocks = P.prefix[P.npairs];
     switch (P.a[0].mode) {
-    case FLOW_ZERO: return launch_chained((phase_iter_kernel<T, R, FLOW_ZERO, TH>), blocks, LK_THREADS, smem, s, P, r, fp64_cond);
-    case FLOW_SAME: return launch_chained((phase_iter_kernel<T, R, FLOW_SAME, TH>), blocks, LK_THREADS, smem, s, P, r, fp64_cond);
-    default: return launch_chained((phase_iter_kernel<T, R, FLOW_UPSAMPLE, TH>), blocks, LK_THREADS, smem, s, P, r, fp64_cond);
+    case FLOW_ZERO:
+        return launch_chained(phase_iter_kernel<T, R, phase_mode<R, TH>(FLOW_ZERO), TH>, blocks, LK_THREADS, smem, s, P, r,
+                              fp64_cond);
+    case FLOW_SAME:
+        return launch_chained(phase_iter_kernel<T, R, phase_mode<R, TH>(FLOW_SAME), TH>, blocks, LK_THREADS, smem, s, P, r,
+                              fp64_cond);
+    default:
+        return launch_chained(phase_iter_kernel<T, R, phase_mode<R, TH>(FLOW_UPSAMPLE), TH>, blocks, LK_THREADS, smem, s, P,
+                              r, fp64_cond);
     }
 }
 
@@ -251,11 +262,7 @@ static cudaError_t phase_for(const IterPhase &P, int r, float fp64_cond, int til
             for (int i = 0; i < P.npairs; ++i) stage = stage || P.a[i].stage_i2 != 0;
             const size_t smem = sizeof(float) * small_smem_floats<R>(stage, (int)sizeof(T));
             const int blocks = P.prefix[P.npairs];
-            switch (P.a[0].mode) {
-            case FLOW_ZERO: return launch_chained(phase_small_kernel<T, R, FLOW_ZERO>, blocks, SM_THREADS, smem, s, P, fp64_cond);
-            case FLOW_SAME: return launch_chained(phase_small_kernel<T, R, FLOW_SAME>, blocks, SM_THREADS, smem, s, P, fp64_cond);
-            default: return launch_chained(phase_small_kernel<T, R, FLOW_UPSAMPLE>, blocks, SM_THREADS, smem, s, P, fp64_cond);
-            }
+            return launch_chained(phase_small_kernel<T, R>, blocks, SM_THREADS, smem, s, P, fp64_cond);
         }
         if constexpr (all_forms<R>())
             if (tile_h == ALT_TH) return phase_for_th<T, R, ALT_TH>(P, r, fp64_cond, s);
@@ -435,8 +442,8 @@ template <int R> cudaError_t radius_configure()
     OF_SET((lk_iter_kernel<float, R>));
     OF_SET((lk_iter_kernel<__half, R>));
     OF_SET((lk_iter_kernel<__nv_bfloat16, R>));
-#define OF_SET_PH(T) OF_SET((phase_iter_kernel<T, R, FLOW_ZERO, LK_TH>)); OF_SET((phase_iter_kernel<T, R, FLOW_SAME, LK_TH>)); \
-    OF_SET((phase_iter_kernel<T, R, FLOW_UPSAMPLE, LK_TH>))
+#define OF_SET_PH(T) OF_SET((phase_iter_kernel<T, R, phase_mode<R, LK_TH>(FLOW_ZERO), LK_TH>)); \
+    OF_SET((phase_iter_kernel<T, R, FLOW_SAME, LK_TH>)); OF_SET((phase_iter_kernel<T, R, phase_mode<R, LK_TH>(FLOW_UPSAMPLE), LK_TH>))
     OF_SET_PH(uint8_t);
     OF_SET_PH(uint16_t);
     OF_SET_PH(float);
@@ -445,12 +452,10 @@ template <int R> cudaError_t radius_configure()
 #undef OF_SET_PH
     if constexpr (R != 0 && all_forms<R>()) {   // the other tile height of the phase kernels
         const int alt = (int)sizeof(float) * lk_tile_smem_floats<R, ALT_TH, strip_kernel<R, ALT_TH>()>(R, true);
-#define OF_SET_ALT(T)                                                                                       \
-    for (const void *fn : {(const void *)phase_iter_kernel<T, R, FLOW_ZERO, ALT_TH>,                        \
-                           (const void *)phase_iter_kernel<T, R, FLOW_SAME, ALT_TH>,                        \
-                           (const void *)phase_iter_kernel<T, R, FLOW_UPSAMPLE, ALT_TH>})                   \
-        if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, alt)) != cudaSuccess) \
-            return e;
+#define OF_SET_ALT(T)                                                                                        \
+    if ((e = cudaFuncSetAttribute((const void *)phase_iter_kernel<T, R, -1, ALT_TH>,                         \
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, alt)) != cudaSuccess)         \
+        return e;
         OF_SET_ALT(uint8_t)
         OF_SET_ALT(uint16_t)
         OF_SET_ALT(float)
@@ -462,9 +467,7 @@ template <int R> cudaError_t radius_configure()
     if constexpr (R != 0) {   // small tiles
         const int sb = (int)sizeof(float) * small_smem_floats<R>(true, 4);
 #define OF_SET_SM(T)                                                                                        \
-    for (const void *fn : {(const void *)lk_small_kernel<T, R>, (const void *)phase_small_kernel<T, R, FLOW_ZERO>, \
-                           (const void *)phase_small_kernel<T, R, FLOW_SAME>,                               \
-                           (const void *)phase_small_kernel<T, R, FLOW_UPSAMPLE>})                          \
+    for (const void *fn : {(const void *)lk_small_kernel<T, R>, (const void *)phase_small_kernel<T, R>})    \
         if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sb)) != cudaSuccess) \
             return e;
         OF_SET_SM(uint8_t)

@@ -14,12 +14,6 @@
 
 #include "batch_device.cuh"
 
-// Strips of the phase launches shrink while a launch would have fewer blocks than this
-// many per resident block slot.
-#ifndef OF_STRIP_WAVES
-#define OF_STRIP_WAVES 2
-#endif
-
 namespace of {
 
 // The bounded-wait test kernel (of_debug_wait_timeout) runs the barrier's wait loop on
@@ -246,8 +240,9 @@ static Resolved resolve(const of_plan &p0, const Tuning &t)
 // up to PHASE_PAIRS pairs (the per-pair arguments are kernel parameters): pyramid passes
 // (after the normalisation of Eq. 2 when the plan asks for it), then the iterations
 // level by level. Stream order separates the phases; there is no grid-wide barrier.
+// sequences: how many such sequences over parts of the batch run concurrently.
 static cudaError_t enqueue_chain(const BatchPair *pairs, int n, const of_plan &p0, const Tuning &t,
-                                 cudaStream_t st)
+                                 cudaStream_t st, int sequences)
 {
     const int L = p0.levels;
     const bool zn = (p0.flags & OF_FLAG_ZNSSD) != 0;
@@ -259,6 +254,8 @@ static cudaError_t enqueue_chain(const BatchPair *pairs, int n, const of_plan &p
     const int32_t prefetch_ahead = sms * t.prefetch;
     // iteration tile height: the tuned one for the grouped sums of a specialised radius
     const int tile_h = (t.tile_h == ALT_TH && !t.generic_sums && radius_specialised(p0.radius)) ? ALT_TH : LK_TH;
+    // blocks a launch keeps before its strips shrink: two per resident slot, counting the other sequences
+    const long slots = (long)lk_slots(p0.radius) * sms * (sequences > 1 ? 1 : 2);
     // tiles per block of the fixed-radius kernels (the run-time-radius kernel takes one)
     const int strip = (!t.generic_sums && radius_strips(p0.radius, tile_h)) ? strip_len(tuning_strip(t)) : 1;
     cudaError_t e;
@@ -348,13 +345,16 @@ static cudaError_t enqueue_chain(const BatchPair *pairs, int n, const of_plan &p
             memset(&I, 0, sizeof(I));
             I.npairs = m;
             I.ahead = prefetch_ahead;
-            // strips as long as the tuning's while the launch keeps OF_STRIP_WAVES blocks per
-            // resident block slot (4 per SM) or more; small tiles where there are few (of the
-            // default tile without a prefetch); the fields do not depend on either
+            // strips as long as the tuning's while the launch has `slots` blocks; small tiles where there
+            // are few (of the default tile without a prefetch); the fields do not depend on
+            // either. A strip's first tile costs twice a later one's time, so fewer, longer strips
+            // pay until slots stay empty: us with strips shrinking below 8, 4, 2 and 1 blocks per SM:
+            // 16 x 1024^2 at r = 4 (4 slots per SM) 1295, 1272, 1297, 1313; 64 x 512^2 1395, 1372,
+            // 1386, 1398; 8 x 1024^2 at r = 10 (2 slots) 1227, 1129, 1079, 1095.
             int kl = strip;
             long tiles_l = 0;
             for (int i = 0; i < m; ++i) tiles_l += strip_units(bp[i].H[l], bp[i].W[l], tile_h, 1);
-            while (kl > 1 && tiles_l < (long)kl * OF_STRIP_WAVES * 4 * sms) kl /= 2;
+            while (kl > 1 && tiles_l < (long)kl * slots) kl /= 2;
             const bool small = !two && tile_h == LK_TH && !t.generic_sums && radius_grouped(p0.radius) &&
                                prefetch_ahead == 0 && use_small_tiles(tiles_l, sms);
             const int th_l = small ? SM_TH : tile_h;
@@ -469,7 +469,7 @@ static cudaError_t enqueue_phased(const std::vector<BatchPair> &pairs, const of_
 {
     const int n = (int)pairs.size();
     const int nb = branches < n ? branches : n;
-    if (nb <= 1) return enqueue_chain(pairs.data(), n, p0, t, st);
+    if (nb <= 1) return enqueue_chain(pairs.data(), n, p0, t, st, 1);
     Forks *f = forks_for_device();
     if (!f) return cudaErrorUnknown;
     double total = 0.0;
@@ -489,7 +489,7 @@ static cudaError_t enqueue_phased(const std::vector<BatchPair> &pairs, const of_
     cudaError_t e = cudaEventRecord(f->fork, st);
     for (int b = 1; b < nb && e == cudaSuccess; ++b) e = cudaStreamWaitEvent(f->s[b - 1], f->fork, 0);
     for (int b = 0; b < nb && e == cudaSuccess; ++b)
-        e = enqueue_chain(pairs.data() + bound[b], bound[b + 1] - bound[b], p0, t, b ? f->s[b - 1] : st);
+        e = enqueue_chain(pairs.data() + bound[b], bound[b + 1] - bound[b], p0, t, b ? f->s[b - 1] : st, nb);
     // join every side stream, also after an error, so that no forked work is left unjoined
     for (int b = 1; b < nb; ++b) {
         const cudaError_t j = cudaEventRecord(f->join[b - 1], f->s[b - 1]) == cudaSuccess

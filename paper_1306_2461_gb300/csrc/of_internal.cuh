@@ -234,6 +234,8 @@ constexpr bool radius_grouped(int r)   // the per-pair and phase launches at lea
 #undef OF_IS_RADIUS
     return radius_specialised(r);
 }
+// Blocks of the 64-wide fixed-radius tiles resident on an SM.
+constexpr int lk_slots(int r) { return r <= 4 ? 4 : (r <= 6 ? 3 : 2); }
 // Strips take over 2r rows of sums from the tile above, which must lie below that tile's own
 // 2r first rows.
 constexpr bool radius_strips(int r, int tile_h) { return radius_grouped(r) && tile_h >= 2 * r; }

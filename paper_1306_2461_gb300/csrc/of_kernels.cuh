@@ -694,16 +694,13 @@ template <int R, int TH = LK_TH, int TW = LK_TW, bool V = false> struct FixedTil
     // written over P01 (strips: see StripTile).
     static constexpr int FLOW_BH = RH;
     static constexpr int FLOW_BOX_BYTES = RWP2 * FLOW_BH * 8;
-#ifndef OF_LK_MIN_BLOCKS
-#define OF_LK_MIN_BLOCKS 4   // resident blocks per SM the fixed-radius kernels are compiled for (R <= 4)
-#endif
     // resident blocks per SM the kernels are compiled for: the measured choice for the
     // default tile height, else as many as the shared memory holds (at most 5). At r = 5 and 6
     // shared memory holds 3 blocks, which leaves 80 registers instead of 64: level-0 launch of 32
     // pairs of 1024^2 at r = 5 416 -> 405 us, a pair 195 -> 193 us
     static constexpr int SMEM_FIT = 233472 / (4 * (PLANES + 4) + 1024);
     static constexpr int MIN_BLOCKS =
-        TH == LK_TH ? (R <= 4 ? OF_LK_MIN_BLOCKS : (R <= 6 ? 3 : 2)) : (SMEM_FIT < 1 ? 1 : (SMEM_FIT > 5 ? 5 : SMEM_FIT));
+        TH == LK_TH ? lk_slots(R) : (SMEM_FIT < 1 ? 1 : (SMEM_FIT > 5 ? 5 : SMEM_FIT));
 };
 
 // Shared memory of a strip's tiles: the planes are rings of RING rows. Region row ry of a tile
@@ -980,7 +977,10 @@ template <int RN> __device__ __forceinline__ int ring_slot(int ry, int base)
 // rows goes to warp (c + woff) mod WARPS. For 64- and 32-wide tiles a warp takes two or
 // four rows and a quarter warp 4 groups of 4 outputs of two of them (with rows RWP2 = 2 mod 4
 // float2 long, its 16-byte reads hit distinct banks); other widths take one row per warp,
-// one group per lane. Each row is read and rewritten by one warp.
+// one group per lane. Each row is read and rewritten by one warp. From r = 7 on a lane of a
+// 64-wide tile takes 8 outputs, whose two groups share the columns between them (2R + 8 read
+// for 8 outputs instead of twice 2R + 4): 8 x 1024^2 at r = 10 1277 -> 1227 us. At r = 4, with 64
+// registers per thread, that costs spills and leaves warps idle (348 -> 390 us per launch).
 template <int R, int TH, int TW = LK_TW, int NT = LK_THREADS, int RN = 0>
 __device__ __forceinline__ void box_h_pairs(float2 *P, int r0 = 0, int woff = 0, int base = 0)
 {
@@ -989,31 +989,35 @@ __device__ __forceinline__ void box_h_pairs(float2 *P, int r0 = 0, int woff = 0,
     constexpr int WARPS = NT / 32;
     constexpr int RW4 = F::RWP2 / 2;   // float4 per row
     const int lane = threadIdx.x & 31;
-    constexpr int NG = TW / 4;
-    constexpr int RPC = TW == 64 ? 2 : (TW == 32 ? 4 : 1);   // rows per warp-sized chunk (r0, RH - r0 even)
-    const int rsub = RPC == 1 ? 0 : ((lane >> 2) & 1) | (RPC == 4 ? (lane >> 4) << 1 : 0);
-    const int g = RPC == 1 ? lane : (lane & 3) | ((lane >> 3) << 2 & (NG - 1));
+    constexpr int GPL = TW == 64 && R > 6 ? 2 : 1;       // groups of 4 outputs per lane
+    constexpr int NL = TW / (4 * GPL);                       // lanes per row
+    constexpr int RPC = TW == 64 || TW == 32 ? 32 / NL : 1;  // rows per warp-sized chunk (r0, RH - r0 even)
+    // quarter warps: 4 lanes of each of 2 rows, or 2 lanes (of 8 outputs) of each of 4 rows
+    const int rsub = RPC == 1 ? 0 : (GPL == 2 ? (lane >> 1) & 3 : ((lane >> 2) & 1) | (RPC == 4 ? (lane >> 4) << 1 : 0));
+    const int g = RPC == 1 ? lane : (GPL == 2 ? (lane & 1) | (lane >> 3) << 1 : (lane & 3) | ((lane >> 3) << 2 & (NL - 1)));
+    constexpr int NV = 4 * (GPL - 1) + 4 * F::NVE;           // float2 columns read per lane
     const int chunks = (F::RH - r0 + RPC - 1) / RPC;
 #pragma unroll 1
     for (int chunk = ((threadIdx.x >> 5) + WARPS - woff) % WARPS; chunk < chunks; chunk += WARPS) {
         const int ry = r0 + RPC * chunk + rsub;
-        const bool act = (RPC != 1 || g < NG) && (RPC != 4 || ry < F::RH);
-        float4 *row = reinterpret_cast<float4 *>(P) + (ring_slot<RN>(ry, base) * RW4 + 2 * g);
-        float2 o[4];
+        const bool act = (RPC != 1 || g < NL) && (RPC != 4 || ry < F::RH);
+        float4 *row = reinterpret_cast<float4 *>(P) + (ring_slot<RN>(ry, base) * RW4 + 2 * GPL * g);
+        float2 o[4 * GPL];
         if (act) {
-            float2 v[4 * F::NVE];
+            float2 v[NV];
 #pragma unroll
-            for (int q = 0; q < 2 * F::NVE; ++q) {
+            for (int q = 0; q < NV / 2; ++q) {
                 const float4 t = row[q];
                 v[2 * q] = f2(t.x, t.y);
                 v[2 * q + 1] = f2(t.z, t.w);
             }
-            box4v<R, F::OFF>(v, o);
+#pragma unroll
+            for (int k = 0; k < GPL; ++k) box4v<R, F::OFF>(v + 4 * k, o + 4 * k);
         }
         __syncwarp();
         if (act) {
-            row[0] = make_float4(o[0].x, o[0].y, o[1].x, o[1].y);
-            row[1] = make_float4(o[2].x, o[2].y, o[3].x, o[3].y);
+#pragma unroll
+            for (int q = 0; q < 2 * GPL; ++q) row[q] = make_float4(o[2 * q].x, o[2 * q].y, o[2 * q + 1].x, o[2 * q + 1].y);
         }
     }
 }

@@ -131,6 +131,7 @@ def dominant_kernel_leg(torch, of, I1, I2, stream, peak, khash, pairs=32, reps=2
     for iters in (2, 6):
         plan = of.Plan.make(H, W, 1, RADIUS, iters, bits=BITS, storage="f16")
         flows = [of.Flow(plan) for _ in range(n)]
+        of.tuning_set(plan, of.batch_size_class(flows), branches=1)   # one launch over all n pairs
         us = [torch.empty((H, W), dtype=torch.float32, device="cuda") for _ in range(n)]
         vs = [torch.empty((H, W), dtype=torch.float32, device="cuda") for _ in range(n)]
         with torch.cuda.stream(stream):
@@ -389,7 +390,7 @@ def main():
     if not args.no_autotune:
         from paper_1306_2461_gb300 import autotune
         tuning = autotune.tune(flows, I1, I2, us, vs, stream=stream, reps=2, save=False)
-    elif args.branches > 1 or args.tile_h or not args.stage:
+    elif args.branches or args.tile_h or not args.stage:
         of.tuning_set(flows[0].plan, of.batch_size_class(flows), branches=max(args.branches, 0),
                       tile_h=args.tile_h, stage_i2=args.stage)
 
@@ -442,7 +443,9 @@ def main():
         return 0
     alg, alg_pyr, alg_it = (algorithmic_bytes_i1grad if args.i1grad else algorithmic_bytes)(H, W, LEVELS, ITERS, 2, 2)
     phased = tuning["best"]["phased"] if tuning else 1
-    branches = (tuning["best"]["branches"] if tuning else max(args.branches, 1)) if phased else 1
+    # without any tuning the library runs a replayed batch as two sequences
+    forced = args.branches or args.tile_h or not args.stage
+    branches = (tuning["best"]["branches"] if tuning else (max(args.branches, 1) if forced else 2)) if phased else 1
     # the batch runs as `branches` concurrent sequences over runs of equal-size pairs (run k
     # ends at the first pair count >= B k / branches), each in launches of at most 64 pairs
     nb = min(branches, B)
@@ -476,7 +479,7 @@ def main():
                    "tuning": ({k: tuning["best"][k] for k in ("generic_sums", "stage_i2", "blocks_per_sm", "phased",
                                                                "prefetch", "tile_h", "branches", "fusion", "strip")}
                               if tuning else ("default (autotuner off)"
-                                              if args.branches <= 1 and not args.tile_h and args.stage else
+                                              if not forced else
                                               f"forced (autotuner off): tile_h {args.tile_h or 'default'}, stage "
                                               f"{args.stage}, {max(args.branches, 1)} concurrent sequences")),
                    "l2": "no flush: per-step working set ~%.1f GB >> 129 MB L2" % (

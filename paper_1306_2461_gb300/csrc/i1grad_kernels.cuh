@@ -30,37 +30,25 @@ template <int R> inline __host__ __device__ int i1_smem_floats(int r, int channe
     if constexpr (R == 0) {
         const int RH = I1_TH + 2 * r, RW = LK_TW + 2 * r;
         return channels * (RH * RW + RH * LK_TW);
-    } else {
-        return channels * FixedTile<R, I1_TH>::PLANE;
+    } else {   // the window matrices: P01 and P4
+        using F = FixedTile<R, I1_TH>;
+        return 2 * F::PAIR_PLANE + F::RH * F::RWP1;
     }
 }
 
-// Plane stride and row length of the product planes (padded rows for a fixed radius).
-template <int R> __device__ __forceinline__ int i1_plane(int RH, int RW)
-{
-    if constexpr (R == 0) return RH * RW;
-    else return FixedTile<R, I1_TH>::PLANE;
-}
-template <int R> __device__ __forceinline__ int i1_rowlen(int RW)
-{
-    if constexpr (R == 0) return RW;
-    else return FixedTile<R, I1_TH>::RWP;
-}
-
-// Window matrix of one level: (Sa, Sb, Sc, 0) at every pixel of one output tile.
-template <typename T, int R>
-__device__ __forceinline__ void i1_hess_tile(const HessArgs &a, int tile, int r, float *smem)
+// Window matrix of one level: (Sa, Sb, Sc, 0) at every pixel of one output tile, for any window
+// radius r given at run time.
+template <typename T>
+__device__ __forceinline__ void i1_hess_tile_generic(const HessArgs &a, int tile, int r, float *smem)
 {
     const int tyi = tile / a.tiles_x;
     const int ty0 = tyi * I1_TH, tx0 = (tile - tyi * a.tiles_x) * LK_TW;
     const T *I1 = static_cast<const T *>(a.I1);
-    const int rr = R == 0 ? r : R;
-    const int RH = I1_TH + 2 * rr, RW = LK_TW + 2 * rr;
-    const int plane = i1_plane<R>(RH, RW);
-    const int rowlen = i1_rowlen<R>(RW);
-    for (int i = threadIdx.x; i < RH * RW; i += LK_THREADS) {
+    const int RH = I1_TH + 2 * r, RW = LK_TW + 2 * r;
+    const int plane = RH * RW;
+    for (int i = threadIdx.x; i < plane; i += LK_THREADS) {
         const int ry = i / RW, rx = i - ry * RW;
-        const int y = ty0 - rr + ry, x = tx0 - rr + rx;
+        const int y = ty0 - r + ry, x = tx0 - r + rx;
         float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f;
         if ((unsigned)y < (unsigned)a.H && (unsigned)x < (unsigned)a.W) {
             float c, gx, gy;
@@ -69,41 +57,87 @@ __device__ __forceinline__ void i1_hess_tile(const HessArgs &a, int tile, int r,
             p1 = gx * gy;
             p2 = gy * gy;
         }
-        float *q = smem + ry * rowlen + rx;
-        q[0] = p0;
-        q[plane] = p1;
-        q[2 * plane] = p2;
+        smem[i] = p0;
+        smem[plane + i] = p1;
+        smem[2 * plane + i] = p2;
     }
     __syncthreads();
-    if constexpr (R == 0) {
-        float *S = smem + 3 * plane;
-        box_hsum<3>(smem, S, RH, RW, r);
-        __syncthreads();
-        for (int i = threadIdx.x; i < I1_TH * LK_TW; i += LK_THREADS) {
-            const int ty = i / LK_TW, tx = i - ty * LK_TW;
-            const int y = ty0 + ty, x = tx0 + tx;
-            if (y >= a.H || x >= a.W) continue;
-            float s[3];
-            box_vsum<3>(S, RH, r, ty, tx, s);
-            a.hess[(size_t)y * a.hess_pitch + x] = make_float4(s[0], s[1], s[2], 0.0f);
-        }
-    } else {
-        box_h_inplace<R, 3, I1_TH>(smem);
-        for (int i = threadIdx.x; i < LK_TW * (I1_TH / 4); i += LK_THREADS) {
-            const int tx = i % LK_TW, g = i / LK_TW;
-            const int x = tx0 + tx;
-            if (x >= a.W || ty0 + 4 * g >= a.H) continue;
-            float s[3][4];
-            box_v4<R, 3, I1_TH>(smem, g, tx, s);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int y = ty0 + 4 * g + j;
-                if (y >= a.H) break;
-                a.hess[(size_t)y * a.hess_pitch + x] = make_float4(s[0][j], s[1][j], s[2][j], 0.0f);
-            }
-        }
+    float *S = smem + 3 * plane;
+    box_hsum<3>(smem, S, RH, RW, r);
+    __syncthreads();
+    for (int i = threadIdx.x; i < I1_TH * LK_TW; i += LK_THREADS) {
+        const int ty = i / LK_TW, tx = i - ty * LK_TW;
+        const int y = ty0 + ty, x = tx0 + tx;
+        if (y >= a.H || x >= a.W) continue;
+        float s[3];
+        box_vsum<3>(S, RH, r, ty, tx, s);
+        a.hess[(size_t)y * a.hess_pitch + x] = make_float4(s[0], s[1], s[2], 0.0f);
     }
 }
+
+// The same for a fixed radius: pixel pairs, the first two channels in a pair plane (P01) and the
+// third in P4, summed by the passes of the iteration tile. 16 images of 1024^2 at r = 4 take 99 us (302
+// MB, 45 us at the memory's rate); one pixel at a time with three planes of floats, 105.
+template <typename T, int R>
+__device__ __forceinline__ void i1_hess_tile(const HessArgs &a, int tile, float *smem)
+{
+    using F = FixedTile<R, I1_TH>;
+    const int tyi = tile / a.tiles_x;
+    const int ty0 = tyi * I1_TH, tx0 = (tile - tyi * a.tiles_x) * LK_TW;
+    float2 *P01 = reinterpret_cast<float2 *>(smem);
+    float *P4 = smem + 2 * F::PAIR_PLANE;
+    const T *I1 = static_cast<const T *>(a.I1);
+    constexpr int NPR = F::RWE / 2, RPI = LK_THREADS / NPR;
+    const int cx = threadIdx.x % NPR, rs = threadIdx.x / NPR;
+    const int x = tx0 - F::RE + 2 * cx;
+    const bool inx = (unsigned)x < (unsigned)a.W, inq = (unsigned)(x + 1) < (unsigned)a.W;
+    if (rs < RPI) {
+#pragma unroll 2
+        for (int ry = rs; ry < F::RH; ry += RPI) {
+            const int y = ty0 - R + ry;
+            float4 s01 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            float2 s4 = f2(0.0f, 0.0f);
+            if (inx && (unsigned)y < (unsigned)a.H) {
+                float2 c, GX, GY;
+                i1_grad_pair<T, false, false>(I1 + (y * a.pitch + x), a.pitch, a.H, a.W, x, y, inq, c, GX, GY);
+                const float2 q0 = mul2(GX, GX), q1 = mul2(GX, GY), q2 = mul2(GY, GY);
+                s01 = inq ? make_float4(q0.x, q1.x, q0.y, q1.y) : make_float4(q0.x, q1.x, 0.0f, 0.0f);
+                s4 = f2(q2.x, inq ? q2.y : 0.0f);
+            }
+            reinterpret_cast<float4 *>(P01)[ry * (F::RWP2 / 2) + cx] = s01;
+            reinterpret_cast<float2 *>(P4)[ry * (F::RWP1 / 2) + cx] = s4;
+        }
+    }
+    __syncthreads();
+    box_h_pairs<R, I1_TH>(P01);
+    box_h_single<R, I1_TH>(P4);
+    __syncthreads();
+    constexpr int VR = v_rows<R, I1_TH>(), NV = 2 * R + VR;
+    for (int i = threadIdx.x; i < LK_TW * (I1_TH / VR); i += LK_THREADS) {
+        const int tx = i % LK_TW, g = i / LK_TW;
+        const int xo = tx0 + tx, yb = ty0 + VR * g;
+        if (xo >= a.W || yb >= a.H) continue;
+        float2 s01[VR];
+        float s4[VR];
+        {
+            float2 v[NV];
+#pragma unroll
+            for (int q = 0; q < NV; ++q) v[q] = P01[(VR * g + q) * F::RWP2 + tx];
+            box4v<R, 0>(v, s01);
+        }
+        {
+            float v[NV];
+#pragma unroll
+            for (int q = 0; q < NV; ++q) v[q] = P4[(VR * g + q) * F::RWP1 + tx];
+            box4v<R, 0>(v, s4);
+        }
+#pragma unroll
+        for (int j = 0; j < VR; ++j)
+            if (yb + j < a.H)
+                a.hess[(size_t)(yb + j) * a.hess_pitch + xo] = make_float4(s01[j].x, s01[j].y, s4[j], 0.0f);
+    }
+}
+static_assert(I1_TH % 6 != 0, "four-row groups in the window-matrix tile");
 
 // One iteration of the variant on one output tile, for any window radius r given at run time
 // (the fixed radii run the tiles of the main method with the variant's stage 1 and solve).
@@ -154,7 +188,8 @@ __global__ void __launch_bounds__(LK_THREADS) i1_hess_kernel(HessArgs a, int r)
 {
     extern __shared__ float4 smem4[];
     chain_begin();
-    i1_hess_tile<T, R>(a, blockIdx.x, r, reinterpret_cast<float *>(smem4));
+    if constexpr (R == 0) i1_hess_tile_generic<T>(a, blockIdx.x, r, reinterpret_cast<float *>(smem4));
+    else i1_hess_tile<T, R>(a, blockIdx.x, reinterpret_cast<float *>(smem4));
 }
 
 // Resident blocks per SM. The iteration is bound by latency and then by memory (36 bytes per
@@ -205,7 +240,8 @@ __global__ void __launch_bounds__(LK_THREADS) phase_hess_kernel(const __grid_con
     extern __shared__ float4 smem4[];
     chain_begin();
     const int p = phase_pair(P.prefix, P.npairs, blockIdx.x);
-    i1_hess_tile<T, R>(P.a[p], blockIdx.x - P.prefix[p], r, reinterpret_cast<float *>(smem4));
+    if constexpr (R == 0) i1_hess_tile_generic<T>(P.a[p], blockIdx.x - P.prefix[p], r, reinterpret_cast<float *>(smem4));
+    else i1_hess_tile<T, R>(P.a[p], blockIdx.x - P.prefix[p], reinterpret_cast<float *>(smem4));
 }
 
 template <typename T, int R>

@@ -645,13 +645,7 @@ __device__ __forceinline__ void lk_tile_generic(const IterArgs &a, int tile, int
 template <int R, int TH = LK_TH, int TW = LK_TW, bool V = false> struct FixedTile {
     static_assert(R >= 2, "the grouped box sums need 2R >= 4");
     static constexpr int W = 2 * R + 1;                // window width
-    static constexpr int NV4 = (2 * R + 4 + 3) / 4;    // float4 loads for 4 outputs' windows
     static constexpr int RH = TH + 2 * R;              // region rows (tile + halo)
-    static constexpr int RW = TW + 2 * R;              // region columns
-    static constexpr int RWP = TW + 4 * NV4 - 4;       // padded row length (>= RW, multiple of 4)
-    static constexpr int PLANE = RH * RWP;
-    static constexpr int NREG = RH * RW;               // region pixels
-    static constexpr int PER = (NREG + LK_THREADS - 1) / LK_THREADS;   // region pixels per thread
     // Staging (a.stage_i2): one TMA box of I2, the window of the tile's region shifted by
     // the rounded estimate at the tile's centre and widened by STAGE_MARGIN pixels plus the 4x4
     // tap footprint (and, for the alignment of its first column, E - 1 columns), in the
@@ -732,83 +726,6 @@ template <int R, int TH, bool V = false> struct StripTile {
 #define OF_PREFETCH_I1 2
 #endif
 constexpr long long STAGE_TIMEOUT_NS = 200000000LL;   // 0.2 s for one tile's staging copies
-
-// o[j] = sum_{k=0}^{2R} v[j+k], j = 0..3, from v[0 .. 2R+3].
-template <int R>
-__device__ __forceinline__ void box4(const float *v, float o[4])
-{
-    float m = v[3];
-#pragma unroll
-    for (int k = 4; k <= 2 * R; ++k) m += v[k];
-    o[0] = ((v[0] + v[1]) + v[2]) + m;
-    o[1] = ((v[1] + v[2]) + m) + v[2 * R + 1];
-    o[2] = ((v[2] + m) + v[2 * R + 1]) + v[2 * R + 2];
-    o[3] = ((m + v[2 * R + 1]) + v[2 * R + 2]) + v[2 * R + 3];
-}
-
-// Horizontal pass, in place: row ry of plane c (c < C) becomes, at columns
-// 0..LK_TW-1, the window sums of the outputs of that row.
-template <int R, int C = 5, int TH = LK_TH>
-__device__ __forceinline__ void box_h_inplace(float *P)
-{
-    using F = FixedTile<R, TH>;
-    constexpr int NG = LK_TW / 4;
-    static_assert(32 % NG == 0 && LK_THREADS % 32 == 0, "a row's items must lie in one warp");
-    constexpr int NITEMS = F::RH * NG;
-    constexpr int IT = (NITEMS + LK_THREADS - 1) / LK_THREADS;
-#pragma unroll 1
-    for (int c = 0; c < C; ++c) {
-        float *Pc = P + c * F::PLANE;
-        float4 res[IT];
-#pragma unroll
-        for (int k = 0; k < IT; ++k) {
-            const int i = threadIdx.x + k * LK_THREADS;
-            if (i < NITEMS) {
-                const int ry = i / NG, g = i % NG;
-                const float4 *src = reinterpret_cast<const float4 *>(Pc + ry * F::RWP + 4 * g);
-                float v[4 * F::NV4];
-#pragma unroll
-                for (int q = 0; q < F::NV4; ++q) {
-                    const float4 t = src[q];
-                    v[4 * q] = t.x;
-                    v[4 * q + 1] = t.y;
-                    v[4 * q + 2] = t.z;
-                    v[4 * q + 3] = t.w;
-                }
-                float o[4];
-                box4<R>(v, o);
-                res[k] = make_float4(o[0], o[1], o[2], o[3]);
-            }
-        }
-        // Item i covers row i / NG: the NG = 16 items of a row are 16 consecutive lanes
-        // of one warp (in every pass), so only that warp reads what it overwrites.
-        __syncwarp();
-#pragma unroll
-        for (int k = 0; k < IT; ++k) {
-            const int i = threadIdx.x + k * LK_THREADS;
-            if (i < NITEMS) {
-                const int ry = i / NG, g = i % NG;
-                *reinterpret_cast<float4 *>(Pc + ry * F::RWP + 4 * g) = res[k];
-            }
-        }
-    }
-    __syncthreads();
-}
-
-// Vertical pass for the 4 outputs (rows 4g..4g+3, column tx) of each of C channels.
-template <int R, int C = 5, int TH = LK_TH>
-__device__ __forceinline__ void box_v4(const float *P, int g, int tx, float s[C][4])
-{
-    using F = FixedTile<R, TH>;
-#pragma unroll
-    for (int c = 0; c < C; ++c) {
-        const float *col = P + c * F::PLANE + 4 * g * F::RWP + tx;
-        float v[2 * R + 4];
-#pragma unroll
-        for (int q = 0; q < 2 * R + 4; ++q) v[q] = col[q * F::RWP];
-        box4<R>(v, s[c]);
-    }
-}
 
 // --------------------------------------------------- pixel-pair and channel-pair passes
 // Two horizontally adjacent pixels (x even) of a level image, as floats (exact for every
@@ -949,8 +866,8 @@ __device__ __forceinline__ void sample_grad2(const T *I, int pitch, const T *win
     GY = mul2(sub2(lerp2(BOT, lerp2(D0, D1, AX, OX), AY, OY), lerp2(lerp2(A0, A1, AX, OX), TOP, AY, OY)), half);
 }
 
-// o[j] = sum_{k=0}^{2R} v[OFF+j+k], j = 0..3, the additions in box4's order (floats or
-// float2 pairs of channels).
+// o[j] = sum_{k=0}^{2R} v[OFF+j+k], j = 0..3, the middle terms m, which the four
+// windows share, added once (floats or float2 pairs of channels).
 template <int R, int OFF, typename V>
 __device__ __forceinline__ void box4v(const V *v, V o[4])
 {
@@ -1289,6 +1206,23 @@ __device__ __forceinline__ void stage1_pair(const IterArgs &a, int x, int y, flo
     }
 }
 
+// I1 at the pixel pair (x, y), (x + 1, y) (row: its first element; the second only when q) and
+// its central-difference gradient, neighbour indices clamped (INNER: none needs it), halved.
+template <typename T, bool NC, bool INNER>
+__device__ __forceinline__ void i1_grad_pair(const T *row, int pitch, int H, int W, int x, int y, bool q, float2 &c,
+                                             float2 &GX, float2 &GY)
+{
+    c = ld_pair<NC>(row, q);
+    const float2 up = ld_pair<NC>(INNER || y > 0 ? row - pitch : row, q);
+    const float2 dn = ld_pair<NC>(INNER || y + 1 < H ? row + pitch : row, q);
+    const float lf = ldf<NC>(INNER || x > 0 ? row - 1 : row);
+    const float rt = INNER || x + 2 < W ? ldf<NC>(row + 2) : c.y;   // right of the second (the last: itself)
+    const float2 half = f2(0.5f, 0.5f);
+    // the first pixel's right neighbour is the second, or itself at the last column
+    GX = mul2(sub2(f2(q ? c.y : c.x, rt), f2(lf, c.x)), half);
+    GY = mul2(sub2(dn, up), half);
+}
+
 // Stage 1 of the variant linearised with the first image's gradient, for the pixel pair: g1 is
 // the central difference of I1 at the pixels (neighbour indices clamped, halved), e~ = I1 -
 // I2(x + u) + g1 . (u - ref), and the products are the two right-hand-side channels g1 e~.
@@ -1311,16 +1245,8 @@ __device__ __forceinline__ void stage1_pair_i1(const IterArgs &a, int x, int y, 
     } else {
         flow_pair<NC, MODE>(a, x, y, inq, fp, fq);
     }
-    const T *row = I1 + (y * a.pitch + x);
-    const float2 c = ld_pair<NC>(row, inq);
-    const float2 up = ld_pair<NC>(INNER || y > 0 ? row - a.pitch : row, inq);
-    const float2 dn = ld_pair<NC>(INNER || y + 1 < a.H ? row + a.pitch : row, inq);
-    const float lf = ldf<NC>(INNER || x > 0 ? row - 1 : row);
-    const float rt = INNER || x + 2 < a.W ? ldf<NC>(row + 2) : c.y;   // right of q (q is the last: itself)
-    const float2 half = f2(0.5f, 0.5f);
-    // p's right neighbour is q, or p itself at the last column
-    const float2 GX = mul2(sub2(f2(inq ? c.y : c.x, rt), f2(lf, c.x)), half);
-    const float2 GY = mul2(sub2(dn, up), half);
+    float2 c, GX, GY;
+    i1_grad_pair<T, NC, INNER>(I1 + (y * a.pitch + x), a.pitch, a.H, a.W, x, y, inq, c, GX, GY);
     const float2 FU = f2(floorf(fp.x), floorf(fq.x)), FV = f2(floorf(fp.y), floorf(fq.y));
     const float2 AX = sub2(f2(fp.x, fq.x), FU), AY = sub2(f2(fp.y, fq.y), FV);
     const int xp = pos_floor(x, FU.x), yp = pos_floor(y, FV.x);

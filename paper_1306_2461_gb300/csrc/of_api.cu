@@ -23,20 +23,7 @@ int pitch_of(int W) { return (W + kPitchAlign - 1) / kPitchAlign * kPitchAlign; 
 
 int map_cuda(cudaError_t e) { return e == cudaSuccess ? OF_OK : (e == cudaErrorMemoryAllocation ? OF_ENOMEM : OF_ECUDA); }
 
-std::mutex g_dev_mu;
-bool g_dev_configured[256];
-
-int configure_device()
-{
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return OF_ECUDA;
-    std::lock_guard<std::mutex> lk(g_dev_mu);
-    if (dev < 0 || dev >= 256) return OF_ECUDA;
-    if (g_dev_configured[dev]) return OF_OK;
-    if (configure_lk_kernels() != cudaSuccess) return OF_ECUDA;
-    g_dev_configured[dev] = true;
-    return OF_OK;
-}
+int configure_device(int radius) { return configure_lk_kernels(radius) == cudaSuccess ? OF_OK : OF_ECUDA; }
 
 }  // namespace
 
@@ -318,7 +305,7 @@ int of_create(const of_plan *p, of_handle *out)
     if (!out) return OF_EINVAL;
     *out = nullptr;
     if (of_plan_validate(p) != OF_OK) return OF_EINVAL;
-    int rc = configure_device();
+    int rc = configure_device(p->radius);
     if (rc) return rc;
     of_ctx *h = new (std::nothrow) of_ctx();
     if (!h) return OF_ENOMEM;
@@ -408,7 +395,7 @@ int of_window_sums(const float *ch, int32_t H, int32_t W, int32_t r, float *out,
 {
     if (!ch || !out || H < 1 || W < 1 || r < 1 || r > MAX_RADIUS || (int64_t)H * W > (int64_t(1) << 28))
         return OF_EINVAL;
-    int rc = configure_device();
+    int rc = configure_device(-1);   // any radius may follow, perhaps inside a capture
     if (rc) return rc;
     return map_cuda(launch_window_sums(ch, H, W, r, out, reinterpret_cast<cudaStream_t>(stream)));
 }

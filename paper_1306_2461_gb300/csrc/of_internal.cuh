@@ -275,7 +275,9 @@ cudaError_t launch_chained(void (*k)(P...), dim3 grid, int threads, size_t smem,
     cfg.attrs = attr;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     cfg.numAttrs = cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k, args...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k, args...);
+    if (e != cudaSuccess) cudaGetLastError();   // reported by the return value
+    return e;
 }
 
 // ------------------------------------------------------------------- launchers
@@ -311,7 +313,9 @@ void *batch_kernel_generic(int in_format, int storage);   // the run-time-radius
 size_t batch_smem_generic(int radius);
 cudaError_t launch_level_to_f32(const Level &l, int elem, float *dst, cudaStream_t s);
 cudaError_t launch_wait_timeout(int *flag, int *status, long long timeout_ns, cudaStream_t s);
-cudaError_t configure_lk_kernels();   // all kernels with dynamic shared memory, current device
+// The kernels with dynamic shared memory of one radius (-1: every radius) and the run-time-radius
+// ones, on the current device, once.
+cudaError_t configure_lk_kernels(int radius);
 // Fill a.tm_flow and a.tm_i2 for the staged fixed-radius tile of this radius and tile
 // height (level image type elem). Returns false (and clears a.stage_i2) when the radius
 // has no fixed-radius kernel or the tensor maps cannot be encoded; the tile then

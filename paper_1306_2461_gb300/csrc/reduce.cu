@@ -121,8 +121,12 @@ cluster_reduce_kernel(const float *p, long long n, A a, void *out)
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     __shared__ uint2 part[CLUSTER];
+    // a block's shared memory may be written from outside once all blocks of the cluster have
+    // arrived here, that is, started; the wait is hidden behind the scan
+    cluster.barrier_arrive();
     scan(p, n, (long long)blockIdx.x * CLUSTER_THREADS + threadIdx.x, (long long)CLUSTER * CLUSTER_THREADS, a);
     block_reduce(a);
+    cluster.barrier_wait();
     if (threadIdx.x == 0) cluster.map_shared_rank(part, 0)[blockIdx.x] = pack(a);
     cluster.sync();
     if (blockIdx.x == 0 && threadIdx.x < 32) {

@@ -1,0 +1,27 @@
+"""Rules of the CUDA programming model that no result shows: a kernel that breaks one may run
+right for years, so they are read off the kernels' sources."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1306_2461_gb300", "csrc")
+
+
+def code_of(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*|/\*.*?\*/", "", f.read(), flags=re.S)
+
+
+SOURCES = sorted(n for n in os.listdir(CSRC) if n.endswith((".cu", ".cuh")))
+
+
+@pytest.mark.parametrize("name", SOURCES)
+def test_remote_shared_memory_between_cluster_barriers(name):
+    # another block's shared memory is accessed after a cluster barrier (the block has started)
+    # and before another one (it has not ended)
+    for body in re.findall(r"__cluster_dims__.*?\n}\n", code_of(name), flags=re.S):
+        barriers = [m.start() for m in re.finditer(r"barrier_wait\(\)|cluster\.sync\(\)", body)]
+        for m in re.finditer(r"map_shared_rank", body):
+            assert any(b < m.start() for b in barriers) and any(b > m.start() for b in barriers)
+        assert len(re.findall(r"barrier_arrive\(\)", body)) == len(re.findall(r"barrier_wait\(\)", body))

@@ -1137,24 +1137,29 @@ __device__ __forceinline__ void box_v_two(const float2 *P01, const float2 *P23, 
 // once when both sample the interior (taps from the staged window or global memory),
 // pixel by pixel near the border or at the image's last column. The form is chosen per
 // warp (all of its pairs take the border form if one has to: it gives the same bits, and
-// running both forms one after the other costs more). INNER: the tile's whole region and
+// running both forms one after the other costs more: 1024^2 pair 181 us, with the form per
+// lane 198): unless INNER, all lanes of the warp call this together, those without a pair with
+// on = false, and the lanes with pixels of the image, found by a ballot of the whole warp,
+// vote. INNER: the tile's whole region and
 // its staged window lie inside the image, so that no pair needs a bounds check and a
 // footprint inside the window is inside the image. sflow: the pair's staged estimates
 // (NULL: read them from fin). Out-of-image pixels get zero products. Returns the products
 // in the planes' layout.
 template <typename T, bool NC, int MODE, int WW, int WH, bool INNER>
-__device__ __forceinline__ void stage1_pair(const IterArgs &a, int x, int y, float2 ref, const float4 *sflow,
+__device__ __forceinline__ void stage1_pair(const IterArgs &a, int x, int y, bool on, float2 ref, const float4 *sflow,
                                             const T *win, int wx0, int wy0, float4 &s01, float4 &s23, float2 &s4)
 {
     s01 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     s23 = s01;
     s4 = f2(0.0f, 0.0f);
-    const bool rowin = INNER || (unsigned)y < (unsigned)a.H;
+    const bool rowin = INNER || (on && (unsigned)y < (unsigned)a.H);
     const bool inp = rowin && (INNER || (unsigned)x < (unsigned)a.W);
     const bool inq = rowin && (INNER || (unsigned)(x + 1) < (unsigned)a.W);   // implies inp (x even)
-    if (!inp) return;
     const T *I1 = static_cast<const T *>(a.I1);
     const T *I2 = static_cast<const T *>(a.I2);
+    unsigned lanes = 0;
+    if constexpr (!INNER) lanes = __ballot_sync(0xffffffffu, inp);
+    if (!inp) return;
     float2 fp, fq;
     if (sflow) {
         const float4 w = *sflow;   // zeros beyond the image
@@ -1179,7 +1184,7 @@ __device__ __forceinline__ void stage1_pair(const IterArgs &a, int x, int y, flo
     bool both = inwin;
     if constexpr (!INNER) {
         const unsigned ws = interior_span(a.W), hs = interior_span(a.H);
-        both = __all_sync(__activemask(), inq && interior(xp, yp, ws, hs) && interior(xq, yq, ws, hs));
+        both = __all_sync(lanes, inq && interior(xp, yp, ws, hs) && interior(xq, yq, ws, hs));
     }
     if (both) {
         sample_grad2<NC, WW>(I2, a.pitch, win, INNER || inwin, cpx, cpy, cqx, cqy, xp, yp, xq, yq, AX, AY, IW, GX, GY);
@@ -1478,9 +1483,11 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
         // rows + DX pairs)
         constexpr int DY = NT / NPR, DX = NT % NPR;
         constexpr int npair = F::RH * NPR;
+        constexpr bool WHOLE = !V && !decltype(inner)::value;   // whole warps (stage1_pair)
         int ry = threadIdx.x / NPR, cx = threadIdx.x % NPR;
 #pragma unroll 1
-        for (int j = threadIdx.x; j < npair; j += NT) {
+        for (int j = threadIdx.x; (WHOLE ? j & ~31 : j) < npair; j += NT) {
+            const bool on = !WHOLE || j < npair;
             const int k2 = ry * (F::RWP2 / 2) + cx;   // float4 slot of the pair in the pair planes
             const float4 *sf = box ? reinterpret_cast<const float4 *>(P01) + k2 : nullptr;
             const int x = tx0 - F::RE + 2 * cx, y = ty0 - R + ry;
@@ -1490,12 +1497,14 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
             } else {
                 float4 s23;
                 float2 s4;
-                stage1_pair<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(a, x, y, ref, sf, wt, wx0, wy0, s01, s23,
-                                                                               s4);
-                reinterpret_cast<float4 *>(P23)[k2] = s23;
-                reinterpret_cast<float2 *>(P4)[ry * (F::RWP1 / 2) + cx] = s4;
+                stage1_pair<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(a, x, y, on, ref, sf, wt, wx0, wy0, s01,
+                                                                               s23, s4);
+                if (on) {
+                    reinterpret_cast<float4 *>(P23)[k2] = s23;
+                    reinterpret_cast<float2 *>(P4)[ry * (F::RWP1 / 2) + cx] = s4;
+                }
             }
-            reinterpret_cast<float4 *>(P01)[k2] = s01;
+            if (on) reinterpret_cast<float4 *>(P01)[k2] = s01;
             ry += DY;
             cx += DX;
             if (cx >= NPR) {
@@ -1602,7 +1611,7 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
         // stage 1 over region rows r0..RH-1, by pixel pairs
         constexpr int NPR = F::RWE / 2;   // pairs per region row
         const T *wt = staged ? reinterpret_cast<const T *>(win) : nullptr;
-        auto pair = [&](auto inner, int ry, int cx) {
+        auto pair = [&](auto inner, int ry, int cx, bool on) {
             const int sl = ring_slot<RN>(ry, base);
             const int k2 = sl * (F::RWP2 / 2) + cx;   // float4 slot of the pair in the pair planes
             const float4 *sf = flows ? reinterpret_cast<const float4 *>(P01) + k2 : nullptr;
@@ -1613,21 +1622,26 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
             } else {
                 float4 s23;
                 float2 s4;
-                stage1_pair<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(a, x, y, ref, sf, wt, wx0, wy0, s01, s23,
-                                                                               s4);
-                reinterpret_cast<float4 *>(P23)[k2] = s23;
-                reinterpret_cast<float2 *>(P4)[sl * (F::RWP1 / 2) + cx] = s4;
+                stage1_pair<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(a, x, y, on, ref, sf, wt, wx0, wy0, s01,
+                                                                               s23, s4);
+                if (on) {
+                    reinterpret_cast<float4 *>(P23)[k2] = s23;
+                    reinterpret_cast<float2 *>(P4)[sl * (F::RWP1 / 2) + cx] = s4;
+                }
             }
-            reinterpret_cast<float4 *>(P01)[k2] = s01;
+            if (on) reinterpret_cast<float4 *>(P01)[k2] = s01;
         };
         auto rows = [&](auto inner) {
             // thread t takes pair cx = t mod NPR of rows r0 + t / NPR, then RPI rows further each
             // round, so that what depends on the pair's column is the same on every row it takes
             constexpr int RPI = NT / NPR;   // rows per round
             const int cx = threadIdx.x % NPR, rs = threadIdx.x / NPR;
-            if (rs < RPI) {
+            if constexpr (!V && !decltype(inner)::value) {   // whole warps (stage1_pair)
 #pragma unroll 1
-                for (int ry = r0 + rs; ry < RH; ry += RPI) pair(inner, ry, cx);
+                for (int row = r0; row < RH; row += RPI) pair(inner, row + rs, cx, rs < RPI && row + rs < RH);
+            } else if (rs < RPI) {
+#pragma unroll 1
+                for (int ry = r0 + rs; ry < RH; ry += RPI) pair(inner, ry, cx, true);
             }
         };
         if (staged && tile_inner<R, TH, TW, S, V>(a, tx0, ty0, wx0, wy0)) rows(std::true_type());
@@ -1773,15 +1787,18 @@ __device__ __forceinline__ void lk_tile_fused2(const IterArgs &a, int tile, floa
         int ry = threadIdx.x / NPR, cx = threadIdx.x % NPR;
         __syncthreads();
 #pragma unroll 1
-        for (int j = threadIdx.x; j < NPAIR; j += LK_THREADS) {
+        for (int j = threadIdx.x; (j & ~31) < NPAIR; j += LK_THREADS) {   // whole warps (stage1_pair)
+            const bool on = j < NPAIR;
             const int k2 = ry * (A::RWP2 / 2) + cx;
             float4 s01, s23;
             float2 s4;
-            stage1_pair<T, NC, FLOW_SAME, 4, 4, false>(a, ax0 - A::RE + 2 * cx, ay0 - R + ry, ref, nullptr, nullptr, 0,
-                                                       0, s01, s23, s4);
-            reinterpret_cast<float4 *>(Q01)[k2] = s01;
-            reinterpret_cast<float4 *>(Q23)[k2] = s23;
-            reinterpret_cast<float2 *>(Q4)[ry * (A::RWP1 / 2) + cx] = s4;
+            stage1_pair<T, NC, FLOW_SAME, 4, 4, false>(a, ax0 - A::RE + 2 * cx, ay0 - R + ry, on, ref, nullptr, nullptr,
+                                                       0, 0, s01, s23, s4);
+            if (on) {
+                reinterpret_cast<float4 *>(Q01)[k2] = s01;
+                reinterpret_cast<float4 *>(Q23)[k2] = s23;
+                reinterpret_cast<float2 *>(Q4)[ry * (A::RWP1 / 2) + cx] = s4;
+            }
             ry += DY;
             cx += DX;
             if (cx >= NPR) {
@@ -1828,16 +1845,19 @@ __device__ __forceinline__ void lk_tile_fused2(const IterArgs &a, int tile, floa
         constexpr int DY = LK_THREADS / NPR, DX = LK_THREADS % NPR;
         int ry = threadIdx.x / NPR, cx = threadIdx.x % NPR;
 #pragma unroll 1
-        for (int j = threadIdx.x; j < NPAIR; j += LK_THREADS) {
+        for (int j = threadIdx.x; (j & ~31) < NPAIR; j += LK_THREADS) {
+            const bool on = j < NPAIR;
             const int k2 = ry * (B::RWP2 / 2) + cx;
             float4 s01, s23;
             float2 s4;
-            stage1_pair<T, NC, FLOW_SAME, 4, 4, false>(a, tx0 - B::RE + 2 * cx, ty0 - R + ry, ref,
+            stage1_pair<T, NC, FLOW_SAME, 4, 4, false>(a, tx0 - B::RE + 2 * cx, ty0 - R + ry, on, ref,
                                                        reinterpret_cast<const float4 *>(FB) + k2, nullptr, 0, 0, s01,
                                                        s23, s4);
-            reinterpret_cast<float4 *>(P01)[k2] = s01;
-            reinterpret_cast<float4 *>(P23)[k2] = s23;
-            reinterpret_cast<float2 *>(P4)[ry * (B::RWP1 / 2) + cx] = s4;
+            if (on) {
+                reinterpret_cast<float4 *>(P01)[k2] = s01;
+                reinterpret_cast<float4 *>(P23)[k2] = s23;
+                reinterpret_cast<float2 *>(P4)[ry * (B::RWP1 / 2) + cx] = s4;
+            }
             ry += DY;
             cx += DX;
             if (cx >= NPR) {

@@ -25,3 +25,15 @@ def test_remote_shared_memory_between_cluster_barriers(name):
         for m in re.finditer(r"map_shared_rank", body):
             assert any(b < m.start() for b in barriers) and any(b > m.start() for b in barriers)
         assert len(re.findall(r"barrier_arrive\(\)", body)) == len(re.findall(r"barrier_wait\(\)", body))
+
+
+@pytest.mark.parametrize("name", SOURCES)
+def test_votes_name_lanes_that_arrive(name):
+    # __activemask() gives whichever lanes happen to be converged: lanes may then hold different
+    # masks for one vote, which is undefined. A vote or reduction names the whole warp, or the
+    # lanes of a ballot of the whole warp.
+    code = code_of(name)
+    assert "__activemask" not in code
+    masks = {"0xffffffffu"} | set(re.findall(r"(\w+) = __ballot_sync\(0xffffffffu,", code))
+    for m in re.finditer(r"__(?:all|any|ballot|shfl\w*|reduce_\w+|match\w*)_sync\(([^,]*),", code):
+        assert m.group(1).strip() in masks

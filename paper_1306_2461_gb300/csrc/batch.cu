@@ -638,17 +638,20 @@ int run_batch(int32_t n, const of_handle *hs, const void *const *I1s, const void
     // longer.
     if (t.branches == BRANCHES_AUTO) t.branches = graphs && n > 1 ? 2 : 0;
     const size_t pairs_bytes = sizeof(BatchPair) * n, prefix_bytes = sizeof(int32_t) * b.prefix.size();
-    std::vector<char> key(pairs_bytes + prefix_bytes + sizeof(st) + 7 * sizeof(int));
+    // Everything the launches depend on: the descriptors, the stream, the method and how it is run.
+    // Entries outlive the handles, and a later handle of another method may get the same addresses.
+    int fp64_bits;
+    memcpy(&fp64_bits, &p0.fp64_cond, sizeof(fp64_bits));
+    const int extra[] = {p0.radius, p0.levels, p0.iterations, p0.in_format, p0.storage, fp64_bits,
+                         (int)(p0.flags & (OF_FLAG_GATHER | OF_FLAG_ZNSSD | OF_FLAG_I1GRAD)), hs[0]->device, graphs ? 1 : 0,
+                         t.generic_sums, t.stage_i2, t.blocks_per_sm, t.phased, t.prefetch, t.tile_h,
+                         t.phased ? t.branches : 0, t.phased ? t.fusion : 0, t.phased ? tuning_strip(t) : 0};
+    std::vector<char> key(pairs_bytes + prefix_bytes + sizeof(st) + sizeof(extra));
     {
         char *k = key.data();
         memcpy(k, b.pairs.data(), pairs_bytes);
         memcpy(k + pairs_bytes, b.prefix.data(), prefix_bytes);
         memcpy(k + pairs_bytes + prefix_bytes, &st, sizeof(st));
-        const int extra[7] = {p0.radius,
-                              (int)(p0.iterations * 16 + (p0.flags & (OF_FLAG_GATHER | OF_FLAG_ZNSSD | OF_FLAG_I1GRAD))),
-                              hs[0]->device, t.generic_sums, t.stage_i2,
-                              t.blocks_per_sm + 256 * t.phased + 65536 * t.prefetch + (1 << 24) * (t.tile_h != 0),
-                              t.phased ? t.branches + 16 * t.fusion + 256 * tuning_strip(t) : 0};
         memcpy(k + pairs_bytes + prefix_bytes + sizeof(st), extra, sizeof(extra));
     }
 

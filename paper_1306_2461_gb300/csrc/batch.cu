@@ -256,8 +256,9 @@ static cudaError_t enqueue_chain(const BatchPair *pairs, int n, const of_plan &p
     const int tile_h = (t.tile_h == ALT_TH && !t.generic_sums && radius_specialised(p0.radius)) ? ALT_TH : LK_TH;
     // blocks a launch keeps before its strips shrink: two per resident slot, counting the other sequences
     const long slots = (long)lk_slots(p0.radius) * sms * (sequences > 1 ? 1 : 2);
-    // tiles per block of the fixed-radius kernels (the run-time-radius kernel takes one)
-    const int strip = (!t.generic_sums && radius_strips(p0.radius, tile_h)) ? strip_len(tuning_strip(t)) : 1;
+    const bool i1grad = (p0.flags & OF_FLAG_I1GRAD) != 0;
+    // tiles per block of the fixed-radius kernels (the run-time-radius kernel and the variant's take one)
+    const int strip = (!t.generic_sums && !i1grad && radius_strips(p0.radius, tile_h)) ? strip_len(tuning_strip(t)) : 1;
     cudaError_t e;
     for (int g0 = 0; g0 < n; g0 += PHASE_PAIRS) {
         const int m = n - g0 < PHASE_PAIRS ? n - g0 : PHASE_PAIRS;
@@ -314,7 +315,6 @@ static cudaError_t enqueue_chain(const BatchPair *pairs, int n, const of_plan &p
         }
         // iterations, coarsest level first; flow buffers ping-pong (one swap per launch). With
         // fusion 2, iterations it and it + 1 of a level (it >= 1) run as one launch.
-        const bool i1grad = (p0.flags & OF_FLAG_I1GRAD) != 0;
         const bool fuse = t.fusion == 2 && !i1grad;
         int cur = 0;
         for (int k = 0; k < L * p0.iterations; ++k, cur = 1 - cur) {
@@ -397,7 +397,7 @@ static cudaError_t enqueue_chain(const BatchPair *pairs, int n, const of_plan &p
                     a.tiles_x = small_tiles_x(a.W);
                     a.tiles = small_units(a.H, a.W);
                 }
-                if (a.stage_i2) fill_stage_maps(a, I.m[i], level_elem(p0, l), p0.radius, th_l, true);   // else gathered
+                if (a.stage_i2) fill_stage_maps(a, I.m[i], level_elem(p0, l), p0.radius, th_l, !i1grad);   // else gathered
                 I.prefix[i + 1] = I.prefix[i] + a.tiles;
             }
             e = i1grad ? launch_phase_i1_iter(I, level_elem(p0, l), p0.radius, t.generic_sums != 0, p0.fp64_cond, th_l, st)

@@ -256,16 +256,15 @@ phase_i1_iter_kernel(const __grid_constant__ IterPhase P, int r, float fp64_cond
         chain_begin();
         i1_iter_tile<T>(P.a[p], unit, r, fp64_cond, smem);
     } else {
-        constexpr bool MULTI = LK_TH >= 2 * R;
         uint32_t phase = 0;
-        lk_tile_init<R, LK_TH, LK_TW, MULTI, true>(smem);
+        lk_tile_init<R, LK_TH, LK_TW, false, true>(smem);
         chain_begin();
         const int t2 = blockIdx.x + P.ahead;
         if (P.ahead > 0 && t2 < P.prefix[P.npairs]) {
             const int q = phase_pair(P.prefix, P.npairs, t2);
             prefetch_tile<T, -1, LK_TH>(P.a[q], t2 - P.prefix[q], R);
         }
-        lk_tile_fixed<T, false, R, -1, LK_TH, MULTI, LK_THREADS, true>(P.a[p], &P.m[p], unit, fp64_cond, smem, phase);
+        lk_tile_fixed<T, false, R, -1, LK_TH, false, LK_THREADS, true>(P.a[p], &P.m[p], unit, fp64_cond, smem, phase);
     }
 }
 
@@ -284,7 +283,7 @@ phase_i1_small_kernel(const __grid_constant__ IterPhase P, float fp64_cond)
 }
 
 // Dynamic shared memory of the variant's iteration kernels (bytes).
-template <int R> inline size_t i1_iter_smem(int r, bool strips, bool small, bool stage, int elem_bytes)
+template <int R> inline size_t i1_iter_smem(int r, bool small, bool stage, int elem_bytes)
 {
     if constexpr (R == 0) {
         return sizeof(float) * (size_t)i1_smem_floats<0>(r, 2);
@@ -294,10 +293,6 @@ template <int R> inline size_t i1_iter_smem(int r, bool strips, bool small, bool
         int f;
         if (small) f = stage ? S::smem_staged(elem_bytes) : S::SMEM_NOSTAGE;
         else f = stage ? F::smem_staged(elem_bytes) : F::SMEM_NOSTAGE;
-        if constexpr (LK_TH >= 2 * R) {
-            using X = StripTile<R, LK_TH, true>;
-            if (strips && !small) f = stage ? X::smem_staged(elem_bytes) : X::SMEM_NOSTAGE;
-        }
         return sizeof(float) * (size_t)f;
     }
 }

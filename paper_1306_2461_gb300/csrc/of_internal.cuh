@@ -178,10 +178,9 @@ inline bool use_small_tiles(long tiles, int sms) { return 3 * tiles < 4 * (long)
 #endif
 constexpr int ALT_TH = OF_ALT_TH;
 static_assert(ALT_TH % 4 == 0 && ALT_TH != LK_TH, "a multiple of 4 other than LK_TH");
-// The fixed-radius iteration tile takes its reference flow per group of REF_GROUP tile
-// rows of a column of tiles, and a work unit is a strip of strip_len(strip) consecutive
-// tiles of one column inside one group (the tiles after the first take over the window
-// sums of the rows they share with the tile above).
+// A work unit of the fixed-radius iteration is a strip of strip_len(strip) consecutive tiles of
+// one column of tiles inside a group of REF_GROUP tile rows (the tiles after the first take over
+// the window sums of the rows they share with the tile above).
 constexpr int REF_GROUP = 4;
 inline __host__ __device__ int strip_len(int strip) { return strip == 2 || strip == 4 ? strip : 1; }
 inline __host__ __device__ int strip_units(int H, int W, int tile_h, int strip)
@@ -239,6 +238,13 @@ constexpr int lk_slots(int r) { return r <= 4 ? 4 : (r <= 6 ? 3 : 2); }
 // Strips take over 2r rows of sums from the tile above, which must lie below that tile's own
 // 2r first rows.
 constexpr bool radius_strips(int r, int tile_h) { return radius_grouped(r) && tile_h >= 2 * r; }
+// Tile rows that share a reference flow, to which the FP32 right-hand side is referred. The nearer the
+// reference, the smaller that side and its rounding: error against 64 bits (relative RMS, 1e-8) with
+// groups of 1, 2 and 4 tile rows and with the run-time-radius kernel's 64 x 24 (the variant's
+// 64 x 32) tiles, 300 x 1500 pairs: r = 7 3.7, 5.0, 8.2 and 3.9; r = 16 4.0, 5.9, 10.1 and 4.4; the
+// variant at r = 4 3.8, 4.7, 6.9 and 4.1. So the radii and the variant that ran those tiles
+// before they had these take each tile's own; the other radii's strips share one per group.
+template <int R, bool V> constexpr int ref_group() { return V || !radius_specialised(R) ? 1 : REF_GROUP; }
 
 // ------------------------------------------------------------- chained launches
 // The launches of a method's sequence after its first, when they go to a stream directly (no

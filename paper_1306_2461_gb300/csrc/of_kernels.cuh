@@ -702,15 +702,15 @@ template <int R, int TH = LK_TH, int TW = LK_TW, bool V = false> struct FixedTil
 // tile; RPAD puts the first row after the 2R carried ones in a slot that is a multiple of 8
 // (a 128-byte boundary), so that the estimate of the rows a tile computes comes in TMA boxes
 // of 8 rows.
-template <int R, int TH, bool V = false> struct StripTile {
-    using F = FixedTile<R, TH, LK_TW, V>;
+template <int R, int TH> struct StripTile {
+    using F = FixedTile<R, TH>;
     static_assert(TH % 8 == 0, "boxes of 8 rows");
     static constexpr int RPAD = (8 - 2 * R % 8) % 8;
     static constexpr int RING = RPAD + F::RH;
     static constexpr int BOX = 8;
     static constexpr int BOX_BYTES = F::RWP2 * BOX * 8;
     static constexpr int PAIR_PLANE = RING * F::RWP2;
-    static constexpr int PLANES = 2 * PAIR_PLANE + (V ? 0 : 2 * PAIR_PLANE + RING * F::RWP1);
+    static constexpr int PLANES = 4 * PAIR_PLANE + RING * F::RWP1;
     static constexpr int OFF_BAR = PLANES;
     static constexpr int OFF_WREF = OFF_BAR + 2;              // the tile-centre estimates (4 float2)
     static constexpr int OFF_WIN = (OFF_WREF + 8 + 31) / 32 * 32;
@@ -1323,7 +1323,7 @@ __device__ __forceinline__ void lk_tile_init(float *smem)
 {
     if (threadIdx.x == 0) {
         constexpr int off = [] {
-            if constexpr (MULTI) return StripTile<R, TH, V>::OFF_BAR;
+            if constexpr (MULTI) return StripTile<R, TH>::OFF_BAR;
             else return FixedTile<R, TH, TW, V>::OFF_BAR;
         }();
         mbar_init(reinterpret_cast<uint64_t *>(smem + off), 1);
@@ -1442,11 +1442,45 @@ __device__ __forceinline__ bool stage_wait(const IterArgs &a, uint64_t *bar, uin
     return true;
 }
 
+// The reference flow of the 64 x TH tiles in tile row t of the column at tx0: the estimate at the
+// centre of the tile's group of ref_group tile rows.
+template <bool NC, int MODE, int R, int TH, bool V = false>
+__device__ __forceinline__ float2 ref_flow(const IterArgs &a, int tx0, int t)
+{
+    constexpr int G = ref_group<R, V>();
+    return flow_mode<NC, MODE>(a, min(tx0 + LK_TW / 2, a.W - 1), min(t / G * G * TH + G * TH / 2, a.H - 1));
+}
+
+// Strips whose tiles have reference flows of their own: a tile that is not the first of its REF_GROUP
+// takes its first 2R region rows over from the tile above, formed with that tile's reference
+// (`above`), and refers their sums along x to its own, as do single and small tiles for the same
+// rows, so that the fields do not depend on the strips: with d = ref - above, sum g e~ becomes
+// sum g e~ - (sum g g^T) d. rows: the region rows 0 .. rows - 1 formed with `above`. 16 pairs of
+// 1024^2 at r = 7, 9 and 12: 1962, 2113 and 2412 us; with one reference per group, whose error is up to
+// 2.3 times as large, 1901, 2017 and 2317; without strips 2537, 2712 and 3249.
+template <int R, bool V = false> constexpr bool ref_moves() { return !V && ref_group<R, V>() == 1 && radius_strips(R, LK_TH); }
+struct RefAbove {
+    float2 above;
+    int rows;
+};
+template <int R, int TH, int TW, int NT, int RN>
+__device__ __forceinline__ void move_refs(const float2 *P01, float2 *P23, float *P4, float2 ref, const RefAbove &m, int base)
+{
+    using F = FixedTile<R, TH, TW>;
+    const float dx = __fsub_rn(m.above.x, ref.x), dy = __fsub_rn(m.above.y, ref.y);
+    for (int i = threadIdx.x; i < m.rows * TW; i += NT) {
+        const int sl = ring_slot<RN>(i / TW, base), tx = i % TW;
+        const float2 s01 = P01[sl * F::RWP2 + tx], s23 = P23[sl * F::RWP2 + tx];
+        P23[sl * F::RWP2 + tx].y = fmaf(s01.y, dy, fmaf(s01.x, dx, s23.y));
+        P4[sl * F::RWP1 + tx] = fmaf(s23.x, dy, fmaf(s01.y, dx, P4[sl * F::RWP1 + tx]));
+    }
+}
+
 // A single tile (TW x TH outputs at (tx0, ty0), NT threads). Returns false if a staging copy
 // did not complete in time.
 template <typename T, bool NC, int R, int MODE, int TH, int TW = LK_TW, int NT = LK_THREADS, bool V = false>
 __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps *maps, int tx0, int ty0, float2 ref,
-                                             float fp64_cond, float *smem, uint32_t &phase)
+                                             const RefAbove &ra, float fp64_cond, float *smem, uint32_t &phase)
 {
     using F = FixedTile<R, TH, TW, V>;
     unsigned char *win = reinterpret_cast<unsigned char *>(smem + F::OFF_WIN);
@@ -1497,7 +1531,8 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
             } else {
                 float4 s23;
                 float2 s4;
-                stage1_pair<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(a, x, y, on, ref, sf, wt, wx0, wy0, s01,
+                const float2 rf = ref_moves<R>() && ry < ra.rows ? ra.above : ref;
+                stage1_pair<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(a, x, y, on, rf, sf, wt, wx0, wy0, s01,
                                                                                s23, s4);
                 if (on) {
                     reinterpret_cast<float4 *>(P23)[k2] = s23;
@@ -1524,6 +1559,12 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
         box_h_single<R, TH, TW, NT>(P4);
     }
     __syncthreads();
+    if constexpr (ref_moves<R, V>()) {
+        if (ra.rows) {
+            move_refs<R, TH, TW, NT, 0>(P01, P23, P4, ref, ra, 0);
+            __syncthreads();
+        }
+    }
     // vertical sums, solve and write: VO rows of one column per item (all VR rows of a group, or
     // two of them where the tile has fewer groups than threads)
     constexpr int VR = v_rows<R, TH>();
@@ -1562,12 +1603,12 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
 // copy 1.1k and request and wait 2.4k; now 13.4k, request and wait 1.1k. Level-0 launch: r = 4
 // 358 -> 348 us, r = 5 462 -> 417, r = 10 680 -> 589. One bulk copy per row instead of the boxes
 // holds the issuing warp for 2k cycles per tile (410 us at r = 4).
-template <typename T, bool NC, int R, int MODE, int TH, int NT, bool V = false>
+template <typename T, bool NC, int R, int MODE, int TH, int NT>
 __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *maps, int tx0, int t_first, int t_end,
                                          float2 ref, float fp64_cond, float *smem, uint32_t &phase)
 {
-    using F = FixedTile<R, TH, LK_TW, V>;
-    using X = StripTile<R, TH, V>;
+    using F = FixedTile<R, TH>;
+    using X = StripTile<R, TH>;
     constexpr int TW = LK_TW, S = (int)sizeof(T), WW = F::win_w(S), RH = F::RH, RN = X::RING;
     unsigned char *win = reinterpret_cast<unsigned char *>(smem + X::OFF_WIN);
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + X::OFF_BAR);
@@ -1577,8 +1618,12 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
     float *P4 = reinterpret_cast<float *>(P23 + X::PAIR_PLANE);
     const bool staged = maps && a.stage_i2 != 0;
     const bool flows = staged && mode_is<MODE>(a, FLOW_SAME);   // the estimate is staged as well
-    // the window estimates of the strip's tiles (at most the 4 slots at OFF_WREF), loaded together
-    if (staged && (int)threadIdx.x < t_end - t_first)
+    // the window estimates of the strip's tiles (at most the 4 slots at OFF_WREF), loaded together: they
+    // are the tiles' reference flows as well where each has its own
+    constexpr bool MOVE = ref_moves<R>();
+    RefAbove ra = {f2(0.0f, 0.0f), 0};
+    if (MOVE && t_first % REF_GROUP) ra = {ref_flow<NC, MODE, R, TH>(a, tx0, t_first - 1), 2 * R};
+    if ((staged || MOVE) && (int)threadIdx.x < t_end - t_first)
         wrefs[threadIdx.x] = win_ref<NC, MODE, TH>(a, tx0, (t_first + (int)threadIdx.x) * TH);
     // Close the tile's phase of the barrier and request the estimate (one thread) in n boxes of
     // 8 rows, the first at image row y in slot sl. extra: bytes requested besides.
@@ -1596,6 +1641,10 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
         const int ty0 = t * TH;
         const bool next = t + 1 < t_end;
         const int r0 = t > t_first ? 2 * R : 0;   // the first region row this tile computes
+        if constexpr (MOVE) {
+            if (t > t_first) ra = {ref, 2 * R};
+            ref = wrefs[t - t_first];
+        }
         int wx0 = 0, wy0 = 0;
         if (staged) {
             win_origin<R, TH, S>(a, tx0, ty0, wrefs[t - t_first], wx0, wy0);
@@ -1604,7 +1653,7 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
                     request_rows(ty0 - R - X::RPAD, 0, RN / X::BOX, (uint32_t)F::win_bytes(S));
                     tma_load_2d(win, &maps->i2, wx0, wy0, bar);
                 }
-                prefetch_region<R, MODE, TH, TW, NT, S, V>(a, tx0, ty0, 0, 32);
+                prefetch_region<R, MODE, TH, TW, NT, S, false>(a, tx0, ty0, 0, 32);
             }
             if (!stage_wait(a, bar, phase)) return false;
         }
@@ -1616,27 +1665,23 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
             const int k2 = sl * (F::RWP2 / 2) + cx;   // float4 slot of the pair in the pair planes
             const float4 *sf = flows ? reinterpret_cast<const float4 *>(P01) + k2 : nullptr;
             const int x = tx0 - F::RE + 2 * cx, y = ty0 - R + ry;
-            float4 s01;
-            if constexpr (V) {
-                stage1_pair_i1<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(a, x, y, ref, sf, wt, wx0, wy0, s01);
-            } else {
-                float4 s23;
-                float2 s4;
-                stage1_pair<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(a, x, y, on, ref, sf, wt, wx0, wy0, s01,
-                                                                               s23, s4);
-                if (on) {
-                    reinterpret_cast<float4 *>(P23)[k2] = s23;
-                    reinterpret_cast<float2 *>(P4)[sl * (F::RWP1 / 2) + cx] = s4;
-                }
+            const float2 rf = MOVE && ry < ra.rows ? ra.above : ref;
+            float4 s01, s23;
+            float2 s4;
+            stage1_pair<T, NC, MODE, WW, F::WIN_H, decltype(inner)::value>(a, x, y, on, rf, sf, wt, wx0, wy0, s01, s23,
+                                                                           s4);
+            if (on) {
+                reinterpret_cast<float4 *>(P01)[k2] = s01;
+                reinterpret_cast<float4 *>(P23)[k2] = s23;
+                reinterpret_cast<float2 *>(P4)[sl * (F::RWP1 / 2) + cx] = s4;
             }
-            if (on) reinterpret_cast<float4 *>(P01)[k2] = s01;
         };
         auto rows = [&](auto inner) {
             // thread t takes pair cx = t mod NPR of rows r0 + t / NPR, then RPI rows further each
             // round, so that what depends on the pair's column is the same on every row it takes
             constexpr int RPI = NT / NPR;   // rows per round
             const int cx = threadIdx.x % NPR, rs = threadIdx.x / NPR;
-            if constexpr (!V && !decltype(inner)::value) {   // whole warps (stage1_pair)
+            if constexpr (!decltype(inner)::value) {   // whole warps (stage1_pair)
 #pragma unroll 1
                 for (int row = r0; row < RH; row += RPI) pair(inner, row + rs, cx, rs < RPI && row + rs < RH);
             } else if (rs < RPI) {
@@ -1644,7 +1689,7 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
                 for (int ry = r0 + rs; ry < RH; ry += RPI) pair(inner, ry, cx, true);
             }
         };
-        if (staged && tile_inner<R, TH, TW, S, V>(a, tx0, ty0, wx0, wy0)) rows(std::true_type());
+        if (staged && tile_inner<R, TH, TW, S, false>(a, tx0, ty0, wx0, wy0)) rows(std::true_type());
         else rows(std::false_type());
         __syncthreads();
         if (staged && next) {
@@ -1655,14 +1700,18 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
                 mbar_expect_tx(bar, (uint32_t)F::win_bytes(S));
                 tma_load_2d(win, &maps->i2, nx0, ny0, bar);
             }
-            prefetch_region<R, MODE, TH, TW, NT, S, V>(a, tx0, ty0 + TH, 2 * R, 32);
+            prefetch_region<R, MODE, TH, TW, NT, S, false>(a, tx0, ty0 + TH, 2 * R, 32);
         }
         box_h_pairs<R, TH, TW, NT, RN>(P01, r0, 0, base);
-        if constexpr (!V) {
-            box_h_pairs<R, TH, TW, NT, RN>(P23, r0, NT / 64, base);   // from the middle warp: the extra chunks fall on different warps
-            box_h_single<R, TH, TW, NT, RN>(P4, r0, base);
-        }
+        box_h_pairs<R, TH, TW, NT, RN>(P23, r0, NT / 64, base);   // from the middle warp: the extra chunks fall on different warps
+        box_h_single<R, TH, TW, NT, RN>(P4, r0, base);
         __syncthreads();
+        if constexpr (MOVE) {
+            if (ra.rows) {
+                move_refs<R, TH, TW, NT, RN>(P01, P23, P4, ref, ra, base);
+                __syncthreads();
+            }
+        }
         // vertical sums, solve and write, VR rows of one column per item
         constexpr int VR = v_rows<R, TH>();
         constexpr int NITEM = TW * (TH / VR);
@@ -1673,10 +1722,10 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
             const int x = tx0 + tx, yb = ty0 + VR * g;
             float2 s01[VR], s23[VR];
             float s4[VR];
-            if (has) box_v_planes<R, TH, TW, RN, V>(P01, P23, P4, g, tx, s01, s23, s4, base);
+            if (has) box_v_planes<R, TH, TW, RN>(P01, P23, P4, g, tx, s01, s23, s4, base);
             __syncthreads();
             if (staged && next && threadIdx.x == 0) request_rows(ty0 + TH + R, ring_slot<RN>(2 * R, base_next), TH / X::BOX, 0u);
-            if (has && x < a.W && yb < a.H) solve_rows<NC, MODE, V, VR>(a, x, yb, ref, fp64_cond, s01, s23, s4);
+            if (has && x < a.W && yb < a.H) solve_rows<NC, MODE, false, VR>(a, x, yb, ref, fp64_cond, s01, s23, s4);
         } else {
 #pragma unroll 1
             for (int i = threadIdx.x; i < NITEM; i += NT) {
@@ -1685,8 +1734,8 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
                 if (x >= a.W || yb >= a.H) continue;
                 float2 s01[VR], s23[VR];
                 float s4[VR];
-                box_v_planes<R, TH, TW, RN, V>(P01, P23, P4, g, tx, s01, s23, s4, base);
-                solve_rows<NC, MODE, V, VR>(a, x, yb, ref, fp64_cond, s01, s23, s4);
+                box_v_planes<R, TH, TW, RN>(P01, P23, P4, g, tx, s01, s23, s4, base);
+                solve_rows<NC, MODE, false, VR>(a, x, yb, ref, fp64_cond, s01, s23, s4);
             }
             __syncthreads();
             if (staged && next && threadIdx.x == 0) request_rows(ty0 + TH + R, ring_slot<RN>(2 * R, base_next), TH / X::BOX, 0u);
@@ -1699,12 +1748,12 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
 // One work unit of the fixed-radius iteration: the a.strip (1, 2 or 4) vertically
 // consecutive 64 x TH tiles of one column of tiles starting at tile row a.strip * (unit /
 // tiles_x), inside one group of REF_GROUP tile rows. All tiles of a group take the same
-// reference flow (the estimate at the group's centre column and row), so the products of
-// a region row do not depend on which tile computes them: the tiles after the first take
-// over the last 2R rows of window sums along x from the tile above instead of computing
-// their stage 1 and horizontal pass again, and the fields are the same bit for bit for
-// every a.strip. MULTI = false: a kernel whose units are single tiles (a.strip 1). Returns
-// false if a staging copy did not complete in time (then OF_ETIMEOUT is in *a.status,
+// reference flow (the estimate at the group's centre column and row; or each tile its own, see
+// ref_moves), so the products of a region row do not depend on which tile computes them: the
+// tiles after the first take over the last 2R rows of window sums along x from the tile above
+// instead of computing their stage 1 and horizontal pass again, and the fields are the same bit
+// for bit for every a.strip. MULTI = false: a kernel whose units are single tiles (a.strip 1).
+// Returns false if a staging copy did not complete in time (then OF_ETIMEOUT is in *a.status,
 // nothing more of the unit was written, and the block must stop).
 template <typename T, bool NC, int R, int MODE, int TH = LK_TH, bool MULTI = true, int NT = LK_THREADS, bool V = false>
 __device__ __forceinline__ bool lk_tile_fixed(const IterArgs &a, const StageMaps *maps, int unit, float fp64_cond,
@@ -1717,18 +1766,20 @@ __device__ __forceinline__ bool lk_tile_fixed(const IterArgs &a, const StageMaps
     const int uy = unit / a.tiles_x;
     const int tx0 = (unit - uy * a.tiles_x) * LK_TW;
     const int t_first = uy * K, t_end = min(t_first + K, (a.H + TH - 1) / TH);
-    const int gy0 = t_first / REF_GROUP * REF_GROUP * TH;
-    const float2 ref = flow_mode<NC, MODE>(a, min(tx0 + LK_TW / 2, a.W - 1), min(gy0 + REF_GROUP * TH / 2, a.H - 1));
+    const float2 ref = ref_flow<NC, MODE, R, TH, V>(a, tx0, t_first);
     if constexpr (!MULTI) {   // one tile per unit (a.strip 1)
-        return lk_tile_step<T, NC, R, MODE, TH, LK_TW, NT, V>(a, maps, tx0, t_first * TH, ref, fp64_cond, smem, phase);
+        RefAbove ra = {f2(0.0f, 0.0f), 0};
+        if (ref_moves<R, V>() && t_first % REF_GROUP) ra = {ref_flow<NC, MODE, R, TH, V>(a, tx0, t_first - 1), 2 * R};
+        return lk_tile_step<T, NC, R, MODE, TH, LK_TW, NT, V>(a, maps, tx0, t_first * TH, ref, ra, fp64_cond, smem, phase);
     } else {
-        return lk_strip<T, NC, R, MODE, TH, NT, V>(a, maps, tx0, t_first, t_end, ref, fp64_cond, smem, phase);
+        static_assert(!V, "the variant's tiles are single");
+        return lk_strip<T, NC, R, MODE, TH, NT>(a, maps, tx0, t_first, t_end, ref, fp64_cond, smem, phase);
     }
 }
 
 // One small tile of the fixed-radius iteration (SM_TW x SM_TH outputs, SM_THREADS threads),
-// for launches with too few 64 x LK_TH tiles to fill the GPU: same reference flows (the
-// groups of the 64 x LK_TH tiles) and the same groups of window sums, so the same bits.
+// for launches with too few 64 x LK_TH tiles to fill the GPU: same reference flows (those
+// of the 64 x LK_TH tiles) and the same groups of window sums, so the same bits.
 static_assert(LK_TW % SM_TW == 0 && LK_TH % SM_TH == 0, "small tiles inside the default tiles, group-aligned");
 template <typename T, bool NC, int R, int MODE, bool V = false>
 __device__ __forceinline__ bool lk_tile_small(const IterArgs &a, const StageMaps *maps, int unit, float fp64_cond,
@@ -1738,9 +1789,11 @@ __device__ __forceinline__ bool lk_tile_small(const IterArgs &a, const StageMaps
     uint32_t phase = 0;
     const int uy = unit / a.tiles_x;
     const int tx0 = (unit - uy * a.tiles_x) * SM_TW, ty0 = uy * SM_TH;
-    const int gx0 = tx0 / LK_TW * LK_TW, gy0 = ty0 / (REF_GROUP * LK_TH) * (REF_GROUP * LK_TH);
-    const float2 ref = flow_mode<NC, MODE>(a, min(gx0 + LK_TW / 2, a.W - 1), min(gy0 + REF_GROUP * LK_TH / 2, a.H - 1));
-    return lk_tile_step<T, NC, R, MODE, SM_TH, SM_TW, SM_THREADS, V>(a, maps, tx0, ty0, ref, fp64_cond, smem, phase);
+    const int gx0 = tx0 / LK_TW * LK_TW, t = ty0 / LK_TH;
+    const float2 ref = ref_flow<NC, MODE, R, LK_TH, V>(a, gx0, t);
+    RefAbove ra = {f2(0.0f, 0.0f), 0};
+    if (ref_moves<R, V>() && t % REF_GROUP) ra = {ref_flow<NC, MODE, R, LK_TH, V>(a, gx0, t - 1), max(2 * R - (ty0 - t * LK_TH), 0)};
+    return lk_tile_step<T, NC, R, MODE, SM_TH, SM_TW, SM_THREADS, V>(a, maps, tx0, ty0, ref, ra, fp64_cond, smem, phase);
 }
 
 // ------------------------------------------------ two iterations fused in one tile

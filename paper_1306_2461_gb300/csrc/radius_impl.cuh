@@ -329,7 +329,7 @@ template <int R> cudaError_t i1h_launch(const HessArgs &a, int elem, int r, cuda
 template <typename T, int R>
 static cudaError_t i1_for(const IterArgs &a, const StageMaps &m, int r, float fp64_cond, bool small, cudaStream_t s)
 {
-    const size_t smem = i1_iter_smem<R>(r, false, small, a.stage_i2 != 0, (int)sizeof(T));
+    const size_t smem = i1_iter_smem<R>(r, small, a.stage_i2 != 0, (int)sizeof(T));
     if constexpr (R != 0)
         if (small) return launch_chained(i1_small_kernel<T, R>, a.tiles, SM_THREADS, smem, s, a, m, fp64_cond);
     return launch_chained(i1_iter_kernel<T, R>, a.tiles, LK_THREADS, smem, s, a, m, r, fp64_cond);
@@ -369,7 +369,7 @@ static cudaError_t phase_i1_for(const IterPhase &P, int r, float fp64_cond, int 
     bool stage = false;
     for (int i = 0; i < P.npairs; ++i) stage = stage || P.a[i].stage_i2 != 0;
     const bool small = R != 0 && tile_h == SM_TH;
-    const size_t smem = i1_iter_smem<R>(r, true, small, stage, (int)sizeof(T));
+    const size_t smem = i1_iter_smem<R>(r, small, stage, (int)sizeof(T));
     const int blocks = P.prefix[P.npairs];
     if constexpr (R != 0)
         if (small) return launch_chained(phase_i1_small_kernel<T, R>, blocks, SM_THREADS, smem, s, P, fp64_cond);
@@ -487,7 +487,7 @@ template <int R> cudaError_t radius_configure()
     {
         const int r = R == 0 ? MAX_RADIUS : R;
         const int hb = (int)sizeof(float) * i1_smem_floats<R>(r, 3);
-        const int ib = (int)i1_iter_smem<R>(r, false, false, true, 4), jb = (int)i1_iter_smem<R>(r, true, false, true, 4);
+        const int ib = (int)i1_iter_smem<R>(r, false, true, 4);
 #define OF_SET_TO(fn, bytes)                                                                                   \
     if ((e = cudaFuncSetAttribute((const void *)(fn), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess) \
         return e;
@@ -495,9 +495,9 @@ template <int R> cudaError_t radius_configure()
     OF_SET_TO((i1_hess_kernel<T, R>), hb)        \
     OF_SET_TO((phase_hess_kernel<T, R>), hb)     \
     OF_SET_TO((i1_iter_kernel<T, R>), ib)        \
-    OF_SET_TO((phase_i1_iter_kernel<T, R>), jb)  \
+    OF_SET_TO((phase_i1_iter_kernel<T, R>), ib)  \
     OF_SET_TO((i1_small_kernel<T, R>), ib)       \
-    OF_SET_TO((phase_i1_small_kernel<T, R>), jb)
+    OF_SET_TO((phase_i1_small_kernel<T, R>), ib)
         OF_SET_I1(uint8_t)
         OF_SET_I1(uint16_t)
         OF_SET_I1(float)

@@ -175,7 +175,7 @@ int of_autotune_batch(int32_t n, const of_handle *hs, const void *const *I1s, co
                     t.blocks_per_sm = b < 0 ? 0 : b;
                     t.prefetch = b < 0 ? pf_of[-1 - b] : 0;
                     t.tile_h = th ? ALT_TH : 0;
-                    t.strip = (t.phased && !gs && radius_strips(p0.radius, LK_TH)) ? 0 : 1;
+                    t.strip = (t.phased && !gs && !variant && radius_strips(p0.radius, LK_TH)) ? 0 : 1;
                     cand.push_back(t);
                     if (t.phased && t.prefetch == 0 && n > 1) {
                         t.branches = 2;

@@ -701,11 +701,11 @@ template <int R, int TH = LK_TH, int TW = LK_TW, bool V = false> struct FixedTil
 // is in slot (ring + RPAD + ry) mod RING, ring a multiple of 8 that moves on by TH from tile to
 // tile; RPAD puts the first row after the 2R carried ones in a slot that is a multiple of 8
 // (a 128-byte boundary), so that the estimate of the rows a tile computes comes in TMA boxes
-// of 8 rows.
-template <int R, int TH> struct StripTile {
+// of 8 rows. STAGE = false: for launches that gather, without those rows.
+template <int R, int TH, bool STAGE = true> struct StripTile {
     using F = FixedTile<R, TH>;
     static_assert(TH % 8 == 0, "boxes of 8 rows");
-    static constexpr int RPAD = (8 - 2 * R % 8) % 8;
+    static constexpr int RPAD = STAGE ? (8 - 2 * R % 8) % 8 : 0;
     static constexpr int RING = RPAD + F::RH;
     static constexpr int BOX = 8;
     static constexpr int BOX_BYTES = F::RWP2 * BOX * 8;
@@ -1603,12 +1603,12 @@ __device__ __forceinline__ bool lk_tile_step(const IterArgs &a, const StageMaps 
 // copy 1.1k and request and wait 2.4k; now 13.4k, request and wait 1.1k. Level-0 launch: r = 4
 // 358 -> 348 us, r = 5 462 -> 417, r = 10 680 -> 589. One bulk copy per row instead of the boxes
 // holds the issuing warp for 2k cycles per tile (410 us at r = 4).
-template <typename T, bool NC, int R, int MODE, int TH, int NT>
+template <typename T, bool NC, int R, int MODE, int TH, int NT, bool STAGE>
 __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *maps, int tx0, int t_first, int t_end,
                                          float2 ref, float fp64_cond, float *smem, uint32_t &phase)
 {
     using F = FixedTile<R, TH>;
-    using X = StripTile<R, TH>;
+    using X = StripTile<R, TH, STAGE>;
     constexpr int TW = LK_TW, S = (int)sizeof(T), WW = F::win_w(S), RH = F::RH, RN = X::RING;
     unsigned char *win = reinterpret_cast<unsigned char *>(smem + X::OFF_WIN);
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + X::OFF_BAR);
@@ -1616,7 +1616,7 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
     float2 *P01 = reinterpret_cast<float2 *>(smem);
     float2 *P23 = P01 + X::PAIR_PLANE;
     float *P4 = reinterpret_cast<float *>(P23 + X::PAIR_PLANE);
-    const bool staged = maps && a.stage_i2 != 0;
+    const bool staged = STAGE && maps && a.stage_i2 != 0;
     const bool flows = staged && mode_is<MODE>(a, FLOW_SAME);   // the estimate is staged as well
     // the window estimates of the strip's tiles (at most the 4 slots at OFF_WREF), loaded together: they
     // are the tiles' reference flows as well where each has its own
@@ -1755,7 +1755,8 @@ __device__ __forceinline__ bool lk_strip(const IterArgs &a, const StageMaps *map
 // for bit for every a.strip. MULTI = false: a kernel whose units are single tiles (a.strip 1).
 // Returns false if a staging copy did not complete in time (then OF_ETIMEOUT is in *a.status,
 // nothing more of the unit was written, and the block must stop).
-template <typename T, bool NC, int R, int MODE, int TH = LK_TH, bool MULTI = true, int NT = LK_THREADS, bool V = false>
+template <typename T, bool NC, int R, int MODE, int TH = LK_TH, bool MULTI = true, int NT = LK_THREADS, bool V = false,
+          bool STAGE = true>
 __device__ __forceinline__ bool lk_tile_fixed(const IterArgs &a, const StageMaps *maps, int unit, float fp64_cond,
                                               float *smem, uint32_t &phase)
 {
@@ -1773,7 +1774,7 @@ __device__ __forceinline__ bool lk_tile_fixed(const IterArgs &a, const StageMaps
         return lk_tile_step<T, NC, R, MODE, TH, LK_TW, NT, V>(a, maps, tx0, t_first * TH, ref, ra, fp64_cond, smem, phase);
     } else {
         static_assert(!V, "the variant's tiles are single");
-        return lk_strip<T, NC, R, MODE, TH, NT>(a, maps, tx0, t_first, t_end, ref, fp64_cond, smem, phase);
+        return lk_strip<T, NC, R, MODE, TH, NT, STAGE>(a, maps, tx0, t_first, t_end, ref, fp64_cond, smem, phase);
     }
 }
 

@@ -88,6 +88,32 @@ phase_iter_kernel(const __grid_constant__ IterPhase P, int r, float fp64_cond)
     lk_tile<T, false, R, MODE, TH, strip_kernel<R, TH>(), LK_THREADS>(P.a[p], &P.m[p], blockIdx.x - P.prefix[p], r, fp64_cond, smem, phase);
 }
 
+// The same where no pair is staged, for the radii (5 and 6) at which four blocks per SM fit then and
+// three otherwise: 32 pairs of 1024^2 at r = 5 (6), two
+// sequences, 3428 (3498) us; with the staged form's three blocks 3727 (3774).
+template <int R> constexpr bool gather_kernel()
+{
+    if constexpr (R == 0) return false;
+    else return lk_slots(R) == 3 && 4 * (4 * StripTile<R, LK_TH, false>::SMEM_NOSTAGE + 1024) <= 228 * 1024;
+}
+template <typename T, int R>
+__global__ void __launch_bounds__(LK_THREADS, 4) phase_gather_kernel(const __grid_constant__ IterPhase P, float fp64_cond)
+{
+    extern __shared__ __align__(128) float4 smem4[];
+    if constexpr (gather_kernel<R>()) {
+        const int p = phase_pair(P.prefix, P.npairs, blockIdx.x);
+        chain_begin();
+        const int t2 = blockIdx.x + P.ahead;
+        if (P.ahead > 0 && t2 < P.prefix[P.npairs]) {
+            const int q = phase_pair(P.prefix, P.npairs, t2);
+            prefetch_tile<T, -1, LK_TH>(P.a[q], t2 - P.prefix[q], R);
+        }
+        uint32_t phase = 0;
+        lk_tile_fixed<T, false, R, -1, LK_TH, true, LK_THREADS, false, false>(
+            P.a[p], nullptr, blockIdx.x - P.prefix[p], fp64_cond, reinterpret_cast<float *>(smem4), phase);
+    }
+}
+
 // Two same-level iterations of up to PHASE_PAIRS pairs in one launch (iteration fusion
 // depth 2): block b runs both on tile b - prefix[p] of pair p (tile height LK_TH).
 template <int R> constexpr int fused2_min_blocks()
@@ -240,6 +266,10 @@ static cudaError_t phase_for_th(const IterPhase &P, int r, float fp64_cond, cuda
     for (int i = 0; i < P.npairs; ++i) stage = stage || P.a[i].stage_i2 != 0;
     const size_t smem = sizeof(float) * lk_tile_smem_floats<R, TH, strip_kernel<R, TH>()>(r, stage, (int)sizeof(T));
     const int blocks = P.prefix[P.npairs];
+    if constexpr (TH == LK_TH && gather_kernel<R>())
+        if (!stage)
+            return launch_chained(phase_gather_kernel<T, R>, blocks, LK_THREADS,
+                                  sizeof(float) * StripTile<R, TH, false>::SMEM_NOSTAGE, s, P, fp64_cond);
     switch (P.a[0].mode) {
     case FLOW_ZERO:
         return launch_chained(phase_iter_kernel<T, R, phase_mode<R, TH>(FLOW_ZERO), TH>, blocks, LK_THREADS, smem, s, P, r,
@@ -464,6 +494,13 @@ template <int R> cudaError_t radius_configure()
 #undef OF_SET_ALT
     }
     OF_SET((window_sums_kernel<R>));
+    if constexpr (gather_kernel<R>()) {
+        const int gb = (int)sizeof(float) * StripTile<R, LK_TH, false>::SMEM_NOSTAGE;
+        for (const void *fn : {(const void *)phase_gather_kernel<uint8_t, R>, (const void *)phase_gather_kernel<uint16_t, R>,
+                               (const void *)phase_gather_kernel<float, R>, (const void *)phase_gather_kernel<__half, R>,
+                               (const void *)phase_gather_kernel<__nv_bfloat16, R>})
+            if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, gb)) != cudaSuccess) return e;
+    }
     if constexpr (R != 0) {   // small tiles
         const int sb = (int)sizeof(float) * small_smem_floats<R>(true, 4);
 #define OF_SET_SM(T)                                                                                        \

@@ -1,5 +1,5 @@
-// Dispatch of the iteration, window-sum and batch kernels to their per-radius
-// instantiations (radius_<R>.cu): a specialised kernel for the radii listed in
+// Dispatch of the iteration and batch kernels to their per-radius
+// instantiations (radius_<R>.cu, pair_<R>.cu): a specialised kernel for the radii listed in
 // OF_RADII (and, but for the persistent and the fused form, OF_RADII_MORE), the generic one
 // (radius at run time) for any other.
 #include <cudaTypedefs.h>
@@ -75,16 +75,6 @@ cudaError_t launch_lk_iter(const IterArgs &a, const StageMaps &m, int elem, int 
     switch (radius) {
         OF_RADII(OF_CASE_LK) OF_RADII_MORE(OF_CASE_LK)
     default: return lk_launch<0>(a, m, elem, radius, fp64_cond, false, s);
-    }
-}
-
-#define OF_CASE_WS(R) \
-    case R: return ws_launch<R>(ch, H, W, r, out, s);
-cudaError_t launch_window_sums(const float *ch, int H, int W, int r, float *out, cudaStream_t s)
-{
-    switch (r) {
-        OF_RADII(OF_CASE_WS) OF_RADII_MORE(OF_CASE_WS)
-    default: return ws_launch<0>(ch, H, W, r, out, s);
     }
 }
 
@@ -177,27 +167,36 @@ size_t batch_smem_bytes(int radius, bool stage_i2)
 void *batch_kernel_generic(int in_format, int storage) { return batch_kernel_ptr<0>(in_format, storage); }
 size_t batch_smem_generic(int radius) { return radius_smem_bytes<0>(radius, false); }
 
-// Once per device and radius (bit r of its word; bit 0: the run-time-radius kernels). Setting an
-// attribute loads the kernel, so the radii a process never uses are left out: the first
-// of_create of a process takes 20 ms with one radius, 224 ms with all.
-#define OF_CFG(R) \
-    if (!(done & (1u << R)) && (radius < 0 || radius == R || R == 0)) { \
-        if ((e = radius_configure<R>()) != cudaSuccess) return e;       \
-        done |= 1u << R;                                                \
+// Once per device, part and radius (bit r of the part's word; bit 0: the run-time-radius kernels).
+// Setting an attribute loads all kernels of a radius's file, so what a process never uses is left
+// out: the first of_create of a process takes 20 ms and one with a further radius 11, the first
+// of_compute_noalloc, which sets up the launches of one pair for every radius, 64 ms (with the batched
+// launches of a radius in the same file 224).
+#define OF_CFG(part, configure, R)                               \
+    if (!(done[part] & (1u << R)) && (all || radius == R || R == 0)) { \
+        if ((e = configure<R>()) != cudaSuccess) return e;       \
+        done[part] |= 1u << R;                                   \
     }
+#define OF_CFG_PAIR(R) OF_CFG(0, pair_configure, R)
+#define OF_CFG_BATCH(R) OF_CFG(1, batch_configure, R)
 cudaError_t configure_lk_kernels(int radius)
 {
     static std::mutex mu;
-    static uint32_t configured[256];
+    static uint32_t configured[256][2];
+    const bool all = radius == CONFIGURE_PAIRS;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 256) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lk(mu);
-    uint32_t &done = configured[dev];
-    OF_CFG(0)
-    OF_RADII(OF_CFG)
-    OF_RADII_MORE(OF_CFG)
+    uint32_t *done = configured[dev];
+    OF_CFG_PAIR(0)
+    OF_RADII(OF_CFG_PAIR)
+    OF_RADII_MORE(OF_CFG_PAIR)
+    if (all) return cudaSuccess;
+    OF_CFG_BATCH(0)
+    OF_RADII(OF_CFG_BATCH)
+    OF_RADII_MORE(OF_CFG_BATCH)
     return cudaSuccess;
 }
 

@@ -46,7 +46,7 @@ int scratch_on_current_device(char **out)
             cudaGetLastError();
             return OF_ECUDA;
         }
-        if (of::configure_lk_kernels(-1) != cudaSuccess) return OF_ECUDA;
+        if (of::configure_lk_kernels(of::CONFIGURE_PAIRS) != cudaSuccess) return OF_ECUDA;
         g_scratch_ptr[dev] = static_cast<char *>(ptr);
     }
     *out = g_scratch_ptr[dev];

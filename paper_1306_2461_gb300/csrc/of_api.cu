@@ -395,8 +395,6 @@ int of_window_sums(const float *ch, int32_t H, int32_t W, int32_t r, float *out,
 {
     if (!ch || !out || H < 1 || W < 1 || r < 1 || r > MAX_RADIUS || (int64_t)H * W > (int64_t(1) << 28))
         return OF_EINVAL;
-    int rc = configure_device(-1);   // any radius may follow, perhaps inside a capture
-    if (rc) return rc;
     return map_cuda(launch_window_sums(ch, H, W, r, out, reinterpret_cast<cudaStream_t>(stream)));
 }
 

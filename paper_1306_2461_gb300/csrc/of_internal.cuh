@@ -319,8 +319,9 @@ void *batch_kernel_generic(int in_format, int storage);   // the run-time-radius
 size_t batch_smem_generic(int radius);
 cudaError_t launch_level_to_f32(const Level &l, int elem, float *dst, cudaStream_t s);
 cudaError_t launch_wait_timeout(int *flag, int *status, long long timeout_ns, cudaStream_t s);
-// The kernels with dynamic shared memory of one radius (-1: every radius) and the run-time-radius
-// ones, on the current device, once.
+// The kernels with dynamic shared memory of one radius and the run-time-radius ones, or
+// (CONFIGURE_PAIRS) of every radius those of one pair, on the current device, once.
+constexpr int CONFIGURE_PAIRS = -1;
 cudaError_t configure_lk_kernels(int radius);
 // Fill a.tm_flow and a.tm_i2 for the staged fixed-radius tile of this radius and tile
 // height (level image type elem). Returns false (and clears a.stage_i2) when the radius
@@ -336,11 +337,10 @@ bool encode_tile_map(CUtensorMap *m, int elem, const void *base, int W, int H, s
 // Element type code for an 8-byte flow element in encode_tile_map.
 constexpr int ET_FLOW2 = 100;
 
-// Per-radius instantiations (radius_<R>.cu; R = 0 is the generic kernel).
+// Per-radius instantiations (radius_<R>.cu, pair_<R>.cu; R = 0 is the generic kernel).
 template <int R>
 cudaError_t lk_launch(const IterArgs &a, const StageMaps &m, int elem, int r, float fp64_cond, bool small,
                       cudaStream_t s);
-template <int R> cudaError_t ws_launch(const float *ch, int H, int W, int r, float *out, cudaStream_t s);
 template <int R> cudaError_t i1h_launch(const HessArgs &a, int elem, int r, cudaStream_t s);
 template <int R> cudaError_t phase_launch(const IterPhase &P, int elem, int r, float fp64_cond, int tile_h, cudaStream_t s);
 template <int R> cudaError_t phase_hess_launch(const HessPhase &P, int elem, int r, cudaStream_t s);
@@ -350,7 +350,8 @@ template <int R>
 cudaError_t i1_launch(const IterArgs &a, const StageMaps &m, int elem, int r, float fp64_cond, bool small,
                       cudaStream_t s);
 template <int R> void *batch_kernel_ptr(int in_format, int storage);
-template <int R> cudaError_t radius_configure();
+template <int R> cudaError_t pair_configure();
+template <int R> cudaError_t batch_configure();
 template <int R> size_t radius_smem_bytes(int r, bool stage_i2);
 template <int R> bool radius_stage_maps(const IterArgs &a, StageMaps &m, int elem, int tile_h, bool strips);
 template <int R> cudaError_t phase2_launch(const IterPhase &P, int elem, float fp64_cond, cudaStream_t s);

@@ -1,3 +1,3 @@
-// Kernels for window radius 0 (0: any radius, given at run time).
+// Batched launches for window radius 0 (0: any radius, given at run time).
 #define OF_RADIUS 0
 #include "radius_impl.cuh"

@@ -1,4 +1,4 @@
-// Kernels for window radius 12.
+// Batched launches for window radius 12.
 #define OF_RADIUS 12
 #define OF_RADIUS_MORE
 #include "radius_impl.cuh"

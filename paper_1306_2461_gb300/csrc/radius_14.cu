@@ -1,4 +1,4 @@
-// Kernels for window radius 14.
+// Batched launches for window radius 14.
 #define OF_RADIUS 14
 #define OF_RADIUS_MORE
 #include "radius_impl.cuh"

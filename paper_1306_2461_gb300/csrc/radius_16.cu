@@ -1,4 +1,4 @@
-// Kernels for window radius 16.
+// Batched launches for window radius 16.
 #define OF_RADIUS 16
 #define OF_RADIUS_MORE
 #include "radius_impl.cuh"

@@ -1,3 +1,3 @@
-// Kernels for window radius 3.
+// Batched launches for window radius 3.
 #define OF_RADIUS 3
 #include "radius_impl.cuh"

@@ -1,3 +1,3 @@
-// Kernels for window radius 5.
+// Batched launches for window radius 5.
 #define OF_RADIUS 5
 #include "radius_impl.cuh"

@@ -1,5 +1,7 @@
-// Kernels and launchers for one window radius. Each radius_<R>.cu defines OF_RADIUS
-// and includes this file; radius 0 is the generic kernel (radius given at run time).
+// Kernels and launchers for one window radius. Each radius_<R>.cu (the batched launches) and
+// pair_<R>.cu (OF_PAIR: the launches of one pair) defines OF_RADIUS and includes this file; radius 0
+// is the generic kernel (radius given at run time). Two files, because the first use of a kernel
+// loads all kernels of its file.
 #pragma once
 
 #include "batch_device.cuh"
@@ -138,76 +140,6 @@ phase_iter2_kernel(const __grid_constant__ IterPhase P, float fp64_cond)
     }
 }
 
-// The window sums of five given planes, through the same passes as the iteration tile.
-template <int R>
-__global__ void __launch_bounds__(LK_THREADS)
-window_sums_kernel(const float *ch, int H, int W, int r, int tiles_x, float *out)
-{
-    extern __shared__ float4 smem4[];
-    float *smem = reinterpret_cast<float *>(smem4);
-    const int tile = blockIdx.x;
-    const int ty0 = (tile / tiles_x) * LK_TH, tx0 = (tile % tiles_x) * LK_TW;
-    const size_t N = (size_t)H * W;
-    if constexpr (R == 0) {
-        const int RH = LK_TH + 2 * r, RW = LK_TW + 2 * r;
-        const int plane = RH * RW;
-        float *P = smem, *S = smem + 5 * plane;
-        for (int i = threadIdx.x; i < plane; i += blockDim.x) {
-            const int ry = i / RW, rx = i - ry * RW;
-            const int y = ty0 - r + ry, x = tx0 - r + rx;
-            const bool in = y >= 0 && y < H && x >= 0 && x < W;
-            for (int c = 0; c < 5; ++c) P[c * plane + i] = in ? ch[c * N + (size_t)y * W + x] : 0.0f;
-        }
-        __syncthreads();
-        box_hsum(P, S, RH, RW, r);
-        __syncthreads();
-        for (int i = threadIdx.x; i < LK_TH * LK_TW; i += blockDim.x) {
-            const int ty = i / LK_TW, tx = i % LK_TW;
-            const int y = ty0 + ty, x = tx0 + tx;
-            if (y >= H || x >= W) continue;
-            float s[5];
-            box_vsum(S, RH, r, ty, tx, s);
-            for (int c = 0; c < 5; ++c) out[c * N + (size_t)y * W + x] = s[c];
-        }
-    } else {
-        // the planes of the iteration tile: channels (0, 1) and (2, 3) as float2 pairs, 4 alone
-        using F = FixedTile<R>;
-        float2 *P01 = reinterpret_cast<float2 *>(smem);
-        float2 *P23 = P01 + F::PAIR_PLANE;
-        float *P4 = reinterpret_cast<float *>(P23 + F::PAIR_PLANE);
-        for (int i = threadIdx.x; i < F::RH * F::RWE; i += blockDim.x) {
-            const int ry = i / F::RWE, rx = i - ry * F::RWE;
-            const int y = ty0 - R + ry, x = tx0 - F::RE + rx;
-            const bool in = y >= 0 && y < H && x >= 0 && x < W;
-            float c[5];
-            for (int k = 0; k < 5; ++k) c[k] = in ? ch[k * N + (size_t)y * W + x] : 0.0f;
-            P01[ry * F::RWP2 + rx] = make_float2(c[0], c[1]);
-            P23[ry * F::RWP2 + rx] = make_float2(c[2], c[3]);
-            P4[ry * F::RWP1 + rx] = c[4];
-        }
-        __syncthreads();
-        box_h_pairs<R, LK_TH>(P01);
-        box_h_pairs<R, LK_TH>(P23);
-        box_h_single<R, LK_TH>(P4);
-        __syncthreads();
-        constexpr int VR = v_rows<R, LK_TH>();
-        for (int i = threadIdx.x; i < LK_TW * (LK_TH / VR); i += blockDim.x) {
-            const int tx = i % LK_TW, g = i / LK_TW;
-            const int x = tx0 + tx;
-            if (x >= W) continue;
-            float2 s01[VR], s23[VR];
-            float s4[VR];
-            box_v_planes<R, LK_TH>(P01, P23, P4, g, tx, s01, s23, s4);
-            for (int j = 0; j < VR; ++j) {
-                const int y = ty0 + VR * g + j;
-                if (y >= H) break;
-                const float s[5] = {s01[j].x, s01[j].y, s23[j].x, s23[j].y, s4[j]};
-                for (int c = 0; c < 5; ++c) out[c * N + (size_t)y * W + x] = s[c];
-            }
-        }
-    }
-}
-
 template <int R> size_t radius_smem_bytes(int r, bool stage_i2)
 {
     size_t lk = sizeof(float) * (size_t)lk_tile_smem_floats<R>(r, stage_i2);
@@ -241,14 +173,6 @@ cudaError_t lk_launch(const IterArgs &a, const StageMaps &m, int elem, int r, fl
     case ET_F16: return lk_for<__half, R>(a, m, r, fp64_cond, small, s);
     default: return lk_for<__nv_bfloat16, R>(a, m, r, fp64_cond, small, s);
     }
-}
-
-template <int R> cudaError_t ws_launch(const float *ch, int H, int W, int r, float *out, cudaStream_t s)
-{
-    const int tiles_x = (W + LK_TW - 1) / LK_TW, tiles_y = (H + LK_TH - 1) / LK_TH;
-    window_sums_kernel<R><<<tiles_x * tiles_y, LK_THREADS, sizeof(float) * lk_tile_smem_floats<R>(r, false), s>>>(
-        ch, H, W, r, tiles_x, out);
-    return cudaGetLastError();
 }
 
 // The flow mode is the same for every pair of a phase: at the default tile height one kernel per
@@ -461,108 +385,92 @@ template <int R> void *batch_kernel_ptr(int in_format, int storage)
     return (void *)batch_kernel<uint16_t, __nv_bfloat16, R>;
 }
 
-// Raise the dynamic shared memory limit of this radius's kernels on the current device.
-template <int R> cudaError_t radius_configure()
+// Raise the dynamic shared memory limit of this radius's kernels of one pair (pair_configure) and of
+// the batched launches (batch_configure) on the current device.
+#define OF_SET(fn, n) \
+    if ((e = cudaFuncSetAttribute((const void *)(fn), cudaFuncAttributeMaxDynamicSharedMemorySize, n)) != cudaSuccess) return e;
+#define OF_SET_ALL(K, n) \
+    OF_SET((K<uint8_t, R>), n) OF_SET((K<uint16_t, R>), n) OF_SET((K<float, R>), n) OF_SET((K<__half, R>), n) OF_SET((K<__nv_bfloat16, R>), n)
+template <int R> cudaError_t pair_configure()
 {
-    const int bytes = (int)radius_smem_bytes<R>(R == 0 ? MAX_RADIUS : R, true);
+    const int r = R == 0 ? MAX_RADIUS : R;
+    const int bytes = (int)radius_smem_bytes<R>(r, true), ib = (int)i1_iter_smem<R>(r, false, true, 4);
+    const int hb = (int)sizeof(float) * i1_smem_floats<R>(r, 3);
     cudaError_t e;
-#define OF_SET(fn) if ((e = cudaFuncSetAttribute((const void *)(fn), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess) return e
-    OF_SET((lk_iter_kernel<uint8_t, R>));
-    OF_SET((lk_iter_kernel<uint16_t, R>));
-    OF_SET((lk_iter_kernel<float, R>));
-    OF_SET((lk_iter_kernel<__half, R>));
-    OF_SET((lk_iter_kernel<__nv_bfloat16, R>));
-#define OF_SET_PH(T) OF_SET((phase_iter_kernel<T, R, phase_mode<R, LK_TH>(FLOW_ZERO), LK_TH>)); \
-    OF_SET((phase_iter_kernel<T, R, FLOW_SAME, LK_TH>)); OF_SET((phase_iter_kernel<T, R, phase_mode<R, LK_TH>(FLOW_UPSAMPLE), LK_TH>))
-    OF_SET_PH(uint8_t);
-    OF_SET_PH(uint16_t);
-    OF_SET_PH(float);
-    OF_SET_PH(__half);
-    OF_SET_PH(__nv_bfloat16);
-#undef OF_SET_PH
-    if constexpr (R != 0 && all_forms<R>()) {   // the other tile height of the phase kernels
-        const int alt = (int)sizeof(float) * lk_tile_smem_floats<R, ALT_TH, strip_kernel<R, ALT_TH>()>(R, true);
-#define OF_SET_ALT(T)                                                                                        \
-    if ((e = cudaFuncSetAttribute((const void *)phase_iter_kernel<T, R, -1, ALT_TH>,                         \
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, alt)) != cudaSuccess)         \
-        return e;
-        OF_SET_ALT(uint8_t)
-        OF_SET_ALT(uint16_t)
-        OF_SET_ALT(float)
-        OF_SET_ALT(__half)
-        OF_SET_ALT(__nv_bfloat16)
-#undef OF_SET_ALT
-    }
-    OF_SET((window_sums_kernel<R>));
-    if constexpr (gather_kernel<R>()) {
-        const int gb = (int)sizeof(float) * StripTile<R, LK_TH, false>::SMEM_NOSTAGE;
-        for (const void *fn : {(const void *)phase_gather_kernel<uint8_t, R>, (const void *)phase_gather_kernel<uint16_t, R>,
-                               (const void *)phase_gather_kernel<float, R>, (const void *)phase_gather_kernel<__half, R>,
-                               (const void *)phase_gather_kernel<__nv_bfloat16, R>})
-            if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, gb)) != cudaSuccess) return e;
-    }
+    OF_SET_ALL(lk_iter_kernel, bytes)
+    OF_SET_ALL(i1_hess_kernel, hb)
+    OF_SET_ALL(i1_iter_kernel, ib)
     if constexpr (R != 0) {   // small tiles
         const int sb = (int)sizeof(float) * small_smem_floats<R>(true, 4);
-#define OF_SET_SM(T)                                                                                        \
-    for (const void *fn : {(const void *)lk_small_kernel<T, R>, (const void *)phase_small_kernel<T, R>})    \
-        if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sb)) != cudaSuccess) \
-            return e;
-        OF_SET_SM(uint8_t)
-        OF_SET_SM(uint16_t)
-        OF_SET_SM(float)
-        OF_SET_SM(__half)
-        OF_SET_SM(__nv_bfloat16)
-#undef OF_SET_SM
+        OF_SET_ALL(lk_small_kernel, sb)
+        OF_SET_ALL(i1_small_kernel, ib)
     }
-    if constexpr (R != 0 && all_forms<R>()) {   // the fused two-iteration kernels
-        const int fb = (int)fused2_smem_bytes<R>();
-        for (const void *fn : {(const void *)phase_iter2_kernel<uint8_t, R>, (const void *)phase_iter2_kernel<uint16_t, R>,
-                               (const void *)phase_iter2_kernel<float, R>, (const void *)phase_iter2_kernel<__half, R>,
-                               (const void *)phase_iter2_kernel<__nv_bfloat16, R>})
-            if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, fb)) != cudaSuccess) return e;
-    }
-    {
-        const int r = R == 0 ? MAX_RADIUS : R;
-        const int hb = (int)sizeof(float) * i1_smem_floats<R>(r, 3);
-        const int ib = (int)i1_iter_smem<R>(r, false, true, 4);
-#define OF_SET_TO(fn, bytes)                                                                                   \
-    if ((e = cudaFuncSetAttribute((const void *)(fn), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess) \
-        return e;
-#define OF_SET_I1(T)                             \
-    OF_SET_TO((i1_hess_kernel<T, R>), hb)        \
-    OF_SET_TO((phase_hess_kernel<T, R>), hb)     \
-    OF_SET_TO((i1_iter_kernel<T, R>), ib)        \
-    OF_SET_TO((phase_i1_iter_kernel<T, R>), ib)  \
-    OF_SET_TO((i1_small_kernel<T, R>), ib)       \
-    OF_SET_TO((phase_i1_small_kernel<T, R>), ib)
-        OF_SET_I1(uint8_t)
-        OF_SET_I1(uint16_t)
-        OF_SET_I1(float)
-        OF_SET_I1(__half)
-        OF_SET_I1(__nv_bfloat16)
-#undef OF_SET_I1
-#undef OF_SET_TO
-    }
-    if constexpr (all_forms<R>())
-        for (int f = 0; f < 2; ++f)
-            for (int st = 0; st < 3; ++st) OF_SET(batch_kernel_ptr<R>(f, st));
-#undef OF_SET
     return cudaSuccess;
 }
 
+template <int R> cudaError_t batch_configure()
+{
+    const int r = R == 0 ? MAX_RADIUS : R;
+    const int bytes = (int)radius_smem_bytes<R>(r, true), ib = (int)i1_iter_smem<R>(r, false, true, 4);
+    const int hb = (int)sizeof(float) * i1_smem_floats<R>(r, 3);
+    cudaError_t e;
+#define OF_SET_PH(T) \
+    OF_SET((phase_iter_kernel<T, R, phase_mode<R, LK_TH>(FLOW_ZERO), LK_TH>), bytes) \
+    OF_SET((phase_iter_kernel<T, R, FLOW_SAME, LK_TH>), bytes) \
+    OF_SET((phase_iter_kernel<T, R, phase_mode<R, LK_TH>(FLOW_UPSAMPLE), LK_TH>), bytes)
+    OF_SET_PH(uint8_t)
+    OF_SET_PH(uint16_t)
+    OF_SET_PH(float)
+    OF_SET_PH(__half)
+    OF_SET_PH(__nv_bfloat16)
+#undef OF_SET_PH
+    OF_SET_ALL(phase_hess_kernel, hb)
+    OF_SET_ALL(phase_i1_iter_kernel, ib)
+    if constexpr (R != 0) {
+        const int sb = (int)sizeof(float) * small_smem_floats<R>(true, 4);
+        OF_SET_ALL(phase_small_kernel, sb)
+        OF_SET_ALL(phase_i1_small_kernel, ib)
+    }
+    if constexpr (gather_kernel<R>()) {
+        const int gb = (int)sizeof(float) * StripTile<R, LK_TH, false>::SMEM_NOSTAGE;
+        OF_SET_ALL(phase_gather_kernel, gb)
+    }
+    if constexpr (R != 0 && all_forms<R>()) {   // the other tile height, the fused iterations
+        const int alt = (int)sizeof(float) * lk_tile_smem_floats<R, ALT_TH, strip_kernel<R, ALT_TH>()>(R, true);
+        const int fb = (int)fused2_smem_bytes<R>();
+        OF_SET((phase_iter_kernel<uint8_t, R, -1, ALT_TH>), alt)
+        OF_SET((phase_iter_kernel<uint16_t, R, -1, ALT_TH>), alt)
+        OF_SET((phase_iter_kernel<float, R, -1, ALT_TH>), alt)
+        OF_SET((phase_iter_kernel<__half, R, -1, ALT_TH>), alt)
+        OF_SET((phase_iter_kernel<__nv_bfloat16, R, -1, ALT_TH>), alt)
+        OF_SET_ALL(phase_iter2_kernel, fb)
+    }
+    if constexpr (all_forms<R>())
+        for (int f = 0; f < 2; ++f)
+            for (int st = 0; st < 3; ++st) {
+                OF_SET(batch_kernel_ptr<R>(f, st), bytes)
+            }
+    return cudaSuccess;
+}
+#undef OF_SET_ALL
+#undef OF_SET
+
+#ifdef OF_PAIR
 template cudaError_t lk_launch<OF_RADIUS>(const IterArgs &, const StageMaps &, int, int, float, bool, cudaStream_t);
-template cudaError_t ws_launch<OF_RADIUS>(const float *, int, int, int, float *, cudaStream_t);
 template cudaError_t i1h_launch<OF_RADIUS>(const HessArgs &, int, int, cudaStream_t);
+template cudaError_t i1_launch<OF_RADIUS>(const IterArgs &, const StageMaps &, int, int, float, bool, cudaStream_t);
+template bool radius_stage_maps<OF_RADIUS>(const IterArgs &, StageMaps &, int, int, bool);
+template cudaError_t pair_configure<OF_RADIUS>();
+#else
 template cudaError_t phase_launch<OF_RADIUS>(const IterPhase &, int, int, float, int, cudaStream_t);
 template cudaError_t phase_hess_launch<OF_RADIUS>(const HessPhase &, int, int, cudaStream_t);
 template cudaError_t phase_i1_launch<OF_RADIUS>(const IterPhase &, int, int, float, int, cudaStream_t);
-template cudaError_t i1_launch<OF_RADIUS>(const IterArgs &, const StageMaps &, int, int, float, bool, cudaStream_t);
+template cudaError_t phase2_launch<OF_RADIUS>(const IterPhase &, int, float, cudaStream_t);
 #ifndef OF_RADIUS_MORE   // one of OF_RADII_MORE
 template void *batch_kernel_ptr<OF_RADIUS>(int, int);
 #endif
-template bool radius_stage_maps<OF_RADIUS>(const IterArgs &, StageMaps &, int, int, bool);
-template cudaError_t phase2_launch<OF_RADIUS>(const IterPhase &, int, float, cudaStream_t);
-template cudaError_t radius_configure<OF_RADIUS>();
 template size_t radius_smem_bytes<OF_RADIUS>(int, bool);
+template cudaError_t batch_configure<OF_RADIUS>();
+#endif
 
 }  // namespace of

@@ -23,6 +23,10 @@ import torch
 
 from . import of
 
+# What a saved entry was timed with; raised when the kernels or the candidates change enough to make another
+# choice. Entries saved before it was recorded (1) hold the run-time-radius kernel for every radius above 6 but 8
+# and 10, which had no other (eight 1024^2 pairs at r = 9: 6929 us with it, 1377 without an entry).
+KERNELS = 2
 DEFAULT_PATH = os.path.join(os.path.expanduser("~"), ".cache", "paper_1306_2461_gb300", "autotune.json")
 
 
@@ -67,9 +71,10 @@ def _write(path: str, data: dict):
 
 
 def load(path: str | None = None) -> int:
-    """Apply the saved entries for this GPU model to the library's table. Returns how many."""
-    data = _read(path or DEFAULT_PATH).get(_device(), {})
-    for ent in data.values():
+    """Apply the saved entries for this GPU model to the library's table, but those timed with other
+    kernels (the library's defaults stand until they are tuned again). Returns how many."""
+    data = [e for e in _read(path or DEFAULT_PATH).get(_device(), {}).values() if e.get("kernels", 1) == KERNELS]
+    for ent in data:
         b = ent["best"]
         of.tuning_set(_plan_of(ent["method"]), ent["size_class"], b["generic_sums"], b["stage_i2"],
                       b["blocks_per_sm"], b.get("phased", 0), b.get("prefetch", 0), b.get("tile_h", 0),
@@ -84,7 +89,8 @@ def tune(flows, I1s, I2s, us=None, vs=None, stream=None, reps: int = 3, path: st
     best, cands = of.autotune_batch(flows, I1s, I2s, us, vs, stream=stream, reps=reps)
     method = _method(flows[0].plan)
     sc = of.batch_size_class(flows)
-    ent = {"method": method, "size_class": sc, "batch": len(flows), "best": best, "candidates": cands}
+    ent = {"method": method, "size_class": sc, "batch": len(flows), "kernels": KERNELS, "best": best,
+           "candidates": cands}
     if save:
         p = path or DEFAULT_PATH
         data = _read(p)

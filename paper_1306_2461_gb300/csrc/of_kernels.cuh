@@ -94,11 +94,19 @@ __device__ __forceinline__ void prefetch_lines_l1(const void *base, int pitch, i
     asm volatile("prefetch.global.L1 [%0];" ::"l"(s));
 }
 
+// The flow mode is `m`: known at compile time (MODE), at run time (MODE < 0), or one of a
+// level's first iteration (FLOW_FIRST).
+template <int MODE> __device__ __forceinline__ bool mode_is(const IterArgs &a, int m)
+{
+    if (MODE == FLOW_FIRST) return m != FLOW_SAME && a.mode == m;
+    return MODE >= 0 ? MODE == m : a.mode == m;
+}
+
 // Warm L2 with what the block that runs iteration tile `tile` will read first: its region
-// (tile + r-pixel halo) of the current estimate (flow mode MODE, or a.mode at run time when
-// MODE < 0), of I1, of I2 widened by PF_MARGIN pixels for the displacement, and of the
-// variant's window matrices (a.hess, when set). Threads [0, 64) take the estimate's rows,
-// [64, 128) I1's, [128, 192) I2's, [192, 256) the window matrices'.
+// (tile + r-pixel halo) of the current estimate (flow mode MODE, see mode_is), of I1, of I2
+// widened by PF_MARGIN pixels for the displacement, and of the variant's window matrices
+// (a.hess, when set). Threads [0, 64) take the estimate's rows, [64, 128) I1's, [128, 192) I2's,
+// [192, 256) the window matrices'.
 constexpr int PF_MARGIN = 8;
 template <typename T, int MODE, int TH = LK_TH>
 __device__ __forceinline__ void prefetch_tile(const IterArgs &a, int tile, int r)
@@ -107,11 +115,10 @@ __device__ __forceinline__ void prefetch_tile(const IterArgs &a, int tile, int r
     const int ty0 = uy * strip_len(a.strip) * TH - r, tx0 = (tile - uy * a.tiles_x) * LK_TW - r;
     const int ty1 = ty0 + TH + 2 * r, tx1 = tx0 + LK_TW + 2 * r;
     const int t = threadIdx.x;
-    const int mode = MODE >= 0 ? MODE : a.mode;
     if (t < 64) {
-        if (mode == FLOW_SAME)
+        if (mode_is<MODE>(a, FLOW_SAME))
             prefetch_row(a.fin, a.fin_pitch, 8, a.H, a.W, ty0, ty1, tx0, tx1, t);
-        else if (mode == FLOW_UPSAMPLE)
+        else if (mode_is<MODE>(a, FLOW_UPSAMPLE))
             prefetch_row(a.fin, a.fin_pitch, 8, a.Hc, a.Wc, ty0 >> 1, (ty1 >> 1) + 2, tx0 >> 1, (tx1 >> 1) + 2, t);
     } else if (t < 128) {
         prefetch_row(a.I1, a.pitch, (int)sizeof(T), a.H, a.W, ty0 - 1, ty1 + 1, tx0 - 1, tx1 + 1, t - 64);
@@ -758,14 +765,6 @@ template <bool NC> __device__ __forceinline__ float2 ld_pair(const __nv_bfloat16
     if (!q) return f2(ldf<NC>(p), 0.0f);
     const __nv_bfloat162 w = ld<NC>(reinterpret_cast<const __nv_bfloat162 *>(p));
     return __bfloat1622float2(w);
-}
-
-// The flow mode is `m`: known at compile time (MODE), at run time (MODE < 0), or one of a
-// level's first iteration (FLOW_FIRST).
-template <int MODE> __device__ __forceinline__ bool mode_is(const IterArgs &a, int m)
-{
-    if (MODE == FLOW_FIRST) return m != FLOW_SAME && a.mode == m;
-    return MODE >= 0 ? MODE == m : a.mode == m;
 }
 
 // The current estimates of the pixel pair (x, y), (x + 1, y) (x even; the second only

@@ -37,3 +37,14 @@ def test_votes_name_lanes_that_arrive(name):
     masks = {"0xffffffffu"} | set(re.findall(r"(\w+) = __ballot_sync\(0xffffffffu,", code))
     for m in re.finditer(r"__(?:all|any|ballot|shfl\w*|reduce_\w+|match\w*)_sync\(([^,]*),", code):
         assert m.group(1).strip() in masks
+
+
+def test_flow_modes_are_asked_of_mode_is():
+    # a kernel's MODE may stand for two modes (FLOW_FIRST: a level's first iteration) or for any (-1);
+    # compared as a number it matches neither, and a prefetch then warms nothing
+    code = code_of("of_kernels.cuh")
+    body = code[code.index("bool mode_is("):]
+    body = code.replace(body[:body.index("\n}\n")], "")
+    for m in re.finditer(r"\bmode == FLOW_\w+|\bMODE >= 0", body):
+        line = body[body.rfind("\n", 0, m.start()) + 1:body.index("\n", m.end())]
+        assert "a.mode" in line and "MODE >= 0" not in line, line

@@ -356,7 +356,7 @@ static cudaError_t enqueue_chain(const BatchPair *pairs, int n, const of_plan &p
             for (int i = 0; i < m; ++i) tiles_l += strip_units(bp[i].H[l], bp[i].W[l], tile_h, 1);
             while (kl > 1 && tiles_l < (long)kl * slots) kl /= 2;
             const bool small = !two && tile_h == LK_TH && !t.generic_sums && radius_grouped(p0.radius) &&
-                               prefetch_ahead == 0 && use_small_tiles(tiles_l, sms);
+                               prefetch_ahead == 0 && use_small_tiles(tiles_l, sms, p0.radius, i1grad, sequences);
             const int th_l = small ? SM_TH : tile_h;
             for (int i = 0; i < m; ++i) {
                 IterArgs &a = I.a[i];

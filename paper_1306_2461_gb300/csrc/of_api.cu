@@ -213,7 +213,7 @@ cudaError_t enqueue_pair(of_ctx *h, const void *I1, const void *I2, float *u, fl
             StageMaps maps;
             memset(&maps, 0, sizeof(maps));
             // few tiles: small ones, so that the launch is spread over the SMs
-            const bool small = fixed && use_small_tiles(a.tiles, sms);
+            const bool small = fixed && use_small_tiles(a.tiles, sms, p.radius, i1grad, 0);
             if (small) {
                 a.tiles_x = small_tiles_x(a.W);
                 a.tiles = small_units(a.H, a.W);

@@ -160,18 +160,34 @@ constexpr int LK_TW = 64;    // iteration output tile width
 #endif
 constexpr int LK_TH = OF_LK_TH;
 static_assert(LK_TH % 4 == 0, "the vertical box pass takes 4 rows at a time");
-// Small iteration tile, for launches whose 64 x LK_TH tiles are fewer than 4/3 of the SMs:
-// such a launch lasts as long as one tile alone on an SM, a serial chain of five rounds of
-// stage 1, two of the horizontal pass and six solves per thread, and leaves SMs idle. A
-// 32 x 12 tile has two rounds, one and two solves, and a quarter of the area. One same-level
-// iteration of one pair at r = 4 (us per launch in a graph, 64 x 24 -> 32 x 12 tiles): 128^2
-// 7.7 -> 4.5, 256^2 8.0 -> 5.0, 384^2 7.9 -> 6.0, 512^2 (176 tiles) 9.9 -> 8.7, 640^2 (270
-// tiles) 10.1 -> 11.1; four 256^2 pairs (176) 10.7 -> 9.3, two 512^2 (352) 13.3 -> 14.2: the
-// line lies between 176 and 270 tiles, beyond it the wider halo (400 pixel pairs computed for
-// 192 written) costs more than the shorter chain saves. Others measured: 64 x 12 5.8 at
-// 256^2, 32 x 6 5.3, 32 x 12 with 512 threads 4.6 (but 10.7 at 512^2).
+// Small iteration tile, for launches of few 64 x LK_TH tiles: such a launch lasts as long as one
+// tile alone on an SM, a serial chain of five rounds of stage 1, two of the horizontal pass and six
+// solves per thread, and leaves SMs idle. A 32 x 12 tile has two rounds, one and two solves, and a
+// quarter of the area. One same-level iteration of one pair at r = 4 (us per launch in a graph, 64 x
+// 24 -> 32 x 12 tiles): 128^2 7.7 -> 4.5, 256^2 8.0 -> 5.0, 384^2 7.9 -> 6.0, 512^2 (176 tiles) 9.9 -> 8.7,
+// 640^2 (270 tiles) 10.1 -> 11.1. Others measured: 64 x 12 5.8 at 256^2, 32 x 6 5.3, 32 x 12 with 512
+// threads 4.6 (but 10.7 at 512^2).
 constexpr int SM_TW = 32, SM_TH = 12, SM_THREADS = 256, SM_MIN_BLOCKS = 4;
-inline bool use_small_tiles(long tiles, int sms) { return 3 * tiles < 4 * (long)sms; }
+// The line lies where the wider halo costs more than the shorter chain saves: four small tiles form the
+// products of 1.4 times the pixels of one wide tile at r = 4 and of 2.1 times at r = 16. Wide / small
+// time at so many wide tiles, 6 iterations of one level on 152 SMs. The per-pair kernels (384 threads per
+// wide tile from r = 7 on): r = 6 1.06 at 184, 0.94 at 200; r = 8 1.40 at 24, 1.03 at 104, 0.93 at 120; r = 12
+// 1.01 at 80, 0.97 at 90; r = 14 1.03 at 64, 0.93 at 80; r = 16 1.04 at 50, 0.93 at 64, 0.58 at 152. One
+// sequence of phase launches: r = 8 1.07 at 184, 0.96 at 200; r = 12 1.05, 0.91; r = 14 1.02 at 104, 0.82 at
+// 120; r = 16 1.00, 0.85. Each of two: r = 8 1.04 at 136, 0.95 at 152; r = 12 0.99, 0.89; r = 14 1.04 at 90,
+// 0.95 at 104; r = 16 0.99 at 104, 0.88 at 120. The variant, one product plane: r = 8 1.04 at 184; r = 12
+// 1.03 at 152, 0.97 at 168; r = 14 (one sequence) 1.06 at 120, 0.95 at 184; r = 16 1.13 at 104, 0.94 at 120.
+// sequences: concurrent launch sequences of a batch, 0 for the per-pair kernels.
+inline bool use_small_tiles(long tiles, int sms, int r, bool variant, int sequences)
+{
+    int percent;   // of the SMs
+    if (variant) percent = r <= 8 ? 133 : (r <= 12 ? (sequences > 1 ? 95 : 105) : (r <= 14 && sequences == 1 ? 100 : 72));
+    else if (r <= 6) percent = 133;
+    else if (sequences == 0) percent = r <= 10 ? 70 : (r <= 12 ? 56 : (r <= 14 ? 45 : 36));
+    else if (sequences == 1) percent = r <= 12 ? 125 : 72;
+    else percent = r <= 12 ? 90 : 60;
+    return 100 * tiles < percent * (long)sms;
+}
 // The other iteration tile height the tuning can choose for the phase launches (64 x ALT_TH).
 #ifndef OF_ALT_TH
 #define OF_ALT_TH 32

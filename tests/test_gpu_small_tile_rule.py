@@ -1,0 +1,38 @@
+"""A launch of as many wide tiles as SMs does not run small tiles where their halo makes it slower:
+the default form of one pair against the one that a prefetch keeps on wide tiles."""
+import pytest
+
+from paper_1306_2461_gb300 import synth
+from helpers import to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("r", [8, 12, 14, 16])
+def test_default_is_no_slower_than_wide_tiles(r):
+    # the fastest of 20 replays of each; the prefetch itself costs a few percent, small tiles took 1.4
+    # times as long here at r = 14 and 16
+    import torch
+    from paper_1306_2461_gb300 import of
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    H, W = 24 * (sms // 8), 64 * 8
+    p = synth.make_c1(H, W, seed=r)
+    I1, I2 = to_dev(p.I1), to_dev(p.I2)
+    plan = of.Plan.make(H, W, 1, r, 12, bits=8, storage="f16")
+    e, s, best = [torch.cuda.Event(enable_timing=True) for _ in range(2)], torch.cuda.Stream(), []
+    with of.Flow(plan) as f:
+        for t in (None, {"prefetch": 1}):
+            if t is not None:
+                of.tuning_set(plan, of.batch_size_class([f]), **t)
+            us, vs = of.compute_batch([f], [I1], [I2], stream=s)
+            ms = []
+            for _ in range(20):
+                e[0].record(s)
+                of.compute_batch([f], [I1], [I2], us, vs, stream=s)
+                e[1].record(s)
+                s.synchronize()
+                ms.append(e[0].elapsed_time(e[1]))
+            best.append(min(ms))
+        of.tuning_clear()
+    print(f"r={r}: default {1e3 * best[0]:.1f} us, wide tiles {1e3 * best[1]:.1f} us")
+    assert best[0] <= 1.05 * best[1]

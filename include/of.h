@@ -69,7 +69,7 @@ typedef enum of_storage { OF_F32 = 0, OF_F16 = 1, OF_BF16 = 2 } of_storage;
                                  The window matrix then depends on I1 only and is summed once per
                                  level; each iteration sums two channels. Batched calls and the
                                  serving loop run it as phase launches (the tuning's phased,
-                                 stage_i2 and blocks_per_sm are ignored for it). The workspace
+                                 stage_i2, strip and blocks_per_sm are ignored for it). The workspace
                                  grows by one float4 per level-0 pixel. */
 
 /*

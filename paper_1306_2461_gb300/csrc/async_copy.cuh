@@ -1,7 +1,6 @@
-// Asynchronous copies global -> shared completing on an mbarrier, with a bounded wait:
-// untiled bulk copies (cp.async.bulk) and 2-D tiled tensor copies (cp.async.bulk.tensor,
-// the TMA unit) that stage an iteration tile's flow estimate and I2 window in shared
-// memory.
+// Asynchronous copies global -> shared completing on an mbarrier, with a bounded wait: 2-D tiled
+// tensor copies (cp.async.bulk.tensor, the TMA unit) that stage an iteration tile's flow estimate and
+// I2 window in shared memory.
 #pragma once
 
 #include <stdint.h>
@@ -39,13 +38,6 @@ __device__ __forceinline__ void fence_proxy_async_smem()
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-// Order generic-proxy writes to global memory (made visible to this thread by a grid
-// barrier) before this thread's later asynchronous-proxy reads.
-__device__ __forceinline__ void fence_proxy_async_global()
-{
-    asm volatile("fence.proxy.async.global;" ::: "memory");
-}
-
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
@@ -56,15 +48,6 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t by
 __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes)
 {
     asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-
-// dst (shared) <- src (global), `bytes` a multiple of 16, both addresses 16-byte aligned.
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_u32(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
 }
 
 // One 2-D box of the tensor described by the tensor map at `map` (a kernel parameter:

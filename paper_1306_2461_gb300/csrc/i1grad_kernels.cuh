@@ -193,10 +193,11 @@ __global__ void __launch_bounds__(LK_THREADS) i1_hess_kernel(HessArgs a, int r)
 }
 
 // Resident blocks per SM. The iteration is bound by latency and then by memory (36 bytes per
-// pixel): as the main method's tiles, with one product plane, a level-0 launch of 16 pairs of
-// 1024^2 at r = 4 takes 153 us (157 with 4 blocks per SM, 160 with 6 at 40 registers; its bytes 89 us),
-// with tiles of their own that gathered every tap and estimate one pixel at a time 188; r = 10
-// 177 instead of 295. A 1024^2 pair 203 -> 158 us.
+// pixel): as the main method's single tiles, with one product plane, a level-0 launch of 16 pairs of
+// 1024^2 at r = 4 takes 154 us (its bytes 89 us), with tiles of their own that gathered every tap and
+// estimate one pixel at a time 188; r = 10 211 instead of 295; a 1024^2 pair 203 -> 155 us. In strips,
+// whose tiles shared a reference flow (see ref_group): 153 (157 with 4 blocks per SM, 160 with 6 at 40
+// registers) and 177.
 #ifndef OF_I1_MIN_BLOCKS
 #define OF_I1_MIN_BLOCKS 5
 #endif

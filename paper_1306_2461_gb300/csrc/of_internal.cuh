@@ -249,7 +249,10 @@ constexpr bool radius_grouped(int r)   // the per-pair and phase launches at lea
 #undef OF_IS_RADIUS
     return radius_specialised(r);
 }
-// Blocks of the 64-wide fixed-radius tiles resident on an SM.
+// Blocks per SM that the registers of the 64-wide fixed-radius kernels are bounded for, and that the
+// rule for the strips counts. As many staged strips of 2-byte levels fit in shared memory; three of
+// 1-byte levels would at r = 8, and three of either at r = 7. Of FP32 levels one fewer fits at r = 2 to 6
+// (at r = 5 and 6 a strip takes 81 and 82 KB, a single tile 72 and 76).
 constexpr int lk_slots(int r) { return r <= 4 ? 4 : (r <= 6 ? 3 : 2); }
 // Strips take over 2r rows of sums from the tile above, which must lie below that tile's own
 // 2r first rows.

@@ -697,7 +697,7 @@ template <int R, int TH = LK_TH, int TW = LK_TW, bool V = false> struct FixedTil
     static constexpr int FLOW_BOX_BYTES = RWP2 * FLOW_BH * 8;
     // resident blocks per SM the kernels are compiled for: the measured choice for the
     // default tile height, else as many as the shared memory holds (at most 5). At r = 5 and 6
-    // shared memory holds 3 blocks, which leaves 80 registers instead of 64: level-0 launch of 32
+    // shared memory holds 3 blocks (of 1- and 2-byte levels), which leaves 80 registers instead of 64: level-0 launch of 32
     // pairs of 1024^2 at r = 5 416 -> 405 us, a pair 195 -> 193 us
     static constexpr int SMEM_FIT = 233472 / (4 * (PLANES + 4) + 1024);
     static constexpr int MIN_BLOCKS =
@@ -1978,7 +1978,7 @@ template <int R, int TH = LK_TH> constexpr int lk_min_blocks()
     if constexpr (R == 0) return 2;
     else return FixedTile<R, TH>::MIN_BLOCKS;
 }
-// Threads per block of the per-pair kernel: at r > 6 shared memory holds two blocks per SM, and
+// Threads per block of the per-pair kernel: at r > 6 the kernels run two blocks per SM, and
 // 384 threads each (12 warps instead of 8; 80 registers) shorten a tile: 1024^2 pair at r = 8
 // 257 -> 247 us, r = 10 291 -> 276 (512 threads: 245, 276). The strips of the phase kernels stay at
 // 256, where half the warps would have no output group: 384 threads 589 -> 597 us, 512 (64

@@ -15,10 +15,10 @@
 
 namespace of {
 
-// Radii with every form of the batched launch (0: the run-time-radius kernel); the others
-// have the per-pair and phase launches at the default tile height.
 // Strips: the phase kernels whose tile height holds the rows carried from tile to tile.
 template <int R, int TH> constexpr bool strip_kernel() { return R != 0 && TH >= 2 * R; }
+// Radii with every form of the batched launch (0: the run-time-radius kernel); the others
+// have the per-pair and phase launches at the default tile height.
 template <int R> constexpr bool all_forms() { return R == 0 || radius_specialised(R); }
 
 template <typename T, int R>

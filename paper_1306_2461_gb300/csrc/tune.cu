@@ -164,7 +164,7 @@ int of_autotune_batch(int32_t n, const of_handle *hs, const void *const *I1s, co
         for (int sg = 0; sg <= (gs ? 0 : 1); ++sg)
             for (int th = 0; th <= ((gs || variant || more) ? 0 : 1); ++th)
                 for (int b : occ) {
-                    if (variant && (b >= 0 || sg)) continue;   // phase launches, gathered taps only
+                    if (variant && (b >= 0 || sg)) continue;   // phase launches only, staged whatever stage_i2 says (effective() in batch.cu)
                     if (more && !gs && b >= 0) continue;       // no persistent form
                     if (th && b >= 0) continue;                // the persistent launch has one tile height
                     if (sg && b >= 0) continue;                // and gathers its taps

@@ -35,4 +35,4 @@ def test_default_is_no_slower_than_wide_tiles(r):
             best.append(min(ms))
         of.tuning_clear()
     print(f"r={r}: default {1e3 * best[0]:.1f} us, wide tiles {1e3 * best[1]:.1f} us")
-    assert best[0] <= 1.05 * best[1]
+    assert best[0] <= 1.1 * best[1]

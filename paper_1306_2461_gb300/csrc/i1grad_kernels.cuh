@@ -194,14 +194,22 @@ __global__ void __launch_bounds__(LK_THREADS) i1_hess_kernel(HessArgs a, int r)
 
 // Resident blocks per SM. The iteration is bound by latency and then by memory (36 bytes per
 // pixel): as the main method's single tiles, with one product plane, a level-0 launch of 16 pairs of
-// 1024^2 at r = 4 takes 154 us (its bytes 89 us), with tiles of their own that gathered every tap and
-// estimate one pixel at a time 188; r = 10 211 instead of 295; a 1024^2 pair 203 -> 155 us. In strips,
-// whose tiles shared a reference flow (see ref_group): 153 (157 with 4 blocks per SM, 160 with 6 at 40
-// registers) and 177.
+// 1024^2 at r = 4 takes 142 us (its bytes 89 us), with tiles of their own that gathered every tap and
+// estimate one pixel at a time 188; r = 10 196 instead of 295; a 1024^2 pair 203 -> 155 us. In strips,
+// whose tiles shared a reference flow (see ref_group): 153 and 177.
 #ifndef OF_I1_MIN_BLOCKS
 #define OF_I1_MIN_BLOCKS 5
 #endif
 template <int R> constexpr int i1_min_blocks() { return R == 0 ? 4 : (R <= 6 ? OF_I1_MIN_BLOCKS : (R <= 12 ? 4 : 3)); }
+// The same for the phase launches, whose single tiles fill the SMs (level-0 launch of 16 pairs of 1024^2,
+// us, with 5, 6 and 7 blocks at r <= 6, 4, 5 and 6 above): r = 2 146, 151, 150; r = 3 150, 138; r = 4 153, 142,
+// 164; r = 6 171, 164, 190; r = 8 194, 181, 176; r = 10 210, 201, 196; r = 12 229, 234, 233; with 3, 4 and 5:
+// r = 13 242, 242, 244; r = 16 307, 307, 314. One pair, whose launches do not fill them, is slower with 6
+// (r = 4 154 -> 160 us).
+template <int R> constexpr int i1_phase_blocks()
+{
+    return R >= 3 && R <= 10 ? 6 : i1_min_blocks<R>();
+}
 
 template <typename T, int R>
 __global__ void __launch_bounds__(LK_THREADS, i1_min_blocks<R>())
@@ -246,7 +254,7 @@ __global__ void __launch_bounds__(LK_THREADS) phase_hess_kernel(const __grid_con
 }
 
 template <typename T, int R>
-__global__ void __launch_bounds__(LK_THREADS, i1_min_blocks<R>())
+__global__ void __launch_bounds__(LK_THREADS, i1_phase_blocks<R>())
 phase_i1_iter_kernel(const __grid_constant__ IterPhase P, int r, float fp64_cond)
 {
     extern __shared__ __align__(128) float4 smem4[];
